@@ -46,11 +46,7 @@ struct BatchArgs {
   const int64_t *walk_off;  // prefix of N_tot over the batch, k+1 entries
   int32_t k;
   int64_t total_walks;
-  const int32_t *row_ptr;
-  const int32_t *col;
-  const uint32_t *adj;
-  const int32_t *npos;
-  int32_t pos_bits;
+  GraphView view;
   uint32_t key0, key1;
   uint32_t shared_key;  // walk key of the shared target walks
   uint4 *M;       // shared walks: M[(i-1) Jmax + j] (.x, .y) bit b = pair j of batch
@@ -91,12 +87,12 @@ __device__ __forceinline__ int find_source(const int64_t *off, int k, int64_t g)
 template <int kLayout>
 __global__ void __launch_bounds__(256) kb_source_walks(const __grid_constant__ BatchArgs A) {
   const RoundKeys rk = round_keys(A.key0, A.key1);
-  const auto G = adj_view<kLayout>(A.adj, A.npos, A.pos_bits, A.row_ptr, A.col);
+  const auto G = adj_view<kLayout>(A.view);
   SRK_BATCH_LOOP(A, {
     const QueryTab &t = *S_.tab;
     const uint32_t s = (uint32_t)S_.s;
     uint32_t deg_s = 0;
-    const int32_t b_s = node_start(G, A.row_ptr, S_.s, deg_s);
+    const int32_t b_s = node_start(G, A.view.row_ptr, S_.s, deg_s);
     const int Ls = S_.L > 0 ? S_.L : 1;
     S_.w.grp_cnt[r_] = 0;
     S_.w.kdraw[r_] = (r_ >= 1) ? fy_draw(rk, s, r_) : 0;
@@ -270,7 +266,7 @@ kb_target_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__
   extern __shared__ int32_t rows[];
   __shared__ PairSet ctx[kBlock / 32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const auto G = adj_view<kLayout>(A.adj, A.npos, A.pos_bits, A.row_ptr, A.col);
+  const auto G = adj_view<kLayout>(A.view);
   int2 *my_rc = reinterpret_cast<int2 *>(rows + (2 * wib) * row_words);
   const int64_t n_items = (int64_t)(*n_act_src_p) * n_act;
   const int64_t limit = item_limit < n_items ? item_limit : n_items;
@@ -308,7 +304,7 @@ kb_target_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__
     uint32_t c = 0, st = 0;
     unsigned long long W = 0;
     uint32_t deg_u = 0;
-    const int32_t b_u = node_start(G, A.row_ptr, u, deg_u);
+    const int32_t b_u = node_start(G, A.view.row_ptr, u, deg_u);
     walk_target(G, ctx[wib], (uint32_t)u, b_u, deg_u, c, W, st);
     for (int off = 16; off > 0; off >>= 1) {
       c += __shfl_xor_sync(0xffffffffu, c, off);
@@ -461,7 +457,7 @@ kb_shared_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__
   __syncthreads();
   const uint32_t key = A.shared_key;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const auto G = adj_view<kLayout>(A.adj, A.npos, A.pos_bits, A.row_ptr, A.col);
+  const auto G = adj_view<kLayout>(A.view);
   const uint4 *M = A.M;
   const int32_t J = A.Jmax;
   const int tbits = A.tbits;
@@ -484,7 +480,7 @@ kb_shared_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__
     wsum[wib][lane + 32] = 0ull;
     if (lane == 0) {
       uint32_t deg_u = 0;
-      w_base[wib] = node_start(G, A.row_ptr, (int32_t)u, deg_u);
+      w_base[wib] = node_start(G, A.view.row_ptr, (int32_t)u, deg_u);
       w_deg[wib] = deg_u;
       w_excl[wib] = excl;
     }
@@ -954,11 +950,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     A.walk_off = d_off;
     A.k = kb;
     A.total_walks = hoff[(size_t)kb];
-    A.row_ptr = g->row_ptr;
-    A.col = g->col;
-    A.adj = g->adj;
-    A.npos = g->npos;
-    A.pos_bits = g->pos_bits;
+    A.view = view_of(g);
     A.key0 = (uint32_t)seed;
     A.key1 = (uint32_t)(seed >> 32);
     A.shared_key = walk_key(seed, kSharedWalkKey);

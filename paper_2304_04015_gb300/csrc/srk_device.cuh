@@ -168,27 +168,17 @@ __host__ __device__ __forceinline__ Small small_view(int32_t *base) {
 //   entry_next(G, e, x, deg): base (returned) and degree of that node x;
 //   node_start(G, row_ptr, v, deg): base and degree of node v, by id.
 
-// The packed adjacency with 4-byte entries: node v's identity is its position
-// pos[v]; a node of degree d < dmax has the word d there and its list right
-// after it; a hub (d >= dmax) has {d, list offset} at an even position of the
-// hub region; entry k of a list is (min(|I(y)|, dmax) << pb) | pos[y].
+// The packed adjacency with 4-byte entries (srk_internal.h): entry =
+// (code << pb) | rank; the list of rank x begins at ctab[code] + x code, a
+// hub's (code = dmax) where its record says.
 struct Adj {
   const uint32_t *adj;
   const int32_t *pos;
+  const uint2 *hub;
+  const uint32_t *ctab;
   int pb;
   uint32_t pmask, dmax;
 };
-
-__host__ __device__ __forceinline__ Adj make_adj(const uint32_t *adj, const int32_t *pos,
-                                                 int pb) {
-  Adj a;
-  a.adj = adj;
-  a.pos = pos;
-  a.pb = pb;
-  a.pmask = (uint32_t)((1ull << pb) - 1ull);
-  a.dmax = (uint32_t)((1ull << (32 - pb)) - 1ull);
-  return a;
-}
 
 __device__ __forceinline__ uint32_t adj_entry(const Adj &G, int32_t base, uint32_t k) {
   return G.adj[base + (int32_t)k];
@@ -196,24 +186,23 @@ __device__ __forceinline__ uint32_t adj_entry(const Adj &G, int32_t base, uint32
 __device__ __forceinline__ int32_t entry_pos(const Adj &G, uint32_t e) {
   return (int32_t)(e & G.pmask);
 }
-// The degree comes with the entry unless x is a hub; a hub's two header
-// words are read together (its position is even).
+// The degree comes with the entry unless x is a hub.
 __device__ __forceinline__ int32_t entry_next(const Adj &G, uint32_t e, int32_t x,
                                               uint32_t &deg) {
   const uint32_t code = e >> G.pb;
   if (code < G.dmax) {
     deg = code;
-    return x + 1;
+    return (int32_t)(G.ctab[code] + (uint32_t)x * code);
   }
-  const uint2 h = *reinterpret_cast<const uint2 *>(G.adj + x);
+  const uint2 h = G.hub[x];
   deg = h.x;
   return (int32_t)h.y;
 }
-__device__ __forceinline__ int32_t node_start(const Adj &G, const int32_t *, int32_t v,
+__device__ __forceinline__ int32_t node_start(const Adj &G, const int32_t *row_ptr, int32_t v,
                                               uint32_t &deg) {
   const int32_t x = G.pos[v];
-  deg = G.adj[x];
-  return deg < G.dmax ? x + 1 : (int32_t)G.adj[x + 1];
+  deg = (uint32_t)(row_ptr[v + 1] - row_ptr[v]);
+  return deg < G.dmax ? (int32_t)(G.ctab[deg] + (uint32_t)x * deg) : (int32_t)G.hub[x].y;
 }
 
 // The wide packed adjacency, for graphs whose positions need more than 28
@@ -225,11 +214,6 @@ struct AdjW {
   const uint2 *adj;
 };
 
-__host__ __device__ __forceinline__ AdjW make_adjw(const uint32_t *words) {
-  AdjW a;
-  a.adj = reinterpret_cast<const uint2 *>(words);
-  return a;
-}
 __device__ __forceinline__ uint2 adj_entry(const AdjW &G, int32_t base, uint32_t k) {
   return G.adj[base + (int32_t)k];
 }
@@ -274,11 +258,17 @@ constexpr int kNarrow = 0, kWide = 1, kCsr = 2;
 
 // The view of a graph's adjacency in layout kLayout.
 template <int kLayout>
-__device__ __forceinline__ auto adj_view(const uint32_t *words, const int32_t *pos, int pb,
-                                         const int32_t *row_ptr, const int32_t *col) {
-  if constexpr (kLayout == kWide) return make_adjw(words);
-  else if constexpr (kLayout == kCsr) return AdjC{row_ptr, col};
-  else return make_adj(words, pos, pb);
+__device__ __forceinline__ auto adj_view(const GraphView &V) {
+  if constexpr (kLayout == kWide) return AdjW{reinterpret_cast<const uint2 *>(V.adj)};
+  else if constexpr (kLayout == kCsr) return AdjC{V.row_ptr, V.col};
+  else
+    return Adj{V.adj,      V.npos, V.hub, V.ctab, V.pos_bits,
+               (uint32_t)((1ull << V.pos_bits) - 1ull), V.deg_max};
+}
+
+// The identity of node v inside the walk kernels.
+__device__ __forceinline__ int32_t node_identity(const GraphView &V, int32_t v) {
+  return V.layout == kNarrow ? V.npos[v] : V.layout == kWide ? v + V.row_ptr[v] : v;
 }
 
 // The entry step i of walk replica r from node v reads (list base b, degree

@@ -199,6 +199,23 @@ __device__ __forceinline__ int32_t edge_owner(const int32_t *row_ptr, int32_t n,
   return lo;
 }
 
+// The owner of every edge; a warp writes the lists of 32 nodes one by one.
+__global__ void k_owners(const int32_t *__restrict__ row_ptr, int32_t n,
+                         int32_t *__restrict__ owner) {
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; v0 < n;
+       v0 += stride) {
+    const int64_t v = v0 + lane;
+    const int32_t b = v < n ? row_ptr[v] : 0, e = v < n ? row_ptr[v + 1] : 0;
+    for (uint32_t todo = __ballot_sync(0xffffffffu, e > b); todo; todo &= todo - 1) {
+      const int l = __ffs(todo) - 1;
+      const int32_t lb = __shfl_sync(0xffffffffu, b, l), le = __shfl_sync(0xffffffffu, e, l);
+      for (int32_t k = lb + lane; k < le; k += 32) owner[k] = (int32_t)(v0 + l);
+    }
+  }
+}
+
 // Expected visits of the walks, used to order the packed adjacency: a walk
 // starts at a uniformly drawn node with in-neighbours and moves to a
 // uniformly drawn in-neighbour.  In 2^-40 fixed point, p_0 = 2^40 / n_act on
@@ -213,15 +230,23 @@ __global__ void k_visit_init(const int32_t *__restrict__ row_ptr, int32_t n, int
     p[v] = row_ptr[v + 1] > row_ptr[v] ? unit : 0ull;
 }
 
-__global__ void k_visit_step(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                             int32_t n, int64_t m, const unsigned long long *__restrict__ p,
+// p becomes the share that each in-neighbour gets.
+__global__ void k_visit_share(const int32_t *__restrict__ row_ptr, int32_t n,
+                              unsigned long long *__restrict__ p) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+    const int32_t d = row_ptr[v + 1] - row_ptr[v];
+    if (d > 1 && p[v]) p[v] /= (unsigned long long)d;
+  }
+}
+
+__global__ void k_visit_step(const int32_t *__restrict__ owner, const int32_t *__restrict__ col,
+                             int64_t m, const unsigned long long *__restrict__ share,
                              unsigned long long *__restrict__ q) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-    const int32_t v = edge_owner(row_ptr, n, e);
-    const unsigned long long share =
-        p[v] / (unsigned long long)(row_ptr[v + 1] - row_ptr[v]);
-    if (share) atomicAdd(&q[col[e]], share);
+    const unsigned long long s = share[owner[e]];
+    if (s) atomicAdd(&q[col[e]], s);
   }
 }
 
@@ -233,32 +258,61 @@ __global__ void k_visit_acc(const unsigned long long *__restrict__ p, int32_t n,
     acc[v] += (unsigned long long)w * p[v];
 }
 
-// Header word of every node that is not a hub: its degree, at its position.
-__global__ void k_narrow_heads(const int32_t *__restrict__ row_ptr, int32_t n, uint32_t dmax,
-                               const int32_t *__restrict__ npos, uint32_t *__restrict__ adj) {
+// Sort key of node v in the narrow layout: its degree code, descending, then
+// its visits, descending, by their leading ten bits (exponent and mantissa).
+__global__ void k_rank_keys(const int32_t *__restrict__ row_ptr, int32_t n, uint32_t dmax,
+                            const unsigned long long *__restrict__ vis,
+                            int32_t *__restrict__ key, int32_t *__restrict__ id,
+                            int32_t *__restrict__ count) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  extern __shared__ int32_t hist[];  // nodes by degree code
+  for (uint32_t c = threadIdx.x; c <= dmax; c += blockDim.x) hist[c] = 0;
+  __syncthreads();
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-    const uint32_t d = (uint32_t)(row_ptr[v + 1] - row_ptr[v]);
-    if (d < dmax) adj[npos[v]] = d;
+    const uint32_t d = (uint32_t)(row_ptr[v + 1] - row_ptr[v]), code = d < dmax ? d : dmax;
+    const unsigned long long w = vis[v];
+    const int e = w ? 64 - __clzll((long long)w) : 0;  // 0..64
+    const uint32_t heat = (uint32_t)e << 9 | (e > 10 ? (uint32_t)(w >> (e - 10)) & 511u
+                                                     : (uint32_t)(w << (10 - e)) & 511u);
+    key[v] = (int32_t)((dmax - code) << 16 | (0xFFFFu - heat));
+    id[v] = (int32_t)v;
+    atomicAdd(&hist[code], 1);
+  }
+  __syncthreads();
+  for (uint32_t c = threadIdx.x; c <= dmax; c += blockDim.x)
+    if (hist[c]) atomicAdd(&count[c], hist[c]);
+}
+
+// npos of the ranked nodes; the hubs' degrees by rank.
+__global__ void k_ranks(const int32_t *__restrict__ row_ptr, int32_t n, int32_t H,
+                        const int32_t *__restrict__ order, int32_t *__restrict__ npos,
+                        int32_t *__restrict__ hub_deg) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
+    const int32_t v = order[x];
+    npos[v] = (int32_t)x;
+    if (x < H) hub_deg[x] = row_ptr[v + 1] - row_ptr[v];
   }
 }
 
-// Edge e of list v lands at base(v) + (e - row_ptr[v]), base(v) = npos[v] + 1
-// or, for a hub, the list offset in its header.
-__global__ void k_narrow_lists(const int32_t *__restrict__ row_ptr,
-                               const int32_t *__restrict__ col, int32_t n, int64_t m,
-                               int pos_bits, const int32_t *__restrict__ npos,
+__global__ void k_hubs(int32_t H, const int32_t *__restrict__ deg, const int32_t *__restrict__ off,
+                       uint2 *__restrict__ hub) {
+  for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < H; x += gridDim.x * blockDim.x)
+    hub[x] = make_uint2((uint32_t)deg[x], (uint32_t)off[x]);
+}
+
+// Edge e of list v lands at first(v) + (e - row_ptr[v]).
+__global__ void k_narrow_lists(GraphView V, const int32_t *__restrict__ owner, int64_t m,
                                uint32_t *__restrict__ adj) {
-  const uint32_t dmax = (uint32_t)((1ull << (32 - pos_bits)) - 1ull);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-    const int32_t v = edge_owner(row_ptr, n, e);
-    const uint32_t dv = (uint32_t)(row_ptr[v + 1] - row_ptr[v]);
-    const int64_t base = dv < dmax ? (int64_t)npos[v] + 1 : (int64_t)adj[npos[v] + 1];
-    const int32_t y = col[e];
-    const uint32_t dy = (uint32_t)(row_ptr[y + 1] - row_ptr[y]);
-    const uint32_t code = dy < dmax ? dy : dmax;
-    adj[base + (e - row_ptr[v])] = (code << pos_bits) | (uint32_t)npos[y];
+    const int32_t v = owner[e];
+    const uint32_t dv = (uint32_t)(V.row_ptr[v + 1] - V.row_ptr[v]), x = (uint32_t)V.npos[v];
+    const uint32_t first = dv < V.deg_max ? V.ctab[dv] + x * dv : V.hub[x].y;
+    const int32_t y = V.col[e];
+    const uint32_t dy = (uint32_t)(V.row_ptr[y + 1] - V.row_ptr[y]);
+    const uint32_t code = dy < V.deg_max ? dy : V.deg_max;
+    adj[first + (uint32_t)(e - V.row_ptr[v])] = (code << V.pos_bits) | (uint32_t)V.npos[y];
   }
 }
 
@@ -281,6 +335,13 @@ __global__ void k_build_adjw_lists(const int32_t *__restrict__ row_ptr,
     adj2[(int64_t)lo + 1 + e] =
         make_uint2((uint32_t)(y + row_ptr[y]), (uint32_t)(row_ptr[y + 1] - row_ptr[y]));
   }
+}
+
+__global__ void k_out_degrees(const int32_t *__restrict__ col, int64_t m,
+                              int32_t *__restrict__ deg) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(&deg[col[e]], 1);
 }
 
 __global__ void k_active_flags(const int32_t *__restrict__ row_ptr, int32_t n,
@@ -355,7 +416,10 @@ extern "C" int srk_graph_free(srk_graph *g) {
     if (g->own_w) cudaFree(g->own_w);
     if (g->adj) cudaFree(g->adj);
     if (g->npos) cudaFree(g->npos);
+    if (g->hub) cudaFree(g->hub);
+    if (g->ctab) cudaFree(g->ctab);
     if (g->act) cudaFree(g->act);
+    if (g->out_deg) cudaFree(g->out_deg);
     if (g->batch_exec) cudaGraphExecDestroy(g->batch_exec);
     free_lin_topo(g);
   }
@@ -370,127 +434,93 @@ static int bits_for(int64_t x) {
   return b;
 }
 
-// Expected visits of every node (k_visit_*): 25 p_1 + 15 p_2 + 9 p_3, the
-// landing mass of the first three steps weighted by survival at c = 0.6
-// (the layout does not depend on a query's c).  Read back to the host.
-static int visit_mass(const srk_graph *g, int dev, int32_t n_act, std::vector<uint64_t> *out) {
-  const int32_t n = g->n;
-  const int64_t m = g->m;
-  unsigned long long *buf = nullptr;
-  cudaError_t e = cudaMalloc(&buf, sizeof(unsigned long long) * 3 * (size_t)n);
-  if (e != cudaSuccess) return cuda_fail(e, "srk_graph_load: visit mass");
-  unsigned long long *p = buf, *q = buf + n, *acc = buf + 2 * (size_t)n;
-  const int blocks = sm_count(dev) * 4;
-  cudaMemset(acc, 0, sizeof(unsigned long long) * (size_t)n);
-  k_visit_init<<<blocks, 256>>>(g->row_ptr, n, n_act, p);
-  const unsigned int w[3] = {25u, 15u, 9u};
-  for (int k = 0; k < 3; ++k) {
-    cudaMemset(q, 0, sizeof(unsigned long long) * (size_t)n);
-    if (m > 0) k_visit_step<<<sm_count(dev) * 8, 256>>>(g->row_ptr, g->col, n, m, p, q);
-    k_visit_acc<<<blocks, 256>>>(q, n, w[k], acc);
-    std::swap(p, q);
-  }
-  out->resize((size_t)n);
-  e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = cudaMemcpy(out->data(), acc, sizeof(unsigned long long) * (size_t)n,
-                   cudaMemcpyDeviceToHost);
-  cudaFree(buf);
-  if (e != cudaSuccess) return cuda_fail(e, "srk_graph_load: visit mass");
-  return SRK_OK;
-}
+// Degree codes of the narrow layout have at most this many bits: a table of
+// list starts that the walk kernels hold in shared memory (8 KB).
+constexpr int kCodeBits = 11;
 
-// Builds the 4-byte-entry adjacency of g (sets adj, npos, n_hubs, pos_bits).
-// The hub count H and the position width pb depend on each other (a hub has
-// degree 2^(32-pb) - 1 or more, and positions run to n + m + H): pb grows
-// from ceil(log2(n + m)) until it holds.  Order: the hubs' headers first, by
-// expected visits (the header of the node a walk lands on is read at the
-// landing), then every node's list (a non-hub's after its header word) by
-// expected visits per list entry, descending, so that the lists read most
-// per byte share sectors and the front of the array; ties by id, nodes
-// without in-neighbours
-// last.  (Measured: on R-MAT 20 this order gives 37.1 queries/s against 37.0
-// for id order; on R-MAT 22-24, where the graph exceeds the L2, it changes
-// nothing measurable, nor did L2 eviction-priority hints that kept its front
-// part resident.)  The layout is a function of the graph alone.
+// Builds the 4-byte-entry adjacency of g (sets adj, npos, hub, ctab, n_hubs,
+// pos_bits, deg_max).  Nodes are ranked by degree code, descending, so that
+// a list's place follows from its node's rank and degree, and within a code by
+// expected visits, descending, so that the lists read most lie together; ties
+// by id.  Expected visits (k_visit_*): 25 p_1 + 15 p_2 + 9 p_3, the landing
+// mass of the first three steps weighted by survival at c = 0.6 (the layout
+// does not depend on a query's c).  The layout is a function of the graph alone
+// and is made on the device: R-MAT 20 in 4 ms, where the same order sorted on
+// the host took 60 ms.
 static int build_narrow(srk_graph *g, int dev) {
   const int32_t n = g->n;
   const int64_t m = g->m;
-  std::vector<int32_t> rp((size_t)n + 1);
-  cudaError_t e = cudaMemcpy(rp.data(), g->row_ptr, sizeof(int32_t) * ((size_t)n + 1),
-                             cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "srk_graph_load: reading row_ptr");
-  auto deg = [&](int32_t v) { return (uint32_t)(rp[(size_t)v + 1] - rp[(size_t)v]); };
-  int32_t n_act = 0;
-  for (int32_t v = 0; v < n; ++v) n_act += deg(v) > 0;
-  int pb = bits_for((int64_t)n + m);
-  int64_t H = 0;
-  for (int it = 0;; ++it) {
-    const uint32_t dmax = (uint32_t)((1ull << (32 - pb)) - 1ull);
-    H = 0;
-    for (int32_t v = 0; v < n; ++v) H += deg(v) >= dmax;
-    const int64_t total = (int64_t)n + m + H;
-    if (total > INT32_MAX || it >= 32)
-      return fail(SRK_EINVAL, "graph too large for 4-byte adjacency entries (n + m + hubs = %lld)",
-                  (long long)total);
-    const int pb2 = bits_for(total);
-    if (pb2 <= pb) break;
-    pb = pb2;
+  const int pb = bits_for(n);
+  const uint32_t dmax = (1u << std::min(32 - pb, kCodeBits)) - 1u;
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t nb = up(sizeof(int32_t) * ((size_t)n + 1)), n8 = up(8 * (size_t)n);
+  const size_t mb = up(sizeof(int32_t) * (size_t)(m > 0 ? m : 1));
+  const size_t sort_b = up(sort_scratch(n)), count_b = up(sizeof(int32_t) * ((size_t)dmax + 1));
+  char *tmp = nullptr;
+  cudaError_t e = cudaMalloc(&tmp, 3 * n8 + 4 * nb + mb + sort_b + count_b);
+  if (e != cudaSuccess) return cuda_fail(e, "srk_graph_load: ranking scratch");
+  unsigned long long *p = (unsigned long long *)tmp, *q = (unsigned long long *)(tmp + n8),
+                     *acc = (unsigned long long *)(tmp + 2 * n8);
+  char *at = tmp + 3 * n8;
+  int32_t *kA = (int32_t *)at, *vA = (int32_t *)(at + nb), *kB = (int32_t *)(at + 2 * nb),
+          *vB = (int32_t *)(at + 3 * nb);
+  at += 4 * nb;
+  int32_t *owner = (int32_t *)at, *sort_tmp = (int32_t *)(at + mb),
+          *count = (int32_t *)(at + mb + sort_b);
+  const int bn = sm_count(dev) * 4, bm = sm_count(dev) * 8;
+  cudaMemsetAsync(acc, 0, 8 * (size_t)n, 0);
+  cudaMemsetAsync(count, 0, sizeof(int32_t) * ((size_t)dmax + 1), 0);
+  if (m > 0) k_owners<<<bm, 256>>>(g->row_ptr, n, owner);
+  k_visit_init<<<bn, 256>>>(g->row_ptr, n, g->n_act, p);
+  const unsigned int w[3] = {25u, 15u, 9u};
+  for (int k = 0; k < 3; ++k) {
+    cudaMemsetAsync(q, 0, 8 * (size_t)n, 0);
+    k_visit_share<<<bn, 256>>>(g->row_ptr, n, p);
+    if (m > 0) k_visit_step<<<bm, 256>>>(owner, g->col, m, p, q);
+    k_visit_acc<<<bn, 256>>>(q, n, w[k], acc);
+    std::swap(p, q);
   }
-  const uint32_t dmax = (uint32_t)((1ull << (32 - pb)) - 1ull);
-  std::vector<uint64_t> vis;
-  int rc = visit_mass(g, dev, n_act, &vis);
-  if (rc) return rc;
-  // hubs by visits; every node by visits per entry
-  std::vector<int32_t> hubs, order((size_t)n);
-  for (int32_t v = 0; v < n; ++v) {
-    order[(size_t)v] = v;
-    if (deg(v) >= dmax) hubs.push_back(v);
+  k_rank_keys<<<bn, 256, sizeof(int32_t) * ((size_t)dmax + 1)>>>(g->row_ptr, n, dmax, acc, kA, vA,
+                                                                 count);
+  const int32_t *order = radix_sort(kA, vA, kB, vB, n, 16 + std::min(32 - pb, kCodeBits), sort_tmp,
+                                    0)
+                             ? vB
+                             : vA;
+  // list starts by degree, from the number of nodes of each code
+  std::vector<int32_t> cnt((size_t)dmax + 1);
+  e = cudaMemcpy(cnt.data(), count, sizeof(int32_t) * cnt.size(), cudaMemcpyDeviceToHost);
+  const int32_t H = e == cudaSuccess ? cnt[dmax] : 0;
+  int64_t rest = m;  // entries of the hubs' lists
+  for (uint32_t d = 1; d < dmax; ++d) rest -= (int64_t)d * cnt[d];
+  std::vector<uint32_t> ctab((size_t)dmax + 1, 0u);
+  uint32_t first = (uint32_t)rest, rank = (uint32_t)H;
+  for (uint32_t d = dmax - 1; d >= 1 && d < dmax; --d) {
+    ctab[d] = first - rank * d;
+    first += d * (uint32_t)cnt[d];
+    rank += (uint32_t)cnt[d];
   }
-  std::stable_sort(hubs.begin(), hubs.end(), [&](int32_t a, int32_t b) {
-    return vis[(size_t)a] > vis[(size_t)b];
-  });
-  std::vector<double> key((size_t)n);
-  for (int32_t v = 0; v < n; ++v)
-    key[(size_t)v] = deg(v) > 0 ? (double)vis[(size_t)v] / (double)deg(v) : -1.0;
-  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-    return key[(size_t)a] > key[(size_t)b];
-  });
-  std::vector<int32_t> npos((size_t)n), hub_rank((size_t)n, -1);
-  std::vector<uint32_t> head(2 * (size_t)std::max<int64_t>(H, 1));
-  for (int64_t r = 0; r < H; ++r) hub_rank[(size_t)hubs[(size_t)r]] = (int32_t)r;
-  int64_t at = 2 * H;
-  for (int32_t v : order) {
-    const uint32_t d = deg(v);
-    if (d < dmax) {
-      npos[(size_t)v] = (int32_t)at;
-      at += 1 + (int64_t)d;
-    } else {
-      const int32_t r = hub_rank[(size_t)v];
-      npos[(size_t)v] = 2 * r;
-      head[2 * (size_t)r] = d;
-      head[2 * (size_t)r + 1] = (uint32_t)at;
-      at += d;
+  if (e == cudaSuccess) e = cudaMalloc(&g->adj, sizeof(uint32_t) * (size_t)(m > 0 ? m : 1));
+  if (e == cudaSuccess) e = cudaMalloc(&g->npos, sizeof(int32_t) * (size_t)n);
+  if (e == cudaSuccess) e = cudaMalloc(&g->hub, sizeof(uint2) * (size_t)(H > 0 ? H : 1));
+  if (e == cudaSuccess) e = cudaMalloc(&g->ctab, sizeof(uint32_t) * ctab.size());
+  if (e == cudaSuccess)
+    e = cudaMemcpy(g->ctab, ctab.data(), sizeof(uint32_t) * ctab.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    g->pos_bits = pb;
+    g->deg_max = dmax;
+    g->n_hubs = H;
+    int32_t *hub_deg = (int32_t *)p, *hub_off = (int32_t *)q;  // n words of 8 bytes each
+    k_ranks<<<bn, 256>>>(g->row_ptr, n, H, order, g->npos, hub_deg);
+    if (H > 0) {
+      scan_i32(hub_deg, hub_off, H, sort_tmp, 0);
+      k_hubs<<<bn, 256>>>(H, hub_deg, hub_off, g->hub);
     }
+    if (m > 0) k_narrow_lists<<<bm, 256>>>(view_of(g), owner, m, g->adj);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
-  const size_t words = (size_t)n + (size_t)m + (size_t)H;
-  if ((size_t)at != words) return fail(SRK_ECUDA, "srk_graph_load: inconsistent layout size");
-  if ((e = cudaMalloc(&g->adj, sizeof(uint32_t) * (words > 0 ? words : 1))) != cudaSuccess ||
-      (e = cudaMalloc(&g->npos, sizeof(int32_t) * (size_t)n)) != cudaSuccess)
-    return cuda_fail(e, "srk_graph_load: packed adjacency");
-  if ((e = cudaMemcpy(g->npos, npos.data(), sizeof(int32_t) * (size_t)n,
-                      cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (H > 0 && (e = cudaMemcpy(g->adj, head.data(), sizeof(uint32_t) * 2 * (size_t)H,
-                                cudaMemcpyHostToDevice)) != cudaSuccess))
-    return cuda_fail(e, "srk_graph_load: positions and hub headers");
-  k_narrow_heads<<<sm_count(dev) * 4, 256>>>(g->row_ptr, n, dmax, g->npos, g->adj);
-  if (m > 0)
-    k_narrow_lists<<<sm_count(dev) * 8, 256>>>(g->row_ptr, g->col, n, m, pb, g->npos, g->adj);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  cudaFree(tmp);
   if (e != cudaSuccess) return cuda_fail(e, "srk_graph_load: building the packed adjacency");
-  g->pos_bits = pb;
-  g->n_hubs = (int32_t)H;
   return SRK_OK;
 }
 
@@ -578,9 +608,40 @@ extern "C" int srk_graph_load(const int32_t *row_ptr, const int32_t *col,
                               "not decrease; col entries must lie in [0, n)");
     }
   }
+  {  // ascending list of the nodes with in-neighbours
+    int32_t *flag = nullptr, *off = nullptr, *scan_tmp = nullptr;
+    const size_t words = ((size_t)n + 64) & ~(size_t)63;
+    if ((e = cudaMalloc(&flag, 2 * sizeof(int32_t) * words + scan_scratch(n))) == cudaSuccess) {
+      off = flag + words;
+      scan_tmp = off + words;
+    } else {
+      int rc = cuda_fail(e, "srk_graph_load: active-node list");
+      srk_graph_free(g);
+      return rc;
+    }
+    k_active_flags<<<sm_count(dev) * 4, 256>>>(g->row_ptr, n, flag);
+    scan_i32(flag, off, n, scan_tmp, 0);
+    int32_t n_act = 0;
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = cudaMemcpy(&n_act, off + n, sizeof(int32_t), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess &&
+        (e = cudaMalloc(&g->act, sizeof(int32_t) * (size_t)(n_act > 0 ? n_act : 1))) ==
+            cudaSuccess) {
+      k_active_scatter<<<sm_count(dev) * 4, 256>>>(flag, off, n, g->act);
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    }
+    cudaFree(flag);
+    if (e != cudaSuccess) {
+      int rc = cuda_fail(e, "srk_graph_load: active-node list");
+      srk_graph_free(g);
+      return rc;
+    }
+    g->n_act = n_act;
+  }
   {
     const int pb = bits_for((int64_t)n + m);  // positions < n + m (wide layout)
-    g->pos_bits = pb;
     // Layout by size (measured on R-MAT graphs 20-24): 4-byte entries up to
     // 28 position bits (degree codes down to 15; the hubs' headers, packed
     // at the front in landing order, stay cached while the entries are half
@@ -611,36 +672,24 @@ extern "C" int srk_graph_load(const int32_t *row_ptr, const int32_t *col,
       return rc;
     }
   }
-  {  // ascending list of the nodes with in-neighbours
-    int32_t *flag = nullptr, *off = nullptr;
-    if ((e = cudaMalloc(&flag, sizeof(int32_t) * (size_t)n)) != cudaSuccess ||
-        (e = cudaMalloc(&off, sizeof(int32_t) * ((size_t)n + 1))) != cudaSuccess) {
-      if (flag) cudaFree(flag);
-      int rc = cuda_fail(e, "srk_graph_load: active-node list");
-      srk_graph_free(g);
-      return rc;
-    }
-    k_active_flags<<<sm_count(dev) * 4, 256>>>(g->row_ptr, n, flag);
-    k_scan<<<1, 1024>>>(flag, off, n);
-    int32_t n_act = 0;
-    e = cudaGetLastError();
-    if (e == cudaSuccess)
-      e = cudaMemcpy(&n_act, off + n, sizeof(int32_t), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess &&
-        (e = cudaMalloc(&g->act, sizeof(int32_t) * (size_t)(n_act > 0 ? n_act : 1))) ==
-            cudaSuccess) {
-      k_active_scatter<<<sm_count(dev) * 4, 256>>>(flag, off, n, g->act);
+  if ((e = allow_lockstep(g->layout)) != cudaSuccess) {
+    int rc = cuda_fail(e, "srk_graph_load: shared memory of the walk kernels");
+    srk_graph_free(g);
+    return rc;
+  }
+  {  // out-degrees (sizes of the queries' filters)
+    e = cudaMalloc(&g->out_deg, sizeof(int32_t) * (size_t)n);
+    if (e == cudaSuccess) e = cudaMemset(g->out_deg, 0, sizeof(int32_t) * (size_t)n);
+    if (e == cudaSuccess && m > 0) {
+      k_out_degrees<<<sm_count(dev) * 8, 256>>>(g->col, m, g->out_deg);
       e = cudaGetLastError();
-      if (e == cudaSuccess) e = cudaDeviceSynchronize();
     }
-    cudaFree(flag);
-    cudaFree(off);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
-      int rc = cuda_fail(e, "srk_graph_load: active-node list");
+      int rc = cuda_fail(e, "srk_graph_load: out-degrees");
       srk_graph_free(g);
       return rc;
     }
-    g->n_act = n_act;
   }
   *out = g;
   return SRK_OK;

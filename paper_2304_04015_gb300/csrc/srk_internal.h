@@ -14,17 +14,16 @@ struct srk_graph {
   const int32_t *row_ptr = nullptr;  // device, n+1
   const int32_t *col = nullptr;      // device, m
   const float *edge_w = nullptr;     // device, m or null
-  // Packed adjacency (owned, n + m + H words, H the hubs below).  Node v's
-  // identity inside the walk kernels is its position npos[v].  A node of
-  // in-degree d < deg_max = 2^(32-pos_bits) - 1 has the word d at its
-  // position and its list right after it; a hub (d >= deg_max) has two words
-  // {d, offset of its list} at position 2r of the hub region at the front,
-  // r its rank by how often walks visit it (so the hot headers share
-  // sectors), and its list after the other nodes'.  The other nodes' words
-  // follow in the order of expected visits per list entry (build_narrow).  Entry k of v's list holds
-  // the k-th in-neighbour y as (min(|I(y)|, deg_max) << pos_bits) | npos[y],
-  // so a walk step learns the next node's degree from the entry it reads and
-  // reads a header only at a hub.
+  // Packed adjacency (owned).  Layout 0 (narrow): the lists of m words, by
+  // rank; node v's identity inside the walk kernels is its rank npos[v] in
+  // the order of build_narrow: in-degree code descending, nodes of one code by
+  // how often walks visit them.  The code of degree d is min(d, deg_max); entry
+  // k of v's list holds the k-th in-neighbour y as (code(y) << pos_bits) |
+  // npos[y].  The d words of a node of degree d < deg_max and rank x begin at
+  // ctab[d] + x d (mod 2^32), since the nodes of one degree follow one another
+  // in rank and in memory; a hub (degree deg_max or more; they come first)
+  // has {degree, first word} in hub[x].  So a walk step learns the next node's
+  // degree and list from the entry it reads and a table of deg_max + 1 words.
   // Wide layout (layout = 1, chosen when n + m needs more than 28 bits or
   // forced by SRK_ADJ_WIDE): 2 (n + m) words forming 8-byte entries at
   // positions v + row_ptr[v], adj[pos(v)] = {0, |I(v)|} and entries
@@ -32,14 +31,18 @@ struct srk_graph {
   // 2, only when forced by SRK_ADJ_CSR): no packed copy; nodes are their ids
   // and a step reads row_ptr and col.
   uint32_t *adj = nullptr;
-  int32_t *npos = nullptr;  // narrow layout: positions, n (owned)
-  int32_t n_hubs = 0;       // narrow layout: H
-  int32_t pos_bits = 1;     // positions < 2^pos_bits
+  int32_t *npos = nullptr;   // narrow layout: ranks, n (owned)
+  uint2 *hub = nullptr;      // narrow layout: hub records, n_hubs (owned)
+  uint32_t *ctab = nullptr;  // narrow layout: list starts by degree (owned)
+  int32_t n_hubs = 0;        // narrow layout: H
+  int32_t pos_bits = 1;      // narrow layout: ranks < 2^pos_bits
+  uint32_t deg_max = 1;      // narrow layout: largest degree code
   int layout = 0;        // 0 narrow, 1 wide, 2 CSR (no packed adjacency; walks read row_ptr/col)
   // Nodes with at least one in-neighbour, ascending (owned): the only targets
   // whose score can be nonzero.
   int32_t *act = nullptr;
   int32_t n_act = 0;
+  int32_t *out_deg = nullptr;  // out-degrees by id, n (owned)
   // Launch shape of the batched target kernel chosen by the autotuner
   // (-1: not tuned yet).
   int batch_cfg = -1;
@@ -54,7 +57,25 @@ struct srk_graph {
   float *own_w = nullptr;
 };
 
+// A graph as the kernels see it (passed by value).
+struct GraphView {
+  const int32_t *row_ptr;  // CSR offsets
+  const int32_t *col;      // in-neighbour lists
+  const uint32_t *adj;     // packed adjacency
+  const int32_t *npos;     // narrow layout: ranks,
+  const uint2 *hub;        //   hub records,
+  const uint32_t *ctab;    //   list starts by degree
+  int32_t pos_bits;
+  uint32_t deg_max;
+  int32_t n, n_hubs, layout;
+};
+
 namespace srk {
+
+inline GraphView view_of(const srk_graph *g) {
+  return GraphView{g->row_ptr, g->col,     g->adj,     g->npos, g->hub,    g->ctab,
+                   g->pos_bits, g->deg_max, g->n,      g->n_hubs, g->layout};
+}
 
 // The output function of SplitMix64 (Steele, Lea, Flood, OOPSLA 2014) and
 // the 32-bit finalizer "lowbias32" (C. Wellons, 2018); both are bijections.
@@ -153,10 +174,25 @@ struct Outputs {
 // number of bytes one query of table `t` needs.
 size_t plan(const QueryTab &t, Workspace *w, char *base);
 // Enqueues steps a2-a5 on `st`; `timing` (may be null) gets two events
-// recorded around the target-walk kernel.
+// recorded around the target-walk kernel; `extra`: scratch for the end filters
+// (see filter_bytes); `count`: step totals are wanted.
 int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
-                  const Outputs &o, cudaStream_t st, const cudaEvent_t *timing,
-                  int32_t u_begin, int32_t u_end);
+                  const Outputs &o, char *extra, size_t extra_bytes, bool count, cudaStream_t st,
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end);
+// srk_single_source with at most extra_limit bytes for the end filters.
+int single_source(const srk_graph *g, int32_t s, double c, double eps, uint64_t seed,
+                  const srk_opts *opt, double *scores, uint32_t *meet_counts,
+                  uint64_t *weight_sums, void *cuda_stream, size_t extra_limit);
+// Bytes of `extra` scratch a query of n_targets targets makes use of (it does
+// with less, or none: its end nodes then have fewer filters, or none).
+size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets);
+// Steps a4-a5 after the source side (sigma, seff, spos and the cap rows of w
+// are made, the outputs of the range cleared): srk_lockstep.cu.
+int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Outputs &o,
+                  char *extra, size_t extra_bytes, bool count, cudaStream_t st,
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end);
+// Shared-memory opt-in of the walk kernels of a layout, in this context.
+cudaError_t allow_lockstep(int layout);
 // [*b, *e): the targets a query computes, from its options (SRK_EINVAL when
 // the range is malformed).
 int target_range(const srk_graph *g, const srk_opts *opt, int32_t *b, int32_t *e);
@@ -164,6 +200,16 @@ int target_range(const srk_graph *g, const srk_opts *opt, int32_t *b, int32_t *e
 __global__ void k_scan(const int32_t *__restrict__ cnt, int32_t *__restrict__ off,
                        int32_t N);
 
+
+// Exclusive scan of cnt[0..N) into off[0..N], with scan_scratch(N) bytes of
+// scratch (srk_sort.cu).
+size_t scan_scratch(int64_t N);
+void scan_i32(const int32_t *cnt, int32_t *off, int64_t N, int32_t *tmp, cudaStream_t st);
+// Stable sort of m pairs (key, value) by the keys' low `bits` bits, with
+// sort_scratch(m) bytes of scratch; returns true when the result is in kB, vB.
+size_t sort_scratch(int64_t m);
+bool radix_sort(int32_t *kA, int32_t *vA, int32_t *kB, int32_t *vB, int64_t m, int bits,
+                int32_t *tmp, cudaStream_t st);
 
 // In-degrees of k sources (ids already checked against n), read from the
 // device CSR on stream st (synchronises st).  SRK_OK or an error code.

@@ -31,6 +31,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "srk_internal.h"
@@ -44,8 +45,6 @@ constexpr int32_t kMid = 512;     // up to this many: one warp
 constexpr int32_t kChunk = 512;   // longer lists: chunks of this many entries, one warp each
 constexpr int kGroup = 8;
 constexpr int kSegBlock = 256;    // threads per block of the reduction kernel
-// Radix sort of the transpose: 8-bit digits, tiles of 256 threads x 16 keys.
-constexpr int kSortBlock = 256, kSortItems = 16, kSortTile = kSortBlock * kSortItems;
 
 // Size-class lists of one direction (in-lists or out-lists) of the graph.
 struct Classes {
@@ -275,71 +274,6 @@ __global__ void k_iota(int32_t *__restrict__ v, int64_t m) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
        k += (int64_t)gridDim.x * blockDim.x)
     v[k] = (int32_t)k;
-}
-
-// Radix sort pass, step 1: digit histogram of each tile, stored digit-major
-// (hist[d * tiles + tile]) so that its exclusive scan gives each
-// (digit, tile) its first output position.
-__global__ void __launch_bounds__(kSortBlock)
-k_sort_hist(const int32_t *__restrict__ keys, int64_t m, int shift, int32_t tiles,
-            int32_t *__restrict__ hist) {
-  __shared__ int32_t cnt[256];
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    const int64_t i = base + (int64_t)r * kSortBlock + threadIdx.x;
-    if (i < m) atomicAdd(&cnt[(keys[i] >> shift) & 255], 1);
-  }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * tiles + blockIdx.x] = cnt[threadIdx.x];
-}
-
-// Radix sort pass, step 2: stable scatter.  Round r of a tile covers 256
-// consecutive keys; a key goes to its (digit, tile) offset plus the number of
-// keys of its digit in earlier rounds, earlier warps and lower lanes.
-__global__ void __launch_bounds__(kSortBlock)
-k_sort_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ vals, int64_t m,
-               int shift, int32_t tiles, const int32_t *__restrict__ off,
-               int32_t *__restrict__ keys_out, int32_t *__restrict__ vals_out) {
-  constexpr int kWarps = kSortBlock / 32;
-  __shared__ int32_t base[256];
-  __shared__ int32_t wcnt[kWarps][256];
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  base[t] = off[(int64_t)t * tiles + blockIdx.x];
-  for (int i = 0; i < kWarps; ++i) wcnt[i][t] = 0;
-  __syncthreads();
-  const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    const int64_t i = tile0 + (int64_t)r * kSortBlock + t;
-    const bool valid = i < m;
-    int32_t key = 0, val = 0, d = 256;  // 256: no key in this slot
-    if (valid) {
-      key = keys[i];
-      val = vals[i];
-      d = (key >> shift) & 255;
-    }
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
-    const int rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid && rank == 0) wcnt[w][d] = __popc(peers);
-    __syncthreads();
-    int32_t run = 0;  // thread t: digit t's counts over the warps, made exclusive
-    for (int k = 0; k < kWarps; ++k) {
-      const int32_t c = wcnt[k][t];
-      wcnt[k][t] = run;
-      run += c;
-    }
-    __syncthreads();
-    if (valid) {
-      const int64_t pos = (int64_t)base[d] + wcnt[w][d] + rank;
-      keys_out[pos] = key;
-      vals_out[pos] = val;
-    }
-    __syncthreads();
-    base[t] += run;
-    for (int k = 0; k < kWarps; ++k) wcnt[k][t] = 0;
-    __syncthreads();
-  }
 }
 
 __global__ void k_gather_i32(const int32_t *__restrict__ src, const int32_t *__restrict__ idx,
@@ -614,11 +548,9 @@ static int build_topo(const srk_graph *g, cudaStream_t st, srk_lin_topo **out) {
   p += class_layout(&T->in, p, n, m);
   class_layout(&T->out, p, n, m);
 
-  // scratch: out-degrees, two key/value buffers, histogram and its scan, counters
-  const int32_t tiles = (int32_t)((m + kSortTile - 1) / kSortTile);
-  const size_t H = (size_t)256 * (size_t)(tiles > 0 ? tiles : 1);
-  const size_t scratch = up256(sizeof(int32_t) * (size_t)n) + 4 * words_m +
-                         up256(sizeof(int32_t) * H) + up256(sizeof(int32_t) * (H + 1)) +
+  // scratch: out-degrees, two key/value buffers, the sort's and the scan's, counters
+  const size_t sort_b = up256(sort_scratch(m)), scan_b = up256(scan_scratch(n));
+  const size_t scratch = up256(sizeof(int32_t) * (size_t)n) + 4 * words_m + sort_b + scan_b +
                          up256(sizeof(int32_t) * 8);
   cudaMemPool_t mp = pool(dev);
   void *sb = nullptr;
@@ -634,10 +566,10 @@ static int build_topo(const srk_graph *g, cudaStream_t st, srk_lin_topo **out) {
   int32_t *kA = (int32_t *)q, *vA = (int32_t *)(q + words_m);
   int32_t *kB = (int32_t *)(q + 2 * words_m), *vB = (int32_t *)(q + 3 * words_m);
   q += 4 * words_m;
-  int32_t *hist = (int32_t *)q;
-  q += up256(sizeof(int32_t) * H);
-  int32_t *hoff = (int32_t *)q;
-  q += up256(sizeof(int32_t) * (H + 1));
+  int32_t *sort_tmp = (int32_t *)q;
+  q += sort_b;
+  int32_t *scan_tmp = (int32_t *)q;
+  q += scan_b;
   int32_t *cnt = (int32_t *)q;
 
   const int gm = grid_of(m, 256, dev), gn = grid_of(n, 256, dev);
@@ -647,22 +579,16 @@ static int build_topo(const srk_graph *g, cudaStream_t st, srk_lin_topo **out) {
     k_erow<<<gm, 256, 0, st>>>(g->row_ptr, n, m, T->erow);
     k_out_degree<<<gm, 256, 0, st>>>(g->col, m, odeg);
   }
-  k_scan<<<1, 1024, 0, st>>>(odeg, T->out_ptr, n);
+  scan_i32(odeg, T->out_ptr, n, scan_tmp, st);
   if (m > 0) {
     // stable LSD radix sort of the edge indices by their source node col[e]
     cudaMemcpyAsync(kA, g->col, sizeof(int32_t) * (size_t)m, cudaMemcpyDeviceToDevice, st);
     k_iota<<<gm, 256, 0, st>>>(vA, m);
     int bits = 0;
     while (bits < 31 && ((int64_t)1 << bits) < (int64_t)n) ++bits;  // keys < n <= 2^bits
-    for (int shift = 0; shift < bits; shift += 8) {
-      k_sort_hist<<<tiles, kSortBlock, 0, st>>>(kA, m, shift, tiles, hist);
-      k_scan<<<1, 1024, 0, st>>>(hist, hoff, (int32_t)H);
-      k_sort_scatter<<<tiles, kSortBlock, 0, st>>>(kA, vA, m, shift, tiles, hoff, kB, vB);
-      int32_t *tk = kA, *tv = vA;
-      kA = kB;
-      vA = vB;
-      kB = tk;
-      vB = tv;
+    if (radix_sort(kA, vA, kB, vB, m, bits, sort_tmp, st)) {
+      std::swap(kA, kB);
+      std::swap(vA, vB);
     }
     cudaMemcpyAsync(T->t_e, vA, sizeof(int32_t) * (size_t)m, cudaMemcpyDeviceToDevice, st);
     k_gather_i32<<<gm, 256, 0, st>>>(T->erow, T->t_e, m, T->t_a);

@@ -1,0 +1,1040 @@
+// Target walks in lockstep (steps a4-a5 of a query): every target with
+// in-neighbours walks its pairs, the first meeting of a pair counts, and the
+// scores follow.
+//
+// A pair j joins the source walk sigma(j), nodes h_1, h_2, ..., with walk j of
+// every target, for cap_j steps at most.  A thread holds a few targets and a
+// block takes its targets through one pair after the other, so a pair's index,
+// nodes, weight and length are the same for all its threads.  Two things follow
+// that a warp per target (lanes over pairs, the earlier form) cannot have:
+//
+//   End filters.  The last step of a pair can only meet when h_cap is an
+//   in-neighbour of the node x the walk is at, that is, when x is in the
+//   out-list of h_cap.  Each end node has a Bloom filter of its out-list (one
+//   hash, 16 bits and more per node), which the block holds in shared memory
+//   while it walks the pair; where it says no, the last step is neither drawn
+//   nor read.  At R-MAT 20 6.5 % of the walks that reach their last step pass,
+//   so of the 1.45 scattered reads a pair costs after its first step 0.92 are
+//   left (CPU model of the walk).  The meetings are the same: the filter has no
+//   false negatives.  A step counts as taken when the walk gets to take it,
+//   whatever its draw, so step counts are the same too.
+//   Pairs of cap 1.  Their only step is their last: 40 % of all pairs, which
+//   meet at one target in 300.  They are not walked at all.  One pass over the
+//   edges (k_edges, which also fills the filters) finds, for every edge from
+//   an end node y to a target u, the pairs that end at y after one step, and
+//   draws u's step for those only.
+//
+// What bounds it (GB300): the misses of the scattered list reads, one 32-byte
+// sector each, 3.1e11 per second with the graph in L2; then issue slots.  At
+// R-MAT 20, eps = 0.02 (10,975 pairs, 546,406 targets): 0.93 sectors and 109
+// warp instructions per 32 pairs and targets, where a warp per target took
+// about 2.0 sectors and 189.  One query 31.5 ms instead of 42.3 ms; R-MAT 16
+// 2.11 ms instead of 2.58 ms; 100,003 nodes with uniform lists of 12, eps =
+// 0.03, 2.17 ms instead of 2.90 ms; R-MAT 22 at eps = 0.05, bound by DRAM (64
+// bytes fetched per missing sector), 51-55 ms instead of 60 ms.
+//
+// Launch shape: 2 blocks of 448 threads per SM, 3 targets a thread (72
+// registers).  Measured at R-MAT 20 in an earlier state of the kernel: 1 target
+// x 704 threads 44.7 ms, 2 x 512 39.9, 3 x 448 38.2, 4 x 384 38.2, 5 x 320 41:
+// several targets share a pair's uniform work, and their chains of dependent
+// loads overlap.  Shared memory is kept to about 76 KB a block, since the rest
+// of the SM's 256 KB holds the lines of reads in flight: 92 KB of it cost
+// nothing against 124 KB, 60 KB 10 %, 28 KB half the speed.
+#include <stdint.h>
+#include <string.h>
+
+#include <algorithm>
+
+#include "srk_device.cuh"
+#include "srk_internal.h"
+
+namespace srk {
+
+// Filters.  A filter of 2^lg words is named by 16 * (its place, in units of
+// kFilterUnit words) + lg; kNoFilter names none.
+constexpr int kFilterUnit = 32;       // words of the smallest filter (lg = 5)
+constexpr int kFilterMaxLg = 10;      // 4 KB
+constexpr int32_t kNoFilter = -1;
+__device__ __forceinline__ int64_t filter_place(int32_t f) { return (int64_t)(f >> 4) * kFilterUnit; }
+__device__ __forceinline__ int filter_lg(int32_t f) { return f & 15; }
+// The bit of the node of identity x in a filter of 2^lg words.
+__device__ __forceinline__ uint32_t filter_bit(int32_t x, int lg) {
+  return ((uint32_t)x * 0x9E3779B1u) >> (27 - lg);
+}
+
+// A slot of the table of end nodes: the node id + 1 (0: empty slot), its
+// filter + 1 (0: none; kWantFilter: some pair ends here), and the pairs of cap
+// 1 that end here, list1[off1 .. off1 + cnt1).
+struct EndSlot {
+  uint32_t key;
+  int32_t filt;
+  int32_t cnt1;
+  int32_t off1;
+};
+constexpr int32_t kWantFilter = -1;
+
+__device__ __forceinline__ uint32_t end_hash(uint32_t id) {
+  id *= 0x85EBCA6Bu;
+  return id ^ (id >> 15);
+}
+
+// End nodes and filters of one query (null slots: the query has none).
+struct Filters {
+  EndSlot *slots;       // 2^slot_bits of them, linear probing
+  uint32_t *bloom;      // 2^bloom_bits bits: ids whose bit is clear are in no slot
+  uint32_t *bits;       // the filters, max_units * kFilterUnit words
+  int32_t *list1;       // pairs of cap 1, grouped by end node
+  int32_t *slot_of;     // per pair: its slot,
+  int32_t *rank1;       //   and its place in the slot's list
+  int32_t *ctl;         // {units of bits handed out, entries of list1 handed out}
+  const int32_t *out_deg;  // out-degrees, by node id
+  int slot_bits, bloom_bits;
+  int32_t max_units;
+};
+
+// What the lockstep kernel needs of one query.
+struct LockQuery {
+  const int4 *rec;              // per pair {j, cap, first node in H, filter}
+  const unsigned long long *w;  // per pair: its quantised weight
+  const int32_t *H;             // nodes of the pairs' source walks, steps 1..cap
+  const uint32_t *bits;         // the filters
+  const int32_t *cnt;           // cnt[i]: pairs with cap >= i (longest first)
+  unsigned long long *W;        // per target: weight sum
+  uint32_t *counts;             // per target: meetings, or null
+  uint32_t *steps;              // per target: steps, or null
+  unsigned long long *steps_total;
+  uint32_t key;                 // walk key of the target walks
+  uint32_t rk[10];              //   and its round keys
+  int32_t s;
+  int32_t min_cap;              // pairs below this cap are not walked here
+};
+
+// -------------------------------------------------- asynchronous copies --
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t *bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// 16-byte aligned addresses, bytes a multiple of 16.
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes,
+                                          uint64_t *bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          smem_addr(dst)),
+      "l"(src), "r"(bytes), "r"(smem_addr(bar))
+      : "memory");
+}
+
+// ------------------------------------------------------ the lockstep block --
+constexpr int kLockThreads = 448;
+constexpr int kLockBlocks = 2;        // per SM
+constexpr int kLockTargets = 3;       // per thread
+constexpr int kLockWarps = kLockThreads / 32;
+constexpr int kStages = 2;            // groups of filters in flight per block,
+constexpr int kStageWords = 2048;     //   this many words of filters each (at least the largest)
+constexpr int kGroup = 16;            //   of at most this many pairs
+constexpr int kListWords = 8192;       // words of targets' own lists held in shared memory
+constexpr int kQueue = 64;            // entries of a warp's queue of last steps
+constexpr int kHubCache = 512;        // hub records held there (narrow layout),
+constexpr int kCodes = 2048;          //   and list starts by degree code
+constexpr size_t kLockSmem = 4 * (size_t)kStages * kStageWords + 4 * kListWords +
+                             16 * kQueue * kLockWarps + 8 * kHubCache + 4 * kCodes;
+
+// The narrow layout's tables in shared memory.
+struct LockTables {
+  uint32_t ctab, hub, n_hub;
+};
+
+struct LockShared {
+  uint64_t full[kStages];   // phase n / kStages: the filters of group n have landed
+  uint64_t empty[kStages];  // phase n / kStages: every warp is done with group n
+  int32_t pairs[kStages];   // pairs of the stage's group
+  int32_t place[kStages][kGroup];  // a pair's filter in the stage: first word, or -1
+  uint32_t sums[4];
+  uint32_t warp_sum[kLockWarps];
+  int32_t unit;
+  int32_t broken;  // a wait gave up: filters are read from global memory from here on
+};
+
+// Waits, a bounded time, for the phase of parity ph.
+__device__ __forceinline__ bool lock_wait(LockShared &S, uint64_t *bar, uint32_t ph) {
+  if (mbar_try(bar, ph)) return *(volatile int32_t *)&S.broken == 0;
+  for (int spin = 0; spin < (1 << 20); ++spin) {
+    if (*(volatile int32_t *)&S.broken) return false;
+    if (mbar_try(bar, ph)) return true;
+  }
+  *(volatile int32_t *)&S.broken = 1;
+  return false;
+}
+
+__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo) {
+  asm("{\n.reg .u64 p;\nmul.wide.u32 p, %2, %3;\nmov.b64 {%1, %0}, p;\n}"
+      : "=r"(hi), "=r"(lo) : "r"(a), "r"(b));
+}
+
+// philox2 with the round keys given (kernel parameters: constant operands).
+__device__ __forceinline__ void philox2k(const uint32_t (&rk)[10], uint32_t c0, uint32_t c1,
+                                         uint32_t &x0, uint32_t &x1) {
+  x0 = c0;
+  x1 = c1;
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    uint32_t hi, lo;
+    mul_wide(kPhilox2M, x0, hi, lo);
+    x0 = hi ^ x1 ^ rk[r];
+    x1 = lo;
+  }
+}
+
+// The indices of step i of walk r below d[t] from the words w[t] (step_entry's
+// draw; 0 where d[t] is 0).  Lemire's test, which almost no word comes near,
+// is one branch for all the thread's targets.
+static __device__ __noinline__ uint32_t rare_index(uint32_t w, uint32_t k, int i, uint32_t r,
+                                                   uint32_t v, uint32_t d) {
+  const uint32_t lo = w * d;
+  return lo < d && lo < (0u - d) % d ? step_index_redraw(k, i, r, v, d) : __umulhi(w, d);
+}
+template <int kT>
+__device__ __forceinline__ void lock_index(const uint32_t (&w)[kT], const uint32_t (&d)[kT],
+                                           uint32_t k, int i, uint32_t r, const int32_t (&v)[kT],
+                                           uint32_t (&idx)[kT]) {
+  bool rare = false;
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    uint32_t lo;
+    mul_wide(w[t], d[t], idx[t], lo);
+    rare |= lo < d[t];
+  }
+  if (rare)
+#pragma unroll
+    for (int t = 0; t < kT; ++t)
+      if (d[t]) idx[t] = rare_index(w[t], k, i, r, (uint32_t)v[t], d[t]);
+}
+
+// Loads under a condition, without a branch: v keeps its value where p is false.
+__device__ __forceinline__ void load_if(bool p, uint32_t smem, uint32_t &v) {
+  asm("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\n@q ld.shared.u32 %0, [%1];\n}"
+      : "+r"(v) : "r"(smem), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void load_if(bool p, uint32_t smem, uint2 &v) {
+  asm("{\n.reg .pred q;\nsetp.ne.u32 q, %3, 0;\n@q ld.shared.v2.u32 {%0, %1}, [%2];\n}"
+      : "+r"(v.x), "+r"(v.y) : "r"(smem), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void load_if(bool p, const uint32_t *g, uint32_t &v) {
+  asm("{\n.reg .pred q;\nsetp.ne.u32 q, %2, 0;\n@q ld.global.u32 %0, [%1];\n}"
+      : "+r"(v) : "l"(g), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void load_if(bool p, const uint2 *g, uint2 &v) {
+  asm("{\n.reg .pred q;\nsetp.ne.u32 q, %3, 0;\n@q ld.global.v2.u32 {%0, %1}, [%2];\n}"
+      : "+r"(v.x), "+r"(v.y) : "l"(g), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void load_if(bool p, uint32_t smem, int32_t &v) {
+  load_if(p, smem, reinterpret_cast<uint32_t &>(v));
+}
+__device__ __forceinline__ void load_if(bool p, const int32_t *g, int32_t &v) {
+  load_if(p, reinterpret_cast<const uint32_t *>(g), reinterpret_cast<uint32_t &>(v));
+}
+__device__ __forceinline__ const uint32_t *entries(const Adj &G) { return G.adj; }
+__device__ __forceinline__ const uint2 *entries(const AdjW &G) { return G.adj; }
+__device__ __forceinline__ const int32_t *entries(const AdjC &G) { return G.col; }
+
+// Base and degree of the node x that entry e names, where p holds; degree 0
+// elsewhere.
+template <class GA, class E>
+__device__ __forceinline__ int32_t lock_next(const GA &G, const LockTables &, bool p, E e,
+                                             int32_t x, uint32_t &deg) {
+  int32_t b = 0;
+  deg = 0;
+  if (p) b = entry_next(G, e, x, deg);
+  return b;
+}
+__device__ __forceinline__ int32_t lock_next(const Adj &G, const LockTables &T, bool p, uint32_t e,
+                                             int32_t x, uint32_t &deg) {
+  const uint32_t code = p ? e >> G.pb : 0u;
+  uint32_t start = 0;
+  load_if(true, T.ctab + 4u * code, start);
+  uint2 h = make_uint2(code, start + (uint32_t)x * code);
+  const bool hub = code == G.dmax, near = (uint32_t)x < T.n_hub;
+  load_if(hub && near, T.hub + 8u * (uint32_t)x, h);
+  load_if(hub && !near, G.hub + (uint32_t)x, h);
+  deg = h.x;
+  return (int32_t)h.y;
+}
+template <class GA, class E>
+__device__ __forceinline__ bool entry_ends(const GA &G, E e, int32_t x) {
+  uint32_t d = 0;
+  entry_next(G, e, x, d);
+  return d == 0;
+}
+__device__ __forceinline__ bool entry_ends(const Adj &G, uint32_t e, int32_t) {
+  return (e >> G.pb) == 0;
+}
+
+template <int kT>
+struct LockTargets {
+  int32_t u[kT], b[kT], at[kT];  // id, list base, list in shared memory (-1: not there,
+                                 // -2: no target)
+  uint32_t d[kT], st[kT];        // in-degree (0: no target), steps
+};
+
+// The first word of an entry (what a queue entry keeps of it; the wide layout
+// finds the degree again at the node's head).
+__device__ __forceinline__ uint32_t entry_word(uint32_t e) { return e; }
+__device__ __forceinline__ uint32_t entry_word(int32_t e) { return (uint32_t)e; }
+__device__ __forceinline__ uint32_t entry_word(uint2 e) { return e.x; }
+__device__ __forceinline__ uint32_t word_entry(const Adj &, uint32_t w) { return w; }
+__device__ __forceinline__ int32_t word_entry(const AdjC &, uint32_t w) { return (int32_t)w; }
+__device__ __forceinline__ uint2 word_entry(const AdjW &G, uint32_t w) {
+  return make_uint2(w, G.adj[w].y);
+}
+
+// Where a pair's filter is: in shared memory (near), or in global.
+struct LockFilter {
+  uint32_t near;
+  const uint32_t *far;
+  int lg;
+  bool has, landed;
+};
+
+// A warp's queue of last steps.  Few walks pass their pair's filter, and
+// their last steps would each hold the whole warp for two dependent loads; the
+// queue collects them until they fill a warp.  Entry {entry of the node before
+// the last step, node to meet, cap << 24 | j, a << 8 | target slot}.
+struct LockQueue {
+  uint4 *at;
+  int32_t n;
+};
+
+template <int kT, class GA>
+__device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, const LockQuery &Q, LockQueue &B, int take,
+                                           const int32_t (&u)[kT]) {
+  __syncwarp();
+  const int lane = threadIdx.x & 31;
+  B.n -= take;
+  const bool p = lane < take;
+  const uint4 it = p ? B.at[B.n + lane] : make_uint4(0u, 0u, 1u << 24, 0u);
+  int32_t v = 0;
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    const int32_t vt = __shfl_sync(0xffffffffu, u[t], it.w & 31);
+    if (((it.w >> 5) & 7) == t) v = vt;
+  }
+  const uint32_t j = it.z & 0xFFFFFFu;
+  const int i = (int)(it.z >> 24);
+  uint32_t deg[1] = {0}, x0[1], x1[1], idx[1];
+  const int32_t vv[1] = {v};
+  int32_t b = 0;
+  if (p) {
+    const auto e = word_entry(G, it.x);
+    b = lock_next(G, T, true, e, entry_pos(G, e), deg[0]);
+  }
+  philox2k(Q.rk, walk_ctr0(i, j), (uint32_t)v, x0[0], x1[0]);
+  if (!(i & 1)) x0[0] = x1[0];
+  lock_index(x0, deg, Q.key, i, j, vv, idx);
+  if (deg[0]) {
+    const auto e = adj_entry(G, b, idx[0]);
+    if (entry_pos(G, e) == (int32_t)it.y) {
+      atomicAdd(&Q.W[v], Q.w[it.w >> 8]);
+      if (Q.counts) atomicAdd(&Q.counts[v], 1u);
+    }
+  }
+  __syncwarp();
+}
+
+// One pair (index j, nodes h at steps 1..cap, step 1..32 in the lanes' h32)
+// for the thread's targets; kCap = cap, or 0 for any.
+template <int kCap, int kT, bool kCount, class GA, class E>
+__device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, const LockQuery &Q, const LockFilter &F,
+                                          uint32_t lists, int32_t a, uint32_t j, int cap_,
+                                          int32_t h32, const int32_t *__restrict__ h,
+                                          LockTargets<kT> &X, LockQueue &B) {
+  const int cap = kCap ? kCap : cap_;
+  const int lane = threadIdx.x & 31;
+  int32_t b[kT];
+  uint32_t deg[kT], x0[kT], x1[kT], idx[kT];
+  E e[kT];
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    philox2k(Q.rk, j, (uint32_t)X.u[t], x0[t], x1[t]);
+    deg[t] = X.d[t];
+  }
+  lock_index(x0, deg, Q.key, 1, j, X.u, idx);
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    e[t] = E{};
+    load_if(X.at[t] >= 0, lists + (uint32_t)sizeof(E) * ((uint32_t)X.at[t] + idx[t]), e[t]);
+    load_if(X.at[t] == -1, entries(G) + ((uint32_t)X.b[t] + idx[t]), e[t]);
+  }
+#pragma unroll(kCap ? kCap : 1)
+  for (int i = 1;; ++i) {
+    // the walks are at the nodes that the entries e of step i name
+    int32_t hi = __shfl_sync(0xffffffffu, h32, (i - 1) & 31);
+    if (kCap == 0 && i > 32) hi = h[i - 1];
+    bool met[kT], meets = false;
+#pragma unroll
+    for (int t = 0; t < kT; ++t) {
+      met[t] = deg[t] != 0 && entry_pos(G, e[t]) == hi;
+      meets |= met[t];
+      if (kCount && (i == cap ? deg[t] != 0 : met[t])) X.st[t] += i;
+    }
+    if (meets) {  // rare: a few times per target and query
+#pragma unroll
+      for (int t = 0; t < kT; ++t)
+        if (met[t]) {
+          atomicAdd(&Q.W[X.u[t]], Q.w[a]);
+          if (Q.counts) atomicAdd(&Q.counts[X.u[t]], 1u);
+          deg[t] = 0;
+        }
+    }
+    if (i == cap) break;  // cap 1
+    if (i == cap - 1) {   // the last step: into the queue, if the filter lets it
+      int32_t he = __shfl_sync(0xffffffffu, h32, i & 31);
+      if (kCap == 0 && i >= 32) he = h[i];
+#pragma unroll
+      for (int t = 0; t < kT; ++t) {
+        const int32_t x = entry_pos(G, e[t]);
+        bool p = deg[t] != 0;
+        if (kCount && p) {
+          const bool ends = entry_ends(G, e[t], x);
+          X.st[t] += ends ? i : cap;
+          p = !ends;
+        }
+        if (F.has) {
+          const uint32_t f = filter_bit(x, F.lg);
+          uint32_t word = 0;
+          if (F.landed) load_if(true, F.near + 4u * (f >> 5), word);
+          else word = F.far[f >> 5];
+          p = p && ((word >> (f & 31)) & 1u);
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, p);
+        if (p)
+          B.at[B.n + __popc(m & lanes_below_mask())] =
+              make_uint4(entry_word(e[t]), (uint32_t)he, (uint32_t)cap << 24 | j,
+                         (uint32_t)a << 8 | (uint32_t)(t * 32 + lane));
+        B.n += __popc(m);
+        if (B.n >= 32) lock_drain(G, T, Q, B, 32, X.u);
+      }
+      break;
+    }
+    uint32_t any = 0;
+#pragma unroll
+    for (int t = 0; t < kT; ++t) {
+      const bool p = deg[t] != 0;
+      b[t] = lock_next(G, T, p, e[t], entry_pos(G, e[t]), deg[t]);
+      if (kCount && p && deg[t] == 0) X.st[t] += i;
+      any |= deg[t];
+    }
+    if (!__any_sync(0xffffffffu, any != 0)) break;
+    if (!(i & 1)) {
+#pragma unroll
+      for (int t = 0; t < kT; ++t)
+        philox2k(Q.rk, walk_ctr0(i + 1, j), (uint32_t)X.u[t], x0[t], x1[t]);
+      lock_index(x0, deg, Q.key, i + 1, j, X.u, idx);
+    } else {
+      lock_index(x1, deg, Q.key, i + 1, j, X.u, idx);
+    }
+#pragma unroll
+    for (int t = 0; t < kT; ++t)
+      load_if(deg[t] != 0, entries(G) + ((uint32_t)b[t] + idx[t]), e[t]);
+  }
+}
+
+// Pairs first, first + stride, ... (len of them) for the block's targets; seq
+// counts the groups of this block.  Warp 0 forms the groups: the next pairs
+// whose filters fit a stage.
+template <int kT, bool kCount, class GA, class E>
+__device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
+                                               const LockQuery &Q, LockShared &S,
+                                               uint32_t *ring, uint4 *queues, const E *lists,
+                                               int32_t first, int32_t stride, int32_t len,
+                                               uint32_t &seq, LockTargets<kT> &X) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool filtered = Q.min_cap == 2;
+  LockQueue B{queues + wid * kQueue, 0};
+  int32_t issued = 0;  // warp 0: pairs in the groups formed so far
+  auto issue = [&](uint32_t n) {  // warp 0: form group n and fetch its filters
+    if (issued >= len) return;
+    const uint32_t sg = n % kStages;
+    int32_t f = kNoFilter, words = 0;
+    const bool in = lane < kGroup && issued + lane < len;
+    if (in) f = Q.rec[first + stride * (issued + lane)].w;
+    if (f != kNoFilter) words = 1 << filter_lg(f);
+    int32_t incl = words;
+    for (int o = 1; o < kGroup; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const uint32_t fits = __ballot_sync(0xffffffffu, in && incl <= kStageWords);
+    const int32_t count = __popc(fits);
+    const int32_t total = __shfl_sync(0xffffffffu, incl, count - 1);
+    const bool mine = lane < count && f != kNoFilter;
+    if (lane < count) S.place[sg][lane] = mine ? incl - words : -1;
+    if (lane == 0) S.pairs[sg] = count;
+    __syncwarp();
+    if (lane == 0) mbar_expect(&S.full[sg], 4u * (uint32_t)total);
+    __syncwarp();
+    if (mine)
+      bulk_load(ring + sg * kStageWords + incl - words, Q.bits + filter_place(f),
+                4u * (uint32_t)words, &S.full[sg]);
+    issued += count;
+  };
+  const uint32_t seq0 = seq;
+  if (filtered && wid == 0)
+    for (uint32_t q = 0; q < kStages - 1; ++q) issue(seq0 + q);
+  int4 nrec = Q.rec[first];
+  int32_t nh = lane < nrec.y ? Q.H[nrec.z + lane] : 0;
+  LockFilter F;
+  F.landed = filtered;
+  for (int32_t gk = 0; gk < len; ++seq) {
+    const uint32_t sg = seq % kStages;
+    int32_t ge = len;
+    if (F.landed) {
+      if (wid == 0 &&
+          __all_sync(0xffffffffu, seq == seq0 || lock_wait(S, &S.empty[(seq - 1) % kStages],
+                                                           ((seq - 1) / kStages) & 1u)))
+        issue(seq + kStages - 1);
+      F.landed = lock_wait(S, &S.full[sg], (seq / kStages) & 1u);
+      F.landed = __all_sync(0xffffffffu, F.landed);
+      if (F.landed) ge = gk + S.pairs[sg];
+    }
+    for (int32_t k = gk; k < ge; ++k) {
+      const int32_t a = first + stride * k;
+      const int4 rec = nrec;
+      const int32_t h32 = nh;
+      if (k + 1 < len) {
+        nrec = Q.rec[a + stride];
+        nh = lane < nrec.y ? Q.H[nrec.z + lane] : 0;
+      }
+      F.has = rec.w != kNoFilter;
+      F.lg = filter_lg(rec.w);
+      F.near = smem_addr(ring + sg * kStageWords + (F.landed ? S.place[sg][(k - gk) & (kGroup - 1)] : 0));
+      F.far = Q.bits + filter_place(rec.w);
+#define SRK_PAIR(C)                                                                           \
+  lock_pair<C, kT, kCount, GA, E>(G, T, Q, F, smem_addr(lists), a, (uint32_t)rec.x, rec.y, h32, \
+                                  Q.H + rec.z, X, B)
+      if (rec.y == 2) SRK_PAIR(2);
+      else if (rec.y == 3) SRK_PAIR(3);
+      else SRK_PAIR(0);
+#undef SRK_PAIR
+    }
+    gk = ge;
+    if (F.landed) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&S.empty[sg]);
+    }
+  }
+  if (B.n > 0) lock_drain(G, T, Q, B, B.n, X.u);
+}
+
+// ------------------------------------- pair records, end nodes, filters --
+
+// Every pair with cap >= 1: its record (pairs sorted by cap, descending), its
+// weight, the identities of its nodes, and its end node in the table.
+__global__ void __launch_bounds__(256)
+k_records(const __grid_constant__ QueryTab tab, GraphView V, Filters F,
+          const int32_t *__restrict__ sigma, const int32_t *__restrict__ seff,
+          const int32_t *__restrict__ spos, int32_t *__restrict__ small_base,
+          int4 *__restrict__ rec, unsigned long long *__restrict__ pair_w,
+          int32_t *__restrict__ H) {
+  __shared__ int32_t P[SRK_MAX_LEN + 2];
+  __shared__ int32_t R[SRK_MAX_LEN + 2];    // cells before the pairs of cap i
+  __shared__ int32_t beg[SRK_MAX_LEN + 2];  // pairs of cap > i
+  Small sm = small_view(small_base);
+  for (int i = threadIdx.x; i <= tab.L + 1; i += blockDim.x) {
+    P[i] = tab.P[i];
+    R[i] = sm.R[i];
+    beg[i] = i <= tab.L ? sm.cnt[i + 1] : 0;
+  }
+  __syncthreads();
+  const int Ls = tab.L > 0 ? tab.L : 1;
+  for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < tab.N_tot;
+       j += gridDim.x * blockDim.x) {
+    const int32_t w = sigma[j];
+    const int l2 = stratum_of(P, tab.L, j);
+    const int32_t cap = min(l2, seff[w]);
+    if (cap < 1) continue;
+    const int l1 = stratum_of(P, tab.L, w);
+    const int32_t a = atomicAdd(&sm.cursor[cap], 1);
+    pair_w[a] = __double2ull_rn(tab.a[l1] * tab.a[l2] * 4294967296.0);
+    const int32_t off = R[cap] + (a - beg[cap]) * cap;
+    rec[a] = make_int4(j, cap, off, kNoFilter);
+    const int32_t *src = spos + (int64_t)w * Ls;
+    for (int i = 0; i < cap; ++i) H[off + i] = node_identity(V, src[i]);
+    if (F.slots) {
+      const uint32_t id = (uint32_t)src[cap - 1], mask = (1u << F.slot_bits) - 1u;
+      const uint32_t hash = end_hash(id), bb = hash >> (32 - F.bloom_bits);
+      atomicOr(&F.bloom[bb >> 5], 1u << (bb & 31));
+      uint32_t sl = hash & mask;
+      for (uint32_t probe = 0; probe <= mask; ++probe, sl = (sl + 1u) & mask) {
+        const uint32_t prev = atomicCAS(&F.slots[sl].key, 0u, id + 1u);
+        if (prev == 0u || prev == id + 1u) break;
+      }
+      F.slot_of[a] = (int32_t)sl;
+      if (cap == 1) F.rank1[a] = atomicAdd(&F.slots[sl].cnt1, 1);
+      else F.slots[sl].filt = kWantFilter;
+    }
+  }
+}
+
+// Room for every slot's list and filter, the filters cleared.
+__global__ void __launch_bounds__(256) k_end_slots(Filters F) {
+  const int lane = threadIdx.x & 31;
+  for (int32_t base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; base < (1 << F.slot_bits);
+       base += gridDim.x * blockDim.x) {
+    EndSlot &S = F.slots[base + lane];
+    if (S.cnt1 > 0) S.off1 = atomicAdd(&F.ctl[1], S.cnt1);
+    int32_t at = -1, units = 0;
+    if (S.filt == kWantFilter) {
+      // 16 bits and more per node of the out-list, so that at most about 6 %
+      // of the other nodes pass, up to the largest size (R-MAT 20: 0.7 KB on
+      // average; one size of 4 KB for all was slower, a block then stops for
+      // its filters every 4 pairs instead of every 11)
+      const int32_t d = F.out_deg[S.key - 1u];
+      int lg = 5;
+      while (lg < kFilterMaxLg && (2 << lg) < d) ++lg;
+      units = (1 << lg) / kFilterUnit;
+      at = atomicAdd(&F.ctl[0], units);
+      if (at > F.max_units - units) at = -1;
+      S.filt = at < 0 ? 0 : 1 + (at << 4 | lg);
+    }
+    for (uint32_t m = __ballot_sync(0xffffffffu, at >= 0); m; m &= m - 1) {
+      const int32_t a0 = __shfl_sync(0xffffffffu, at, __ffs(m) - 1),
+                    nu = __shfl_sync(0xffffffffu, units, __ffs(m) - 1);
+      for (int32_t x = lane; x < nu * kFilterUnit; x += 32)
+        F.bits[(int64_t)a0 * kFilterUnit + x] = 0u;
+    }
+  }
+}
+
+// Every pair's place in its end node's list, or its filter.
+__global__ void __launch_bounds__(256)
+k_end_lists(Filters F, const int32_t *__restrict__ small_base, int4 *__restrict__ rec) {
+  const Small sm = small_view(const_cast<int32_t *>(small_base));
+  for (int32_t a = blockIdx.x * blockDim.x + threadIdx.x; a < sm.cnt[1];
+       a += gridDim.x * blockDim.x) {
+    const EndSlot S = F.slots[F.slot_of[a]];
+    if (a >= sm.cnt[2]) F.list1[S.off1 + F.rank1[a]] = a;
+    else rec[a].w = S.filt - 1;
+  }
+}
+
+// One pass over the edges y -> u (entry k of u's list).  Where y is an end
+// node, u joins its filter, and if u is a target, the pairs of cap 1 that end
+// at y are decided for u, the warp's lanes over the pairs: pair j meets here
+// exactly when its step draws k.  (Every entry that holds y is its own edge,
+// so repeated in-neighbours count once each, as the draw does.)  A bitmap in
+// L1 turns most edges away; R-MAT 20: 0.37 ms for 16.1 M edges.
+__global__ void __launch_bounds__(256)
+k_edges(Filters F, GraphView V, int64_t m,
+        const int4 *__restrict__ rec, const unsigned long long *__restrict__ pair_w, uint32_t key,
+        int32_t s, int32_t u_begin, int32_t u_end, unsigned long long *__restrict__ W,
+        uint32_t *__restrict__ counts) {
+  const int lane = threadIdx.x & 31;
+  const int32_t *row_ptr = V.row_ptr;
+  const uint32_t mask = (1u << F.slot_bits) - 1u;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; e0 < m;
+       e0 += stride) {
+    const int64_t e = e0 + lane;
+    EndSlot S{0u, 0, 0, 0};
+    if (e < m) {
+      const uint32_t y = (uint32_t)V.col[e], hash = end_hash(y), bb = hash >> (32 - F.bloom_bits);
+      if ((F.bloom[bb >> 5] >> (bb & 31)) & 1u) {
+        uint32_t sl = hash & mask;
+        for (uint32_t probe = 0; probe <= mask; ++probe, sl = (sl + 1u) & mask) {
+          const EndSlot T = F.slots[sl];
+          if (T.key == y + 1u) S = T;
+          if (T.key == y + 1u || T.key == 0u) break;
+        }
+      }
+    }
+    int32_t u = 0;
+    uint32_t k = 0, d = 1;
+    if (S.key) {
+      int32_t lo = 0, hi = V.n - 1;  // the node whose list holds edge e
+      while (lo < hi) {
+        const int32_t mid = lo + (hi - lo + 1) / 2;
+        if ((int64_t)row_ptr[mid] <= e) lo = mid; else hi = mid - 1;
+      }
+      u = lo;
+      const int32_t b = row_ptr[u];
+      k = (uint32_t)(e - b);
+      d = (uint32_t)(row_ptr[u + 1] - b);
+      if (S.filt > 0) {
+        const uint32_t f = filter_bit(node_identity(V, u), filter_lg(S.filt - 1));
+        atomicOr(&F.bits[filter_place(S.filt - 1) + (f >> 5)], 1u << (f & 31));
+      }
+    }
+    const bool todo = S.key && S.cnt1 > 0 && u >= u_begin && u < u_end && u != s;
+    for (uint32_t mm = __ballot_sync(0xffffffffu, todo); mm; mm &= mm - 1) {
+      const int l = __ffs(mm) - 1;
+      const int32_t uu = __shfl_sync(0xffffffffu, u, l), cnt = __shfl_sync(0xffffffffu, S.cnt1, l),
+                    off = __shfl_sync(0xffffffffu, S.off1, l);
+      const uint32_t kk = __shfl_sync(0xffffffffu, k, l), dd = __shfl_sync(0xffffffffu, d, l);
+      uint32_t c = 0;
+      unsigned long long ws = 0;
+      for (int32_t q = lane; q < cnt; q += 32) {
+        const int32_t a = F.list1[off + q];
+        const uint32_t j = (uint32_t)rec[a].x;
+        uint32_t x0, x1;
+        philox2(key, walk_ctr0(1, j), (uint32_t)uu, x0, x1);
+        uint32_t idx = __umulhi(x0, dd);
+        const uint32_t lo = x0 * dd;
+        if (lo < dd && lo < (0u - dd) % dd) idx = step_index_redraw(key, 1, j, (uint32_t)uu, dd);
+        if (idx == kk) {
+          ++c;
+          ws += pair_w[a];
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        c += __shfl_xor_sync(0xffffffffu, c, o);
+        ws += __shfl_xor_sync(0xffffffffu, ws, o);
+      }
+      if (lane == 0 && c) {
+        atomicAdd(&W[uu], ws);
+        if (counts) atomicAdd(&counts[uu], c);
+      }
+    }
+  }
+}
+
+// Into how many strided sets the pairs are cut, so that sets x target blocks
+// are units of equal work: up to 16 a block, of at least 128 pairs where there
+// are as many, and as near below a whole number of rounds over the grid as a
+// count within a quarter of the largest gets.
+__device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb, int32_t grid) {
+  const int64_t per_block = (int64_t)n_pairs * n_tb / grid;
+  const int32_t rounds = max(1, (int32_t)min((int64_t)16, per_block / 128));
+  const int32_t most = max(1, min(n_pairs, rounds * grid / n_tb));
+  int32_t best = most;
+  float fill = 0.0f;
+  for (int32_t c = most, k = 0; c > 0 && c >= most - most / 4 && k < 16; --c, ++k) {
+    const float units = (float)(c * n_tb);  // at most rounds x grid, or n_tb: exact
+    const float f = units / ((float)grid * ceilf(units / (float)grid));
+    if (f > fill) {
+      fill = f;
+      best = c;
+    }
+  }
+  return best;
+}
+
+// The walks.  A unit of work is a block of targets and a strided set of
+// pairs; blocks take units from a counter.  A unit's targets keep their lists
+// in shared memory where they fit, for their first steps.  W[u] (in the scores
+// until k_finish) and the counts grow by atomics, at the rare meetings.
+template <int kLayout, bool kCount, int kT>
+__global__ void __launch_bounds__(kLockThreads, kLockBlocks)
+k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act, int32_t *bounds,
+           const __grid_constant__ LockQuery Q) {
+  extern __shared__ __align__(128) unsigned char dyn[];
+  __shared__ LockShared S;
+  const auto G = adj_view<kLayout>(V);
+  using E = decltype(adj_entry(G, 0, 0u));
+  uint32_t *ring = reinterpret_cast<uint32_t *>(dyn);
+  E *lists = reinterpret_cast<E *>(ring + kStages * kStageWords);
+  uint4 *queues = reinterpret_cast<uint4 *>(ring + kStages * kStageWords + kListWords);
+  uint2 *hub = reinterpret_cast<uint2 *>(queues + kQueue * kLockWarps);
+  uint32_t *ctab = reinterpret_cast<uint32_t *>(hub + kHubCache);
+  LockTables tabs{smem_addr(ctab), smem_addr(hub), 0u};
+  constexpr int32_t kLists = kListWords * 4 / (int)sizeof(E);
+  const int32_t act_lo = bounds[2], act_hi = bounds[1];
+  const int32_t n_pairs = Q.cnt[Q.min_cap], n_t = act_hi - act_lo;
+  if (n_pairs == 0 || n_t <= 0) return;
+  const int32_t T = kLockThreads * kT, n_tb = (n_t + T - 1) / T;
+  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
+  const int64_t units = (int64_t)n_tb * n_chunks;
+  if ((int64_t)blockIdx.x >= units) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (threadIdx.x < kStages) {
+    mbar_init(&S.full[threadIdx.x], 1);
+    mbar_init(&S.empty[threadIdx.x], kLockWarps);
+  }
+  if (threadIdx.x == 0) S.broken = 0;
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if constexpr (kLayout == kNarrow) {
+    tabs.n_hub = (uint32_t)min(V.n_hubs, kHubCache);
+    for (uint32_t i = threadIdx.x; i < tabs.n_hub; i += kLockThreads) hub[i] = V.hub[i];
+    for (uint32_t i = threadIdx.x; i <= V.deg_max; i += kLockThreads) ctab[i] = V.ctab[i];
+  }
+  unsigned long long total = 0;
+  uint32_t seq = 0;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) S.unit = atomicAdd(bounds, 1);
+    if (threadIdx.x < 4) S.sums[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t unit = S.unit;
+    if (unit >= units) break;
+    const int32_t tb = (int32_t)(unit % n_tb);
+    const int32_t first = (int32_t)(unit / n_tb), len = (n_pairs - first + n_chunks - 1) / n_chunks;
+    LockTargets<kT> X;
+#pragma unroll
+    for (int t = 0; t < kT; ++t) {
+      const int32_t i = act_lo + tb * T + t * kLockThreads + threadIdx.x;
+      X.u[t] = i < act_hi ? act[i] : 0;
+      X.b[t] = node_start(G, V.row_ptr, X.u[t], X.d[t]);
+      if (i >= act_hi || X.u[t] == Q.s) X.d[t] = 0;
+      X.st[t] = 0;
+      X.at[t] = X.d[t] ? -1 : -2;
+    }
+    if (len >= 32) {
+      // lists of at most 64, 32, 16 or 8 entries go to shared memory: the
+      // largest bound whose lists fit
+      uint32_t sum[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int t = 0; t < kT; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (X.d[t] <= (64u >> q)) sum[q] += X.d[t];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint32_t v = sum[q];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) atomicAdd(&S.sums[q], v);
+      }
+      __syncthreads();
+      int q = 0;
+      while (q < 4 && S.sums[q] > (uint32_t)kLists) ++q;
+      // first the lists below that bound, then the longer ones while they fit
+      uint32_t base = 0;
+      for (int pass = 0; pass < 2; ++pass) {
+        auto wanted = [&](uint32_t d) {
+          return d <= 64u && (pass == (q < 4 && d <= (64u >> q) ? 0 : 1));
+        };
+        uint32_t mine = 0;
+#pragma unroll
+        for (int t = 0; t < kT; ++t)
+          if (wanted(X.d[t])) mine += X.d[t];
+        uint32_t incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        if (lane == 31) S.warp_sum[wid] = incl;
+        __syncthreads();
+        uint32_t at = base + incl - mine;
+        for (int w = 0; w < kLockWarps; ++w) {
+          if (w < wid) at += S.warp_sum[w];
+          base += S.warp_sum[w];
+        }
+#pragma unroll
+        for (int t = 0; t < kT; ++t)
+          if (X.d[t] && wanted(X.d[t])) {
+            if (at + X.d[t] <= (uint32_t)kLists) {
+              X.at[t] = (int32_t)at;
+              for (uint32_t k = 0; k < X.d[t]; ++k) lists[at + k] = adj_entry(G, X.b[t], k);
+            }
+            at += X.d[t];
+          }
+        __syncthreads();
+      }
+    }
+    lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len, seq,
+                               X);
+#pragma unroll
+    for (int t = 0; t < kT; ++t) {
+      if (kCount && X.st[t]) {
+        if (Q.steps) atomicAdd(&Q.steps[X.u[t]], X.st[t]);
+        total += X.st[t];
+      }
+    }
+  }
+  if (kCount) {
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    if (lane == 0 && total) atomicAdd(Q.steps_total, total);
+  }
+}
+
+// Scores from the weight sums, and the steps of the pairs that k_edges decided.
+__global__ void __launch_bounds__(256)
+k_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ bounds,
+         const int32_t *__restrict__ cnt, int32_t s, int32_t u_begin, int32_t u_end, double z,
+         int32_t skipped, double *__restrict__ scores, unsigned long long *__restrict__ wsums,
+         uint32_t *__restrict__ steps, unsigned long long *__restrict__ steps_total) {
+  // pairs of cap 1 decided per edge: one step each of every target
+  const uint32_t one = skipped ? (uint32_t)(cnt[1] - cnt[2]) : 0u;
+  for (int64_t u = (int64_t)u_begin + blockIdx.x * blockDim.x + threadIdx.x; u < u_end;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long W = (unsigned long long)__double_as_longlong(scores[u]);
+    if (wsums) wsums[u] = W;
+    // most targets meet nowhere, and an FP64 division is slow: 0 is 0 / z
+    scores[u] = u == s ? 1.0 : W ? (double)W * 2.3283064365386963e-10 / z : 0.0;
+    if (steps && one && u != s && row_ptr[u + 1] > row_ptr[u]) steps[u] += one;
+  }
+  if (one && blockIdx.x == 0 && threadIdx.x == 0) {
+    int64_t t = bounds[1] - bounds[2];
+    if (s >= u_begin && s < u_end && row_ptr[s + 1] > row_ptr[s]) --t;
+    atomicAdd(steps_total, (unsigned long long)t * one);
+  }
+}
+
+// ------------------------------------------------------------ host side --
+// Sizes (and, with a base, places) the end nodes and filters of one query in
+// at most `avail` bytes; F->slots stays null when the query does without.
+// Returns the bytes taken.
+static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+
+static size_t plan_filters(const srk_graph *g, const QueryTab &t, int64_t n_targets, size_t avail,
+                           Filters *F, char *base) {
+  memset(F, 0, sizeof *F);
+  // They cost a pass over the edges and save about a last step in every pair
+  // and target, some hundred times less each: not for fewer than 8 pairs x
+  // targets an edge (a short target range, a tiny z).  Beyond 2^20 walks the
+  // table of end nodes would outgrow the caches.
+  const int64_t pairs = t.L >= 1 ? t.N_tot - t.P[1] : 0;
+  if (t.literal || pairs == 0 || g->m == 0 || t.N_tot > (1 << 20) ||
+      (double)pairs * (double)n_targets < 8.0 * (double)g->m)
+    return 0;
+  int sb = 5;
+  while (((int64_t)1 << sb) < 2 * std::min<int64_t>(pairs, g->n)) ++sb;
+  F->slot_bits = sb;
+  F->bloom_bits = std::min(20, sb + 3);
+  const size_t fixed = align_up((size_t)16 << sb) + align_up((size_t)1 << (F->bloom_bits - 3)) + 256;
+  if (avail < fixed) return 0;
+  // room for 2 KB per end node of a longer pair; those beyond do without
+  const size_t unit = 4 * kFilterUnit;
+  const int64_t wanted = std::min<int64_t>(t.L >= 2 ? t.N_tot - t.P[2] : 0, g->n);
+  const size_t room = std::min<size_t>(std::min<size_t>(avail - fixed, (size_t)32 << 20),
+                                       (size_t)wanted * 2048 + 65536);
+  F->max_units = (int32_t)(room / unit);
+  F->out_deg = g->out_deg;
+  F->slots = reinterpret_cast<EndSlot *>(base);
+  F->bloom = reinterpret_cast<uint32_t *>(base + align_up((size_t)16 << sb));
+  F->ctl = reinterpret_cast<int32_t *>(base + fixed - 256);
+  F->bits = reinterpret_cast<uint32_t *>(base + fixed);
+  return fixed + unit * (size_t)F->max_units;
+}
+
+size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets) {
+  Filters F;
+  return plan_filters(g, t, n_targets, SIZE_MAX, &F, nullptr);
+}
+
+
+static int grid_for(int64_t work, int threads, int device) {
+  const int64_t want = (work + threads - 1) / threads;
+  const int64_t cap = (int64_t)sm_count(device) * 8;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
+}
+
+// Lets the lockstep kernels take their shared memory (above the default 48 KB
+// a kernel must opt in).  Called at graph load, in the context the queries
+// run in and outside any capture.
+template <int kLayout>
+static cudaError_t allow_lock_t() {
+  cudaError_t e = cudaSuccess;
+  auto set = [&](const void *f) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLockSmem);
+  };
+  set((const void *)k_lockstep<kLayout, false, 1>);
+  set((const void *)k_lockstep<kLayout, true, 1>);
+  set((const void *)k_lockstep<kLayout, false, kLockTargets>);
+  set((const void *)k_lockstep<kLayout, true, kLockTargets>);
+  return e;
+}
+cudaError_t allow_lockstep(int layout) {
+  return layout == kWide ? allow_lock_t<kWide>()
+         : layout == kCsr ? allow_lock_t<kCsr>()
+                          : allow_lock_t<kNarrow>();
+}
+
+template <int kLayout, bool kCount>
+static void launch_lockstep(const GraphView &V, const int32_t *act, int32_t *bounds,
+                            const LockQuery &Q, bool one, int grid, cudaStream_t st) {
+  if (one)
+    k_lockstep<kLayout, kCount, 1><<<grid, kLockThreads, kLockSmem, st>>>(V, act, bounds, Q);
+  else
+    k_lockstep<kLayout, kCount, kLockTargets><<<grid, kLockThreads, kLockSmem, st>>>(V, act, bounds,
+                                                                                     Q);
+}
+
+int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Outputs &o,
+                  char *extra, size_t extra_bytes, bool count, cudaStream_t st,
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end) {
+  const int dev = g->device;
+  const int gN = grid_for(t.N_tot, 256, dev);
+  const int64_t nr = (int64_t)u_end - u_begin;
+  const GraphView V = view_of(g);
+  Filters F;
+  plan_filters(g, t, nr, extra ? extra_bytes : 0, &F, extra);
+  // the Fisher-Yates arrays are free after k_pairs; the pair records take the
+  // first four (16 bytes a pair), kdraw to grp_off
+  F.list1 = w.items;
+  F.slot_of = w.first;
+  F.rank1 = w.succ;
+  int4 *rec = reinterpret_cast<int4 *>(w.kdraw);
+  const Small sm = small_view(w.small);
+  int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
+  unsigned long long *W = reinterpret_cast<unsigned long long *>(o.scores);
+  cudaError_t e = cudaSuccess;
+  if (F.slots) {
+    e = cudaMemsetAsync(F.slots, 0, (size_t)((char *)F.ctl + 256 - (char *)F.slots), st);
+    if (e != cudaSuccess) return cuda_fail(e, "clearing the end nodes");
+  }
+  k_records<<<gN, 256, 0, st>>>(t, V, F, w.sigma, w.seff, w.spos, w.small, rec, w.pair_w, w.Hc);
+  if (F.slots) {
+    k_end_slots<<<grid_for((int64_t)1 << F.slot_bits, 256, dev), 256, 0, st>>>(F);
+    k_end_lists<<<gN, 256, 0, st>>>(F, w.small, rec);
+    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, rec, w.pair_w, t.tkey, t.s,
+                                                      u_begin, u_end, W, o.counts);
+  }
+  LockQuery Q;
+  Q.rec = rec;
+  Q.w = w.pair_w;
+  Q.H = w.Hc;
+  Q.bits = F.bits;
+  Q.cnt = sm.cnt;
+  Q.W = W;
+  Q.counts = o.counts;
+  Q.steps = o.steps;
+  Q.steps_total = sm.ctr;
+  Q.key = t.tkey;
+  for (int r = 0; r < 10; ++r) Q.rk[r] = t.tkey + (uint32_t)r * kPhiloxW0;
+  Q.s = t.s;
+  Q.min_cap = F.slots ? 2 : 1;
+  if (timing) cudaEventRecord(timing[0], st);
+  const int grid = sm_count(dev) * kLockBlocks;
+  const bool one = nr <= kLockThreads;  // too few targets to give a thread several
+  if (g->layout == kWide) {
+    if (count) launch_lockstep<kWide, true>(V, g->act, bounds, Q, one, grid, st);
+    else launch_lockstep<kWide, false>(V, g->act, bounds, Q, one, grid, st);
+  } else if (g->layout == kCsr) {
+    if (count) launch_lockstep<kCsr, true>(V, g->act, bounds, Q, one, grid, st);
+    else launch_lockstep<kCsr, false>(V, g->act, bounds, Q, one, grid, st);
+  } else {
+    if (count) launch_lockstep<kNarrow, true>(V, g->act, bounds, Q, one, grid, st);
+    else launch_lockstep<kNarrow, false>(V, g->act, bounds, Q, one, grid, st);
+  }
+  if (timing) cudaEventRecord(timing[1], st);
+  if (nr > 0)
+    k_finish<<<grid_for(nr, 256, dev), 256, 0, st>>>(g->row_ptr, bounds, sm.cnt, t.s, u_begin,
+                                                     u_end, t.z, F.slots ? 1 : 0, o.scores,
+                                                     o.wsums, o.steps, sm.ctr);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
+  return SRK_OK;
+}
+
+}  // namespace srk

@@ -134,7 +134,8 @@ extern "C" int srk_single_source_noalloc(const srk_graph *g, int32_t s, double c
   o.wsums = reinterpret_cast<unsigned long long *>(weight_sums);
   o.steps = step_counts;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  rc = enqueue_query(g, t, w, o, st,
+  rc = enqueue_query(g, t, w, o, base + need, SRK_NOALLOC_SCRATCH_BYTES - need,
+                     o.steps || (opt && opt->stats), st,
                      opt ? (const cudaEvent_t *)opt->timing_events : nullptr, u_begin, u_end);
   if (!rc && opt && opt->stats) rc = read_stats(t, w, st, opt->stats, false);
   return rc;

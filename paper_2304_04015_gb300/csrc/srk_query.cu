@@ -7,13 +7,13 @@
 //                        the Fisher-Yates permutation sigma (Section 4.1(b),
 //                        Section 5.2), resolved in parallel (see k_pairs), and
 //                        each pair's step cap min(l2, steps of source walk)
-//       k_rows, k_hit_table
-//                        pairs sorted by cap (descending) and the step-major
-//                        hit table: row i holds, for every pair that can still
-//                        meet at step i, the source walk's node at step i
-//   a4+a5 k_target_walks the hot loop: every target walks its pairs, detects
-//                        the first meeting (Lemma 2, Algorithm 2, Section 5.5)
-//                        and writes count, weight sum and score
+//       k_rows           pairs sorted by cap (descending): where each cap's
+//                        pairs begin
+//   a4+a5 enqueue_walks  (srk_lockstep.cu) the targets' walks
+//       k_literal_walks  the same with the literal target shuffle, on a
+//                        step-major hit table (k_hit_table): row i holds, for
+//                        every pair that can still meet at step i, the source
+//                        walk's node at step i
 #include <stdint.h>
 #include <string.h>
 
@@ -28,15 +28,13 @@ namespace srk {
 // Walk r of the source has length l = stratum(r).  Step i >= 1 moves to
 // I(x)[k], k the bounded draw below |I(x)| from word (i-1)&1 of the
 // Philox2x32-10 block (((i-1)>>1) << 24 | r, s) under the source's walk key
-// (step_entry); it stops early at a node with no in-neighbours.  Walks run
-// on the graph's adjacency layout (a packed copy
-// in which nodes are identified by their position, or the CSR itself).  The
-// same thread computes Fisher-Yates draw t = r, k_t = floor(R * (t+1) / 2^64)
-// with R from counter (t>>1, ~0, ~0, s).
-template <int kLayout>
+// (step_entry); it stops early at a node with no in-neighbours.  The source's
+// walks run on the CSR, so spos holds node ids: the filters (srk_filter.cu)
+// look ids up, and the hit lists translate them once.  The same thread
+// computes Fisher-Yates draw t = r, k_t = floor(R * (t+1) / 2^64) with R from
+// counter (t>>1, ~0, ~0, s).
 __global__ void __launch_bounds__(256)
 k_source_walks(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-               const uint32_t *__restrict__ adj, const int32_t *__restrict__ npos, int pos_bits,
                const __grid_constant__ QueryTab tab,
                int32_t *__restrict__ spos, int32_t *__restrict__ seff,
                int32_t *__restrict__ kdraw, int32_t *__restrict__ grp_cnt,
@@ -47,7 +45,7 @@ k_source_walks(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ 
   const RoundKeys rk = round_keys(tab.key0, tab.key1);
   const int Ls = tab.L > 0 ? tab.L : 1;
   const uint32_t s = (uint32_t)tab.s;
-  const auto G = adj_view<kLayout>(adj, npos, pos_bits, row_ptr, col);
+  const AdjC G{row_ptr, col};
   uint32_t deg_s = 0;
   const int32_t b_s = node_start(G, row_ptr, tab.s, deg_s);
   unsigned long long steps = 0;
@@ -185,13 +183,15 @@ k_pairs(const __grid_constant__ QueryTab tab, const int32_t *__restrict__ kdraw,
     if (hist[i]) atomicAdd(&sm.cap_hist[i], hist[i]);
 }
 
-// Hit-table geometry: pairs sorted by cap, descending.  Row i (i = 1..L) has
-// cnt[i] = #pairs with cap >= i entries and starts at R[i].
-// Also finds [act_lo, act_hi), the part of the ascending active-target list
-// `act` inside [u_begin, u_end): the target kernel's work counter starts at
-// act_lo, and act_hi is stored in the word after it.
-__global__ void k_rows(int L, int32_t *__restrict__ small_base, const int32_t *__restrict__ act,
-                       int32_t n_act, int32_t n, int32_t u_begin, int32_t u_end) {
+// Pairs sorted by cap, descending: cnt[i] = #pairs with cap >= i.  R[i] is
+// where the nodes of the pairs of cap i begin, or, in the literal mode, where
+// row i of the hit table begins.  Also finds [act_lo, act_hi), the part of the
+// ascending active-target list `act` inside [u_begin, u_end): words 1 and 2
+// after the work counter, which starts at 0 (units) or, in the literal mode, at
+// act_lo.
+__global__ void k_rows(int L, bool literal, int32_t *__restrict__ small_base,
+                       const int32_t *__restrict__ act, int32_t n_act, int32_t n, int32_t u_begin,
+                       int32_t u_end) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   Small sm = small_view(small_base);
   int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);  // counter, act_hi
@@ -204,7 +204,8 @@ __global__ void k_rows(int L, int32_t *__restrict__ small_base, const int32_t *_
     }
     return lo;
   };
-  bounds[0] = u_begin == 0 ? 0 : lower_bound(u_begin);
+  bounds[2] = u_begin == 0 ? 0 : lower_bound(u_begin);
+  bounds[0] = literal ? bounds[2] : 0;
   bounds[1] = u_end == n ? n_act : lower_bound(u_end);
   int32_t c = 0;
   sm.cnt[L + 1] = 0;
@@ -214,9 +215,17 @@ __global__ void k_rows(int L, int32_t *__restrict__ small_base, const int32_t *_
     sm.cnt[i] = c;
   }
   int32_t r = 0;
-  for (int i = 1; i <= L + 1; ++i) {
-    sm.R[i] = r;
-    if (i <= L) r += sm.cnt[i];
+  if (literal) {
+    for (int i = 1; i <= L + 1; ++i) {
+      sm.R[i] = r;
+      if (i <= L) r += sm.cnt[i];
+    }
+  } else {
+    for (int i = L; i >= 1; --i) {  // the nodes of longer pairs come first
+      sm.R[i] = r;
+      r += i * sm.cap_hist[i];
+    }
+    sm.R[L + 1] = r;
   }
   sm.cnt[0] = c;
   sm.R[0] = 0;
@@ -226,7 +235,7 @@ __global__ void k_rows(int L, int32_t *__restrict__ small_base, const int32_t *_
 // hit table with the source walk's nodes at steps 1..cap.  The pair's Lemma 7
 // weight is round(a(l1) a(l2) 2^32) with l1 the source walk's length.
 __global__ void __launch_bounds__(256)
-k_hit_table(const __grid_constant__ QueryTab tab, const int32_t *__restrict__ sigma,
+k_hit_table(const __grid_constant__ QueryTab tab, GraphView V, const int32_t *__restrict__ sigma,
             const int32_t *__restrict__ seff, const int32_t *__restrict__ spos,
             int32_t *__restrict__ small_base, int32_t *__restrict__ pair_j,
             unsigned long long *__restrict__ pair_w, int32_t *__restrict__ Hc) {
@@ -252,18 +261,17 @@ k_hit_table(const __grid_constant__ QueryTab tab, const int32_t *__restrict__ si
     pair_w[a] = tab.literal ? (unsigned long long)l1
                             : __double2ull_rn(tab.a[l1] * tab.a[l2] * 4294967296.0);
     const int32_t *src = spos + (int64_t)w * Ls;
-    for (int i = 1; i <= cap; ++i) Hc[R[i] + a] = src[i - 1];
+    for (int i = 1; i <= cap; ++i) Hc[R[i] + a] = node_identity(V, src[i - 1]);
   }
 }
 
-// -------------------------------------------------------------- steps a4-a5 --
+// ---------------------------------- steps a4-a5 with the literal shuffle --
 // Each warp takes targets u from a global counter.  Its 32 lanes walk the
 // target's pairs a = 0, 1, ... of the cap-sorted list; a lane whose walk ends
 // takes the next unassigned pair at once (lane refill), so walks that end
-// early (cap, meeting, no in-neighbours) do not idle the warp.  Walks run on
-// the packed adjacency: from a node at position p with degree d, a step reads
-// entry adj[p + 1 + index], which holds the next node's position and, unless
-// that node's degree is large, its degree as well.  Pair a (original index
+// early (cap, meeting, no in-neighbours) do not idle the warp.  (Pairs differ
+// from target to target here, so the lockstep form has nothing to share.)
+// Walks run on the packed adjacency.  Pair a (original index
 // j) walks from u: one Philox2x32-10 block, counter (((i-1)>>1) << 24 | j, u)
 // under the target walks' key, serves the odd step i (word 0) and the even
 // step i+1 (word 1).  A step moves to I(x)[k], k the bounded draw below |I(x)|
@@ -273,11 +281,7 @@ k_hit_table(const __grid_constant__ QueryTab tab, const int32_t *__restrict__ si
 // to W_u.  The warp then reduces and writes count, W and s~(s,u) = W 2^-32 / z
 // (s~(s,s) = 1).
 struct TargetArgs {
-  const int32_t *row_ptr;  // CSR offsets (wide and CSR layouts locate nodes by them)
-  const int32_t *col;      // in-neighbour lists (CSR layout)
-  const uint32_t *adj;     // packed adjacency (see srk_internal.h)
-  const int32_t *npos;     // 4-byte-entry layout: node positions
-  int32_t pos_bits;
+  GraphView view;
   int32_t n, s, L;
   uint32_t walk_key;       // walk key of the target walks (the source's or the shared one)
   uint32_t key0, key1;
@@ -294,10 +298,10 @@ struct TargetArgs {
   int32_t *target_counter;  // next index into act (from act_lo), then act_hi
   const int32_t *act;       // the targets with in-neighbours, ascending
   int32_t u_begin, u_end;   // targets computed: [u_begin, u_end)
-  int32_t N_tot;            // literal mode: the permutation's domain
+  int32_t N_tot;            // the permutation's domain
 };
 
-// Literal mode also needs the stratum prefix and the Lemma 7 weights.
+// The stratum prefix and the Lemma 7 weights.
 struct LiteralArgs {
   int32_t P[SRK_MAX_LEN + 2];
   double a[SRK_MAX_LEN + 1];
@@ -305,24 +309,24 @@ struct LiteralArgs {
 
 // 8 blocks of 256 threads per SM (32 registers): the kernel is bound by the
 // rate of scattered L1 misses, and full occupancy keeps the most misses in
-// flight.  kLiteral: the literal target shuffle (walk_target_literal).
-template <bool kLiteral, int kLayout>
+// flight.
+template <int kLayout>
 __global__ void __launch_bounds__(256, 8)
-k_target_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ LiteralArgs X) {
+k_literal_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ LiteralArgs X) {
   __shared__ int2 rc[SRK_MAX_LEN + 3];  // {R[i], cnt[i+1]}, one load per step
-  __shared__ int32_t Psh[kLiteral ? SRK_MAX_LEN + 2 : 1];
+  __shared__ int32_t Psh[SRK_MAX_LEN + 2];
   {
     const Small sm = small_view(const_cast<int32_t *>(A.small_base));
     for (int i = threadIdx.x; i <= A.L + 2; i += blockDim.x) {
       rc[i] = make_int2((i <= A.L + 1) ? sm.R[i] : 0,
                         (i + 1 <= A.L + 1) ? sm.cnt[i + 1] : 0);  // cnt[L+1] = cnt[L+2] = 0
-      if (kLiteral && i <= A.L + 1) Psh[i] = X.P[i];
+      if (i <= A.L + 1) Psh[i] = X.P[i];
     }
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const uint32_t lanes_below = (1u << lane) - 1u;
-  const auto G = adj_view<kLayout>(A.adj, A.npos, A.pos_bits, A.row_ptr, A.col);
+  const auto G = adj_view<kLayout>(A.view);
   PairSet S;
   S.rc = rc;
   S.pair_j = A.pair_j;
@@ -330,9 +334,8 @@ k_target_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ Lit
   S.Hc = A.Hc;
   S.n_pairs = rc[0].y;  // cnt[1]
   S.key = A.walk_key;
-  FeistelShape fs;
-  if constexpr (kLiteral)
-    fs = feistel_shape(A.N_tot, ((uint64_t)A.key1 << 32) | A.key0, (uint32_t)A.s);
+  const FeistelShape fs =
+      feistel_shape(A.N_tot, ((uint64_t)A.key1 << 32) | A.key0, (uint32_t)A.s);
   unsigned long long warp_steps = 0;
   // the active targets act[counter .. act_hi) (k_rows set the counter to the
   // range's first index and act_hi beside it); the outputs of the others
@@ -351,14 +354,10 @@ k_target_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ Lit
     uint32_t c = 0, st = 0;
     unsigned long long W = 0;
     uint32_t deg_u = 0;
-    const int32_t b_u = node_start(G, A.row_ptr, u, deg_u);
-    if (u != A.s && deg_u > 0) {
-      if (kLiteral)
-        walk_target_literal(G, S, fs, Psh, A.L, X.a, (uint32_t)u, b_u, deg_u,
-                            lanes_below, c, W, st);
-      else
-        walk_target(G, S, (uint32_t)u, b_u, deg_u, c, W, st);
-    }
+    const int32_t b_u = node_start(G, A.view.row_ptr, u, deg_u);
+    if (u != A.s && deg_u > 0)
+      walk_target_literal(G, S, fs, Psh, A.L, X.a, (uint32_t)u, b_u, deg_u, lanes_below, c, W,
+                          st);
     for (int off = 16; off > 0; off >>= 1) {
       c += __shfl_xor_sync(0xffffffffu, c, off);
       st += __shfl_xor_sync(0xffffffffu, st, off);
@@ -419,7 +418,7 @@ static int target_grid(int device) {
   static int blocks_per_sm[64] = {};
   int b = (device >= 0 && device < 64) ? blocks_per_sm[device] : 0;
   if (!b) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_target_walks<false, kNarrow>, 256, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_literal_walks<kNarrow>, 256, 0) !=
             cudaSuccess || b < 1)
       b = 1;
     if (device >= 0 && device < 64) blocks_per_sm[device] = b;
@@ -430,92 +429,74 @@ static int target_grid(int device) {
 // Enqueues one query on `st` with device-resident outputs `o`.  Workspace
 // `w` (already carved) must hold plan(t) bytes.
 int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
-                  const Outputs &o, cudaStream_t st, const cudaEvent_t *timing,
-                  int32_t u_begin, int32_t u_end) {
+                  const Outputs &o, char *extra, size_t extra_bytes, bool count, cudaStream_t st,
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end) {
   const int dev = g->device;
   const int N = t.N_tot;
   const int gN = grid_for(N, 256, dev);
   cudaError_t e = cudaMemsetAsync(w.small, 0, kSmallBytes, st);
   if (e != cudaSuccess) return cuda_fail(e, "clearing query counters");
-  if (g->layout == kWide)
-    k_source_walks<kWide><<<gN, 256, 0, st>>>(g->row_ptr, g->col, g->adj, g->npos, g->pos_bits, t,
-                                              w.spos, w.seff, w.kdraw, w.grp_cnt, w.small);
-  else if (g->layout == kCsr)
-    k_source_walks<kCsr><<<gN, 256, 0, st>>>(g->row_ptr, g->col, g->adj, g->npos, g->pos_bits, t,
-                                             w.spos, w.seff, w.kdraw, w.grp_cnt, w.small);
-  else
-    k_source_walks<kNarrow><<<gN, 256, 0, st>>>(g->row_ptr, g->col, g->adj, g->npos, g->pos_bits, t,
-                                                w.spos, w.seff, w.kdraw, w.grp_cnt, w.small);
+  k_source_walks<<<gN, 256, 0, st>>>(g->row_ptr, g->col, t, w.spos, w.seff, w.kdraw, w.grp_cnt,
+                                     w.small);
   k_fy_rank<<<gN, 256, 0, st>>>(w.kdraw, w.grp_cnt, w.rank, N);
   k_scan<<<1, 1024, 0, st>>>(w.grp_cnt, w.grp_off, N);
   k_fy_scatter<<<gN, 256, 0, st>>>(w.kdraw, w.grp_off, w.rank, w.items, N);
   k_fy_groups<<<gN, 256, 0, st>>>(w.grp_off, w.items, w.first, w.succ, N);
   k_pairs<<<gN, 256, 0, st>>>(t, w.kdraw, w.first, w.succ, w.seff, w.sigma, w.small);
-  k_rows<<<1, 32, 0, st>>>(t.L, w.small, g->act, g->n_act, g->n, u_begin, u_end);
+  k_rows<<<1, 32, 0, st>>>(t.L, t.literal != 0, w.small, g->act, g->n_act, g->n, u_begin, u_end);
   // targets without in-neighbours have zero outputs (and s, if it is one of
-  // them, the score 1 the kernel writes): clear the range, then walk only
-  // the active targets
+  // them, the score 1): clear the range, then walk only the active targets
   const size_t nr = (size_t)(u_end - u_begin);
   if (nr > 0) {
     e = cudaMemsetAsync(o.scores + u_begin, 0, sizeof(double) * nr, st);
     if (e == cudaSuccess && o.counts)
       e = cudaMemsetAsync(o.counts + u_begin, 0, sizeof(uint32_t) * nr, st);
-    if (e == cudaSuccess && o.wsums)
+    if (e == cudaSuccess && o.wsums && t.literal)
       e = cudaMemsetAsync(o.wsums + u_begin, 0, sizeof(unsigned long long) * nr, st);
     if (e == cudaSuccess && o.steps)
       e = cudaMemsetAsync(o.steps + u_begin, 0, sizeof(uint32_t) * nr, st);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the outputs of the target range");
   }
-  k_hit_table<<<gN, 256, 0, st>>>(t, w.sigma, w.seff, w.spos, w.small, w.pair_j,
-                                  w.pair_w, w.Hc);
-  TargetArgs A;
-  A.row_ptr = g->row_ptr;
-  A.col = g->col;
-  A.adj = g->adj;
-  A.npos = g->npos;
-  A.pos_bits = g->pos_bits;
-  A.n = g->n;
-  A.s = t.s;
-  A.walk_key = t.tkey;
-  A.L = t.L;
-  A.key0 = t.key0;
-  A.key1 = t.key1;
-  A.z = t.z;
-  A.small_base = w.small;
-  A.pair_j = w.pair_j;
-  A.pair_w = w.pair_w;
-  A.Hc = w.Hc;
-  A.scores = o.scores;
-  A.counts = o.counts;
-  A.wsums = o.wsums;
-  A.steps_per_target = o.steps;
-  A.steps_total = small_view(w.small).ctr;
-  A.target_counter = reinterpret_cast<int32_t *>(small_view(w.small).ctr + 2);
-  A.act = g->act;
-  A.u_begin = u_begin;
-  A.u_end = u_end;
-  A.N_tot = t.N_tot;
-  LiteralArgs X;
+  const GraphView V = view_of(g);
   if (t.literal) {
+    k_hit_table<<<gN, 256, 0, st>>>(t, V, w.sigma, w.seff, w.spos, w.small, w.pair_j, w.pair_w,
+                                    w.Hc);
+    TargetArgs A;
+    A.view = V;
+    A.n = g->n;
+    A.s = t.s;
+    A.walk_key = t.tkey;
+    A.L = t.L;
+    A.key0 = t.key0;
+    A.key1 = t.key1;
+    A.z = t.z;
+    A.small_base = w.small;
+    A.pair_j = w.pair_j;
+    A.pair_w = w.pair_w;
+    A.Hc = w.Hc;
+    A.scores = o.scores;
+    A.counts = o.counts;
+    A.wsums = o.wsums;
+    A.steps_per_target = o.steps;
+    A.steps_total = small_view(w.small).ctr;
+    A.target_counter = reinterpret_cast<int32_t *>(small_view(w.small).ctr + 2);
+    A.act = g->act;
+    A.u_begin = u_begin;
+    A.u_end = u_end;
+    A.N_tot = t.N_tot;
+    LiteralArgs X;
     memcpy(X.P, t.P, sizeof X.P);
     memcpy(X.a, t.a, sizeof X.a);
-  } else {
-    memset(&X, 0, sizeof X);
+    if (timing) cudaEventRecord(timing[0], st);
+    const int tg = target_grid(dev);
+    if (g->layout == kWide) k_literal_walks<kWide><<<tg, 256, 0, st>>>(A, X);
+    else if (g->layout == kCsr) k_literal_walks<kCsr><<<tg, 256, 0, st>>>(A, X);
+    else k_literal_walks<kNarrow><<<tg, 256, 0, st>>>(A, X);
+    if (timing) cudaEventRecord(timing[1], st);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? SRK_OK : cuda_fail(e, "kernel launch");
   }
-  if (timing) cudaEventRecord(timing[0], st);
-  const int tg = target_grid(dev);
-  switch (g->layout * 2 + (t.literal ? 1 : 0)) {
-    case 2 * kWide: k_target_walks<false, kWide><<<tg, 256, 0, st>>>(A, X); break;
-    case 2 * kWide + 1: k_target_walks<true, kWide><<<tg, 256, 0, st>>>(A, X); break;
-    case 2 * kCsr: k_target_walks<false, kCsr><<<tg, 256, 0, st>>>(A, X); break;
-    case 2 * kCsr + 1: k_target_walks<true, kCsr><<<tg, 256, 0, st>>>(A, X); break;
-    case 2 * kNarrow + 1: k_target_walks<true, kNarrow><<<tg, 256, 0, st>>>(A, X); break;
-    default: k_target_walks<false, kNarrow><<<tg, 256, 0, st>>>(A, X); break;
-  }
-  if (timing) cudaEventRecord(timing[1], st);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
-  return SRK_OK;
+  return enqueue_walks(g, t, w, o, extra, extra_bytes, count, st, timing, u_begin, u_end);
 }
 
 // The target range of a query from its options: [0, n) by default.
@@ -566,6 +547,13 @@ extern "C" int srk_single_source(const srk_graph *g, int32_t s, double c,
                                  double eps, uint64_t seed, const srk_opts *opt,
                                  double *scores, uint32_t *meet_counts,
                                  uint64_t *weight_sums, void *cuda_stream) {
+  return single_source(g, s, c, eps, seed, opt, scores, meet_counts, weight_sums, cuda_stream,
+                       SIZE_MAX);
+}
+
+int srk::single_source(const srk_graph *g, int32_t s, double c, double eps, uint64_t seed,
+                       const srk_opts *opt, double *scores, uint32_t *meet_counts,
+                       uint64_t *weight_sums, void *cuda_stream, size_t extra_limit) {
   clear_error();
   if (!g) return fail(SRK_EINVAL, "null graph");
   if (!scores) return fail(SRK_EINVAL, "scores is null");
@@ -598,8 +586,15 @@ extern "C" int srk_single_source(const srk_graph *g, int32_t s, double c,
   if (!d_steps) ws += align_up(4 * n);
   cudaMemPool_t mp = pool(g->device);
   if (!mp) return fail(SRK_ECUDA, "cannot create the device memory pool");
+  const size_t o_extra = ws;
+  size_t extra = std::min(extra_limit, filter_bytes(g, t, (int64_t)(u_end - u_begin)));
   char *base = nullptr;
-  cudaError_t e = cudaMallocFromPoolAsync((void **)&base, ws, mp, st);
+  cudaError_t e = cudaMallocFromPoolAsync((void **)&base, ws + extra, mp, st);
+  if (e == cudaErrorMemoryAllocation && extra > 0) {  // the query can do without filters
+    cudaGetLastError();
+    extra = 0;
+    e = cudaMallocFromPoolAsync((void **)&base, ws, mp, st);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");
   plan(t, &w, base);
   Outputs o;
@@ -608,7 +603,7 @@ extern "C" int srk_single_source(const srk_graph *g, int32_t s, double c,
   o.wsums = d_wsums ? (unsigned long long *)weight_sums
                     : (unsigned long long *)(base + o_wsums);
   o.steps = d_steps ? step_counts : (uint32_t *)(base + o_steps);
-  rc = enqueue_query(g, t, w, o, st,
+  rc = enqueue_query(g, t, w, o, base + o_extra, extra, o.steps || (opt && opt->stats), st,
                      opt ? (const cudaEvent_t *)opt->timing_events : nullptr, u_begin, u_end);
   bool host_out = !d_scores || !d_counts || !d_wsums || !d_steps;
   if (!rc) {  // host outputs: copy back the computed range only

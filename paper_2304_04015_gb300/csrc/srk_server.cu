@@ -44,6 +44,7 @@ struct Request {
   uint64_t seed, tag;
   double *host_scores;
   size_t bytes;  // reserved device memory
+  size_t extra;  // end-filter scratch it runs with when the budget has room
   double pairs;  // (targets with in-neighbours) x N_tot, 0 when s has none
   double work;   // estimated seconds of service
   uint64_t order;
@@ -72,6 +73,10 @@ struct srk_server {
   std::vector<std::thread> workers;
   bool stop = false;
   size_t reserved = 0, reserved_peak = 0;
+  // Device bytes of the requests now running, and the filter scratch some of
+  // them run with on top (only ever from what the budget has left).
+  size_t running_bytes = 0, extra_bytes = 0;
+  std::condition_variable cv_extra;
   int running = 0;
   uint64_t submitted = 0, admitted = 0, shed = 0, completed = 0, failed = 0;
   uint64_t target_steps = 0;
@@ -100,6 +105,15 @@ static void worker_main(srk_server *srv, int device) {
       r = *pick;
       srv->queue.erase(pick);
       ++srv->running;
+      // requests admitted after others took filter scratch may find the budget
+      // full: that scratch comes back as those finish
+      srv->cv_extra.wait(lk, [&] {
+        return srv->running_bytes + srv->extra_bytes + r.bytes <= srv->budget ||
+               srv->extra_bytes == 0;
+      });
+      srv->running_bytes += r.bytes;
+      if (srv->reserved + srv->extra_bytes + r.extra <= srv->budget) srv->extra_bytes += r.extra;
+      else r.extra = 0;
     }
     const srk_graph *g = srv->graphs[(size_t)r.graph];
     double *d_scores = nullptr;
@@ -114,7 +128,8 @@ static void worker_main(srk_server *srv, int device) {
                                             pool(g->device), st);
     if (e != cudaSuccess) rc = SRK_ENOMEM;
     if (rc == SRK_OK)
-      rc = srk_single_source(g, r.s, r.c, r.eps, r.seed, &opt, d_scores, nullptr, nullptr, st);
+      rc = single_source(g, r.s, r.c, r.eps, r.seed, &opt, d_scores, nullptr, nullptr, st,
+                         r.extra);
     if (rc == SRK_OK && r.host_scores)
       e = cudaMemcpyAsync(r.host_scores, d_scores, sizeof(double) * (size_t)g->n,
                           cudaMemcpyDeviceToHost, st);
@@ -125,6 +140,9 @@ static void worker_main(srk_server *srv, int device) {
       std::lock_guard<std::mutex> lk(srv->mu);
       --srv->running;
       srv->reserved -= r.bytes;
+      srv->running_bytes -= r.bytes;
+      srv->extra_bytes -= r.extra;
+      srv->cv_extra.notify_all();
       srv->queued_work -= r.work;
       if (srv->queued_work < 0.0) srv->queued_work = 0.0;
       if (rc == SRK_OK) {
@@ -278,6 +296,7 @@ extern "C" int srk_server_submit(srk_server *srv, int32_t graph, int32_t s, doub
   r.tag = tag;
   r.host_scores = host_scores;
   r.bytes = bytes;
+  r.extra = filter_bytes(g, t, g->n);
   r.pairs = pairs;
   r.t_submit = Clock::now();
   std::lock_guard<std::mutex> lk(srv->mu);

@@ -1,0 +1,92 @@
+"""The lockstep target walks and their end filters against the CPU oracle.
+
+All outputs are integers or functions of one integer, so every comparison is
+exact.  The cases sit at the edges of the kernel's tiles: 448 targets per pass
+of a block's threads, 3 per thread, groups of 16 pairs, 32 nodes of a pair in
+a warp's lanes, the smallest and the largest filter, lists around the bounds
+of what goes to shared memory, hubs within and beyond the cached records.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_parity import assert_parity, gpu_query, oracle_query, srk  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def ring_lists(n, d, seed):
+    """Every node has exactly d in-neighbours (so the number of targets is n)."""
+    rng = np.random.default_rng(seed)
+    col = np.sort((np.arange(n)[:, None] + rng.integers(1, n, size=(n, d))) % n, axis=1)
+    return np.arange(0, n * d + 1, d, dtype=np.int32), col.astype(np.int32).ravel()
+
+
+@pytest.mark.parametrize("n", [2, 31, 447, 448, 449, 1343, 1345, 2689])
+def test_target_blocks(srk, n):
+    # repeated entries in a list are separate draws: keep the duplicates
+    rp, col = ring_lists(n, 3, n)
+    kw = dict(z_override=700.0, L_override=12)
+    assert_parity(gpu_query(srk, rp, col, n // 2, 0.5, 3, **kw),
+                  oracle_query(rp, col, n // 2, 0.5, 3, **kw))
+
+
+@pytest.mark.parametrize("d", [1, 8, 9, 33, 64, 65, 200])
+def test_own_lists(srk, d):
+    rp, col = ring_lists(1500, d, d)
+    kw = dict(z_override=3000.0, L_override=9)
+    assert_parity(gpu_query(srk, rp, col, 7, 0.5, 4, **kw),
+                  oracle_query(rp, col, 7, 0.5, 4, **kw))
+
+
+@pytest.mark.parametrize("z,L", [(1.0, 0), (2.0, 1), (40.0, 2), (90.0, 3), (60.0, 33), (50.0, 70),
+                                 (9000.0, 34)])
+def test_pair_counts_and_lengths(srk, z, L):
+    # long pairs: two nodes with one shared in-neighbour chain that never ends
+    rp, col = ring_lists(400, 2, 11)
+    kw = dict(z_override=z, L_override=L)
+    assert_parity(gpu_query(srk, rp, col, 3, 0.5, 5, **kw), oracle_query(rp, col, 3, 0.5, 5, **kw))
+
+
+@pytest.mark.parametrize("layout", ["narrow", "wide", "csr"])
+@pytest.mark.parametrize("hubs", [1, 600])
+def test_hubs_and_filter_sizes(srk, layout, hubs):
+    """Hubs of in-degree 2,500 (600 of them: more than the cached records) that
+    are also in-neighbours of up to 12,000 nodes (filters of the largest size),
+    beside nodes that are in-neighbours of one or two (the smallest)."""
+    import torch
+    from srk_inputs import csr_from_edges
+    rng = np.random.default_rng(hubs)
+    n = 12000
+    h = rng.choice(n, size=hubs, replace=False)
+    src = [rng.integers(0, n, size=2500) for _ in h]
+    dst = [np.full(2500, x) for x in h]
+    src += [h[rng.integers(0, hubs, size=n)], rng.integers(0, n, size=n)]
+    dst += [np.arange(n), np.arange(n)]
+    rp, col = csr_from_edges(n, np.concatenate(src), np.concatenate(dst))
+    s = int(h[0])
+    dev = torch.device("cuda:0")
+    with srk.srk_graph_load(torch.from_numpy(rp).to(dev), torch.from_numpy(col).to(dev),
+                            layout=layout) as g:
+        scores = torch.empty(n, dtype=torch.float64, device=dev)
+        out = [torch.empty(n, dtype=t, device=dev) for t in (torch.int32, torch.int64, torch.int32)]
+        stats = srk.SrkStats()
+        srk.srk_single_source(g, s, 0.6, 0.5, 9, scores, out[0], out[1], step_counts=out[2],
+                              stats=stats, z_override=900.0, L_override=15)
+        again = torch.empty_like(scores)
+        srk.srk_single_source(g, s, 0.6, 0.5, 9, again, z_override=900.0, L_override=15)
+        torch.cuda.synchronize()
+    gpu = (scores.cpu().numpy(), out[0].cpu().numpy().view(np.uint32),
+           out[1].cpu().numpy().view(np.uint64), out[2].cpu().numpy().view(np.uint32), stats)
+    assert_parity(gpu, oracle_query(rp, col, s, 0.5, 9, z_override=900.0, L_override=15))
+    assert torch.equal(again, scores)  # the kernel that does not count steps
+
+
+@pytest.mark.parametrize("lo,hi", [(0, 1), (100, 100), (17, 465), (999, 1000)])
+def test_short_target_ranges_without_filters(srk, lo, hi):
+    rp, col = ring_lists(1000, 5, 2)
+    kw = dict(z_override=300.0, L_override=10)
+    ref = oracle_query(rp, col, 20, 0.5, 6, **kw)
+    got = gpu_query(srk, rp, col, 20, 0.5, 6, target_range=(lo, hi), **kw)
+    for a, b in zip(got[:4], (ref.scores, ref.count, ref.wsum, ref.steps)):
+        assert np.array_equal(a[lo:hi].astype(b.dtype), b[lo:hi])
+    assert got[4].target_steps == int(ref.steps[lo:hi].sum())
