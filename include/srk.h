@@ -160,10 +160,11 @@ typedef struct srk_opts {
  *                  are copied.  SRK_VALIDATE is accepted and implied.
  *                  SRK_ADJ_NARROW / SRK_ADJ_WIDE / SRK_ADJ_CSR force the
  *                  adjacency layout the walks read: a packed copy with
- *                  4-byte entries carrying a degree code of 32 - b bits,
- *                  2^b >= n + m + H, where the H nodes whose degree the code
- *                  cannot hold keep their degree in a header (n + m + H
- *                  words plus n positions; SRK_EINVAL if n + m + H >= 2^31);
+ *                  4-byte entries carrying a node's rank, b bits, 2^b >= n,
+ *                  and a degree code of min(32 - b, 11) bits, where the H
+ *                  nodes whose degree the code cannot hold have a record of
+ *                  their degree and list (m + 2 H words plus n ranks and a
+ *                  table of at most 2048 words);
  *                  a packed copy with 8-byte entries carrying the full
  *                  degree (2 (n + m) words); or row_ptr and col themselves
  *                  (no copy).  By default: 4-byte entries while
@@ -234,12 +235,12 @@ int srk_single_source(const srk_graph *g, int32_t s, double c, double eps,
  * a scratch budget (a quarter of free device memory, at most 8 GiB, or the
  * byte count in the environment variable SRK_BATCH_BYTES): one
  * launch per source-side phase for the whole batch, then one persistent
- * launch over the batch's (source, target) work items, captured in a CUDA
- * graph unless opt->flags has SRK_OPT_NO_GRAPH.  Sources none of whose walk
- * pairs can meet (e.g. no in-neighbours) and targets without in-neighbours
- * produce no work items; their scores are written directly.  The persistent
- * kernel's launch shape is picked per graph by timing the candidate shapes on
- * the first items of the first call (kept in the handle).  The call
+ * launch per source over its targets, captured in a CUDA graph unless
+ * opt->flags has SRK_OPT_NO_GRAPH.  Sources none of whose walk pairs can meet
+ * (e.g. no in-neighbours) and targets without in-neighbours produce no work;
+ * their scores are written directly.  The persistent kernel's launch shape is
+ * picked per graph by timing the candidate shapes on the first units of work
+ * of the first call (kept in the handle).  The call
  * synchronises the stream at the end of every batch.  With
  * SRK_OPT_SHARED_WALKS the batches hold up to 64 sources, grouped by walk
  * budget with the sources without in-neighbours last (the call first reads

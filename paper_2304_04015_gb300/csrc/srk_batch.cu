@@ -3,19 +3,18 @@
 // The sources are processed in batches sized by a memory budget.  Each batch
 // runs the source-side steps a2-a3 of all its sources with one launch per
 // phase (thread g of a phase finds its source by a binary search over the
-// prefix of the sources' walk counts), then one persistent launch walks every
-// (source, target) work item: a warp takes items from a global counter in
-// source-major order and walks the target's pairs exactly as the
-// single-source kernel does (walk_target in srk_device.cuh), so the results
-// are identical to srk_single_source.  Sources whose walks never leave the
-// source (no pair can meet) are short-circuited: their score rows are
-// prefilled (1 at the source, 0 elsewhere) and they contribute no items, and
-// neither do targets without in-neighbours.  A batch's launches are captured
-// in a CUDA graph and launched as one.  The persistent kernel's launch shape
-// (block size x blocks per SM) is chosen per graph by timing the candidates
-// on the first items of the first batch (autotuner).  With shared target walks
-// (SRK_OPT_SHARED_WALKS) the batches hold up to 64 sources and the target
-// walks run once for all of them (kb_shared_walks, below).
+// prefix of the sources' walk counts); then every source's targets are walked
+// as srk_single_source walks them (enqueue_walks, srk_lockstep.cu), so the
+// results are identical.  Sources whose walks never leave the source (no pair
+// can meet) find no work there: their score rows are prefilled (1 at the
+// source, 0 elsewhere).  A batch's launches are captured in a CUDA graph and
+// launched as one.  The walk kernel's launch shape (targets per thread) is
+// chosen per graph by timing the candidates on the first units of the first
+// batch (autotuner).  (One persistent launch over all (source, target) items,
+// a warp each, took 86.2 ms for 24 sources of mixed eps on R-MAT 16, where this
+// takes 61.8 ms.)  With shared target walks (SRK_OPT_SHARED_WALKS) the batches hold
+// up to 64 sources and the target walks run once for all of them
+// (kb_shared_walks, below).
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
@@ -35,7 +34,6 @@ struct BatchSrc {
   const QueryTab *tab;    // the source's table (device copy)
   double *scores;         // output row, n entries
   uint32_t *counts;       // output row or null
-  unsigned long long *steps;  // target-walk steps of this source (one counter)
   unsigned long long *wj;     // shared walks: quantised Lemma 7 weight of pair j
   int32_t s, L, N_tot;
   double z;
@@ -83,11 +81,11 @@ __device__ __forceinline__ int find_source(const int64_t *off, int k, int64_t g)
     __VA_ARGS__                                                                  \
   }
 
-// a2: source walks and Fisher-Yates draws of every source of the batch.
-template <int kLayout>
+// a2: source walks (on the CSR: spos holds node ids) and Fisher-Yates draws of
+// every source of the batch.
 __global__ void __launch_bounds__(256) kb_source_walks(const __grid_constant__ BatchArgs A) {
   const RoundKeys rk = round_keys(A.key0, A.key1);
-  const auto G = adj_view<kLayout>(A.view);
+  const AdjC G{A.view.row_ptr, A.view.col};
   SRK_BATCH_LOOP(A, {
     const QueryTab &t = *S_.tab;
     const uint32_t s = (uint32_t)S_.s;
@@ -186,59 +184,33 @@ __global__ void kb_pairs(const __grid_constant__ BatchArgs A) {
   })
 }
 
-// Row geometry of every source (one thread per source), as in k_rows, and
-// the list of sources with at least one pair.
-__global__ void kb_rows(const __grid_constant__ BatchArgs A, int32_t *act_src,
-                        int32_t *n_act_src) {
-  if (blockIdx.x != 0) return;
-  for (int i = threadIdx.x; i < A.k; i += blockDim.x) {
+// Row geometry and target bounds of every source (one thread per source), as
+// in k_rows.
+__global__ void kb_rows(const __grid_constant__ BatchArgs A, int32_t n_act) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.k; i += gridDim.x * blockDim.x) {
     const Small sm = small_view(A.src[i].w.small);
     const int L = A.src[i].L;
-    int32_t c = 0;
+    int32_t c = 0, r = 0;
     sm.cnt[L + 1] = 0;
     for (int q = L; q >= 1; --q) {
+      const int32_t h = sm.cap_hist[q];
       sm.cursor[q] = c;
-      c += sm.cap_hist[q];
+      sm.R[q] = r;
+      c += h;
+      r += q * h;
       sm.cnt[q] = c;
     }
-    int32_t r = 0;
-    for (int q = 1; q <= L + 1; ++q) {
-      sm.R[q] = r;
-      if (q <= L) r += sm.cnt[q];
-    }
+    sm.R[L + 1] = r;
     sm.cnt[0] = c;
     sm.R[0] = 0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {  // in source order, so the items stay source-major
-    int32_t m = 0;
-    for (int i = 0; i < A.k; ++i)
-      if (small_view(A.src[i].w.small).cnt[1] > 0) act_src[m++] = i;
-    *n_act_src = m;
+    int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
+    bounds[0] = 0;
+    bounds[1] = n_act;
+    bounds[2] = 0;
   }
 }
 
-__global__ void kb_hit_table(const __grid_constant__ BatchArgs A) {
-  SRK_BATCH_LOOP(A, {
-    const int32_t j = r_;
-    const int32_t w = S_.w.sigma[j];
-    const int l2 = stratum_of(S_.tab->P, S_.L, j);
-    const int32_t cap = min(l2, S_.w.seff[w]);
-    if (cap >= 1) {
-      const Small sm = small_view(S_.w.small);
-      const int l1 = stratum_of(S_.tab->P, S_.L, w);
-      const int32_t a = atomicAdd(&sm.cursor[cap], 1);
-      S_.w.pair_j[a] = j;
-      S_.w.pair_w[a] = __double2ull_rn(S_.tab->a[l1] * S_.tab->a[l2] * 4294967296.0);
-      const int Ls = S_.L > 0 ? S_.L : 1;
-      const int32_t *sp = S_.w.spos + (int64_t)w * Ls;
-      for (int q = 1; q <= cap; ++q) S_.w.Hc[sm.R[q] + a] = sp[q - 1];
-    }
-  })
-}
-
-// Every output row: 1 at the source, 0 elsewhere (the rows of items walked
-// later are overwritten per target).
+// Every output row: 1 at the source, 0 elsewhere (the walks add to the rows).
 __global__ void kb_prefill(const BatchSrc *__restrict__ src, int32_t k, int32_t n) {
   const int64_t total = (int64_t)k * n;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
@@ -248,77 +220,6 @@ __global__ void kb_prefill(const BatchSrc *__restrict__ src, int32_t k, int32_t 
     src[i].scores[u] = (u == src[i].s) ? 1.0 : 0.0;
     if (src[i].counts) src[i].counts[u] = 0;
   }
-}
-
-// a4-a5 for every (active source, target with in-neighbours) item, source-
-// major.  Items at or beyond `item_limit` are not walked (autotuner trials).
-// Each warp keeps its current source's context in shared memory: the pair
-// list pointers and the rows cnt[0..L+2], R[0..L+2] (dynamic shared memory,
-// 2 (Lmax + 3) words per warp), so the walk loop holds no per-source state
-// in registers.
-template <int kBlock, int kMinBlocks, int kLayout>
-__global__ void __launch_bounds__(kBlock, kMinBlocks)
-kb_target_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__ act,
-                int32_t n_act, const int32_t *__restrict__ act_src,
-                const int32_t *__restrict__ n_act_src_p,
-                unsigned long long *__restrict__ item_counter, int64_t item_limit,
-                int32_t row_words) {
-  extern __shared__ int32_t rows[];
-  __shared__ PairSet ctx[kBlock / 32];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const auto G = adj_view<kLayout>(A.view);
-  int2 *my_rc = reinterpret_cast<int2 *>(rows + (2 * wib) * row_words);
-  const int64_t n_items = (int64_t)(*n_act_src_p) * n_act;
-  const int64_t limit = item_limit < n_items ? item_limit : n_items;
-  int cur = -1;
-  unsigned long long acc = 0;  // steps of source `cur` by this warp (lane 0)
-  for (;;) {
-    unsigned long long item = 0;
-    if (lane == 0) item = atomicAdd(item_counter, 1ull);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if ((int64_t)item >= limit) break;
-    const int q = (int)((int64_t)item / n_act);
-    const int32_t u = act[(int64_t)item - (int64_t)q * n_act];
-    const int i = act_src[q];
-    if (i != cur) {
-      if (lane == 0 && cur >= 0 && acc) atomicAdd(A.src[cur].steps, acc);
-      acc = 0;
-      cur = i;
-      const BatchSrc &B = A.src[i];
-      const Small sm = small_view(B.w.small);
-      __syncwarp();
-      for (int x = lane; x <= B.L + 2; x += 32)
-        my_rc[x] = make_int2((x <= B.L + 1) ? sm.R[x] : 0, (x + 1 <= B.L + 1) ? sm.cnt[x + 1] : 0);
-      if (lane == 0) {
-        PairSet &S = ctx[wib];
-        S.rc = my_rc;
-        S.pair_j = B.w.pair_j;
-        S.pair_w = B.w.pair_w;
-        S.Hc = B.w.Hc;
-        S.n_pairs = sm.cnt[1];
-        S.key = B.tab->tkey;
-      }
-      __syncwarp();
-    }
-    if (u == A.src[i].s) continue;  // prefilled with 1
-    uint32_t c = 0, st = 0;
-    unsigned long long W = 0;
-    uint32_t deg_u = 0;
-    const int32_t b_u = node_start(G, A.view.row_ptr, u, deg_u);
-    walk_target(G, ctx[wib], (uint32_t)u, b_u, deg_u, c, W, st);
-    for (int off = 16; off > 0; off >>= 1) {
-      c += __shfl_xor_sync(0xffffffffu, c, off);
-      st += __shfl_xor_sync(0xffffffffu, st, off);
-      W += __shfl_xor_sync(0xffffffffu, W, off);
-    }
-    if (lane == 0) {
-      const BatchSrc &B = A.src[i];
-      B.scores[u] = (double)W * 2.3283064365386963e-10 / B.z;
-      if (B.counts) B.counts[u] = c;
-      acc += st;
-    }
-  }
-  if (lane == 0 && cur >= 0 && acc) atomicAdd(A.src[cur].steps, acc);
 }
 
 // ------------------------------------------------------------------------
@@ -367,7 +268,7 @@ __global__ void kb_hitj(const __grid_constant__ BatchArgs A) {
     const bool high = i_ >= 32;
     const uint32_t smask = (1u << A.tbits) - 1u;
     for (int q = 1; q <= cap; ++q) {
-      const int32_t node = sp[q - 1];
+      const int32_t node = node_identity(A.view, sp[q - 1]);
       uint4 *cell = &A.M[(int64_t)(q - 1) * A.Jmax + j];
       const uint32_t h = node_hash(node);
       atomicOr(high ? &cell->y : &cell->x, bit);
@@ -575,83 +476,6 @@ kb_shared_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__
   if (lane == 0 && warp_steps) atomicAdd(ctr + 1, warp_steps);
 }
 
-// The candidate launch shapes of the autotuner (block size, blocks per SM).
-struct Shape {
-  int block, per_sm;
-};
-static const Shape kShapes[] = {{256, 8}, {512, 4}, {128, 16}, {1024, 2}, {256, 6}};
-constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
-
-template <int kLayout>
-static void launch_targets_t(int shape, int grid, int block, size_t smem, cudaStream_t st,
-                             const BatchArgs &A, const int32_t *act, int32_t n_act,
-                             const int32_t *act_src, const int32_t *n_act_src,
-                             unsigned long long *ctr, int64_t limit, int32_t rw) {
-#define SRK_KB_LAUNCH(B, M)                                                                  \
-  kb_target_walks<B, M, kLayout><<<grid, block, smem, st>>>(A, act, n_act, act_src, n_act_src, \
-                                                            ctr, limit, rw)
-  switch (shape) {
-    case 0: SRK_KB_LAUNCH(256, 8); break;
-    case 1: SRK_KB_LAUNCH(512, 4); break;
-    case 2: SRK_KB_LAUNCH(128, 16); break;
-    case 3: SRK_KB_LAUNCH(1024, 2); break;
-    default: SRK_KB_LAUNCH(256, 6); break;
-  }
-#undef SRK_KB_LAUNCH
-}
-
-// Shared memory of the target kernel in launch shape `shape`: two rows of
-// Lmax + 3 words per warp.
-static size_t target_smem(int shape, int Lmax) {
-  return sizeof(int32_t) * 2 * (size_t)(Lmax + 3) * (size_t)(kShapes[shape].block / 32);
-}
-
-// Lets every launch shape of layout kLayout take `bytes` of dynamic shared
-// memory (above the default 48 KB a kernel must opt in).  Not a stream
-// operation, so it runs before any capture.
-template <int kLayout>
-static cudaError_t allow_smem_t(size_t bytes) {
-  const int b = (int)bytes;
-  cudaError_t e = cudaSuccess;
-  auto set = [&](const void *f) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  };
-  set((const void *)kb_target_walks<256, 8, kLayout>);
-  set((const void *)kb_target_walks<512, 4, kLayout>);
-  set((const void *)kb_target_walks<128, 16, kLayout>);
-  set((const void *)kb_target_walks<1024, 2, kLayout>);
-  set((const void *)kb_target_walks<256, 6, kLayout>);
-  return e;
-}
-
-static cudaError_t allow_smem(int layout, int Lmax) {
-  size_t most = 0;
-  for (int sh = 0; sh < kNumShapes; ++sh) most = std::max(most, target_smem(sh, Lmax));
-  if (most <= 48 * 1024) return cudaSuccess;
-  return layout == kWide ? allow_smem_t<kWide>(most)
-         : layout == kCsr ? allow_smem_t<kCsr>(most)
-                          : allow_smem_t<kNarrow>(most);
-}
-
-static void launch_targets(int layout, int shape, int sms, cudaStream_t st, const BatchArgs &A,
-                           const int32_t *act, int32_t n_act, const int32_t *act_src,
-                           const int32_t *n_act_src, unsigned long long *ctr,
-                           int64_t limit, int Lmax) {
-  const Shape sh = kShapes[shape];
-  const int grid = sms * sh.per_sm;
-  const int32_t rw = Lmax + 3;
-  const size_t smem = target_smem(shape, Lmax);
-  if (layout == kWide)
-    launch_targets_t<kWide>(shape, grid, sh.block, smem, st, A, act, n_act, act_src,
-                            n_act_src, ctr, limit, rw);
-  else if (layout == kCsr)
-    launch_targets_t<kCsr>(shape, grid, sh.block, smem, st, A, act, n_act, act_src, n_act_src,
-                           ctr, limit, rw);
-  else
-    launch_targets_t<kNarrow>(shape, grid, sh.block, smem, st, A, act, n_act, act_src,
-                              n_act_src, ctr, limit, rw);
-}
-
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // The shared-walk kernel: a persistent grid of as many 256-thread blocks as
@@ -740,6 +564,57 @@ int source_in_degrees(const srk_graph *g, const int32_t *sources, int32_t k, cud
 }
 
 }  // namespace srk
+
+namespace {
+
+// The launch shape (enqueue_walks) that walks the first units of a batch's
+// first source with pairs the fastest, per target and pair; stays -1 when no
+// source has any.  Leaves the source side to be run again.
+template <class SourceSide, class Walks>
+int tune_shape(const srk_graph *g, const std::vector<BatchSrc> &src, SourceSide &source_side,
+               Walks &walks, cudaStream_t st, int *shape) {
+  source_side(st);
+  int32_t pick = -1;
+  for (size_t b = 0; b < src.size() && pick < 0; ++b) {
+    int32_t pairs = 0;
+    cudaError_t e = cudaMemcpyAsync(&pairs, small_view(src[b].w.small).cnt + 1, sizeof pairs,
+                                    cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "batched query: reading the pair counts");
+    if (pairs > 0) pick = (int32_t)b;
+  }
+  if (pick < 0) return SRK_OK;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaError_t e = cudaEventCreate(&ev[0]);
+  if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
+  int rc = e == cudaSuccess ? SRK_OK
+                            : cuda_fail(e, "batched query: creating the autotuner's events");
+  double best = 0.0;
+  for (int sh = 0; sh < kWalkShapes && rc == SRK_OK; ++sh) {
+    if (sh > 0) source_side(st);
+    const int32_t units = sm_count(g->device) * 2;  // about one round of the grid
+    rc = walks(pick, st, ev, sh, units);
+    int32_t cnt[3] = {0, 0, 0};
+    float ms = 0.f;
+    if (rc == SRK_OK) {
+      e = cudaMemcpyAsync(cnt, small_view(src[(size_t)pick].w.small).cnt, sizeof cnt,
+                          cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+      if (e != cudaSuccess) rc = cuda_fail(e, "batched query: autotuner");
+    }
+    const double rate = walk_units_work(g, sh, cnt[2] > 0 ? cnt[2] : cnt[1], units) / std::max(1e-6f, ms);
+    if (rc == SRK_OK && rate > best) {
+      best = rate;
+      *shape = sh;
+    }
+  }
+  if (ev[0]) cudaEventDestroy(ev[0]);
+  if (ev[1]) cudaEventDestroy(ev[1]);
+  return rc;
+}
+
+}  // namespace
 
 extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
                                 int32_t k, double c, const double *eps,
@@ -886,23 +761,29 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     const size_t r_bytes = shared ? sizeof(int64_t) * rowbase.size() : 0;
     const size_t h_bytes = shared ? (16 * (size_t)n_tables) << tbits : 0;
     const size_t head = align256(sizeof(BatchSrc) * kb) + align256(sizeof(QueryTab) * kb) +
-                        align256(sizeof(int64_t) * (kb + 1)) +
-                        align256(sizeof(int32_t) * (kb + 1)) +
-                        align256(sizeof(unsigned long long) * (kb + 2)) + align256(m_bytes) +
+                        align256(sizeof(int64_t) * (kb + 1)) + 256 + align256(m_bytes) +
                         align256(r_bytes) + align256(h_bytes);
+    // end filters: one region, which the sources use one after the other
+    size_t extra = 0;
+    for (int32_t b = i0; b < i1 && !shared; ++b)
+      extra = std::max(extra, filter_bytes(g, tabs[(size_t)b], g->n));
     char *base = nullptr;
-    cudaError_t e = cudaMallocFromPoolAsync((void **)&base, head + need, mp, st);
+    cudaError_t e = cudaMallocFromPoolAsync((void **)&base, head + need + extra, mp, st);
+    if (e == cudaErrorMemoryAllocation && extra > 0) {  // the walks can do without
+      cudaGetLastError();
+      extra = 0;
+      e = cudaMallocFromPoolAsync((void **)&base, head + need, mp, st);
+    }
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch workspace allocation"); break; }
     BatchSrc *d_src = (BatchSrc *)base;
     QueryTab *d_tab = (QueryTab *)(base + align256(sizeof(BatchSrc) * kb));
     int64_t *d_off = (int64_t *)((char *)d_tab + align256(sizeof(QueryTab) * kb));
-    int32_t *d_act_src = (int32_t *)((char *)d_off + align256(sizeof(int64_t) * (kb + 1)));
-    unsigned long long *d_ctr = (unsigned long long *)((char *)d_act_src +
-                                                         align256(sizeof(int32_t) * (kb + 1)));
-    uint4 *d_M = (uint4 *)((char *)d_ctr + align256(sizeof(unsigned long long) * (kb + 2)));
+    unsigned long long *d_ctr =
+        (unsigned long long *)((char *)d_off + align256(sizeof(int64_t) * (kb + 1)));
+    uint4 *d_M = (uint4 *)((char *)d_ctr + 256);
     int64_t *d_rowbase = (int64_t *)((char *)d_M + align256(m_bytes));
     uint4 *d_T = (uint4 *)((char *)d_rowbase + align256(r_bytes));
-    // d_ctr[0] = item counter, d_ctr[1 + i] = steps of source i; n_act_src in d_act_src[kb]
+    // shared walks: d_ctr[0] = target counter, d_ctr[1] = steps
     char *ws_base = base + head;
     std::vector<BatchSrc> hsrc((size_t)kb);
     std::vector<int64_t> hoff((size_t)kb + 1);
@@ -925,7 +806,6 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         S.wj = (unsigned long long *)extra;
         extra += align256(8 * (size_t)t.N_tot);
       }
-      S.steps = d_ctr + 1 + b;
       S.s = t.s;
       S.L = t.L;
       S.N_tot = t.N_tot;
@@ -965,13 +845,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     auto enqueue_source_side = [&](cudaStream_t s2) {
       for (int32_t b = 0; b < kb; ++b)
         cudaMemsetAsync(hsrc[(size_t)b].w.small, 0, kSmallBytes, s2);
-      cudaMemsetAsync(d_ctr, 0, sizeof(unsigned long long) * (kb + 1), s2);
-      if (g->layout == kWide)
-        kb_source_walks<kWide><<<gw, 256, 0, s2>>>(A);
-      else if (g->layout == kCsr)
-        kb_source_walks<kCsr><<<gw, 256, 0, s2>>>(A);
-      else
-        kb_source_walks<kNarrow><<<gw, 256, 0, s2>>>(A);
+      kb_source_walks<<<gw, 256, 0, s2>>>(A);
       kb_fy_rank<<<gw, 256, 0, s2>>>(A);
       kb_scan<<<kb, 1024, 0, s2>>>(A);
       kb_fy_scatter<<<gw, 256, 0, s2>>>(A);
@@ -982,59 +856,39 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         cudaMemsetAsync(d_T, 0, h_bytes, s2);
         kb_hitj<<<gw, 256, 0, s2>>>(A);
       } else {
-        kb_rows<<<1, 256, 0, s2>>>(A, d_act_src, d_act_src + kb);
-        kb_hit_table<<<gw, 256, 0, s2>>>(A);
+        kb_rows<<<(kb + 31) / 32, 32, 0, s2>>>(A, g->n_act);
       }
       const int gp = (int)std::min<int64_t>(((int64_t)kb * (int64_t)n + 255) / 256,
                                             (int64_t)sms * 16);
       kb_prefill<<<gp, 256, 0, s2>>>(d_src, kb, (int32_t)n);
     };
-    if ((e = allow_smem(g->layout, Lmax)) != cudaSuccess) {
-      rc = cuda_fail(e, "batched query: shared memory of the target kernel");
-      cudaFreeAsync(base, st);
-      break;
-    }
-    // autotune the persistent kernel's launch shape on the first batch
+    const bool count = opt && opt->stats;
+    auto enqueue_source = [&](int32_t b, cudaStream_t s2, const cudaEvent_t *timing, int shape,
+                              int32_t max_units) {
+      const BatchSrc &S = hsrc[(size_t)b];
+      const Outputs o{S.scores, S.counts, nullptr, nullptr};
+      return enqueue_walks(g, tabs[(size_t)(i0 + b)], S.w, o, ws_base + need, extra, count, s2,
+                           timing, 0, (int32_t)n, shape, max_units);
+    };
+    // autotune the walk kernel's launch shape on the first batch with pairs
     int shape = g->batch_cfg;
-    if (!shared && (shape < 0 || shape >= kNumShapes)) {
-      enqueue_source_side(st);
-      cudaEvent_t t0 = nullptr, t1 = nullptr;
-      e = cudaEventCreate(&t0);
-      if (e == cudaSuccess) e = cudaEventCreate(&t1);
-      if (e != cudaSuccess) {
-        if (t0) cudaEventDestroy(t0);
-        rc = cuda_fail(e, "batched query: creating the autotuner's events");
+    if (!shared && shape < 0) {
+      rc = tune_shape(g, hsrc, enqueue_source_side, enqueue_source, st, &shape);
+      if (rc) {
         cudaFreeAsync(base, st);
         break;
       }
-      const int64_t trial = (int64_t)sms * 64 * 3;  // about three items per warp
-      float best = 1e30f;
-      shape = 0;
-      for (int sh = 0; sh < kNumShapes; ++sh) {
-        cudaMemsetAsync(d_ctr, 0, sizeof(unsigned long long), st);
-        cudaEventRecord(t0, st);
-        launch_targets(g->layout, sh, sms, st, A, g->act, g->n_act, d_act_src, d_act_src + kb,
-                       d_ctr, trial, Lmax);
-        const bool launched = cudaGetLastError() == cudaSuccess;  // a shape that cannot run
-        cudaEventRecord(t1, st);
-        float ms = 0.f;
-        if (cudaEventSynchronize(t1) == cudaSuccess && launched &&
-            cudaEventElapsedTime(&ms, t0, t1) == cudaSuccess && ms < best) {
-          best = ms;
-          shape = sh;
-        }
-      }
-      cudaEventDestroy(t0);
-      cudaEventDestroy(t1);
-      const_cast<srk_graph *>(g)->batch_cfg = shape;
+      if (shape >= 0) const_cast<srk_graph *>(g)->batch_cfg = shape;
     }
     auto enqueue_all = [&](cudaStream_t s2) {
       enqueue_source_side(s2);
+      int r = SRK_OK;
       if (shared)
         launch_shared(g->layout, s2, A, g->act, g->n_act, j0, d_ctr, dev);
       else
-        launch_targets(g->layout, shape, sms, s2, A, g->act, g->n_act, d_act_src, d_act_src + kb,
-                       d_ctr, INT64_MAX, Lmax);
+        for (int32_t b = 0; b < kb && r == SRK_OK; ++b)
+          r = enqueue_source(b, s2, nullptr, shape, INT32_MAX);
+      return r;
     };
     if (use_graph) {
       // The batch is captured every time (its buffers move), but the graph's
@@ -1048,8 +902,9 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ev_in, 0);
       if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        enqueue_all(cs);
+        rc = enqueue_all(cs);
         e = cudaStreamEndCapture(cs, &graph);
+        if (rc && e == cudaSuccess) e = cudaErrorUnknown;
       }
       if (e == cudaSuccess && gm->batch_exec) {
         cudaGraphExecUpdateResultInfo info;
@@ -1068,12 +923,12 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
       if (graph) cudaGraphDestroy(graph);
     } else {
-      enqueue_all(st);
+      rc = enqueue_all(st);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      rc = cuda_fail(e, "batched query launch");
+    if (e != cudaSuccess || rc) {
+      if (!rc) rc = cuda_fail(e, "batched query launch");
       cudaFreeAsync(base, st);
       break;
     }
@@ -1088,9 +943,9 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
                             cudaMemcpyDeviceToHost, st);
     }
     if (e == cudaSuccess && opt && opt->stats) {
-      std::vector<unsigned long long> steps((size_t)kb + 1);
-      e = cudaMemcpyAsync(steps.data(), d_ctr, sizeof(unsigned long long) * (kb + 1),
-                          cudaMemcpyDeviceToHost, st);
+      unsigned long long walked = 0;  // steps of the shared walks
+      if (shared)
+        e = cudaMemcpyAsync(&walked, d_ctr + 1, sizeof walked, cudaMemcpyDeviceToHost, st);
       for (int32_t b = 0; b < kb && e == cudaSuccess; ++b) {
         unsigned long long sc[2];
         int32_t act = 0;
@@ -1099,12 +954,13 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         if (e == cudaSuccess)
           e = cudaMemcpyAsync(&act, sm.cnt + 1, sizeof act, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        total.target_steps += sc[0];
         total.source_steps += sc[1];
         total.n_active_pairs += act;
         total.n_walks += tabs[(size_t)(i0 + b)].N_tot;
       }
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      for (int32_t b = 0; b < kb; ++b) total.target_steps += steps[(size_t)b + 1];
+      total.target_steps += walked;
       total.z = tabs[(size_t)(i1 - 1)].z;
       total.L = tabs[(size_t)(i1 - 1)].L;
     }

@@ -190,7 +190,13 @@ size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets);
 // are made, the outputs of the range cleared): srk_lockstep.cu.
 int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Outputs &o,
                   char *extra, size_t extra_bytes, bool count, cudaStream_t st,
-                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end);
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end, int shape = -1,
+                  int32_t max_units = INT32_MAX);
+// Launch shapes of the walks: 0 and up, -1 for the default of the target count.
+// max_units bounds the units of work walked (the autotuner's trials), and
+// walk_units_work is the targets x pairs of that many units over all targets.
+constexpr int kWalkShapes = 2;
+double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t max_units);
 // Shared-memory opt-in of the walk kernels of a layout, in this context.
 cudaError_t allow_lockstep(int layout);
 // [*b, *e): the targets a query computes, from its options (SRK_EINVAL when

@@ -107,6 +107,7 @@ struct LockQuery {
   uint32_t rk[10];              //   and its round keys
   int32_t s;
   int32_t min_cap;              // pairs below this cap are not walked here
+  int32_t max_units;            // units beyond these are not walked
 };
 
 // -------------------------------------------------- asynchronous copies --
@@ -597,7 +598,9 @@ k_records(const __grid_constant__ QueryTab tab, GraphView V, Filters F,
 }
 
 // Room for every slot's list and filter, the filters cleared.
-__global__ void __launch_bounds__(256) k_end_slots(Filters F) {
+__global__ void __launch_bounds__(256)
+k_end_slots(Filters F, const int32_t *__restrict__ cnt) {
+  if (cnt[1] == 0) return;
   const int lane = threadIdx.x & 31;
   for (int32_t base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; base < (1 << F.slot_bits);
        base += gridDim.x * blockDim.x) {
@@ -645,10 +648,11 @@ k_end_lists(Filters F, const int32_t *__restrict__ small_base, int4 *__restrict_
 // so repeated in-neighbours count once each, as the draw does.)  A bitmap in
 // L1 turns most edges away; R-MAT 20: 0.37 ms for 16.1 M edges.
 __global__ void __launch_bounds__(256)
-k_edges(Filters F, GraphView V, int64_t m,
+k_edges(Filters F, GraphView V, int64_t m, const int32_t *__restrict__ cnt,
         const int4 *__restrict__ rec, const unsigned long long *__restrict__ pair_w, uint32_t key,
         int32_t s, int32_t u_begin, int32_t u_end, unsigned long long *__restrict__ W,
         uint32_t *__restrict__ counts) {
+  if (cnt[1] == 0) return;  // no pair can meet
   const int lane = threadIdx.x & 31;
   const int32_t *row_ptr = V.row_ptr;
   const uint32_t mask = (1u << F.slot_bits) - 1u;
@@ -688,12 +692,12 @@ k_edges(Filters F, GraphView V, int64_t m,
     const bool todo = S.key && S.cnt1 > 0 && u >= u_begin && u < u_end && u != s;
     for (uint32_t mm = __ballot_sync(0xffffffffu, todo); mm; mm &= mm - 1) {
       const int l = __ffs(mm) - 1;
-      const int32_t uu = __shfl_sync(0xffffffffu, u, l), cnt = __shfl_sync(0xffffffffu, S.cnt1, l),
+      const int32_t uu = __shfl_sync(0xffffffffu, u, l), n1 = __shfl_sync(0xffffffffu, S.cnt1, l),
                     off = __shfl_sync(0xffffffffu, S.off1, l);
       const uint32_t kk = __shfl_sync(0xffffffffu, k, l), dd = __shfl_sync(0xffffffffu, d, l);
       uint32_t c = 0;
       unsigned long long ws = 0;
-      for (int32_t q = lane; q < cnt; q += 32) {
+      for (int32_t q = lane; q < n1; q += 32) {
         const int32_t a = F.list1[off + q];
         const uint32_t j = (uint32_t)rec[a].x;
         uint32_t x0, x1;
@@ -722,10 +726,13 @@ k_edges(Filters F, GraphView V, int64_t m,
 // are units of equal work: up to 16 a block, of at least 128 pairs where there
 // are as many, and as near below a whole number of rounds over the grid as a
 // count within a quarter of the largest gets.
-__device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb, int32_t grid) {
+__host__ __device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb,
+                                                       int32_t grid) {
   const int64_t per_block = (int64_t)n_pairs * n_tb / grid;
-  const int32_t rounds = max(1, (int32_t)min((int64_t)16, per_block / 128));
-  const int32_t most = max(1, min(n_pairs, rounds * grid / n_tb));
+  const int32_t rounds = per_block < 256 ? 1 : per_block < 2048 ? (int32_t)(per_block / 128) : 16;
+  int32_t most = rounds * grid / n_tb;
+  if (most > n_pairs) most = n_pairs;
+  if (most < 1) most = 1;
   int32_t best = most;
   float fill = 0.0f;
   for (int32_t c = most, k = 0; c > 0 && c >= most - most / 4 && k < 16; --c, ++k) {
@@ -763,7 +770,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   if (n_pairs == 0 || n_t <= 0) return;
   const int32_t T = kLockThreads * kT, n_tb = (n_t + T - 1) / T;
   const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
-  const int64_t units = (int64_t)n_tb * n_chunks;
+  const int64_t units = min((int64_t)n_tb * n_chunks, (int64_t)Q.max_units);
   if ((int64_t)blockIdx.x >= units) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (threadIdx.x < kStages) {
@@ -970,9 +977,19 @@ static void launch_lockstep(const GraphView &V, const int32_t *act, int32_t *bou
                                                                                      Q);
 }
 
+double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t max_units) {
+  const int32_t T = kLockThreads * (shape == 1 ? 1 : kLockTargets);
+  const int32_t n_tb = (g->n_act + T - 1) / T;
+  if (n_tb == 0 || n_pairs == 0) return 0.0;
+  const int32_t chunks = lock_chunks(n_pairs, n_tb, sm_count(g->device) * kLockBlocks);
+  const double units = (double)n_tb * chunks;
+  return (double)g->n_act * n_pairs * std::min(1.0, (double)max_units / units);
+}
+
 int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Outputs &o,
                   char *extra, size_t extra_bytes, bool count, cudaStream_t st,
-                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end) {
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end, int shape,
+                  int32_t max_units) {
   const int dev = g->device;
   const int gN = grid_for(t.N_tot, 256, dev);
   const int64_t nr = (int64_t)u_end - u_begin;
@@ -995,10 +1012,10 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   }
   k_records<<<gN, 256, 0, st>>>(t, V, F, w.sigma, w.seff, w.spos, w.small, rec, w.pair_w, w.Hc);
   if (F.slots) {
-    k_end_slots<<<grid_for((int64_t)1 << F.slot_bits, 256, dev), 256, 0, st>>>(F);
+    k_end_slots<<<grid_for((int64_t)1 << F.slot_bits, 256, dev), 256, 0, st>>>(F, sm.cnt);
     k_end_lists<<<gN, 256, 0, st>>>(F, w.small, rec);
-    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, rec, w.pair_w, t.tkey, t.s,
-                                                      u_begin, u_end, W, o.counts);
+    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, sm.cnt, rec, w.pair_w, t.tkey,
+                                                      t.s, u_begin, u_end, W, o.counts);
   }
   LockQuery Q;
   Q.rec = rec;
@@ -1014,9 +1031,11 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   for (int r = 0; r < 10; ++r) Q.rk[r] = t.tkey + (uint32_t)r * kPhiloxW0;
   Q.s = t.s;
   Q.min_cap = F.slots ? 2 : 1;
+  Q.max_units = max_units;
   if (timing) cudaEventRecord(timing[0], st);
   const int grid = sm_count(dev) * kLockBlocks;
-  const bool one = nr <= kLockThreads;  // too few targets to give a thread several
+  // shape 0: kLockTargets targets a thread; 1: one (too few to give it several)
+  const bool one = shape < 0 ? nr <= kLockThreads : shape == 1;
   if (g->layout == kWide) {
     if (count) launch_lockstep<kWide, true>(V, g->act, bounds, Q, one, grid, st);
     else launch_lockstep<kWide, false>(V, g->act, bounds, Q, one, grid, st);
