@@ -164,7 +164,8 @@ typedef struct srk_opts {
  *                  and a degree code of min(32 - b, 11) bits, where the H
  *                  nodes whose degree the code cannot hold have a record of
  *                  their degree and list (m + 2 H words plus n ranks and a
- *                  table of at most 2048 words);
+ *                  table of at most 2048 words; SRK_EINVAL if n + m > 2^30 and
+ *                  n + m plus the nodes with in-neighbours reach 2^31);
  *                  a packed copy with 8-byte entries carrying the full
  *                  degree (2 (n + m) words); or row_ptr and col themselves
  *                  (no copy).  By default: 4-byte entries while

@@ -14,7 +14,7 @@
 // a warp each, took 86.2 ms for 24 sources of mixed eps on R-MAT 16, where this
 // takes 61.8 ms.)  With shared target walks (SRK_OPT_SHARED_WALKS) the batches hold
 // up to 64 sources and the target walks run once for all of them
-// (kb_shared_walks, below).
+// (k_lock_shared, srk_lockstep.cu).
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
@@ -47,10 +47,10 @@ struct BatchArgs {
   GraphView view;
   uint32_t key0, key1;
   uint32_t shared_key;  // walk key of the shared target walks
-  uint4 *M;       // shared walks: M[(i-1) Jmax + j] (.x, .y) bit b = pair j of batch
-                  // source b may still meet at step i (cap_b(j) >= i); (.z, .w) = the
-                  // 64-bit signature of those sources' nodes at step i (bit
-                  // node_hash(node) per node); Lmax + 1 rows
+  uint2 *M;       // shared walks: M[j (Lmax + 1) + i - 1] bit b = pair j of batch source b
+                  // may still meet at step i (cap_b(j) >= i)
+  uint32_t *sig;  // shared walks: 32 words per meeting table, bit sig_bit(node) set for
+                  // every node of the table
   uint4 *T;       // shared walks: the meeting tables, one per (step i, pair j) with
                   // j >= Pmin_i (below, no pair of the batch reaches step i) at
                   // T + ((rowbase[i] + j) << tbits): 2^tbits slots {node + 1,
@@ -210,7 +210,7 @@ __global__ void kb_rows(const __grid_constant__ BatchArgs A, int32_t n_act) {
   }
 }
 
-// Every output row: 1 at the source, 0 elsewhere (the walks add to the rows).
+// Every output row: 0 (the walks add to the rows), and 1 at the source.
 __global__ void kb_prefill(const BatchSrc *__restrict__ src, int32_t k, int32_t n) {
   const int64_t total = (int64_t)k * n;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
@@ -232,26 +232,11 @@ __global__ void kb_prefill(const BatchSrc *__restrict__ src, int32_t k, int32_t 
 // srk_single_source with the same flag decides it.  Those nodes of all the
 // batch's sources sit in one small hash table per (step, pair), so a walk
 // tests every pending source with one lookup of its own node (one sector,
-// rarely two).  Batches hold at most 64 sources (one mask bit each).
-
-// One of 64 bits for a node: the signature of a (step, pair) has the bits of
-// the pending sources' nodes there, so a walk whose node's bit is clear
-// meets no source there.
-__device__ __forceinline__ uint32_t node_hash(int32_t x) {
-  return ((uint32_t)x * 0x9E3779B9u) >> 26;
-}
-// Is the bit of node x set in the signature (sig.x: bits 0-31, sig.y: 32-63)?
-__device__ __forceinline__ bool sig_has(uint2 sig, int32_t x) {
-  const uint32_t h = node_hash(x);
-  return ((h < 32 ? sig.x : sig.y) >> (h & 31)) & 1u;
-}
-// The first slot of node x in a meeting table of 2^tbits slots.
-__device__ __forceinline__ uint32_t slot_of(int32_t x, int tbits) {
-  return ((uint32_t)x * 0x85EBCA6Bu) >> (32 - tbits);
-}
+// rarely two).  Batches hold at most 64 sources (one mask bit each).  The walks
+// are k_lock_shared's (srk_lockstep.cu).
 
 // Per source and pair j: the pair's weight, its bit in the step masks, its
-// node's bit in the step signatures and its bit in the meeting tables of
+// node's bit in the tables' signatures and its bit in the meeting tables of
 // steps 1..cap(j) (source walk sigma(j)).  A table holds at most k nodes in
 // 2^tbits >= 2k slots, so an insertion always finds its node or a free slot.
 __global__ void kb_hitj(const __grid_constant__ BatchArgs A) {
@@ -269,10 +254,10 @@ __global__ void kb_hitj(const __grid_constant__ BatchArgs A) {
     const uint32_t smask = (1u << A.tbits) - 1u;
     for (int q = 1; q <= cap; ++q) {
       const int32_t node = node_identity(A.view, sp[q - 1]);
-      uint4 *cell = &A.M[(int64_t)(q - 1) * A.Jmax + j];
-      const uint32_t h = node_hash(node);
+      uint2 *cell = &A.M[(int64_t)j * (A.Lmax + 1) + q - 1];
+      const uint32_t h = sig_bit(node);
       atomicOr(high ? &cell->y : &cell->x, bit);
-      atomicOr(h < 32 ? &cell->z : &cell->w, 1u << (h & 31));
+      atomicOr(&A.sig[(A.rowbase[q] + j) * 32 + (h >> 5)], 1u << (h & 31));
       uint4 *tab = A.T + ((A.rowbase[q] + j) << A.tbits);
       const uint32_t key = (uint32_t)node + 1u;
       uint32_t sl = slot_of(node, A.tbits);
@@ -287,226 +272,12 @@ __global__ void kb_hitj(const __grid_constant__ BatchArgs A) {
   })
 }
 
-// The batch's sources as the shared-walk kernel reads them (shared memory).
-struct ShSrc {
-  const unsigned long long *wj;
-  double *scores;
-  uint32_t *counts;
-  double z;
-  int32_t N, s;
-};
-
-// The meeting test after a step: a stepping lane whose node x has its bit
-// in the step's signature looks x up in the step's meeting table (tab); the
-// pending sources among the slot's are those that meet here.  Their counts
-// and weight sums go to the warp's shared words cnt[b], wsum[b] (atomics:
-// lanes of a warp can meet the same source at once).  Returns them.
-__device__ __forceinline__ unsigned long long shared_meet(
-    const ShSrc *src, const uint4 *tab, int tbits, bool stepped, int32_t x,
-    unsigned long long pend, uint2 sig, int32_t j, uint32_t *cnt, unsigned long long *wsum) {
-  unsigned long long hits = 0ull;
-  if (stepped && pend != 0ull && sig_has(sig, x)) {
-    const uint32_t smask = (1u << tbits) - 1u, key = (uint32_t)x + 1u;
-    uint32_t sl = slot_of(x, tbits);
-    for (uint32_t probe = 0; probe <= smask; ++probe, sl = (sl + 1u) & smask) {
-      const uint4 e = tab[sl];
-      if (e.x == key) {
-        hits = (((unsigned long long)e.z << 32) | e.y) & pend;
-        break;
-      }
-      if (e.x == 0u) break;
-    }
-    for (unsigned long long m = hits; m; m &= m - 1) {
-      const int b = __ffsll((long long)m) - 1;
-      atomicAdd(&cnt[b], 1u);
-      atomicAdd(&wsum[b], src[b].wj[j]);
-    }
-  }
-  return hits;
-}
-
-// a4+a5 of a batch with shared target walks: warps take targets (the nodes
-// with in-neighbours) from a counter; the 32 lanes walk the target's pairs
-// j = j0, j0 + 1, ... with lane refill, one Philox2x32-10 block (counter
-// (((i-1)>>1) << 24 | j, u) under the shared walk key) per odd and following
-// even step; after
-// every step the stepping lanes' nodes are tested against their pending
-// sources (shared_meet), and lane b writes source b's count, weight sum and
-// score at the end of the target.  A source's own row
-// keeps its prefilled 1.
-// 6 blocks of 256 threads per SM (40 registers): at 8 (32 registers) every
-// form spilled.
-template <int kLayout>
-__global__ void __launch_bounds__(256, 6)
-kb_shared_walks(const __grid_constant__ BatchArgs A, const int32_t *__restrict__ act,
-                int32_t n_act, int32_t j0, unsigned long long *__restrict__ ctr) {
-  __shared__ ShSrc src[64];
-  __shared__ uint32_t cnt[8][64];
-  __shared__ unsigned long long wsum[8][64];
-  // per warp: the sources whose own row the target is, and the target's list
-  // (read at refills only, so they hold no registers across the walk)
-  __shared__ unsigned long long w_excl[8];
-  __shared__ uint32_t w_deg[8];
-  __shared__ int32_t w_base[8];
-  __shared__ long long rowbase[SRK_MAX_LEN + 2];  // meeting-table rows (A.rowbase)
-  for (int i = threadIdx.x; i <= SRK_MAX_LEN + 1; i += blockDim.x)
-    rowbase[i] = (i <= A.Lmax) ? A.rowbase[i] : 0;
-  for (int b = threadIdx.x; b < A.k; b += blockDim.x) {
-    const BatchSrc &B = A.src[b];
-    src[b] = ShSrc{B.wj, B.scores, B.counts, B.z, B.N_tot, B.s};
-  }
-  __syncthreads();
-  const uint32_t key = A.shared_key;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const auto G = adj_view<kLayout>(A.view);
-  const uint4 *M = A.M;
-  const int32_t J = A.Jmax;
-  const int tbits = A.tbits;
-  unsigned long long warp_steps = 0;
-  for (;;) {
-    int32_t q = 0;
-    if (lane == 0) q = (int32_t)atomicAdd(ctr, 1ull);
-    q = __shfl_sync(0xffffffffu, q, 0);
-    if (q >= n_act) break;
-    const uint32_t u = (uint32_t)act[q];
-    // sources whose own row this target is
-    const unsigned long long excl =
-        __ballot_sync(0xffffffffu, lane < A.k && src[lane].s == (int32_t)u) |
-        ((unsigned long long)__ballot_sync(0xffffffffu, lane + 32 < A.k &&
-                                                       src[lane + 32].s == (int32_t)u)
-         << 32);
-    cnt[wib][lane] = 0u;            // meetings of sources `lane`, `lane` + 32 at this target
-    cnt[wib][lane + 32] = 0u;
-    wsum[wib][lane] = 0ull;         // and their weight sums
-    wsum[wib][lane + 32] = 0ull;
-    if (lane == 0) {
-      uint32_t deg_u = 0;
-      w_base[wib] = node_start(G, A.view.row_ptr, (int32_t)u, deg_u);
-      w_deg[wib] = deg_u;
-      w_excl[wib] = excl;
-    }
-    __syncwarp();
-    uint32_t st = 0;
-    int32_t next = j0, j = 0, i = 1, b = 0;
-    bool live = false;
-    uint32_t deg = 0;
-    unsigned long long pend = 0ull;
-    uint2 sg = make_uint2(0u, 0u);  // the signature of the next test
-    // pend &= the mask of row `row`; sg = its signature
-    auto next_mask = [&](int64_t row) {
-      const uint4 mn = M[row];
-      pend &= ((unsigned long long)mn.y << 32) | mn.x;
-      sg = make_uint2(mn.z, mn.w);
-    };
-    for (;;) {
-      const uint32_t idle = __ballot_sync(0xffffffffu, !live);
-      if (idle) {
-        if (!live) {
-          j = next + __popc(idle & lanes_below_mask());
-          if (j < J) {
-            const uint4 m1 = M[j];
-            pend = (((unsigned long long)m1.y << 32) | m1.x) & ~w_excl[wib];
-            sg = make_uint2(m1.z, m1.w);
-            live = pend != 0ull;
-            i = 1;
-            b = w_base[wib];
-            deg = w_deg[wib];
-          }
-        }
-        next += __popc(idle);
-      }
-      if (!__any_sync(0xffffffffu, live)) {
-        if (next >= J) break;
-        continue;  // every pair of this round was dead: take the next ones
-      }
-      uint32_t x0 = 0, x1 = 0;
-      int32_t x = 0;
-      decltype(adj_entry(G, 0, 0u)) e{};
-      // odd step i
-      bool stepped = live;
-      if (stepped) {
-        philox2(key, walk_ctr0(i, (uint32_t)j), u, x0, x1);
-        e = step_entry(G, b, x0, deg, key, i, (uint32_t)j, u);
-        x = entry_pos(G, e);
-        ++st;
-      }
-      pend &= ~shared_meet(src, A.T + ((rowbase[i] + j) << tbits), tbits, stepped, x, pend,
-                           sg, j, cnt[wib], wsum[wib]);
-      if (stepped) {
-        next_mask((int64_t)i * J + j);  // still able to meet at step i + 1
-        if (!pend) {
-          live = false;
-        } else {
-          b = entry_next(G, e, x, deg);
-          if (deg == 0) live = false;
-        }
-      }
-      // even step i + 1
-      stepped = live;
-      if (stepped) {
-        e = step_entry(G, b, x1, deg, key, i + 1, (uint32_t)j, u);
-        x = entry_pos(G, e);
-        ++st;
-      }
-      pend &= ~shared_meet(src, A.T + ((rowbase[i + 1] + j) << tbits), tbits, stepped, x,
-                           pend, sg, j, cnt[wib], wsum[wib]);
-      if (stepped) {
-        next_mask((int64_t)(i + 1) * J + j);
-        if (!pend) {
-          live = false;
-        } else {
-          b = entry_next(G, e, x, deg);
-          if (deg == 0) live = false;
-          i += 2;
-        }
-      }
-    }
-    for (int off = 16; off > 0; off >>= 1) st += __shfl_xor_sync(0xffffffffu, st, off);
-    warp_steps += st;
-    __syncwarp();
-    for (int bb = lane; bb < A.k; bb += 32) {
-      if ((w_excl[wib] >> bb) & 1ull) continue;
-      const ShSrc &S = src[bb];
-      const unsigned long long W = wsum[wib][bb];
-      S.scores[u] = (double)W * 2.3283064365386963e-10 / S.z;
-      if (S.counts) S.counts[u] = cnt[wib][bb];
-    }
-    __syncwarp();
-  }
-  if (lane == 0 && warp_steps) atomicAdd(ctr + 1, warp_steps);
-}
-
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The shared-walk kernel: a persistent grid of as many 256-thread blocks as
-// fit at once (ctr[0]: the target counter, cleared here; ctr[1]: the steps).
 // The first walk index of source table t whose length is at least i (walks
 // are in stratum order): pairs below it cannot reach step i.
 static int32_t first_reaching(const QueryTab &t, int i) {
   return i <= t.L ? t.P[i] : t.N_tot;
-}
-
-static void launch_shared(int layout, cudaStream_t st, const BatchArgs &A,
-                          const int32_t *act, int32_t n_act, int32_t j0,
-                          unsigned long long *ctr, int dev) {
-  static int per_sm[3][64] = {};
-  auto grid = [&](const void *f, int l) {
-    int b = (dev >= 0 && dev < 64) ? per_sm[l][dev] : 0;
-    if (!b) {
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, 256, 0) != cudaSuccess || b < 1)
-        b = 1;
-      if (dev >= 0 && dev < 64) per_sm[l][dev] = b;
-    }
-    return sm_count(dev) * b;
-  };
-#define SRK_SH_LAUNCH(L)                                                         \
-  kb_shared_walks<L><<<grid((const void *)kb_shared_walks<L>, L), 256, 0, st>>>( \
-      A, act, n_act, j0, ctr)
-  cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), st);
-  if (layout == kWide) SRK_SH_LAUNCH(kWide);
-  else if (layout == kCsr) SRK_SH_LAUNCH(kCsr);
-  else SRK_SH_LAUNCH(kNarrow);
-#undef SRK_SH_LAUNCH
 }
 
 static std::mutex g_stream_mu;
@@ -718,7 +489,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         size_t tables = 0;
         for (int i = 1; i <= L1; ++i)
           tables += (size_t)(N1 - std::min<int64_t>(pmin[(size_t)i], first_reaching(t, i)));
-        sb = 16 * (size_t)(L1 + 1) * (size_t)N1 + ((16 * tables) << tb);
+        sb = 8 * (size_t)(L1 + 1) * (size_t)N1 + 128 * tables + ((16 * tables) << tb);
       }
       Workspace w;
       const QueryTab &t1 = tabs[(size_t)i1];
@@ -755,14 +526,17 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       rowbase[(size_t)i] = n_tables - pm;
       n_tables += Jmax - pm;
     }
-    // shared walks: the step masks and signatures, Lmax + 1 rows of Jmax
-    // 16-byte cells, the table rows and the tables
-    const size_t m_bytes = shared ? 16 * (size_t)(Lmax + 1) * (size_t)Jmax : 0;
+    // shared walks: the step masks (Jmax rows of Lmax + 1), the table rows, the
+    // signatures and the tables
+    const size_t m_bytes = shared ? 8 * (size_t)(Lmax + 1) * (size_t)Jmax : 0;
     const size_t r_bytes = shared ? sizeof(int64_t) * rowbase.size() : 0;
+    const size_t g_bytes = shared ? 128 * (size_t)n_tables : 0;
     const size_t h_bytes = shared ? (16 * (size_t)n_tables) << tbits : 0;
+    const size_t c_bytes = shared ? sizeof(SharedSrc) * (size_t)kb : 0;
     const size_t head = align256(sizeof(BatchSrc) * kb) + align256(sizeof(QueryTab) * kb) +
                         align256(sizeof(int64_t) * (kb + 1)) + 256 + align256(m_bytes) +
-                        align256(r_bytes) + align256(h_bytes);
+                        align256(r_bytes) + align256(g_bytes) + align256(h_bytes) +
+                        align256(c_bytes);
     // end filters: one region, which the sources use one after the other
     size_t extra = 0;
     for (int32_t b = i0; b < i1 && !shared; ++b)
@@ -780,9 +554,11 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     int64_t *d_off = (int64_t *)((char *)d_tab + align256(sizeof(QueryTab) * kb));
     unsigned long long *d_ctr =
         (unsigned long long *)((char *)d_off + align256(sizeof(int64_t) * (kb + 1)));
-    uint4 *d_M = (uint4 *)((char *)d_ctr + 256);
+    uint2 *d_M = (uint2 *)((char *)d_ctr + 256);
     int64_t *d_rowbase = (int64_t *)((char *)d_M + align256(m_bytes));
-    uint4 *d_T = (uint4 *)((char *)d_rowbase + align256(r_bytes));
+    uint32_t *d_sig = (uint32_t *)((char *)d_rowbase + align256(r_bytes));
+    uint4 *d_T = (uint4 *)((char *)d_sig + align256(g_bytes));
+    SharedSrc *d_ssrc = (SharedSrc *)((char *)d_T + align256(h_bytes));
     // shared walks: d_ctr[0] = target counter, d_ctr[1] = steps
     char *ws_base = base + head;
     std::vector<BatchSrc> hsrc((size_t)kb);
@@ -812,6 +588,12 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       S.z = t.z;
       hoff[(size_t)b + 1] = hoff[(size_t)b] + t.N_tot;
     }
+    std::vector<SharedSrc> ssrc;
+    for (int32_t b = 0; shared && b < kb; ++b) {
+      const BatchSrc &S = hsrc[(size_t)b];
+      ssrc.push_back(SharedSrc{S.wj, reinterpret_cast<unsigned long long *>(S.scores), S.counts,
+                               S.z, S.s});
+    }
     // tables and source descriptors (synchronous staging of pageable memory)
     if ((e = cudaMemcpyAsync(d_tab, tabs.data() + i0, sizeof(QueryTab) * kb,
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
@@ -820,7 +602,9 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         (e = cudaMemcpyAsync(d_off, hoff.data(), sizeof(int64_t) * (kb + 1),
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (shared && (e = cudaMemcpyAsync(d_rowbase, rowbase.data(), r_bytes,
-                                        cudaMemcpyHostToDevice, st)) != cudaSuccess)) {
+                                        cudaMemcpyHostToDevice, st)) != cudaSuccess) ||
+        (shared && (e = cudaMemcpyAsync(d_ssrc, ssrc.data(), c_bytes, cudaMemcpyHostToDevice,
+                                        st)) != cudaSuccess)) {
       rc = cuda_fail(e, "batch descriptors");
       cudaFreeAsync(base, st);
       break;
@@ -835,6 +619,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     A.key1 = (uint32_t)(seed >> 32);
     A.shared_key = walk_key(seed, kSharedWalkKey);
     A.M = d_M;
+    A.sig = d_sig;
     A.T = d_T;
     A.rowbase = d_rowbase;
     A.tbits = tbits;
@@ -852,8 +637,9 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       kb_fy_groups<<<gw, 256, 0, s2>>>(A);
       kb_pairs<<<gw, 256, 0, s2>>>(A);
       if (shared) {
+        cudaMemsetAsync(d_ctr, 0, 256, s2);
         cudaMemsetAsync(d_M, 0, m_bytes, s2);
-        cudaMemsetAsync(d_T, 0, h_bytes, s2);
+        cudaMemsetAsync(d_sig, 0, align256(g_bytes) + h_bytes, s2);
         kb_hitj<<<gw, 256, 0, s2>>>(A);
       } else {
         kb_rows<<<(kb + 31) / 32, 32, 0, s2>>>(A, g->n_act);
@@ -863,6 +649,25 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       kb_prefill<<<gp, 256, 0, s2>>>(d_src, kb, (int32_t)n);
     };
     const bool count = opt && opt->stats;
+    SharedWalks SW;
+    memset(&SW, 0, sizeof SW);
+    if (shared) {
+      SW.mask = d_M;
+      SW.sig = d_sig;
+      SW.T = d_T;
+      SW.rowbase = d_rowbase;
+      SW.src = d_ssrc;
+      SW.k = kb;
+      SW.rows = Lmax + 1;
+      SW.tbits = tbits;
+      SW.j0 = j0;
+      SW.J = Jmax;
+      SW.Lmax = Lmax;
+      SW.key = A.shared_key;
+      for (int r = 0; r < 10; ++r) SW.rk[r] = A.shared_key + (uint32_t)r * kPhiloxW0;
+      SW.steps = count ? d_ctr + 1 : nullptr;
+      SW.counter = reinterpret_cast<int32_t *>(d_ctr);
+    }
     auto enqueue_source = [&](int32_t b, cudaStream_t s2, const cudaEvent_t *timing, int shape,
                               int32_t max_units) {
       const BatchSrc &S = hsrc[(size_t)b];
@@ -884,7 +689,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       enqueue_source_side(s2);
       int r = SRK_OK;
       if (shared)
-        launch_shared(g->layout, s2, A, g->act, g->n_act, j0, d_ctr, dev);
+        r = enqueue_shared_walks(g, SW, s2);
       else
         for (int32_t b = 0; b < kb && r == SRK_OK; ++b)
           r = enqueue_source(b, s2, nullptr, shape, INT32_MAX);

@@ -450,6 +450,10 @@ constexpr int kCodeBits = 11;
 static int build_narrow(srk_graph *g, int dev) {
   const int32_t n = g->n;
   const int64_t m = g->m;
+  // the documented bound of this layout (n + m + n_act past 2^30 edges and nodes)
+  if ((int64_t)n + m > (1 << 30) && (int64_t)n + m + g->n_act > INT32_MAX)
+    return fail(SRK_EINVAL, "graph too large for 4-byte adjacency entries (n + m + hubs = %lld)",
+                (long long)n + (long long)m + (long long)g->n_act);
   const int pb = bits_for(n);
   const uint32_t dmax = (1u << std::min(32 - pb, kCodeBits)) - 1u;
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };

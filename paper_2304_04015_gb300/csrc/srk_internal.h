@@ -197,6 +197,33 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
 // walk_units_work is the targets x pairs of that many units over all targets.
 constexpr int kWalkShapes = 2;
 double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t max_units);
+// Shared target walks of up to 64 sources (srk_batch.cu makes the tables).
+struct SharedSrc {
+  const unsigned long long *wj;  // quantised Lemma 7 weight of pair j
+  unsigned long long *W;         // per target: weight sum (in the score row)
+  uint32_t *counts;              // per target: meetings, or null
+  double z;
+  int32_t s;
+};
+struct SharedWalks {
+  const uint2 *mask;       // [j rows + i - 1]: sources whose pair j may meet at step i
+  const uint32_t *sig;     // per meeting table: 1024 bits, one for each node of it
+  const uint4 *T;          // the meeting tables (BatchArgs in srk_batch.cu)
+  const int64_t *rowbase;  // table of (step i, pair j): rowbase[i] + j
+  const SharedSrc *src;
+  int32_t k, rows, tbits, j0, J, Lmax;
+  uint32_t key, rk[10];
+  unsigned long long *steps;  // null: not counted
+  int32_t *counter;           // units handed out (zero at the start)
+};
+int enqueue_shared_walks(const srk_graph *g, const SharedWalks &Q, cudaStream_t st);
+// The bit of a node in a signature, the first slot in a table of 2^tbits slots.
+__host__ __device__ __forceinline__ uint32_t sig_bit(int32_t x) {
+  return ((uint32_t)x * 0x9E3779B9u) >> 22;
+}
+__host__ __device__ __forceinline__ uint32_t slot_of(int32_t x, int tbits) {
+  return ((uint32_t)x * 0x85EBCA6Bu) >> (32 - tbits);
+}
 // Shared-memory opt-in of the walk kernels of a layout, in this context.
 cudaError_t allow_lockstep(int layout);
 // [*b, *e): the targets a query computes, from its options (SRK_EINVAL when

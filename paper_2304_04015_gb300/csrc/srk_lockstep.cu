@@ -746,6 +746,80 @@ __host__ __device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t
   return best;
 }
 
+// The targets act[from .. to) of a block (all but `skip`), at most kT a thread;
+// with `stage`, their lists of up to 64 entries go to shared memory while they
+// fit.  S.sums is zero on entry; every thread of the block calls.
+template <int kT, class GA, class E>
+__device__ __forceinline__ void lock_targets(const GA &G, const int32_t *__restrict__ row_ptr,
+                                             LockShared &S, E *lists,
+                                             const int32_t *__restrict__ act, int32_t from,
+                                             int32_t to, int32_t skip, bool stage,
+                                             LockTargets<kT> &X) {
+  constexpr uint32_t lists_max = kListWords * 4 / (uint32_t)sizeof(E);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int t = 0; t < kT; ++t) {
+    const int32_t i = from + t * kLockThreads + (int32_t)threadIdx.x;
+    X.u[t] = i < to ? act[i] : 0;
+    X.b[t] = node_start(G, row_ptr, X.u[t], X.d[t]);
+    if (i >= to || X.u[t] == skip) X.d[t] = 0;
+    X.st[t] = 0;
+    X.at[t] = X.d[t] ? -1 : -2;
+  }
+  if (stage) {
+    // lists of at most 64, 32, 16 or 8 entries go to shared memory: the
+    // largest bound whose lists fit
+    uint32_t sum[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int t = 0; t < kT; ++t)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (X.d[t] <= (64u >> q)) sum[q] += X.d[t];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t v = sum[q];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) atomicAdd(&S.sums[q], v);
+    }
+    __syncthreads();
+    int q = 0;
+    while (q < 4 && S.sums[q] > lists_max) ++q;
+    // first the lists below that bound, then the longer ones while they fit
+    uint32_t base = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+      auto wanted = [&](uint32_t d) {
+        return d <= 64u && (pass == (q < 4 && d <= (64u >> q) ? 0 : 1));
+      };
+      uint32_t mine = 0;
+#pragma unroll
+      for (int t = 0; t < kT; ++t)
+        if (wanted(X.d[t])) mine += X.d[t];
+      uint32_t incl = mine;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) S.warp_sum[wid] = incl;
+      __syncthreads();
+      uint32_t at = base + incl - mine;
+      for (int w = 0; w < kLockWarps; ++w) {
+        if (w < wid) at += S.warp_sum[w];
+        base += S.warp_sum[w];
+      }
+#pragma unroll
+      for (int t = 0; t < kT; ++t)
+        if (X.d[t] && wanted(X.d[t])) {
+          if (at + X.d[t] <= lists_max) {
+            X.at[t] = (int32_t)at;
+            for (uint32_t k = 0; k < X.d[t]; ++k) lists[at + k] = adj_entry(G, X.b[t], k);
+          }
+          at += X.d[t];
+        }
+      __syncthreads();
+    }
+  }
+}
+
 // The walks.  A unit of work is a block of targets and a strided set of
 // pairs; blocks take units from a counter.  A unit's targets keep their lists
 // in shared memory where they fit, for their first steps.  W[u] (in the scores
@@ -764,7 +838,6 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   uint2 *hub = reinterpret_cast<uint2 *>(queues + kQueue * kLockWarps);
   uint32_t *ctab = reinterpret_cast<uint32_t *>(hub + kHubCache);
   LockTables tabs{smem_addr(ctab), smem_addr(hub), 0u};
-  constexpr int32_t kLists = kListWords * 4 / (int)sizeof(E);
   const int32_t act_lo = bounds[2], act_hi = bounds[1];
   const int32_t n_pairs = Q.cnt[Q.min_cap], n_t = act_hi - act_lo;
   if (n_pairs == 0 || n_t <= 0) return;
@@ -772,7 +845,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
   const int64_t units = min((int64_t)n_tb * n_chunks, (int64_t)Q.max_units);
   if ((int64_t)blockIdx.x >= units) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   if (threadIdx.x < kStages) {
     mbar_init(&S.full[threadIdx.x], 1);
     mbar_init(&S.empty[threadIdx.x], kLockWarps);
@@ -796,67 +869,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
     const int32_t tb = (int32_t)(unit % n_tb);
     const int32_t first = (int32_t)(unit / n_tb), len = (n_pairs - first + n_chunks - 1) / n_chunks;
     LockTargets<kT> X;
-#pragma unroll
-    for (int t = 0; t < kT; ++t) {
-      const int32_t i = act_lo + tb * T + t * kLockThreads + threadIdx.x;
-      X.u[t] = i < act_hi ? act[i] : 0;
-      X.b[t] = node_start(G, V.row_ptr, X.u[t], X.d[t]);
-      if (i >= act_hi || X.u[t] == Q.s) X.d[t] = 0;
-      X.st[t] = 0;
-      X.at[t] = X.d[t] ? -1 : -2;
-    }
-    if (len >= 32) {
-      // lists of at most 64, 32, 16 or 8 entries go to shared memory: the
-      // largest bound whose lists fit
-      uint32_t sum[4] = {0, 0, 0, 0};
-#pragma unroll
-      for (int t = 0; t < kT; ++t)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (X.d[t] <= (64u >> q)) sum[q] += X.d[t];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t v = sum[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) atomicAdd(&S.sums[q], v);
-      }
-      __syncthreads();
-      int q = 0;
-      while (q < 4 && S.sums[q] > (uint32_t)kLists) ++q;
-      // first the lists below that bound, then the longer ones while they fit
-      uint32_t base = 0;
-      for (int pass = 0; pass < 2; ++pass) {
-        auto wanted = [&](uint32_t d) {
-          return d <= 64u && (pass == (q < 4 && d <= (64u >> q) ? 0 : 1));
-        };
-        uint32_t mine = 0;
-#pragma unroll
-        for (int t = 0; t < kT; ++t)
-          if (wanted(X.d[t])) mine += X.d[t];
-        uint32_t incl = mine;
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        if (lane == 31) S.warp_sum[wid] = incl;
-        __syncthreads();
-        uint32_t at = base + incl - mine;
-        for (int w = 0; w < kLockWarps; ++w) {
-          if (w < wid) at += S.warp_sum[w];
-          base += S.warp_sum[w];
-        }
-#pragma unroll
-        for (int t = 0; t < kT; ++t)
-          if (X.d[t] && wanted(X.d[t])) {
-            if (at + X.d[t] <= (uint32_t)kLists) {
-              X.at[t] = (int32_t)at;
-              for (uint32_t k = 0; k < X.d[t]; ++k) lists[at + k] = adj_entry(G, X.b[t], k);
-            }
-            at += X.d[t];
-          }
-        __syncthreads();
-      }
-    }
+    lock_targets(G, V.row_ptr, S, lists, act, act_lo + tb * T, act_hi, Q.s, len >= 32, X);
     lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len, seq,
                                X);
 #pragma unroll
@@ -893,6 +906,198 @@ k_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ bounds
     int64_t t = bounds[1] - bounds[2];
     if (s >= u_begin && s < u_end && row_ptr[s + 1] > row_ptr[s]) --t;
     atomicAdd(steps_total, (unsigned long long)t * one);
+  }
+}
+
+// ---------------------------------------------------- shared target walks --
+// SRK_OPT_SHARED_WALKS: walk j of a target serves pair j of every source of
+// the batch, as long as some source's pair can still meet.  In lockstep the
+// pending sources, the nodes they wait at and the table of those nodes are the
+// same for all targets; a target only keeps the sources that its walk j has
+// met.  A node is looked up in the step's table when its bit is set in the
+// table's signature: 1024 bits, one L1 line that all the block's warps read,
+// so at most 6 % of the walks that meet nobody go to the table (with a 64-bit
+// signature in a register, the form before, half of them did).
+// A warp per target with lanes over pairs took 10.4 ms for 48 sources on R-MAT
+// 18, eps = 0.05; this takes 6.2 ms, with 54 % of the issue slots and 62 % of the
+// request cycles to the L2 in use; 2 targets a thread 6.6
+// ms, 1 8.6 ms.
+constexpr int kSharedTargets = 3;  // per thread
+
+template <int kLayout, bool kCount>
+__global__ void __launch_bounds__(kLockThreads, kLockBlocks)
+k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ act, int32_t n_act,
+              const __grid_constant__ SharedWalks Q) {
+  constexpr int kT = kSharedTargets;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  __shared__ LockShared S;
+  __shared__ int64_t rowbase[SRK_MAX_LEN + 2];
+  __shared__ int32_t src_s[64];
+  __shared__ int32_t own_rows;  // some target of the unit is a source
+  const auto G = adj_view<kLayout>(V);
+  using E = decltype(adj_entry(G, 0, 0u));
+  E *lists = reinterpret_cast<E *>(dyn);
+  uint2 *hub = reinterpret_cast<uint2 *>(dyn + 4 * kListWords);
+  uint32_t *ctab = reinterpret_cast<uint32_t *>(hub + kHubCache);
+  unsigned long long *excl = reinterpret_cast<unsigned long long *>(ctab + kCodes);
+  LockTables tabs{smem_addr(ctab), smem_addr(hub), 0u};
+  const int32_t n_pairs = Q.J - Q.j0;
+  if (n_pairs <= 0 || n_act <= 0) return;
+  const int32_t T = kLockThreads * kT, n_tb = (n_act + T - 1) / T;
+  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
+  const int64_t units = (int64_t)n_tb * n_chunks;
+  if ((int64_t)blockIdx.x >= units) return;
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i <= SRK_MAX_LEN + 1; i += kLockThreads)
+    rowbase[i] = (i >= 1 && i <= Q.Lmax) ? Q.rowbase[i] : 0;
+  for (int i = threadIdx.x; i < 64; i += kLockThreads) src_s[i] = i < Q.k ? Q.src[i].s : -1;
+  if constexpr (kLayout == kNarrow) {
+    tabs.n_hub = (uint32_t)min(V.n_hubs, kHubCache);
+    for (uint32_t i = threadIdx.x; i < tabs.n_hub; i += kLockThreads) hub[i] = V.hub[i];
+    for (uint32_t i = threadIdx.x; i <= V.deg_max; i += kLockThreads) ctab[i] = V.ctab[i];
+  }
+  const uint32_t lists_at = smem_addr(lists), smask = (1u << Q.tbits) - 1u;
+  unsigned long long total = 0;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      S.unit = atomicAdd(Q.counter, 1);
+      own_rows = 0;
+    }
+    if (threadIdx.x < 4) S.sums[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t unit = S.unit;
+    if (unit >= units) break;
+    const int32_t tb = (int32_t)(unit % n_tb), first = (int32_t)(unit / n_tb);
+    LockTargets<kT> X;
+    lock_targets(G, V.row_ptr, S, lists, act, tb * T, n_act, -1, (n_pairs - first) / n_chunks >= 32,
+                 X);
+#pragma unroll
+    for (int t = 0; t < kT; ++t) {
+      unsigned long long m = 0ull;
+      for (int b = 0; b < Q.k; ++b)
+        if (X.d[t] && src_s[b] == X.u[t]) m |= 1ull << b;
+      excl[t * kLockThreads + threadIdx.x] = m;
+      if (m) own_rows = 1;
+    }
+    __syncthreads();
+    const bool any_own = own_rows != 0;
+    uint2 m0 = Q.mask[(int64_t)(Q.j0 + first) * Q.rows];
+    for (int32_t q = first; q < n_pairs; q += n_chunks) {
+      const int32_t j = Q.j0 + q;
+      uint2 m = m0;
+      if (q + n_chunks < n_pairs) m0 = Q.mask[(int64_t)(j + n_chunks) * Q.rows];
+      if (!(m.x | m.y)) continue;
+      const uint2 *mask = Q.mask + (int64_t)j * Q.rows;
+      int32_t b[kT];
+      uint32_t deg[kT], x0[kT], x1[kT], idx[kT];
+      uint2 gone[kT];  // sources met, or whose own row this is
+      E e[kT];
+#pragma unroll
+      for (int t = 0; t < kT; ++t) {
+        philox2k(Q.rk, (uint32_t)j, (uint32_t)X.u[t], x0[t], x1[t]);
+        gone[t] = make_uint2(0u, 0u);
+        deg[t] = X.d[t];
+        if (any_own) {
+          const unsigned long long g = excl[t * kLockThreads + threadIdx.x];
+          gone[t] = make_uint2((uint32_t)g, (uint32_t)(g >> 32));
+          if (!((m.x & ~gone[t].x) | (m.y & ~gone[t].y))) deg[t] = 0;
+        }
+      }
+      lock_index(x0, deg, Q.key, 1, (uint32_t)j, X.u, idx);
+#pragma unroll
+      for (int t = 0; t < kT; ++t) {
+        e[t] = E{};
+        const bool p = deg[t] != 0;
+        load_if(p && X.at[t] >= 0, lists_at + (uint32_t)sizeof(E) * ((uint32_t)X.at[t] + idx[t]),
+                e[t]);
+        load_if(p && X.at[t] < 0, entries(G) + ((uint32_t)X.b[t] + idx[t]), e[t]);
+      }
+      for (int i = 1;; ++i) {
+        // the walks are at the nodes that the entries e of step i name
+        const uint2 mn = mask[i];
+        const int64_t table = rowbase[i] + j;
+        const uint32_t *sig = Q.sig + table * 32;
+        bool cand[kT], any = false;
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+          const uint32_t h = sig_bit(entry_pos(G, e[t]));
+          uint32_t word = 0;
+          load_if(deg[t] != 0, sig + (h >> 5), word);
+          cand[t] = (word >> (h & 31)) & 1u;
+          any |= cand[t];
+          if (kCount && deg[t]) ++X.st[t];
+        }
+        if (any) {
+#pragma unroll
+          for (int t = 0; t < kT; ++t) {
+            if (!cand[t]) continue;
+            const int32_t x = entry_pos(G, e[t]);
+            const uint4 *tab = Q.T + (table << Q.tbits);
+            uint32_t sl = slot_of(x, Q.tbits);
+            for (uint32_t probe = 0; probe <= smask; ++probe, sl = (sl + 1u) & smask) {
+              const uint4 c = tab[sl];
+              if (c.x == (uint32_t)x + 1u) {
+                const uint32_t lo = c.y & m.x & ~gone[t].x, hi = c.z & m.y & ~gone[t].y;
+                gone[t].x |= lo;
+                gone[t].y |= hi;
+                for (unsigned long long w = ((unsigned long long)hi << 32) | lo; w; w &= w - 1) {
+                  const SharedSrc &B = Q.src[__ffsll((long long)w) - 1];
+                  atomicAdd(&B.W[X.u[t]], B.wj[j]);
+                  if (B.counts) atomicAdd(&B.counts[X.u[t]], 1u);
+                }
+                break;
+              }
+              if (c.x == 0u) break;
+            }
+          }
+        }
+        if (!(mn.x | mn.y)) break;  // no source's pair j reaches step i + 1
+        m = mn;
+        uint32_t live = 0;
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+          const bool p = deg[t] != 0 && ((m.x & ~gone[t].x) | (m.y & ~gone[t].y)) != 0;
+          b[t] = lock_next(G, tabs, p, e[t], entry_pos(G, e[t]), deg[t]);
+          live |= deg[t];
+        }
+        if (!__any_sync(0xffffffffu, live != 0)) break;
+        if (!(i & 1)) {
+#pragma unroll
+          for (int t = 0; t < kT; ++t)
+            philox2k(Q.rk, walk_ctr0(i + 1, (uint32_t)j), (uint32_t)X.u[t], x0[t], x1[t]);
+          lock_index(x0, deg, Q.key, i + 1, (uint32_t)j, X.u, idx);
+        } else {
+          lock_index(x1, deg, Q.key, i + 1, (uint32_t)j, X.u, idx);
+        }
+#pragma unroll
+        for (int t = 0; t < kT; ++t)
+          load_if(deg[t] != 0, entries(G) + ((uint32_t)b[t] + idx[t]), e[t]);
+      }
+    }
+    if (kCount) {
+#pragma unroll
+      for (int t = 0; t < kT; ++t) total += X.st[t];
+    }
+  }
+  if (kCount) {
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    if (lane == 0 && total) atomicAdd(Q.steps, total);
+  }
+}
+
+// The rows' scores from their weight sums.
+__global__ void __launch_bounds__(256)
+k_finish_rows(const SharedSrc *__restrict__ src, int32_t k, int32_t n) {
+  const int64_t total = (int64_t)k * n;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
+       g += (int64_t)gridDim.x * blockDim.x) {
+    const int i = (int)(g / n);
+    const int32_t u = (int32_t)(g - (int64_t)i * n);
+    double *scores = reinterpret_cast<double *>(src[i].W);
+    const unsigned long long W = src[i].W[u];
+    if (u == src[i].s) scores[u] = 1.0;
+    else if (W) scores[u] = (double)W * 2.3283064365386963e-10 / src[i].z;
   }
 }
 
@@ -959,6 +1164,8 @@ static cudaError_t allow_lock_t() {
   set((const void *)k_lockstep<kLayout, true, 1>);
   set((const void *)k_lockstep<kLayout, false, kLockTargets>);
   set((const void *)k_lockstep<kLayout, true, kLockTargets>);
+  set((const void *)k_lock_shared<kLayout, false>);
+  set((const void *)k_lock_shared<kLayout, true>);
   return e;
 }
 cudaError_t allow_lockstep(int layout) {
@@ -1054,6 +1261,28 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return SRK_OK;
+}
+
+int enqueue_shared_walks(const srk_graph *g, const SharedWalks &Q, cudaStream_t st) {
+  const GraphView V = view_of(g);
+  const int grid = sm_count(g->device) * kLockBlocks;
+  const size_t smem = 4 * (size_t)kListWords + 8 * kHubCache + 4 * kCodes +
+                      8 * (size_t)kSharedTargets * kLockThreads;
+  static_assert(4 * (size_t)kListWords + 8 * kHubCache + 4 * kCodes +
+                        8 * (size_t)kSharedTargets * kLockThreads <= kLockSmem,
+                "the opt-in covers both kernels");
+#define SRK_SHARED(L)                                                                       \
+  do {                                                                                      \
+    if (Q.steps) k_lock_shared<L, true><<<grid, kLockThreads, smem, st>>>(V, g->act, g->n_act, Q); \
+    else k_lock_shared<L, false><<<grid, kLockThreads, smem, st>>>(V, g->act, g->n_act, Q);  \
+  } while (0)
+  if (g->layout == kWide) SRK_SHARED(kWide);
+  else if (g->layout == kCsr) SRK_SHARED(kCsr);
+  else SRK_SHARED(kNarrow);
+#undef SRK_SHARED
+  k_finish_rows<<<grid_for((int64_t)Q.k * g->n, 1024, g->device), 256, 0, st>>>(Q.src, Q.k, g->n);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? SRK_OK : cuda_fail(e, "shared walks: launch");
 }
 
 }  // namespace srk
