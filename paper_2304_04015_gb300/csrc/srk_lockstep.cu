@@ -886,21 +886,47 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   }
 }
 
-// Scores from the weight sums, and the steps of the pairs that k_edges decided.
+// Scores from weight sums.  Most sums are 0, whose bits are the score 0.0
+// already; the others of a tile are gathered first, since an FP64 division
+// holds a warp for as long with one active lane as with 32 (1.05 M targets: 48
+// us with a division in every warp).  row[u] for u in [u0, u1), one tile.
+constexpr int kFinishTile = 2048;
+__device__ __forceinline__ void finish_tile(double *__restrict__ row, int64_t u0, int64_t u1,
+                                            double z, uint16_t *list, int32_t *n_list) {
+  if (threadIdx.x == 0) *n_list = 0;
+  __syncthreads();
+  for (int64_t u = u0 + threadIdx.x; u < u1; u += blockDim.x)
+    if (__double_as_longlong(row[u]) != 0) list[atomicAdd(n_list, 1)] = (uint16_t)(u - u0);
+  __syncthreads();
+  for (int32_t q = threadIdx.x; q < *n_list; q += blockDim.x) {
+    const int64_t u = u0 + list[q];
+    row[u] = (double)(unsigned long long)__double_as_longlong(row[u]) * 2.3283064365386963e-10 / z;
+  }
+  __syncthreads();
+}
+
+// Scores of a query, and the steps of the pairs that k_edges decided.
 __global__ void __launch_bounds__(256)
 k_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ bounds,
          const int32_t *__restrict__ cnt, int32_t s, int32_t u_begin, int32_t u_end, double z,
          int32_t skipped, double *__restrict__ scores, unsigned long long *__restrict__ wsums,
          uint32_t *__restrict__ steps, unsigned long long *__restrict__ steps_total) {
+  __shared__ uint16_t list[kFinishTile];
+  __shared__ int32_t n_list;
   // pairs of cap 1 decided per edge: one step each of every target
   const uint32_t one = skipped ? (uint32_t)(cnt[1] - cnt[2]) : 0u;
-  for (int64_t u = (int64_t)u_begin + blockIdx.x * blockDim.x + threadIdx.x; u < u_end;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long W = (unsigned long long)__double_as_longlong(scores[u]);
-    if (wsums) wsums[u] = W;
-    // most targets meet nowhere, and an FP64 division is slow: 0 is 0 / z
-    scores[u] = u == s ? 1.0 : W ? (double)W * 2.3283064365386963e-10 / z : 0.0;
-    if (steps && one && u != s && row_ptr[u + 1] > row_ptr[u]) steps[u] += one;
+  for (int64_t u0 = (int64_t)u_begin + (int64_t)blockIdx.x * kFinishTile; u0 < u_end;
+       u0 += (int64_t)gridDim.x * kFinishTile) {
+    const int64_t u1 = min((int64_t)u_end, u0 + kFinishTile);
+    if (wsums || (steps && one))
+      for (int64_t u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
+        // (the batched path hands in a row that is 1 at s; s has no sum)
+        if (wsums) wsums[u] = u == s ? 0ull : (unsigned long long)__double_as_longlong(scores[u]);
+        if (steps && one && u != s && row_ptr[u + 1] > row_ptr[u]) steps[u] += one;
+      }
+    if (cnt[1] > 0) finish_tile(scores, u0, u1, z, list, &n_list);
+    __syncthreads();
+    if (threadIdx.x == 0 && s >= u0 && s < u1) scores[s] = 1.0;
   }
   if (one && blockIdx.x == 0 && threadIdx.x == 0) {
     int64_t t = bounds[1] - bounds[2];
@@ -1086,18 +1112,18 @@ k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ a
   }
 }
 
-// The rows' scores from their weight sums.
+// The rows' scores from their weight sums (blockIdx.y: the row).
 __global__ void __launch_bounds__(256)
-k_finish_rows(const SharedSrc *__restrict__ src, int32_t k, int32_t n) {
-  const int64_t total = (int64_t)k * n;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(g / n);
-    const int32_t u = (int32_t)(g - (int64_t)i * n);
-    double *scores = reinterpret_cast<double *>(src[i].W);
-    const unsigned long long W = src[i].W[u];
-    if (u == src[i].s) scores[u] = 1.0;
-    else if (W) scores[u] = (double)W * 2.3283064365386963e-10 / src[i].z;
+k_finish_rows(const SharedSrc *__restrict__ src, int32_t n) {
+  __shared__ uint16_t list[kFinishTile];
+  __shared__ int32_t n_list;
+  const SharedSrc B = src[blockIdx.y];
+  double *scores = reinterpret_cast<double *>(B.W);
+  for (int64_t u0 = (int64_t)blockIdx.x * kFinishTile; u0 < n;
+       u0 += (int64_t)gridDim.x * kFinishTile) {
+    const int64_t u1 = min((int64_t)n, u0 + kFinishTile);
+    finish_tile(scores, u0, u1, B.z, list, &n_list);
+    if (threadIdx.x == 0 && B.s >= u0 && B.s < u1) scores[B.s] = 1.0;
   }
 }
 
@@ -1255,8 +1281,8 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   }
   if (timing) cudaEventRecord(timing[1], st);
   if (nr > 0)
-    k_finish<<<grid_for(nr, 256, dev), 256, 0, st>>>(g->row_ptr, bounds, sm.cnt, t.s, u_begin,
-                                                     u_end, t.z, F.slots ? 1 : 0, o.scores,
+    k_finish<<<grid_for(nr, kFinishTile, dev), 256, 0, st>>>(g->row_ptr, bounds, sm.cnt, t.s,
+                                                             u_begin, u_end, t.z, F.slots ? 1 : 0, o.scores,
                                                      o.wsums, o.steps, sm.ctr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
@@ -1280,7 +1306,10 @@ int enqueue_shared_walks(const srk_graph *g, const SharedWalks &Q, cudaStream_t 
   else if (g->layout == kCsr) SRK_SHARED(kCsr);
   else SRK_SHARED(kNarrow);
 #undef SRK_SHARED
-  k_finish_rows<<<grid_for((int64_t)Q.k * g->n, 1024, g->device), 256, 0, st>>>(Q.src, Q.k, g->n);
+  const dim3 rows((unsigned)std::min<int64_t>((g->n + (int64_t)kFinishTile - 1) / kFinishTile,
+                                              (int64_t)sm_count(g->device) * 4),
+                  (unsigned)Q.k);
+  k_finish_rows<<<rows, 256, 0, st>>>(Q.src, g->n);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SRK_OK : cuda_fail(e, "shared walks: launch");
 }

@@ -7,9 +7,10 @@
 // device, and the selection runs on those rows.
 //
 // Selection of one row (scores are non-negative doubles, whose IEEE bit
-// patterns order like unsigned integers): eight radix-select passes over the
-// 64-bit key, one byte per pass from the top, find the key T of the top-th
-// largest entry and how many entries equal to T are still needed; then every
+// patterns order like unsigned integers): six radix-select passes over the
+// key, eleven bits per pass from the top (the first the exponent), find the key
+// T of the top-th largest entry and how many entries equal to T are still
+// needed; then every
 // entry above T is taken, and of the entries equal to T the ones with the
 // smallest ids (a chunked scan keeps id order); a block sorts the selection by
 // (score descending, id ascending).
@@ -24,7 +25,12 @@
 namespace srk {
 namespace {
 
-constexpr int kChunk = 65536;     // targets per block of the tie scan
+constexpr int kChunk = 8192;      // targets per block of the tie scan
+constexpr int kBins = 2048;       // of a pass's digit
+constexpr int kPasses = 6;
+// The passes' digits: bits [shift, shift + 11), the last one 8 bits.
+__host__ __device__ constexpr int pass_shift(int p) { return p < 5 ? 52 - 11 * p : 0; }
+__host__ __device__ constexpr int pass_bins(int p) { return p < 5 ? kBins : 256; }
 constexpr int kMaxTop = 4096;     // largest `top` (the final sort is one block)
 
 struct RowSel {
@@ -41,70 +47,84 @@ __device__ __forceinline__ unsigned long long key_of(const double *row, int32_t 
   return (unsigned long long)__double_as_longlong(row[u]);
 }
 
-// Nonzero scores per row, the source excluded.
-__global__ void k_topk_count(const double *__restrict__ rows, int64_t n, int32_t R,
-                             const int32_t *__restrict__ src, RowSel *__restrict__ sel) {
-  const int r = blockIdx.y;
-  const double *row = rows + (int64_t)r * n;
-  int64_t c = 0;
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x)
-    c += (u != src[r] && key_of(row, (int32_t)u) != 0ull) ? 1 : 0;
-  for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd((unsigned long long *)&sel[r].nnz,
-                                              (unsigned long long)c);
-}
-
-// Histogram of key byte `shift` over the row's candidates (nonzero keys
-// matching the prefix so far).
-__global__ void k_topk_hist(const double *__restrict__ rows, int64_t n,
-                            const int32_t *__restrict__ src, const RowSel *__restrict__ sel,
-                            int shift, unsigned int *__restrict__ hist) {
-  __shared__ unsigned int h[256];
-  const int r = blockIdx.y;
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
-  __syncthreads();
+// Histogram of pass p's digit over the row's candidates: the nonzero keys that
+// match the prefix so far, the source excluded; pass 0 counts them.
+__global__ void __launch_bounds__(256)
+k_topk_hist(const double *__restrict__ rows, int64_t n, const int32_t *__restrict__ src,
+            RowSel *__restrict__ sel, int p, unsigned int *__restrict__ hist) {
+  __shared__ unsigned int h[kBins];
+  const int r = blockIdx.y, bins = pass_bins(p), shift = pass_shift(p);
   const RowSel S = sel[r];
-  if (S.nnz > S.need || S.mask != 0ull) {  // rows with nnz <= top take every nonzero key
-    const double *row = rows + (int64_t)r * n;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-         u += (int64_t)gridDim.x * blockDim.x) {
-      const unsigned long long k = key_of(row, (int32_t)u);
-      if (k != 0ull && u != src[r] && (k & S.mask) == S.prefix)
-        atomicAdd(&h[(k >> shift) & 255ull], 1u);
+  if (p > 0 && S.mask == 0ull) return;  // rows with nnz <= top take every nonzero key
+  for (int i = threadIdx.x; i < bins; i += blockDim.x) h[i] = 0;
+  __syncthreads();
+  const double *row = rows + (int64_t)r * n;
+  const int32_t s = src[r];
+  unsigned int c = 0;
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long k = key_of(row, (int32_t)u);
+    if (k != 0ull && u != s && (k & S.mask) == S.prefix) {
+      atomicAdd(&h[(k >> shift) & (unsigned)(bins - 1)], 1u);
+      ++c;
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[r * 256 + i], h[i]);
+  for (int i = threadIdx.x; i < bins; i += blockDim.x)
+    if (h[i]) atomicAdd(&hist[r * kBins + i], h[i]);
+  if (p == 0) {
+    for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+    if ((threadIdx.x & 31) == 0 && c)
+      atomicAdd((unsigned long long *)&sel[r].nnz, (unsigned long long)c);
+  }
 }
 
-// One thread per row: the byte at `shift` of the need-th largest candidate.
-__global__ void k_topk_pick(int32_t R, int shift, unsigned int *__restrict__ hist,
-                            RowSel *__restrict__ sel) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
-  RowSel &S = sel[r];
-  unsigned int *h = hist + r * 256;
-  if (S.nnz > S.need || S.mask != 0ull) {
-    int64_t above = 0;
-    int b = 255;
-    for (; b > 0; --b) {
-      if (above + (int64_t)h[b] >= S.need) break;
-      above += h[b];
-    }
-    S.prefix |= (unsigned long long)b << shift;
-    S.mask |= 255ull << shift;
-    S.need -= above;
+// One block per row: the digit of the need-th largest candidate in pass p; the
+// histogram is cleared for the next pass.  (One thread a row took 30 us a pass.)
+__global__ void __launch_bounds__(256)
+k_topk_pick(int p, unsigned int *__restrict__ hist, RowSel *__restrict__ sel) {
+  constexpr int kPer = kBins / 256;
+  __shared__ unsigned int warp_sum[8];
+  RowSel &S = sel[blockIdx.x];
+  unsigned int *h = hist + (int64_t)blockIdx.x * kBins;
+  const int64_t need = S.need, nnz = S.nnz;
+  const bool run = p == 0 ? nnz > need : S.mask != 0ull;
+  const int bins = pass_bins(p), shift = pass_shift(p);
+  // thread t has bins [top - 8 t - 7, top - 8 t], the largest first
+  unsigned int v[kPer], sum = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int b = kBins - 1 - (int)threadIdx.x * kPer - k;
+    v[k] = run && b < bins ? h[b] : 0u;
+    sum += v[k];
+    h[b] = 0u;
   }
-  for (int i = 0; i < 256; ++i) h[i] = 0;
-  if (shift == 0) {  // done: entries above T, then `need` entries equal to T
-    if (S.mask == 0ull) {  // nnz <= top: every nonzero key, none by tie rank
-      S.thr = 0ull;
-      S.take_eq = 0;
-    } else {
-      S.thr = S.prefix;
-      S.take_eq = S.need;
+  unsigned int incl = sum;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) warp_sum[wid] = incl;
+  __syncthreads();
+  int64_t above = (int64_t)incl - sum;
+  for (int w = 0; w < wid; ++w) above += warp_sum[w];
+  if (run && above < need && above + (int64_t)sum >= need) {  // one thread
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (above < need && above + (int64_t)v[k] >= need) {
+        const int b = kBins - 1 - (int)threadIdx.x * kPer - k;
+        S.prefix |= (unsigned long long)b << shift;
+        S.mask |= (unsigned long long)(bins - 1) << shift;
+        S.need = need - above;
+        if (p == kPasses - 1) {  // entries above T, then `need` entries equal to T
+          S.thr = S.prefix;
+          S.take_eq = need - above;
+        }
+        above = need;  // done
+      } else {
+        above += v[k];
+      }
     }
   }
 }
@@ -135,7 +155,9 @@ __global__ void k_topk_ties(const double *__restrict__ rows, int64_t n,
 
 // The selection: every entry above T (slots by atomics), then the entries
 // equal to T in id order until take_eq are taken (each chunk knows how many
-// ties precede it; inside the chunk a block-wide ordered scan ranks them).
+// ties precede it; a chunk that has some to take ranks them by a block-wide
+// ordered scan, the others never wait for one another: 64 rows of 131,072 in
+// 26 us, 237 with the scan in every chunk of 65,536).
 __global__ void __launch_bounds__(256)
 k_topk_collect(const double *__restrict__ rows, int64_t n, const int32_t *__restrict__ src,
                RowSel *__restrict__ sel, int32_t n_chunks, const int32_t *__restrict__ ties,
@@ -144,45 +166,47 @@ k_topk_collect(const double *__restrict__ rows, int64_t n, const int32_t *__rest
   const int r = blockIdx.y, ch = blockIdx.x;
   const RowSel S = sel[r];
   const double *row = rows + (int64_t)r * n;
-  __shared__ int64_t before;
-  __shared__ int wsum[8];
-  if (threadIdx.x == 0) {
-    int64_t t = 0;
-    for (int c = 0; c < ch; ++c) t += ties[r * n_chunks + c];
-    before = t;
-  }
-  __syncthreads();
+  const int32_t s = src[r];
   const int64_t n_gt_total = S.mask == 0ull ? S.nnz : (int64_t)top - S.take_eq;
   unsigned long long *ok = out_key + (int64_t)r * top;
   int32_t *oi = out_id + (int64_t)r * top;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t run = before;  // ties before this tile (same in every thread)
   const int64_t b = (int64_t)ch * kChunk, e = std::min<int64_t>(n, b + kChunk);
-  for (int64_t t0 = b; t0 < e; t0 += blockDim.x) {
-    const int64_t u = t0 + threadIdx.x;
-    unsigned long long k = 0ull;
-    bool valid = u < e && u != src[r];
-    if (valid) k = key_of(row, (int32_t)u);
-    if (valid && k > S.thr) {
+  for (int64_t u = b + threadIdx.x; u < e; u += blockDim.x) {
+    const unsigned long long k = key_of(row, (int32_t)u);
+    if (k > S.thr && u != s) {
       const int slot = atomicAdd(&sel[r].n_gt, 1);
       if (slot < n_gt_total && slot < top) {
         ok[slot] = k;
         oi[slot] = (int32_t)u;
       }
     }
-    const bool tie = valid && S.take_eq > 0 && k == S.thr;
+  }
+  if (S.take_eq <= 0 || ties[r * n_chunks + ch] == 0) return;
+  __shared__ int64_t part[8];
+  __shared__ int wsum[8];
+  int64_t run = 0;  // ties before this tile (same in every thread)
+  for (int c = threadIdx.x; c < ch; c += blockDim.x) run += ties[r * n_chunks + c];
+  for (int off = 16; off > 0; off >>= 1) run += __shfl_xor_sync(0xffffffffu, run, off);
+  if (lane == 0) part[w] = run;
+  __syncthreads();
+  run = 0;
+  for (int x = 0; x < 8; ++x) run += part[x];
+  for (int64_t t0 = b; t0 < e && run < S.take_eq; t0 += blockDim.x) {
+    const int64_t u = t0 + threadIdx.x;
+    const bool tie = u < e && u != s && key_of(row, (int32_t)u) == S.thr;
     const unsigned int bal = __ballot_sync(0xffffffffu, tie);
     if (lane == 0) wsum[w] = __popc(bal);
     __syncthreads();
     int64_t rank = run + __popc(bal & ((1u << lane) - 1u));
     int64_t tile = 0;
-    for (int x = 0; x < (int)(blockDim.x >> 5); ++x) {
+    for (int x = 0; x < 8; ++x) {
       if (x < w) rank += wsum[x];
       tile += wsum[x];
     }
     if (tie && rank < S.take_eq) {
       const int64_t slot = n_gt_total + rank;
-      ok[slot] = k;
+      ok[slot] = S.thr;
       oi[slot] = (int32_t)u;
     }
     run += tile;
@@ -285,7 +309,7 @@ extern "C" int srk_multi_source_topk(const srk_graph *g, const int32_t *sources,
   // scratch: rows, per-row state, histograms, tie counts, selection, sources
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t b_rows = al(8 * (size_t)R * n), b_sel = al(sizeof(RowSel) * R),
-               b_hist = al(4 * 256 * (size_t)R), b_ties = al(4 * (size_t)R * n_chunks),
+               b_hist = al(4 * kBins * (size_t)R), b_ties = al(4 * (size_t)R * n_chunks),
                b_key = al(8 * (size_t)R * top), b_id = al(4 * (size_t)R * top),
                b_src = al(4 * (size_t)R), b_dst = al(4 * (size_t)R);
   cudaMemPool_t mp = pool(g->device);
@@ -365,16 +389,15 @@ extern "C" int srk_multi_source_topk(const srk_graph *g, const int32_t *sources,
                              st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(ddst, order.data() + i0, 4 * (size_t)r, cudaMemcpyHostToDevice,
                              st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(hist, 0, 4 * 256 * (size_t)r, st)) != cudaSuccess) {
+        (e = cudaMemsetAsync(hist, 0, 4 * kBins * (size_t)r, st)) != cudaSuccess) {
       rc = cuda_fail(e, "srk_multi_source_topk: row state");
       break;
     }
-    const dim3 grid_rows((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 1023) / 1024, (int64_t)sms * 4)),
+    const dim3 grid_rows((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 4095) / 4096, (int64_t)sms * 4)),
                          (unsigned)r);
-    k_topk_count<<<grid_rows, 256, 0, st>>>(rows, n, r, dsrc, sel);
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      k_topk_hist<<<grid_rows, 256, 0, st>>>(rows, n, dsrc, sel, shift, hist);
-      k_topk_pick<<<(r + 127) / 128, 128, 0, st>>>(r, shift, hist, sel);
+    for (int p = 0; p < kPasses; ++p) {
+      k_topk_hist<<<grid_rows, 256, 0, st>>>(rows, n, dsrc, sel, p, hist);
+      k_topk_pick<<<r, 256, 0, st>>>(p, hist, sel);
     }
     const dim3 grid_chunks((unsigned)n_chunks, (unsigned)r);
     k_topk_ties<<<grid_chunks, 256, 0, st>>>(rows, n, dsrc, sel, n_chunks, ties);
