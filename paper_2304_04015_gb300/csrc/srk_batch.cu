@@ -81,135 +81,6 @@ __device__ __forceinline__ int find_source(const int64_t *off, int k, int64_t g)
     __VA_ARGS__                                                                  \
   }
 
-// a2: source walks (on the CSR: spos holds node ids) and Fisher-Yates draws of
-// every source of the batch.
-__global__ void __launch_bounds__(256) kb_source_walks(const __grid_constant__ BatchArgs A) {
-  const RoundKeys rk = round_keys(A.key0, A.key1);
-  const AdjC G{A.view.row_ptr, A.view.col};
-  SRK_BATCH_LOOP(A, {
-    const QueryTab &t = *S_.tab;
-    const uint32_t s = (uint32_t)S_.s;
-    uint32_t deg_s = 0;
-    const int32_t b_s = node_start(G, A.view.row_ptr, S_.s, deg_s);
-    const int Ls = S_.L > 0 ? S_.L : 1;
-    S_.w.grp_cnt[r_] = 0;
-    S_.w.kdraw[r_] = (r_ >= 1) ? fy_draw(rk, s, r_) : 0;
-    const int len = stratum_of(t.P, S_.L, r_);
-    const int eff = source_walk(t.skey, G, s, b_s, deg_s, r_, len,
-                                S_.w.spos + (int64_t)r_ * Ls);
-    S_.w.seff[r_] = eff;
-    atomicAdd(small_view(S_.w.small).ctr + 1, (unsigned long long)eff);
-  })
-}
-
-__global__ void kb_fy_rank(const __grid_constant__ BatchArgs A) {
-  SRK_BATCH_LOOP(A, {
-    if (r_ >= 1) S_.w.rank[r_] = atomicAdd(&S_.w.grp_cnt[S_.w.kdraw[r_]], 1);
-  })
-}
-
-// Exclusive scan of each source's group counts: block b scans source b.
-__global__ void __launch_bounds__(1024) kb_scan(const __grid_constant__ BatchArgs A) {
-  __shared__ int32_t warp_sum[32];
-  __shared__ int32_t carry;
-  const BatchSrc &S = A.src[blockIdx.x];
-  const int32_t N = S.N_tot;
-  const int32_t *cnt = S.w.grp_cnt;
-  int32_t *off = S.w.grp_off;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t base = 0; base < N; base += 4096) {
-    const int64_t i0 = base + 4 * (int64_t)threadIdx.x;
-    int32_t v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = (i0 + q < N) ? cnt[i0 + q] : 0;
-    const int32_t local = v[0] + v[1] + v[2] + v[3];
-    int32_t incl = local;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_sum[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-      int32_t ws = warp_sum[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, ws, o);
-        if (lane >= o) ws += y;
-      }
-      warp_sum[lane] = ws;
-    }
-    __syncthreads();
-    int32_t run = carry + (wid ? warp_sum[wid - 1] : 0) + incl - local;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (i0 + q < N) off[i0 + q] = run;
-      run += v[q];
-    }
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = run;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) off[N] = carry;
-}
-
-__global__ void kb_fy_scatter(const __grid_constant__ BatchArgs A) {
-  SRK_BATCH_LOOP(A, {
-    if (r_ >= 1) S_.w.items[S_.w.grp_off[S_.w.kdraw[r_]] + S_.w.rank[r_]] = r_;
-  })
-}
-
-__global__ void kb_fy_groups(const __grid_constant__ BatchArgs A) {
-  SRK_BATCH_LOOP(A, {
-    const int32_t b = S_.w.grp_off[r_], e = S_.w.grp_off[r_ + 1];
-    int32_t *items = S_.w.items;
-    for (int32_t x = b + 1; x < e; ++x) {  // insertion sort (groups are tiny)
-      const int32_t y = items[x];
-      int32_t q = x - 1;
-      while (q >= b && items[q] > y) { items[q + 1] = items[q]; --q; }
-      items[q + 1] = y;
-    }
-    S_.w.first[r_] = (e > b) ? items[b] : -1;
-    for (int32_t x = b; x < e; ++x) S_.w.succ[items[x]] = (x + 1 < e) ? items[x + 1] : -1;
-  })
-}
-
-__global__ void kb_pairs(const __grid_constant__ BatchArgs A) {
-  SRK_BATCH_LOOP(A, {
-    const int32_t p = resolve_sigma(r_, S_.w.kdraw, S_.w.first, S_.w.succ, S_.N_tot);
-    S_.w.sigma[r_] = p;
-    const int32_t cap = min(stratum_of(S_.tab->P, S_.L, r_), S_.w.seff[p]);
-    if (cap >= 1) atomicAdd(&small_view(S_.w.small).cap_hist[cap], 1);
-  })
-}
-
-// Row geometry and target bounds of every source (one thread per source), as
-// in k_rows.
-__global__ void kb_rows(const __grid_constant__ BatchArgs A, int32_t n_act) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.k; i += gridDim.x * blockDim.x) {
-    const Small sm = small_view(A.src[i].w.small);
-    const int L = A.src[i].L;
-    int32_t c = 0, r = 0;
-    sm.cnt[L + 1] = 0;
-    for (int q = L; q >= 1; --q) {
-      const int32_t h = sm.cap_hist[q];
-      sm.cursor[q] = c;
-      sm.R[q] = r;
-      c += h;
-      r += q * h;
-      sm.cnt[q] = c;
-    }
-    sm.R[L + 1] = r;
-    sm.cnt[0] = c;
-    sm.R[0] = 0;
-    int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
-    bounds[0] = 0;
-    bounds[1] = n_act;
-    bounds[2] = 0;
-  }
-}
-
 // Every output row: 0 (the walks add to the rows), and 1 at the source.
 __global__ void kb_prefill(const BatchSrc *__restrict__ src, int32_t k, int32_t n) {
   const int64_t total = (int64_t)k * n;
@@ -253,7 +124,7 @@ __global__ void kb_hitj(const __grid_constant__ BatchArgs A) {
     const bool high = i_ >= 32;
     const uint32_t smask = (1u << A.tbits) - 1u;
     for (int q = 1; q <= cap; ++q) {
-      const int32_t node = node_identity(A.view, sp[q - 1]);
+      const int32_t node = walk_identity(A.view, sp[q - 1]);
       uint2 *cell = &A.M[(int64_t)j * (A.Lmax + 1) + q - 1];
       const uint32_t h = sig_bit(node);
       atomicOr(high ? &cell->y : &cell->x, bit);
@@ -344,7 +215,8 @@ namespace {
 template <class SourceSide, class Walks>
 int tune_shape(const srk_graph *g, const std::vector<BatchSrc> &src, SourceSide &source_side,
                Walks &walks, cudaStream_t st, int *shape) {
-  source_side(st);
+  int rc = source_side(st);
+  if (rc) return rc;
   int32_t pick = -1;
   for (size_t b = 0; b < src.size() && pick < 0; ++b) {
     int32_t pairs = 0;
@@ -358,13 +230,12 @@ int tune_shape(const srk_graph *g, const std::vector<BatchSrc> &src, SourceSide 
   cudaEvent_t ev[2] = {nullptr, nullptr};
   cudaError_t e = cudaEventCreate(&ev[0]);
   if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
-  int rc = e == cudaSuccess ? SRK_OK
-                            : cuda_fail(e, "batched query: creating the autotuner's events");
+  if (e != cudaSuccess) rc = cuda_fail(e, "batched query: creating the autotuner's events");
   double best = 0.0;
   for (int sh = 0; sh < kWalkShapes && rc == SRK_OK; ++sh) {
-    if (sh > 0) source_side(st);
+    if (sh > 0) rc = source_side(st);
     const int32_t units = sm_count(g->device) * 2;  // about one round of the grid
-    rc = walks(pick, st, ev, sh, units);
+    if (rc == SRK_OK) rc = walks(pick, st, ev, sh, units);
     int32_t cnt[3] = {0, 0, 0};
     float ms = 0.f;
     if (rc == SRK_OK) {
@@ -536,7 +407,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     const size_t head = align256(sizeof(BatchSrc) * kb) + align256(sizeof(QueryTab) * kb) +
                         align256(sizeof(int64_t) * (kb + 1)) + 256 + align256(m_bytes) +
                         align256(r_bytes) + align256(g_bytes) + align256(h_bytes) +
-                        align256(c_bytes);
+                        align256(c_bytes) + align256(sizeof(SourceJob) * (size_t)kb);
     // end filters: one region, which the sources use one after the other
     size_t extra = 0;
     for (int32_t b = i0; b < i1 && !shared; ++b)
@@ -559,6 +430,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     uint32_t *d_sig = (uint32_t *)((char *)d_rowbase + align256(r_bytes));
     uint4 *d_T = (uint4 *)((char *)d_sig + align256(g_bytes));
     SharedSrc *d_ssrc = (SharedSrc *)((char *)d_T + align256(h_bytes));
+    SourceJob *d_jobs = (SourceJob *)((char *)d_ssrc + align256(c_bytes));
     // shared walks: d_ctr[0] = target counter, d_ctr[1] = steps
     char *ws_base = base + head;
     std::vector<BatchSrc> hsrc((size_t)kb);
@@ -588,6 +460,9 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       S.z = t.z;
       hoff[(size_t)b + 1] = hoff[(size_t)b] + t.N_tot;
     }
+    std::vector<SourceJob> jobs;
+    for (int32_t b = 0; b < kb; ++b)
+      jobs.push_back(SourceJob{hsrc[(size_t)b].w, hsrc[(size_t)b].tab});
     std::vector<SharedSrc> ssrc;
     for (int32_t b = 0; shared && b < kb; ++b) {
       const BatchSrc &S = hsrc[(size_t)b];
@@ -597,6 +472,8 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     // tables and source descriptors (synchronous staging of pageable memory)
     if ((e = cudaMemcpyAsync(d_tab, tabs.data() + i0, sizeof(QueryTab) * kb,
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(SourceJob) * kb, cudaMemcpyHostToDevice,
+                             st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(d_src, hsrc.data(), sizeof(BatchSrc) * kb,
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(d_off, hoff.data(), sizeof(int64_t) * (kb + 1),
@@ -628,25 +505,17 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     const int gw = (int)std::max<int64_t>(1, std::min<int64_t>((A.total_walks + 255) / 256,
                                                                 (int64_t)sms * 8));
     auto enqueue_source_side = [&](cudaStream_t s2) {
-      for (int32_t b = 0; b < kb; ++b)
-        cudaMemsetAsync(hsrc[(size_t)b].w.small, 0, kSmallBytes, s2);
-      kb_source_walks<<<gw, 256, 0, s2>>>(A);
-      kb_fy_rank<<<gw, 256, 0, s2>>>(A);
-      kb_scan<<<kb, 1024, 0, s2>>>(A);
-      kb_fy_scatter<<<gw, 256, 0, s2>>>(A);
-      kb_fy_groups<<<gw, 256, 0, s2>>>(A);
-      kb_pairs<<<gw, 256, 0, s2>>>(A);
+      int r = enqueue_sources(g, d_jobs, kb, shared, s2);
       if (shared) {
         cudaMemsetAsync(d_ctr, 0, 256, s2);
         cudaMemsetAsync(d_M, 0, m_bytes, s2);
         cudaMemsetAsync(d_sig, 0, align256(g_bytes) + h_bytes, s2);
         kb_hitj<<<gw, 256, 0, s2>>>(A);
-      } else {
-        kb_rows<<<(kb + 31) / 32, 32, 0, s2>>>(A, g->n_act);
       }
       const int gp = (int)std::min<int64_t>(((int64_t)kb * (int64_t)n + 255) / 256,
                                             (int64_t)sms * 16);
       kb_prefill<<<gp, 256, 0, s2>>>(d_src, kb, (int32_t)n);
+      return r;
     };
     const bool count = opt && opt->stats;
     SharedWalks SW;
@@ -671,9 +540,14 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     auto enqueue_source = [&](int32_t b, cudaStream_t s2, const cudaEvent_t *timing, int shape,
                               int32_t max_units) {
       const BatchSrc &S = hsrc[(size_t)b];
+      const QueryTab &t = tabs[(size_t)(i0 + b)];
       const Outputs o{S.scores, S.counts, nullptr, nullptr};
-      return enqueue_walks(g, tabs[(size_t)(i0 + b)], S.w, o, ws_base + need, extra, count, s2,
-                           timing, 0, (int32_t)n, shape, max_units);
+      Filters F;
+      plan_filters(g, t, S.w, g->n, extra, &F, ws_base + need);
+      int r = enqueue_ends(g, S.w, F, s2);
+      if (r == SRK_OK)
+        r = enqueue_walks(g, t, S.w, F, o, count, s2, timing, 0, (int32_t)n, shape, max_units);
+      return r;
     };
     // autotune the walk kernel's launch shape on the first batch with pairs
     int shape = g->batch_cfg;
@@ -686,8 +560,8 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       if (shape >= 0) const_cast<srk_graph *>(g)->batch_cfg = shape;
     }
     auto enqueue_all = [&](cudaStream_t s2) {
-      enqueue_source_side(s2);
-      int r = SRK_OK;
+      int r = enqueue_source_side(s2);
+      if (r) return r;
       if (shared)
         r = enqueue_shared_walks(g, SW, s2);
       else

@@ -270,6 +270,32 @@ __device__ __forceinline__ auto adj_view(const GraphView &V) {
 __device__ __forceinline__ int32_t node_identity(const GraphView &V, int32_t v) {
   return V.layout == kNarrow ? V.npos[v] : V.layout == kWide ? v + V.row_ptr[v] : v;
 }
+// The source's walks (Workspace::spos) hold ranks in the narrow layout and
+// node ids in the others: the identity and the id of such a node.
+__device__ __forceinline__ int32_t walk_identity(const GraphView &V, int32_t x) {
+  return V.layout == kWide ? x + V.row_ptr[x] : x;
+}
+__device__ __forceinline__ int32_t walk_id(const GraphView &V, int32_t x) {
+  return V.layout == kNarrow ? V.order[x] : x;
+}
+
+// Filters.  A filter of 2^lg words is named by 16 * (its place, in units of
+// kFilterUnit words) + lg; kNoFilter names none.
+constexpr int kFilterUnit = 32;       // words of the smallest filter (lg = 5)
+constexpr int kFilterMaxLg = 10;      // 4 KB
+constexpr int32_t kNoFilter = -1;
+__device__ __forceinline__ int64_t filter_place(int32_t f) { return (int64_t)(f >> 4) * kFilterUnit; }
+__device__ __forceinline__ int filter_lg(int32_t f) { return f & 15; }
+// The bit of the node of identity x in a filter of 2^lg words.
+__device__ __forceinline__ uint32_t filter_bit(int32_t x, int lg) {
+  return ((uint32_t)x * 0x9E3779B1u) >> (27 - lg);
+}
+// The hash of node id in the table of end nodes: its low bits the first slot,
+// its high ones the bit of the bitmap.
+__device__ __forceinline__ uint32_t end_hash(uint32_t id) {
+  id *= 0x85EBCA6Bu;
+  return id ^ (id >> 15);
+}
 
 // The entry step i of walk replica r from node v reads (list base b, degree
 // d), from the step's word w of block (walk_ctr0(i, r), v) under key k.  The
@@ -317,7 +343,7 @@ __device__ __forceinline__ int32_t fy_draw(const RoundKeys &rk, uint32_t s, int3
 }
 
 // sigma[j] of the sequential Fisher-Yates loop, from the draws and the
-// "next write of a position" links (see k_pairs in srk_query.cu).
+// "next write of a position" links (see srk_source.cu).
 __device__ __forceinline__ int32_t resolve_sigma(int32_t j, const int32_t *kdraw,
                                                  const int32_t *first,
                                                  const int32_t *succ, int32_t N) {

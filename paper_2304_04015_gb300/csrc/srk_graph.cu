@@ -416,6 +416,7 @@ extern "C" int srk_graph_free(srk_graph *g) {
     if (g->own_w) cudaFree(g->own_w);
     if (g->adj) cudaFree(g->adj);
     if (g->npos) cudaFree(g->npos);
+    if (g->order) cudaFree(g->order);
     if (g->hub) cudaFree(g->hub);
     if (g->ctab) cudaFree(g->ctab);
     if (g->act) cudaFree(g->act);
@@ -505,6 +506,9 @@ static int build_narrow(srk_graph *g, int dev) {
   }
   if (e == cudaSuccess) e = cudaMalloc(&g->adj, sizeof(uint32_t) * (size_t)(m > 0 ? m : 1));
   if (e == cudaSuccess) e = cudaMalloc(&g->npos, sizeof(int32_t) * (size_t)n);
+  if (e == cudaSuccess) e = cudaMalloc(&g->order, sizeof(int32_t) * (size_t)n);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(g->order, order, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, 0);
   if (e == cudaSuccess) e = cudaMalloc(&g->hub, sizeof(uint2) * (size_t)(H > 0 ? H : 1));
   if (e == cudaSuccess) e = cudaMalloc(&g->ctab, sizeof(uint32_t) * ctab.size());
   if (e == cudaSuccess)

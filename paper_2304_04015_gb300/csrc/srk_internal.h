@@ -31,7 +31,8 @@ struct srk_graph {
   // 2, only when forced by SRK_ADJ_CSR): no packed copy; nodes are their ids
   // and a step reads row_ptr and col.
   uint32_t *adj = nullptr;
-  int32_t *npos = nullptr;   // narrow layout: ranks, n (owned)
+  int32_t *npos = nullptr;   // narrow layout: ranks, n (owned),
+  int32_t *order = nullptr;  //   and the nodes by rank, n (owned)
   uint2 *hub = nullptr;      // narrow layout: hub records, n_hubs (owned)
   uint32_t *ctab = nullptr;  // narrow layout: list starts by degree (owned)
   int32_t n_hubs = 0;        // narrow layout: H
@@ -63,6 +64,7 @@ struct GraphView {
   const int32_t *col;      // in-neighbour lists
   const uint32_t *adj;     // packed adjacency
   const int32_t *npos;     // narrow layout: ranks,
+  const int32_t *order;    //   nodes by rank,
   const uint2 *hub;        //   hub records,
   const uint32_t *ctab;    //   list starts by degree
   int32_t pos_bits;
@@ -73,8 +75,8 @@ struct GraphView {
 namespace srk {
 
 inline GraphView view_of(const srk_graph *g) {
-  return GraphView{g->row_ptr, g->col,     g->adj,     g->npos, g->hub,    g->ctab,
-                   g->pos_bits, g->deg_max, g->n,      g->n_hubs, g->layout};
+  return GraphView{g->row_ptr, g->col,      g->adj,     g->npos, g->order,  g->hub,
+                   g->ctab,    g->pos_bits, g->deg_max, g->n,    g->n_hubs, g->layout};
 }
 
 // The output function of SplitMix64 (Steele, Lea, Flood, OOPSLA 2014) and
@@ -160,6 +162,9 @@ struct Workspace {
       *succ, *sigma, *pair_j, *Hc, *small;
   unsigned long long *pair_w;
   size_t bytes;
+  // the pair records {j, cap, first node in Hc, filter}, longest pairs first:
+  // 16 bytes a pair in kdraw to grp_off, which the shuffle no longer needs then
+  __host__ __device__ int4 *rec() const { return reinterpret_cast<int4 *>(kdraw); }
 };
 
 // Device outputs of one query (null = not wanted, except scores).
@@ -169,6 +174,48 @@ struct Outputs {
   unsigned long long *wsums;
   uint32_t *steps;
 };
+
+// A slot of the table of end nodes: the node id + 1 (0: empty slot), its
+// filter + 1 (0: none; kWantFilter: some pair ends here), and the pairs of cap
+// 1 that end here, list1[off1 .. off1 + cnt1).
+struct EndSlot {
+  uint32_t key;
+  int32_t filt;
+  int32_t cnt1;
+  int32_t off1;
+};
+constexpr int32_t kWantFilter = -1;
+// End nodes and filters of one query (srk_lockstep.cu; null slots: it has none).
+struct Filters {
+  EndSlot *slots;       // 2^slot_bits of them, linear probing
+  uint32_t *bloom;      // 2^bloom_bits bits: ids whose bit is clear are in no slot
+  uint32_t *bits;       // the filters, max_units * kFilterUnit words
+  int32_t *list1;       // pairs of cap 1, grouped by end node
+  int32_t *slot_of;     // per pair: its slot,
+  int32_t *rank1;       //   and its place in the slot's list
+  int32_t *ctl;         // {units of bits handed out, entries of list1 handed out}
+  const int32_t *out_deg;  // out-degrees, by node id
+  int slot_bits, bloom_bits;
+  int32_t max_units;
+};
+// The query's end nodes and filters in `avail` bytes at `extra` (0 bytes or a
+// null pointer: none); returns the bytes taken.
+size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, int64_t n_targets,
+                    size_t avail, Filters *F, char *extra);
+
+// The source side of queries (srk_source.cu).  enqueue_source: one query, steps
+// a2-a3 to the pair records (the cap rows only with the literal shuffle) and
+// the end nodes of F.  enqueue_sources: of k queries, to the pair records or,
+// with `shared`, to sigma.  enqueue_ends: the end nodes of one of them.
+struct SourceJob {
+  Workspace w;
+  const QueryTab *tab;  // device
+};
+int enqueue_source(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
+                   int32_t u_begin, int32_t u_end, cudaStream_t st);
+int enqueue_sources(const srk_graph *g, const SourceJob *jobs, int32_t k, bool shared,
+                    cudaStream_t st);
+int enqueue_ends(const srk_graph *g, const Workspace &w, const Filters &F, cudaStream_t st);
 
 // Carves `base` (or only sizes the plan when base is null); returns the
 // number of bytes one query of table `t` needs.
@@ -186,10 +233,10 @@ int single_source(const srk_graph *g, int32_t s, double c, double eps, uint64_t 
 // Bytes of `extra` scratch a query of n_targets targets makes use of (it does
 // with less, or none: its end nodes then have fewer filters, or none).
 size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets);
-// Steps a4-a5 after the source side (sigma, seff, spos and the cap rows of w
-// are made, the outputs of the range cleared): srk_lockstep.cu.
-int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Outputs &o,
-                  char *extra, size_t extra_bytes, bool count, cudaStream_t st,
+// Steps a4-a5 after the source side (the pair records of w and the end nodes
+// of F are made, the outputs of the range cleared): srk_lockstep.cu.
+int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
+                  const Outputs &o, bool count, cudaStream_t st,
                   const cudaEvent_t *timing, int32_t u_begin, int32_t u_end, int shape = -1,
                   int32_t max_units = INT32_MAX);
 // Launch shapes of the walks: 0 and up, -1 for the default of the target count.
@@ -229,11 +276,6 @@ cudaError_t allow_lockstep(int layout);
 // [*b, *e): the targets a query computes, from its options (SRK_EINVAL when
 // the range is malformed).
 int target_range(const srk_graph *g, const srk_opts *opt, int32_t *b, int32_t *e);
-// Exclusive scan of cnt[0..N) into off[0..N] (one block of 1024 threads).
-__global__ void k_scan(const int32_t *__restrict__ cnt, int32_t *__restrict__ off,
-                       int32_t N);
-
-
 // Exclusive scan of cnt[0..N) into off[0..N], with scan_scratch(N) bytes of
 // scratch (srk_sort.cu).
 size_t scan_scratch(int64_t N);

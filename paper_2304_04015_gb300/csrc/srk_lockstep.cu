@@ -50,48 +50,6 @@
 
 namespace srk {
 
-// Filters.  A filter of 2^lg words is named by 16 * (its place, in units of
-// kFilterUnit words) + lg; kNoFilter names none.
-constexpr int kFilterUnit = 32;       // words of the smallest filter (lg = 5)
-constexpr int kFilterMaxLg = 10;      // 4 KB
-constexpr int32_t kNoFilter = -1;
-__device__ __forceinline__ int64_t filter_place(int32_t f) { return (int64_t)(f >> 4) * kFilterUnit; }
-__device__ __forceinline__ int filter_lg(int32_t f) { return f & 15; }
-// The bit of the node of identity x in a filter of 2^lg words.
-__device__ __forceinline__ uint32_t filter_bit(int32_t x, int lg) {
-  return ((uint32_t)x * 0x9E3779B1u) >> (27 - lg);
-}
-
-// A slot of the table of end nodes: the node id + 1 (0: empty slot), its
-// filter + 1 (0: none; kWantFilter: some pair ends here), and the pairs of cap
-// 1 that end here, list1[off1 .. off1 + cnt1).
-struct EndSlot {
-  uint32_t key;
-  int32_t filt;
-  int32_t cnt1;
-  int32_t off1;
-};
-constexpr int32_t kWantFilter = -1;
-
-__device__ __forceinline__ uint32_t end_hash(uint32_t id) {
-  id *= 0x85EBCA6Bu;
-  return id ^ (id >> 15);
-}
-
-// End nodes and filters of one query (null slots: the query has none).
-struct Filters {
-  EndSlot *slots;       // 2^slot_bits of them, linear probing
-  uint32_t *bloom;      // 2^bloom_bits bits: ids whose bit is clear are in no slot
-  uint32_t *bits;       // the filters, max_units * kFilterUnit words
-  int32_t *list1;       // pairs of cap 1, grouped by end node
-  int32_t *slot_of;     // per pair: its slot,
-  int32_t *rank1;       //   and its place in the slot's list
-  int32_t *ctl;         // {units of bits handed out, entries of list1 handed out}
-  const int32_t *out_deg;  // out-degrees, by node id
-  int slot_bits, bloom_bits;
-  int32_t max_units;
-};
-
 // What the lockstep kernel needs of one query.
 struct LockQuery {
   const int4 *rec;              // per pair {j, cap, first node in H, filter}
@@ -255,6 +213,19 @@ __device__ __forceinline__ void load_if(bool p, uint32_t smem, int32_t &v) {
 __device__ __forceinline__ void load_if(bool p, const int32_t *g, int32_t &v) {
   load_if(p, reinterpret_cast<const uint32_t *>(g), reinterpret_cast<uint32_t &>(v));
 }
+// The same for a store, and its plain counterpart for a warp's queue.
+__device__ __forceinline__ void store_if(bool p, uint32_t smem, uint32_t x, uint32_t y, uint32_t z,
+                                         uint32_t w) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.u32 q, %5, 0;\n@q st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n}"
+               ::"r"(smem), "r"(x), "r"(y), "r"(z), "r"(w), "r"((uint32_t)p)
+               : "memory");
+}
+__device__ __forceinline__ uint4 load_shared(uint32_t smem) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem) : "memory");
+  return v;
+}
 __device__ __forceinline__ const uint32_t *entries(const Adj &G) { return G.adj; }
 __device__ __forceinline__ const uint2 *entries(const AdjW &G) { return G.adj; }
 __device__ __forceinline__ const int32_t *entries(const AdjC &G) { return G.col; }
@@ -322,7 +293,7 @@ struct LockFilter {
 // queue collects them until they fill a warp.  Entry {entry of the node before
 // the last step, node to meet, cap << 24 | j, a << 8 | target slot}.
 struct LockQueue {
-  uint4 *at;
+  uint32_t at;  // shared memory
   int32_t n;
 };
 
@@ -333,7 +304,8 @@ __device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, con
   const int lane = threadIdx.x & 31;
   B.n -= take;
   const bool p = lane < take;
-  const uint4 it = p ? B.at[B.n + lane] : make_uint4(0u, 0u, 1u << 24, 0u);
+  uint4 it = make_uint4(0u, 0u, 1u << 24, 0u);
+  if (p) it = load_shared(B.at + 16u * (uint32_t)(B.n + lane));
   int32_t v = 0;
 #pragma unroll
   for (int t = 0; t < kT; ++t) {
@@ -398,7 +370,7 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
       meets |= met[t];
       if (kCount && (i == cap ? deg[t] != 0 : met[t])) X.st[t] += i;
     }
-    if (meets) {  // rare: a few times per target and query
+    if (__any_sync(0xffffffffu, meets)) {  // rare: a few times per target and query
 #pragma unroll
       for (int t = 0; t < kT; ++t)
         if (met[t]) {
@@ -428,10 +400,9 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
           p = p && ((word >> (f & 31)) & 1u);
         }
         const uint32_t m = __ballot_sync(0xffffffffu, p);
-        if (p)
-          B.at[B.n + __popc(m & lanes_below_mask())] =
-              make_uint4(entry_word(e[t]), (uint32_t)he, (uint32_t)cap << 24 | j,
-                         (uint32_t)a << 8 | (uint32_t)(t * 32 + lane));
+        store_if(p, B.at + 16u * (uint32_t)(B.n + __popc(m & lanes_below_mask())),
+                 entry_word(e[t]), (uint32_t)he, (uint32_t)cap << 24 | j,
+                 (uint32_t)a << 8 | (uint32_t)(t * 32 + lane));
         B.n += __popc(m);
         if (B.n >= 32) lock_drain(G, T, Q, B, 32, X.u);
       }
@@ -471,7 +442,7 @@ __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
                                                uint32_t &seq, LockTargets<kT> &X) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const bool filtered = Q.min_cap == 2;
-  LockQueue B{queues + wid * kQueue, 0};
+  LockQueue B{smem_addr(queues + wid * kQueue), 0};
   int32_t issued = 0;  // warp 0: pairs in the groups formed so far
   auto issue = [&](uint32_t n) {  // warp 0: form group n and fetch its filters
     if (issued >= len) return;
@@ -547,106 +518,40 @@ __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
   if (B.n > 0) lock_drain(G, T, Q, B, B.n, X.u);
 }
 
-// ------------------------------------- pair records, end nodes, filters --
-
-// Every pair with cap >= 1: its record (pairs sorted by cap, descending), its
-// weight, the identities of its nodes, and its end node in the table.
-__global__ void __launch_bounds__(256)
-k_records(const __grid_constant__ QueryTab tab, GraphView V, Filters F,
-          const int32_t *__restrict__ sigma, const int32_t *__restrict__ seff,
-          const int32_t *__restrict__ spos, int32_t *__restrict__ small_base,
-          int4 *__restrict__ rec, unsigned long long *__restrict__ pair_w,
-          int32_t *__restrict__ H) {
-  __shared__ int32_t P[SRK_MAX_LEN + 2];
-  __shared__ int32_t R[SRK_MAX_LEN + 2];    // cells before the pairs of cap i
-  __shared__ int32_t beg[SRK_MAX_LEN + 2];  // pairs of cap > i
-  Small sm = small_view(small_base);
-  for (int i = threadIdx.x; i <= tab.L + 1; i += blockDim.x) {
-    P[i] = tab.P[i];
-    R[i] = sm.R[i];
-    beg[i] = i <= tab.L ? sm.cnt[i + 1] : 0;
-  }
-  __syncthreads();
-  const int Ls = tab.L > 0 ? tab.L : 1;
-  for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < tab.N_tot;
-       j += gridDim.x * blockDim.x) {
-    const int32_t w = sigma[j];
-    const int l2 = stratum_of(P, tab.L, j);
-    const int32_t cap = min(l2, seff[w]);
-    if (cap < 1) continue;
-    const int l1 = stratum_of(P, tab.L, w);
-    const int32_t a = atomicAdd(&sm.cursor[cap], 1);
-    pair_w[a] = __double2ull_rn(tab.a[l1] * tab.a[l2] * 4294967296.0);
-    const int32_t off = R[cap] + (a - beg[cap]) * cap;
-    rec[a] = make_int4(j, cap, off, kNoFilter);
-    const int32_t *src = spos + (int64_t)w * Ls;
-    for (int i = 0; i < cap; ++i) H[off + i] = node_identity(V, src[i]);
-    if (F.slots) {
-      const uint32_t id = (uint32_t)src[cap - 1], mask = (1u << F.slot_bits) - 1u;
-      const uint32_t hash = end_hash(id), bb = hash >> (32 - F.bloom_bits);
-      atomicOr(&F.bloom[bb >> 5], 1u << (bb & 31));
-      uint32_t sl = hash & mask;
-      for (uint32_t probe = 0; probe <= mask; ++probe, sl = (sl + 1u) & mask) {
-        const uint32_t prev = atomicCAS(&F.slots[sl].key, 0u, id + 1u);
-        if (prev == 0u || prev == id + 1u) break;
-      }
-      F.slot_of[a] = (int32_t)sl;
-      if (cap == 1) F.rank1[a] = atomicAdd(&F.slots[sl].cnt1, 1);
-      else F.slots[sl].filt = kWantFilter;
-    }
-  }
-}
-
-// Room for every slot's list and filter, the filters cleared.
-__global__ void __launch_bounds__(256)
-k_end_slots(Filters F, const int32_t *__restrict__ cnt) {
-  if (cnt[1] == 0) return;
-  const int lane = threadIdx.x & 31;
-  for (int32_t base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; base < (1 << F.slot_bits);
-       base += gridDim.x * blockDim.x) {
-    EndSlot &S = F.slots[base + lane];
-    if (S.cnt1 > 0) S.off1 = atomicAdd(&F.ctl[1], S.cnt1);
-    int32_t at = -1, units = 0;
-    if (S.filt == kWantFilter) {
-      // 16 bits and more per node of the out-list, so that at most about 6 %
-      // of the other nodes pass, up to the largest size (R-MAT 20: 0.7 KB on
-      // average; one size of 4 KB for all was slower, a block then stops for
-      // its filters every 4 pairs instead of every 11)
-      const int32_t d = F.out_deg[S.key - 1u];
-      int lg = 5;
-      while (lg < kFilterMaxLg && (2 << lg) < d) ++lg;
-      units = (1 << lg) / kFilterUnit;
-      at = atomicAdd(&F.ctl[0], units);
-      if (at > F.max_units - units) at = -1;
-      S.filt = at < 0 ? 0 : 1 + (at << 4 | lg);
-    }
-    for (uint32_t m = __ballot_sync(0xffffffffu, at >= 0); m; m &= m - 1) {
-      const int32_t a0 = __shfl_sync(0xffffffffu, at, __ffs(m) - 1),
-                    nu = __shfl_sync(0xffffffffu, units, __ffs(m) - 1);
-      for (int32_t x = lane; x < nu * kFilterUnit; x += 32)
-        F.bits[(int64_t)a0 * kFilterUnit + x] = 0u;
-    }
-  }
-}
-
-// Every pair's place in its end node's list, or its filter.
-__global__ void __launch_bounds__(256)
-k_end_lists(Filters F, const int32_t *__restrict__ small_base, int4 *__restrict__ rec) {
-  const Small sm = small_view(const_cast<int32_t *>(small_base));
-  for (int32_t a = blockIdx.x * blockDim.x + threadIdx.x; a < sm.cnt[1];
-       a += gridDim.x * blockDim.x) {
-    const EndSlot S = F.slots[F.slot_of[a]];
-    if (a >= sm.cnt[2]) F.list1[S.off1 + F.rank1[a]] = a;
-    else rec[a].w = S.filt - 1;
-  }
-}
+// ------------------------------------------------------- edges, and walks --
 
 // One pass over the edges y -> u (entry k of u's list).  Where y is an end
 // node, u joins its filter, and if u is a target, the pairs of cap 1 that end
-// at y are decided for u, the warp's lanes over the pairs: pair j meets here
-// exactly when its step draws k.  (Every entry that holds y is its own edge,
-// so repeated in-neighbours count once each, as the draw does.)  A bitmap in
-// L1 turns most edges away; R-MAT 20: 0.37 ms for 16.1 M edges.
+// at y are decided for u: pair j meets here exactly when its step draws k.
+// (Every entry that holds y is its own edge, so repeated in-neighbours count
+// once each, as the draw does.)  A bitmap in L1 turns most edges away.  A warp
+// takes kEdgeRun consecutive edges and follows their owners along row_ptr, 32
+// nodes at a time; a binary search per edge of an end node took 0.37 ms at
+// R-MAT 20 (16.1 M edges), this 0.26 ms (R-MAT 16, 0.95 M edges: 0.037, 0.046).
+constexpr int kEdgeRun = 1024;
+
+// Meetings of the pairs of cap 1 list1[off + q], q = q0, q0 + dq, ... < cnt, with
+// target u, whose entry k of d is the end node.
+__device__ __forceinline__ void last_steps(const Filters &F, const int4 *__restrict__ rec,
+                                           const unsigned long long *__restrict__ pair_w,
+                                           uint32_t key, int32_t u, uint32_t k, uint32_t d,
+                                           int32_t off, int32_t cnt, int32_t q0, int32_t dq,
+                                           uint32_t &c, unsigned long long &ws) {
+  for (int32_t q = q0; q < cnt; q += dq) {
+    const int32_t a = F.list1[off + q];
+    const uint32_t j = (uint32_t)rec[a].x;
+    uint32_t x0, x1;
+    philox2(key, walk_ctr0(1, j), (uint32_t)u, x0, x1);
+    uint32_t idx = __umulhi(x0, d);
+    const uint32_t lo = x0 * d;
+    if (lo < d && lo < (0u - d) % d) idx = step_index_redraw(key, 1, j, (uint32_t)u, d);
+    if (idx == k) {
+      ++c;
+      ws += pair_w[a];
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256)
 k_edges(Filters F, GraphView V, int64_t m, const int32_t *__restrict__ cnt,
         const int4 *__restrict__ rec, const unsigned long long *__restrict__ pair_w, uint32_t key,
@@ -654,69 +559,96 @@ k_edges(Filters F, GraphView V, int64_t m, const int32_t *__restrict__ cnt,
         uint32_t *__restrict__ counts) {
   if (cnt[1] == 0) return;  // no pair can meet
   const int lane = threadIdx.x & 31;
-  const int32_t *row_ptr = V.row_ptr;
+  const int32_t *__restrict__ row_ptr = V.row_ptr;
   const uint32_t mask = (1u << F.slot_bits) - 1u;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; e0 < m;
-       e0 += stride) {
-    const int64_t e = e0 + lane;
-    EndSlot S{0u, 0, 0, 0};
-    if (e < m) {
-      const uint32_t y = (uint32_t)V.col[e], hash = end_hash(y), bb = hash >> (32 - F.bloom_bits);
-      if ((F.bloom[bb >> 5] >> (bb & 31)) & 1u) {
-        uint32_t sl = hash & mask;
-        for (uint32_t probe = 0; probe <= mask; ++probe, sl = (sl + 1u) & mask) {
-          const EndSlot T = F.slots[sl];
-          if (T.key == y + 1u) S = T;
-          if (T.key == y + 1u || T.key == 0u) break;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  // short runs when there are few edges, so that all warps have some
+  int64_t run = (m + warps - 1) / warps;
+  run = run > kEdgeRun ? kEdgeRun : (run + 31) & ~31ll;
+  for (int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * run; r0 < m;
+       r0 += warps * run) {
+    int32_t v = -1;  // owners so far are below v + 32 (-1: not looked up yet)
+    const int64_t r1 = r0 + run < m ? r0 + run : m;
+    for (int64_t e0 = r0; e0 < r1; e0 += 32) {
+      const int64_t e = e0 + lane;
+      EndSlot S{0u, 0, 0, 0};
+      if (e < r1) {
+        const uint32_t y = (uint32_t)V.col[e], hash = end_hash(y),
+                       bb = hash >> (32 - F.bloom_bits);
+        if ((F.bloom[bb >> 5] >> (bb & 31)) & 1u) {
+          uint32_t sl = hash & mask;
+          for (uint32_t probe = 0; probe <= mask; ++probe, sl = (sl + 1u) & mask) {
+            const EndSlot T = F.slots[sl];
+            if (T.key == y + 1u) S = T;
+            if (T.key == y + 1u || T.key == 0u) break;
+          }
         }
       }
-    }
-    int32_t u = 0;
-    uint32_t k = 0, d = 1;
-    if (S.key) {
-      int32_t lo = 0, hi = V.n - 1;  // the node whose list holds edge e
-      while (lo < hi) {
-        const int32_t mid = lo + (hi - lo + 1) / 2;
-        if ((int64_t)row_ptr[mid] <= e) lo = mid; else hi = mid - 1;
+      bool open = S.key != 0u;  // owner wanted
+      if (!__any_sync(0xffffffffu, open)) continue;
+      if (v < 0) {  // the owner of the run's first edge: 32 probes a round
+        int32_t lo = 0, hi = V.n;  // row_ptr[lo] <= e0 < row_ptr[hi]
+        while (hi - lo > 1) {
+          const int64_t step = ((int64_t)hi - lo + 31) / 32;
+          const int32_t at = (int32_t)min((int64_t)hi, lo + (lane + 1) * step);
+          const uint32_t above = __ballot_sync(0xffffffffu, (int64_t)row_ptr[at] > e0);
+          const int f = __ffs(above) - 1;  // the first probe past e0 (row_ptr[hi] is)
+          hi = (int32_t)min((int64_t)hi, lo + (f + 1) * step);
+          lo += (int32_t)(f * step);
+        }
+        v = lo;
       }
-      u = lo;
-      const int32_t b = row_ptr[u];
-      k = (uint32_t)(e - b);
-      d = (uint32_t)(row_ptr[u + 1] - b);
+      int32_t u = 0;
+      uint32_t k = 0, d = 1;
+      for (;;) {  // the owner is v plus the number of lists that end at or before e
+        const int32_t end = row_ptr[min(V.n, v + 1 + lane)];
+        int q = 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if ((int64_t)__shfl_sync(0xffffffffu, end, q + o - 1) <= e) q += o;
+        const bool in = (int64_t)__shfl_sync(0xffffffffu, end, 31) > e;
+        const int32_t b = __shfl_sync(0xffffffffu, end, q > 0 ? q - 1 : 0),
+                      f = __shfl_sync(0xffffffffu, end, q);
+        if (open && in) {
+          u = v + q;
+          const int32_t beg = q > 0 ? b : row_ptr[v];
+          k = (uint32_t)(e - beg);
+          d = (uint32_t)(f - beg);
+          open = false;
+        }
+        if (!__any_sync(0xffffffffu, open)) break;
+        v += 32;
+      }
       if (S.filt > 0) {
         const uint32_t f = filter_bit(node_identity(V, u), filter_lg(S.filt - 1));
         atomicOr(&F.bits[filter_place(S.filt - 1) + (f >> 5)], 1u << (f & 31));
       }
-    }
-    const bool todo = S.key && S.cnt1 > 0 && u >= u_begin && u < u_end && u != s;
-    for (uint32_t mm = __ballot_sync(0xffffffffu, todo); mm; mm &= mm - 1) {
-      const int l = __ffs(mm) - 1;
-      const int32_t uu = __shfl_sync(0xffffffffu, u, l), n1 = __shfl_sync(0xffffffffu, S.cnt1, l),
-                    off = __shfl_sync(0xffffffffu, S.off1, l);
-      const uint32_t kk = __shfl_sync(0xffffffffu, k, l), dd = __shfl_sync(0xffffffffu, d, l);
+      const bool todo = S.cnt1 > 0 && u >= u_begin && u < u_end && u != s;
+      // a few pairs: each lane decides its edge's; many: the warp's lanes share them
       uint32_t c = 0;
       unsigned long long ws = 0;
-      for (int32_t q = lane; q < n1; q += 32) {
-        const int32_t a = F.list1[off + q];
-        const uint32_t j = (uint32_t)rec[a].x;
-        uint32_t x0, x1;
-        philox2(key, walk_ctr0(1, j), (uint32_t)uu, x0, x1);
-        uint32_t idx = __umulhi(x0, dd);
-        const uint32_t lo = x0 * dd;
-        if (lo < dd && lo < (0u - dd) % dd) idx = step_index_redraw(key, 1, j, (uint32_t)uu, dd);
-        if (idx == kk) {
-          ++c;
-          ws += pair_w[a];
+      if (todo && S.cnt1 <= 8)
+        last_steps(F, rec, pair_w, key, u, k, d, S.off1, S.cnt1, 0, 1, c, ws);
+      for (uint32_t mm = __ballot_sync(0xffffffffu, todo && S.cnt1 > 8); mm; mm &= mm - 1) {
+        const int l = __ffs(mm) - 1;
+        uint32_t cl = 0;
+        unsigned long long wl = 0;
+        last_steps(F, rec, pair_w, key, __shfl_sync(0xffffffffu, u, l),
+                   __shfl_sync(0xffffffffu, k, l), __shfl_sync(0xffffffffu, d, l),
+                   __shfl_sync(0xffffffffu, S.off1, l), __shfl_sync(0xffffffffu, S.cnt1, l), lane,
+                   32, cl, wl);
+        for (int o = 16; o > 0; o >>= 1) {
+          cl += __shfl_xor_sync(0xffffffffu, cl, o);
+          wl += __shfl_xor_sync(0xffffffffu, wl, o);
+        }
+        if (lane == l) {
+          c = cl;
+          ws = wl;
         }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-        ws += __shfl_xor_sync(0xffffffffu, ws, o);
-      }
-      if (lane == 0 && c) {
-        atomicAdd(&W[uu], ws);
-        if (counts) atomicAdd(&counts[uu], c);
+      if (c) {
+        atomicAdd(&W[u], ws);
+        if (counts) atomicAdd(&counts[u], c);
       }
     }
   }
@@ -1133,9 +1065,13 @@ k_finish_rows(const SharedSrc *__restrict__ src, int32_t n) {
 // Returns the bytes taken.
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
-static size_t plan_filters(const srk_graph *g, const QueryTab &t, int64_t n_targets, size_t avail,
-                           Filters *F, char *base) {
+size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, int64_t n_targets,
+                    size_t avail, Filters *F, char *base) {
   memset(F, 0, sizeof *F);
+  // (arrays of the shuffle, free by then)
+  F->list1 = w.items;
+  F->slot_of = w.first;
+  F->rank1 = w.succ;
   // They cost a pass over the edges and save about a last step in every pair
   // and target, some hundred times less each: not for fewer than 8 pairs x
   // targets an edge (a short target range, a tiny z).  Beyond 2^20 walks the
@@ -1166,7 +1102,9 @@ static size_t plan_filters(const srk_graph *g, const QueryTab &t, int64_t n_targ
 
 size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets) {
   Filters F;
-  return plan_filters(g, t, n_targets, SIZE_MAX, &F, nullptr);
+  Workspace w;
+  memset(&w, 0, sizeof w);
+  return plan_filters(g, t, w, n_targets, SIZE_MAX, &F, nullptr);
 }
 
 
@@ -1219,39 +1157,20 @@ double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t m
   return (double)g->n_act * n_pairs * std::min(1.0, (double)max_units / units);
 }
 
-int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Outputs &o,
-                  char *extra, size_t extra_bytes, bool count, cudaStream_t st,
-                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end, int shape,
-                  int32_t max_units) {
+int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
+                  const Outputs &o, bool count, cudaStream_t st, const cudaEvent_t *timing,
+                  int32_t u_begin, int32_t u_end, int shape, int32_t max_units) {
   const int dev = g->device;
-  const int gN = grid_for(t.N_tot, 256, dev);
   const int64_t nr = (int64_t)u_end - u_begin;
   const GraphView V = view_of(g);
-  Filters F;
-  plan_filters(g, t, nr, extra ? extra_bytes : 0, &F, extra);
-  // the Fisher-Yates arrays are free after k_pairs; the pair records take the
-  // first four (16 bytes a pair), kdraw to grp_off
-  F.list1 = w.items;
-  F.slot_of = w.first;
-  F.rank1 = w.succ;
-  int4 *rec = reinterpret_cast<int4 *>(w.kdraw);
   const Small sm = small_view(w.small);
   int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
   unsigned long long *W = reinterpret_cast<unsigned long long *>(o.scores);
-  cudaError_t e = cudaSuccess;
-  if (F.slots) {
-    e = cudaMemsetAsync(F.slots, 0, (size_t)((char *)F.ctl + 256 - (char *)F.slots), st);
-    if (e != cudaSuccess) return cuda_fail(e, "clearing the end nodes");
-  }
-  k_records<<<gN, 256, 0, st>>>(t, V, F, w.sigma, w.seff, w.spos, w.small, rec, w.pair_w, w.Hc);
-  if (F.slots) {
-    k_end_slots<<<grid_for((int64_t)1 << F.slot_bits, 256, dev), 256, 0, st>>>(F, sm.cnt);
-    k_end_lists<<<gN, 256, 0, st>>>(F, w.small, rec);
-    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, sm.cnt, rec, w.pair_w, t.tkey,
+  if (F.slots)
+    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, sm.cnt, w.rec(), w.pair_w, t.tkey,
                                                       t.s, u_begin, u_end, W, o.counts);
-  }
   LockQuery Q;
-  Q.rec = rec;
+  Q.rec = w.rec();
   Q.w = w.pair_w;
   Q.H = w.Hc;
   Q.bits = F.bits;
@@ -1267,30 +1186,36 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   Q.max_units = max_units;
   if (timing) cudaEventRecord(timing[0], st);
   const int grid = sm_count(dev) * kLockBlocks;
+  // The targets: by rank where all of them are wanted (the narrow layout ranks
+  // the nodes with in-neighbours first), so that a block's lists are of one
+  // length: the short ones all fit its shared memory, the heavy units come
+  // first.  By id for a part of them.
+  const int32_t *act = nr == g->n && g->layout == kNarrow ? g->order : g->act;
   // shape 0: kLockTargets targets a thread; 1: one (too few to give it several)
   const bool one = shape < 0 ? nr <= kLockThreads : shape == 1;
   if (g->layout == kWide) {
-    if (count) launch_lockstep<kWide, true>(V, g->act, bounds, Q, one, grid, st);
-    else launch_lockstep<kWide, false>(V, g->act, bounds, Q, one, grid, st);
+    if (count) launch_lockstep<kWide, true>(V, act, bounds, Q, one, grid, st);
+    else launch_lockstep<kWide, false>(V, act, bounds, Q, one, grid, st);
   } else if (g->layout == kCsr) {
-    if (count) launch_lockstep<kCsr, true>(V, g->act, bounds, Q, one, grid, st);
-    else launch_lockstep<kCsr, false>(V, g->act, bounds, Q, one, grid, st);
+    if (count) launch_lockstep<kCsr, true>(V, act, bounds, Q, one, grid, st);
+    else launch_lockstep<kCsr, false>(V, act, bounds, Q, one, grid, st);
   } else {
-    if (count) launch_lockstep<kNarrow, true>(V, g->act, bounds, Q, one, grid, st);
-    else launch_lockstep<kNarrow, false>(V, g->act, bounds, Q, one, grid, st);
+    if (count) launch_lockstep<kNarrow, true>(V, act, bounds, Q, one, grid, st);
+    else launch_lockstep<kNarrow, false>(V, act, bounds, Q, one, grid, st);
   }
   if (timing) cudaEventRecord(timing[1], st);
   if (nr > 0)
     k_finish<<<grid_for(nr, kFinishTile, dev), 256, 0, st>>>(g->row_ptr, bounds, sm.cnt, t.s,
                                                              u_begin, u_end, t.z, F.slots ? 1 : 0, o.scores,
                                                      o.wsums, o.steps, sm.ctr);
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return SRK_OK;
 }
 
 int enqueue_shared_walks(const srk_graph *g, const SharedWalks &Q, cudaStream_t st) {
   const GraphView V = view_of(g);
+  const int32_t *act = g->layout == kNarrow ? g->order : g->act;  // (see enqueue_walks)
   const int grid = sm_count(g->device) * kLockBlocks;
   const size_t smem = 4 * (size_t)kListWords + 8 * kHubCache + 4 * kCodes +
                       8 * (size_t)kSharedTargets * kLockThreads;
@@ -1299,8 +1224,8 @@ int enqueue_shared_walks(const srk_graph *g, const SharedWalks &Q, cudaStream_t 
                 "the opt-in covers both kernels");
 #define SRK_SHARED(L)                                                                       \
   do {                                                                                      \
-    if (Q.steps) k_lock_shared<L, true><<<grid, kLockThreads, smem, st>>>(V, g->act, g->n_act, Q); \
-    else k_lock_shared<L, false><<<grid, kLockThreads, smem, st>>>(V, g->act, g->n_act, Q);  \
+    if (Q.steps) k_lock_shared<L, true><<<grid, kLockThreads, smem, st>>>(V, act, g->n_act, Q); \
+    else k_lock_shared<L, false><<<grid, kLockThreads, smem, st>>>(V, act, g->n_act, Q);  \
   } while (0)
   if (g->layout == kWide) SRK_SHARED(kWide);
   else if (g->layout == kCsr) SRK_SHARED(kCsr);

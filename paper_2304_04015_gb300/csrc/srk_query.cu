@@ -1,15 +1,9 @@
 // Single- and multi-source queries: the sqrt(c)-walk Monte Carlo estimator of
 // arXiv 2304.04015 as kernel phases on one stream.
 //
-//   a2  k_source_walks   N_tot fixed-length walks from s (Algorithm 1 lines
-//                        4-7) and the Fisher-Yates draws of the shuffle
-//   a3  k_fy_rank .. k_pairs
-//                        the Fisher-Yates permutation sigma (Section 4.1(b),
-//                        Section 5.2), resolved in parallel (see k_pairs), and
-//                        each pair's step cap min(l2, steps of source walk)
-//       k_rows           pairs sorted by cap (descending): where each cap's
-//                        pairs begin
-//   a4+a5 enqueue_walks  (srk_lockstep.cu) the targets' walks
+//   a2-a3 enqueue_source (srk_source.cu) the source's walks, their shuffle and
+//                        the walk pairs, sorted by step cap (descending)
+//   a4-a5 enqueue_walks  (srk_lockstep.cu) the targets' walks
 //       k_literal_walks  the same with the literal target shuffle, on a
 //                        step-major hit table (k_hit_table): row i holds, for
 //                        every pair that can still meet at step i, the source
@@ -23,213 +17,6 @@
 #include "srk_internal.h"
 
 namespace srk {
-
-// ---------------------------------------------------------------- step a2 --
-// Walk r of the source has length l = stratum(r).  Step i >= 1 moves to
-// I(x)[k], k the bounded draw below |I(x)| from word (i-1)&1 of the
-// Philox2x32-10 block (((i-1)>>1) << 24 | r, s) under the source's walk key
-// (step_entry); it stops early at a node with no in-neighbours.  The source's
-// walks run on the CSR, so spos holds node ids: the filters (srk_filter.cu)
-// look ids up, and the hit lists translate them once.  The same thread
-// computes Fisher-Yates draw t = r, k_t = floor(R * (t+1) / 2^64) with R from
-// counter (t>>1, ~0, ~0, s).
-__global__ void __launch_bounds__(256)
-k_source_walks(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-               const __grid_constant__ QueryTab tab,
-               int32_t *__restrict__ spos, int32_t *__restrict__ seff,
-               int32_t *__restrict__ kdraw, int32_t *__restrict__ grp_cnt,
-               int32_t *__restrict__ small_base) {
-  __shared__ int32_t P[SRK_MAX_LEN + 2];
-  for (int i = threadIdx.x; i <= tab.L + 1; i += blockDim.x) P[i] = tab.P[i];
-  __syncthreads();
-  const RoundKeys rk = round_keys(tab.key0, tab.key1);
-  const int Ls = tab.L > 0 ? tab.L : 1;
-  const uint32_t s = (uint32_t)tab.s;
-  const AdjC G{row_ptr, col};
-  uint32_t deg_s = 0;
-  const int32_t b_s = node_start(G, row_ptr, tab.s, deg_s);
-  unsigned long long steps = 0;
-  for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < tab.N_tot;
-       r += gridDim.x * blockDim.x) {
-    grp_cnt[r] = 0;
-    kdraw[r] = (r >= 1) ? fy_draw(rk, s, r) : 0;
-    const int len = stratum_of(P, tab.L, r);
-    const int eff = source_walk(tab.skey, G, s, b_s, deg_s, r, len, spos + (int64_t)r * Ls);
-    seff[r] = eff;
-    steps += (unsigned long long)eff;
-  }
-  // source-step total (one atomic per warp)
-  for (int off = 16; off > 0; off >>= 1) steps += __shfl_xor_sync(0xffffffffu, steps, off);
-  if ((threadIdx.x & 31) == 0 && steps)
-    atomicAdd(small_view(small_base).ctr + 1, steps);
-}
-
-// ---------------------------------------------------------------- step a3 --
-// The permutation sigma of the sequential Fisher-Yates loop "for t = N-1
-// down to 1: swap(sigma[t], sigma[k_t])" is resolved in parallel.  Position
-// t >= 1 is final after step t and receives the value that position k_t held
-// just before step t.  Position p (p <= t) was last written before step t by
-// the step t' = min{t' > t : k_t' = p}, which moved in the value position t'
-// held before step t'; if no such step exists it still holds p.  Following
-// these links gives sigma[t] (sigma[0]: the value of position 0 after all
-// steps).  Steps are grouped by k (counting sort) to find the links.
-
-__global__ void k_fy_rank(const int32_t *__restrict__ kdraw, int32_t *grp_cnt,
-                          int32_t *__restrict__ rank, int32_t N) {
-  for (int32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < N;
-       t += gridDim.x * blockDim.x)
-    if (t >= 1) rank[t] = atomicAdd(&grp_cnt[kdraw[t]], 1);
-}
-
-// Exclusive scan of cnt[0..N) into off[0..N], one block of 1024 threads.
-__global__ void __launch_bounds__(1024)
-k_scan(const int32_t *__restrict__ cnt, int32_t *__restrict__ off, int32_t N) {
-  __shared__ int32_t warp_sum[32];
-  __shared__ int32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int64_t base = 0; base < N; base += 4096) {
-    const int64_t i0 = base + 4 * (int64_t)threadIdx.x;
-    int32_t v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = (i0 + k < N) ? cnt[i0 + k] : 0;
-    const int32_t local = v[0] + v[1] + v[2] + v[3];
-    int32_t incl = local;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_sum[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-      int32_t ws = warp_sum[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, ws, o);
-        if (lane >= o) ws += y;
-      }
-      warp_sum[lane] = ws;  // inclusive over warps
-    }
-    __syncthreads();
-    int32_t run = carry + (wid ? warp_sum[wid - 1] : 0) + incl - local;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (i0 + k < N) off[i0 + k] = run;
-      run += v[k];
-    }
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = run;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) off[N] = carry;
-}
-
-__global__ void k_fy_scatter(const int32_t *__restrict__ kdraw,
-                             const int32_t *__restrict__ off,
-                             const int32_t *__restrict__ rank,
-                             int32_t *__restrict__ items, int32_t N) {
-  for (int32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < N;
-       t += gridDim.x * blockDim.x)
-    if (t >= 1) items[off[kdraw[t]] + rank[t]] = t;
-}
-
-// Per group q = {t : k_t = q}: sort ascending, first[q] = its smallest step,
-// succ[t] = the next larger step of t's group (-1 for the largest).
-__global__ void k_fy_groups(const int32_t *__restrict__ off,
-                            int32_t *__restrict__ items,
-                            int32_t *__restrict__ first,
-                            int32_t *__restrict__ succ, int32_t N) {
-  for (int32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < N;
-       q += gridDim.x * blockDim.x) {
-    const int32_t b = off[q], e = off[q + 1];
-    for (int32_t i = b + 1; i < e; ++i) {  // insertion sort (groups are tiny)
-      const int32_t x = items[i];
-      int32_t k = i - 1;
-      while (k >= b && items[k] > x) { items[k + 1] = items[k]; --k; }
-      items[k + 1] = x;
-    }
-    first[q] = (e > b) ? items[b] : -1;
-    for (int32_t i = b; i < e; ++i) succ[items[i]] = (i + 1 < e) ? items[i + 1] : -1;
-  }
-}
-
-// sigma[j] by following the links, then the pair's step cap
-// cap_j = min(l2 = stratum(j), steps taken by source walk sigma[j]);
-// pairs with cap >= 1 are counted per cap value.
-__global__ void __launch_bounds__(256)
-k_pairs(const __grid_constant__ QueryTab tab, const int32_t *__restrict__ kdraw,
-        const int32_t *__restrict__ first, const int32_t *__restrict__ succ,
-        const int32_t *__restrict__ seff, int32_t *__restrict__ sigma,
-        int32_t *__restrict__ small_base) {
-  __shared__ int32_t P[SRK_MAX_LEN + 2];
-  __shared__ int32_t hist[SRK_MAX_LEN + 2];
-  for (int i = threadIdx.x; i <= tab.L + 1; i += blockDim.x) {
-    P[i] = tab.P[i];
-    hist[i] = 0;
-  }
-  __syncthreads();
-  const int32_t N = tab.N_tot;
-  for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < N;
-       j += gridDim.x * blockDim.x) {
-    const int32_t p = resolve_sigma(j, kdraw, first, succ, N);
-    sigma[j] = p;
-    // literal mode: the target walk is pi_u(j), so only the source bounds the cap
-    const int32_t cap = tab.literal ? seff[p] : min(stratum_of(P, tab.L, j), seff[p]);
-    if (cap >= 1) atomicAdd(&hist[cap], 1);
-  }
-  __syncthreads();
-  Small sm = small_view(small_base);
-  for (int i = threadIdx.x; i <= tab.L + 1; i += blockDim.x)
-    if (hist[i]) atomicAdd(&sm.cap_hist[i], hist[i]);
-}
-
-// Pairs sorted by cap, descending: cnt[i] = #pairs with cap >= i.  R[i] is
-// where the nodes of the pairs of cap i begin, or, in the literal mode, where
-// row i of the hit table begins.  Also finds [act_lo, act_hi), the part of the
-// ascending active-target list `act` inside [u_begin, u_end): words 1 and 2
-// after the work counter, which starts at 0 (units) or, in the literal mode, at
-// act_lo.
-__global__ void k_rows(int L, bool literal, int32_t *__restrict__ small_base,
-                       const int32_t *__restrict__ act, int32_t n_act, int32_t n, int32_t u_begin,
-                       int32_t u_end) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  Small sm = small_view(small_base);
-  int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);  // counter, act_hi
-  auto lower_bound = [&](int32_t v) {  // first index with act[index] >= v
-    int32_t lo = 0, hi = n_act;
-    while (lo < hi) {
-      const int32_t mid = lo + (hi - lo) / 2;
-      if (act[mid] < v) lo = mid + 1;
-      else hi = mid;
-    }
-    return lo;
-  };
-  bounds[2] = u_begin == 0 ? 0 : lower_bound(u_begin);
-  bounds[0] = literal ? bounds[2] : 0;
-  bounds[1] = u_end == n ? n_act : lower_bound(u_end);
-  int32_t c = 0;
-  sm.cnt[L + 1] = 0;
-  for (int i = L; i >= 1; --i) {
-    sm.cursor[i] = c;  // cap-i pairs follow all pairs with a larger cap
-    c += sm.cap_hist[i];
-    sm.cnt[i] = c;
-  }
-  int32_t r = 0;
-  if (literal) {
-    for (int i = 1; i <= L + 1; ++i) {
-      sm.R[i] = r;
-      if (i <= L) r += sm.cnt[i];
-    }
-  } else {
-    for (int i = L; i >= 1; --i) {  // the nodes of longer pairs come first
-      sm.R[i] = r;
-      r += i * sm.cap_hist[i];
-    }
-    sm.R[L + 1] = r;
-  }
-  sm.cnt[0] = c;
-  sm.R[0] = 0;
-}
 
 // Places every pair with cap >= 1 in its cap group and fills its column of the
 // hit table with the source walk's nodes at steps 1..cap.  The pair's Lemma 7
@@ -261,7 +48,7 @@ k_hit_table(const __grid_constant__ QueryTab tab, GraphView V, const int32_t *__
     pair_w[a] = tab.literal ? (unsigned long long)l1
                             : __double2ull_rn(tab.a[l1] * tab.a[l2] * 4294967296.0);
     const int32_t *src = spos + (int64_t)w * Ls;
-    for (int i = 1; i <= cap; ++i) Hc[R[i] + a] = node_identity(V, src[i - 1]);
+    for (int i = 1; i <= cap; ++i) Hc[R[i] + a] = walk_identity(V, src[i - 1]);
   }
 }
 
@@ -432,18 +219,11 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
                   const Outputs &o, char *extra, size_t extra_bytes, bool count, cudaStream_t st,
                   const cudaEvent_t *timing, int32_t u_begin, int32_t u_end) {
   const int dev = g->device;
-  const int N = t.N_tot;
-  const int gN = grid_for(N, 256, dev);
-  cudaError_t e = cudaMemsetAsync(w.small, 0, kSmallBytes, st);
-  if (e != cudaSuccess) return cuda_fail(e, "clearing query counters");
-  k_source_walks<<<gN, 256, 0, st>>>(g->row_ptr, g->col, t, w.spos, w.seff, w.kdraw, w.grp_cnt,
-                                     w.small);
-  k_fy_rank<<<gN, 256, 0, st>>>(w.kdraw, w.grp_cnt, w.rank, N);
-  k_scan<<<1, 1024, 0, st>>>(w.grp_cnt, w.grp_off, N);
-  k_fy_scatter<<<gN, 256, 0, st>>>(w.kdraw, w.grp_off, w.rank, w.items, N);
-  k_fy_groups<<<gN, 256, 0, st>>>(w.grp_off, w.items, w.first, w.succ, N);
-  k_pairs<<<gN, 256, 0, st>>>(t, w.kdraw, w.first, w.succ, w.seff, w.sigma, w.small);
-  k_rows<<<1, 32, 0, st>>>(t.L, t.literal != 0, w.small, g->act, g->n_act, g->n, u_begin, u_end);
+  cudaError_t e = cudaSuccess;
+  Filters F;
+  plan_filters(g, t, w, (int64_t)u_end - u_begin, extra ? extra_bytes : 0, &F, extra);
+  const int rc = enqueue_source(g, t, w, F, u_begin, u_end, st);
+  if (rc) return rc;
   // targets without in-neighbours have zero outputs (and s, if it is one of
   // them, the score 1): clear the range, then walk only the active targets
   const size_t nr = (size_t)(u_end - u_begin);
@@ -457,9 +237,9 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
       e = cudaMemsetAsync(o.steps + u_begin, 0, sizeof(uint32_t) * nr, st);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the outputs of the target range");
   }
-  const GraphView V = view_of(g);
   if (t.literal) {
-    k_hit_table<<<gN, 256, 0, st>>>(t, V, w.sigma, w.seff, w.spos, w.small, w.pair_j, w.pair_w,
+    const GraphView V = view_of(g);
+    k_hit_table<<<grid_for(t.N_tot, 256, dev), 256, 0, st>>>(t, V, w.sigma, w.seff, w.spos, w.small, w.pair_j, w.pair_w,
                                     w.Hc);
     TargetArgs A;
     A.view = V;
@@ -496,7 +276,7 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
     e = cudaGetLastError();
     return e == cudaSuccess ? SRK_OK : cuda_fail(e, "kernel launch");
   }
-  return enqueue_walks(g, t, w, o, extra, extra_bytes, count, st, timing, u_begin, u_end);
+  return enqueue_walks(g, t, w, F, o, count, st, timing, u_begin, u_end);
 }
 
 // The target range of a query from its options: [0, n) by default.

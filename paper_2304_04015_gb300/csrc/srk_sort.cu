@@ -76,6 +76,49 @@ k_sort_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ val
   }
 }
 
+// Exclusive scan of cnt[0..N) into off[0..N], one block of 1024 threads.
+static __global__ void __launch_bounds__(1024)
+k_scan(const int32_t *__restrict__ cnt, int32_t *__restrict__ off, int32_t N) {
+  __shared__ int32_t warp_sum[32];
+  __shared__ int32_t carry;
+  if (threadIdx.x == 0) carry = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int64_t base = 0; base < N; base += 4096) {
+    const int64_t i0 = base + 4 * (int64_t)threadIdx.x;
+    int32_t v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = (i0 + k < N) ? cnt[i0 + k] : 0;
+    const int32_t local = v[0] + v[1] + v[2] + v[3];
+    int32_t incl = local;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_sum[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+      int32_t ws = warp_sum[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, ws, o);
+        if (lane >= o) ws += y;
+      }
+      warp_sum[lane] = ws;  // inclusive over warps
+    }
+    __syncthreads();
+    int32_t run = carry + (wid ? warp_sum[wid - 1] : 0) + incl - local;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (i0 + k < N) off[i0 + k] = run;
+      run += v[k];
+    }
+    __syncthreads();
+    if (threadIdx.x == 1023) carry = run;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) off[N] = carry;
+}
+
 // Sums of the scan's tiles.
 __global__ void __launch_bounds__(1024)
 k_scan_sums(const int32_t *__restrict__ cnt, int64_t N, int32_t *__restrict__ sums) {
