@@ -112,8 +112,8 @@ constexpr int kLockWarps = kLockThreads / 32;
 constexpr int kStages = 2;            // groups of filters in flight per block,
 constexpr int kStageWords = 2048;     //   this many words of filters each (at least the largest)
 constexpr int kGroup = 16;            //   of at most this many pairs
-constexpr int kListWords = 8192;       // words of targets' own lists held in shared memory
-constexpr int kQueue = 64;            // entries of a warp's queue of last steps
+constexpr int kListWords = 2048;       // words of targets' own lists held in shared memory
+constexpr int kQueue = 128;           // entries of a warp's queue of last steps
 constexpr int kHubCache = 512;        // hub records held there (narrow layout),
 constexpr int kCodes = 2048;          //   and list starts by degree code
 constexpr size_t kLockSmem = 4 * (size_t)kStages * kStageWords + 4 * kListWords +
@@ -184,7 +184,7 @@ __device__ __forceinline__ void lock_index(const uint32_t (&w)[kT], const uint32
     mul_wide(w[t], d[t], idx[t], lo);
     rare |= lo < d[t];
   }
-  if (rare)
+  if (__any_sync(0xffffffffu, rare))
 #pragma unroll
     for (int t = 0; t < kT; ++t)
       if (d[t]) idx[t] = rare_index(w[t], k, i, r, (uint32_t)v[t], d[t]);
@@ -295,6 +295,7 @@ struct LockFilter {
 struct LockQueue {
   uint32_t at;  // shared memory
   int32_t n;
+  uint32_t below;  // the mask of the lower lanes
 };
 
 template <int kT, class GA>
@@ -335,13 +336,13 @@ __device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, con
 }
 
 // One pair (index j, nodes h at steps 1..cap, step 1..32 in the lanes' h32)
-// for the thread's targets; kCap = cap, or 0 for any.
+// for the thread's targets; kCap = cap, or 0 for any up to 32, or -1 for any.
 template <int kCap, int kT, bool kCount, class GA, class E>
 __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, const LockQuery &Q, const LockFilter &F,
                                           uint32_t lists, int32_t a, uint32_t j, int cap_,
                                           int32_t h32, const int32_t *__restrict__ h,
                                           LockTargets<kT> &X, LockQueue &B) {
-  const int cap = kCap ? kCap : cap_;
+  const int cap = kCap > 0 ? kCap : cap_;
   const int lane = threadIdx.x & 31;
   int32_t b[kT];
   uint32_t deg[kT], x0[kT], x1[kT], idx[kT];
@@ -358,54 +359,68 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
     load_if(X.at[t] >= 0, lists + (uint32_t)sizeof(E) * ((uint32_t)X.at[t] + idx[t]), e[t]);
     load_if(X.at[t] == -1, entries(G) + ((uint32_t)X.b[t] + idx[t]), e[t]);
   }
-#pragma unroll(kCap ? kCap : 1)
+#pragma unroll(kCap > 0 ? kCap : 1)
   for (int i = 1;; ++i) {
     // the walks are at the nodes that the entries e of step i name
     int32_t hi = __shfl_sync(0xffffffffu, h32, (i - 1) & 31);
-    if (kCap == 0 && i > 32) hi = h[i - 1];
-    bool met[kT], meets = false;
+    if (kCap < 0 && i > 32) hi = h[i - 1];
+    bool meets = false;
 #pragma unroll
     for (int t = 0; t < kT; ++t) {
-      met[t] = deg[t] != 0 && entry_pos(G, e[t]) == hi;
-      meets |= met[t];
-      if (kCount && (i == cap ? deg[t] != 0 : met[t])) X.st[t] += i;
+      meets |= entry_pos(G, e[t]) == hi;  // (or a walk that has ended was there)
+      if (kCount && i == cap && deg[t]) X.st[t] += i;
     }
     if (__any_sync(0xffffffffu, meets)) {  // rare: a few times per target and query
 #pragma unroll
       for (int t = 0; t < kT; ++t)
-        if (met[t]) {
+        if (deg[t] != 0 && entry_pos(G, e[t]) == hi) {
           atomicAdd(&Q.W[X.u[t]], Q.w[a]);
           if (Q.counts) atomicAdd(&Q.counts[X.u[t]], 1u);
           deg[t] = 0;
+          if (kCount && i < cap) X.st[t] += i;
         }
     }
     if (i == cap) break;  // cap 1
     if (i == cap - 1) {   // the last step: into the queue, if the filter lets it
       int32_t he = __shfl_sync(0xffffffffu, h32, i & 31);
-      if (kCap == 0 && i >= 32) he = h[i];
+      if (kCap < 0 && i >= 32) he = h[i];
+      uint32_t word[kT], f[kT];
+      if (F.has) {
+#pragma unroll
+        for (int t = 0; t < kT; ++t) f[t] = filter_bit(entry_pos(G, e[t]), F.lg);
+        if (F.landed) {
+#pragma unroll
+          for (int t = 0; t < kT; ++t) {
+            word[t] = 0;
+            load_if(true, F.near + 4u * (f[t] >> 5), word[t]);
+          }
+        } else {
+#pragma unroll
+          for (int t = 0; t < kT; ++t) word[t] = F.far[f[t] >> 5];
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+          word[t] = ~0u;
+          f[t] = 0;
+        }
+      }
+      const uint32_t len_j = (uint32_t)cap << 24 | j, a_lane = (uint32_t)a << 8 | (uint32_t)lane;
 #pragma unroll
       for (int t = 0; t < kT; ++t) {
-        const int32_t x = entry_pos(G, e[t]);
         bool p = deg[t] != 0;
         if (kCount && p) {
-          const bool ends = entry_ends(G, e[t], x);
+          const bool ends = entry_ends(G, e[t], entry_pos(G, e[t]));
           X.st[t] += ends ? i : cap;
           p = !ends;
         }
-        if (F.has) {
-          const uint32_t f = filter_bit(x, F.lg);
-          uint32_t word = 0;
-          if (F.landed) load_if(true, F.near + 4u * (f >> 5), word);
-          else word = F.far[f >> 5];
-          p = p && ((word >> (f & 31)) & 1u);
-        }
+        p = p && ((word[t] >> (f[t] & 31)) & 1u);
         const uint32_t m = __ballot_sync(0xffffffffu, p);
-        store_if(p, B.at + 16u * (uint32_t)(B.n + __popc(m & lanes_below_mask())),
-                 entry_word(e[t]), (uint32_t)he, (uint32_t)cap << 24 | j,
-                 (uint32_t)a << 8 | (uint32_t)(t * 32 + lane));
+        store_if(p, B.at + 16u * (uint32_t)(B.n + __popc(m & B.below)), entry_word(e[t]),
+                 (uint32_t)he, len_j, a_lane + 32u * t);
         B.n += __popc(m);
-        if (B.n >= 32) lock_drain(G, T, Q, B, 32, X.u);
       }
+      while (B.n >= 32) lock_drain(G, T, Q, B, 32, X.u);
       break;
     }
     uint32_t any = 0;
@@ -442,7 +457,7 @@ __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
                                                uint32_t &seq, LockTargets<kT> &X) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const bool filtered = Q.min_cap == 2;
-  LockQueue B{smem_addr(queues + wid * kQueue), 0};
+  LockQueue B{smem_addr(queues + wid * kQueue), 0, lanes_below_mask()};
   int32_t issued = 0;  // warp 0: pairs in the groups formed so far
   auto issue = [&](uint32_t n) {  // warp 0: form group n and fetch its filters
     if (issued >= len) return;
@@ -506,7 +521,8 @@ __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
                                   Q.H + rec.z, X, B)
       if (rec.y == 2) SRK_PAIR(2);
       else if (rec.y == 3) SRK_PAIR(3);
-      else SRK_PAIR(0);
+      else if (rec.y <= 32) SRK_PAIR(0);
+      else SRK_PAIR(-1);
 #undef SRK_PAIR
     }
     gk = ge;
