@@ -415,12 +415,7 @@ extern "C" int srk_graph_free(srk_graph *g) {
     if (g->own_col) cudaFree(g->own_col);
     if (g->own_w) cudaFree(g->own_w);
     if (g->adj) cudaFree(g->adj);
-    if (g->npos) cudaFree(g->npos);
-    if (g->order) cudaFree(g->order);
-    if (g->hub) cudaFree(g->hub);
-    if (g->ctab) cudaFree(g->ctab);
     if (g->act) cudaFree(g->act);
-    if (g->out_deg) cudaFree(g->out_deg);
     if (g->batch_exec) cudaGraphExecDestroy(g->batch_exec);
     free_lin_topo(g);
   }
@@ -504,13 +499,19 @@ static int build_narrow(srk_graph *g, int dev) {
     first += d * (uint32_t)cnt[d];
     rank += (uint32_t)cnt[d];
   }
-  if (e == cudaSuccess) e = cudaMalloc(&g->adj, sizeof(uint32_t) * (size_t)(m > 0 ? m : 1));
-  if (e == cudaSuccess) e = cudaMalloc(&g->npos, sizeof(int32_t) * (size_t)n);
-  if (e == cudaSuccess) e = cudaMalloc(&g->order, sizeof(int32_t) * (size_t)n);
+  // one block: the lists, ranks, nodes by rank, hub records and list starts
+  const size_t adj_b = up(sizeof(uint32_t) * (size_t)(m > 0 ? m : 1)),
+               hub_b = up(sizeof(uint2) * (size_t)(H > 0 ? H : 1));
   if (e == cudaSuccess)
+    e = cudaMalloc(&g->adj, adj_b + 2 * nb + hub_b + sizeof(uint32_t) * ctab.size());
+  if (e == cudaSuccess) {
+    char *p8 = (char *)g->adj + adj_b;
+    g->npos = (int32_t *)p8;
+    g->order = (int32_t *)(p8 + nb);
+    g->hub = (uint2 *)(p8 + 2 * nb);
+    g->ctab = (uint32_t *)(p8 + 2 * nb + hub_b);
     e = cudaMemcpyAsync(g->order, order, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, 0);
-  if (e == cudaSuccess) e = cudaMalloc(&g->hub, sizeof(uint2) * (size_t)(H > 0 ? H : 1));
-  if (e == cudaSuccess) e = cudaMalloc(&g->ctab, sizeof(uint32_t) * ctab.size());
+  }
   if (e == cudaSuccess)
     e = cudaMemcpy(g->ctab, ctab.data(), sizeof(uint32_t) * ctab.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
@@ -591,62 +592,49 @@ extern "C" int srk_graph_load(const int32_t *row_ptr, const int32_t *col,
     g->col = g->own_col;
     g->edge_w = g->own_w;
   }
-  {  // always validate: the walk kernels index with these values
-    int *bad = nullptr;
-    int hbad = 0;
-    if ((e = cudaMalloc(&bad, sizeof(int))) != cudaSuccess) {
-      int rc = cuda_fail(e, "srk_graph_load: validation flag");
+  {
+    // Always validate: the walk kernels index with these values.  In the same
+    // go, the ascending list of the nodes with in-neighbours and the
+    // out-degrees (sizes of the queries' filters): few allocations and waits,
+    // since those are what a small graph's load consists of.
+    const size_t words = ((size_t)n + 64) & ~(size_t)63;  // at least n + 1
+    int32_t *flag = nullptr;
+    if ((e = cudaMalloc(&flag, sizeof(int32_t) * (2 * words + 64) + scan_scratch(n))) !=
+        cudaSuccess) {
+      int rc = cuda_fail(e, "srk_graph_load: active-node list");
       srk_graph_free(g);
       return rc;
     }
-    cudaMemset(bad, 0, sizeof(int));
+    int32_t *off = flag + words, *bad = off + n + 1, *scan_tmp = off + words + 64;
     const int blocks = sm_count(dev) * 4;
+    cudaMemsetAsync(bad, 0, sizeof(int), 0);
     k_validate_csr<<<blocks, 256>>>(g->row_ptr, g->col, n, m, bad);
+    k_active_flags<<<blocks, 256>>>(g->row_ptr, n, flag);
+    scan_i32(flag, off, n, scan_tmp, 0);
+    int32_t got[2] = {0, 0};  // nodes with in-neighbours, malformed
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaFree(bad);
+    if (e == cudaSuccess) e = cudaMemcpy(got, off + n, sizeof got, cudaMemcpyDeviceToHost);
+    const size_t act_words = ((size_t)got[0] + 64) & ~(size_t)63;
+    if (e == cudaSuccess && !got[1] &&
+        (e = cudaMalloc(&g->act, sizeof(int32_t) * (act_words + (size_t)n))) == cudaSuccess) {
+      g->n_act = got[0];
+      g->out_deg = g->act + act_words;
+      cudaMemsetAsync(g->out_deg, 0, sizeof(int32_t) * (size_t)n, 0);
+      k_active_scatter<<<blocks, 256>>>(flag, off, n, g->act);
+      if (m > 0) k_out_degrees<<<2 * blocks, 256>>>(g->col, m, g->out_deg);
+      e = cudaGetLastError();
+    }
+    cudaFree(flag);
     if (e != cudaSuccess) {
-      int rc = cuda_fail(e, "srk_graph_load: validation");
+      int rc = cuda_fail(e, "srk_graph_load: validation and target list");
       srk_graph_free(g);
       return rc;
     }
-    if (hbad) {
+    if (got[1]) {
       srk_graph_free(g);
       return fail(SRK_EINVAL, "malformed CSR: row_ptr must start at 0, end at m and "
                               "not decrease; col entries must lie in [0, n)");
     }
-  }
-  {  // ascending list of the nodes with in-neighbours
-    int32_t *flag = nullptr, *off = nullptr, *scan_tmp = nullptr;
-    const size_t words = ((size_t)n + 64) & ~(size_t)63;
-    if ((e = cudaMalloc(&flag, 2 * sizeof(int32_t) * words + scan_scratch(n))) == cudaSuccess) {
-      off = flag + words;
-      scan_tmp = off + words;
-    } else {
-      int rc = cuda_fail(e, "srk_graph_load: active-node list");
-      srk_graph_free(g);
-      return rc;
-    }
-    k_active_flags<<<sm_count(dev) * 4, 256>>>(g->row_ptr, n, flag);
-    scan_i32(flag, off, n, scan_tmp, 0);
-    int32_t n_act = 0;
-    e = cudaGetLastError();
-    if (e == cudaSuccess)
-      e = cudaMemcpy(&n_act, off + n, sizeof(int32_t), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess &&
-        (e = cudaMalloc(&g->act, sizeof(int32_t) * (size_t)(n_act > 0 ? n_act : 1))) ==
-            cudaSuccess) {
-      k_active_scatter<<<sm_count(dev) * 4, 256>>>(flag, off, n, g->act);
-      e = cudaGetLastError();
-      if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    }
-    cudaFree(flag);
-    if (e != cudaSuccess) {
-      int rc = cuda_fail(e, "srk_graph_load: active-node list");
-      srk_graph_free(g);
-      return rc;
-    }
-    g->n_act = n_act;
   }
   {
     const int pb = bits_for((int64_t)n + m);  // positions < n + m (wide layout)
@@ -685,19 +673,10 @@ extern "C" int srk_graph_load(const int32_t *row_ptr, const int32_t *col,
     srk_graph_free(g);
     return rc;
   }
-  {  // out-degrees (sizes of the queries' filters)
-    e = cudaMalloc(&g->out_deg, sizeof(int32_t) * (size_t)n);
-    if (e == cudaSuccess) e = cudaMemset(g->out_deg, 0, sizeof(int32_t) * (size_t)n);
-    if (e == cudaSuccess && m > 0) {
-      k_out_degrees<<<sm_count(dev) * 8, 256>>>(g->col, m, g->out_deg);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) {
-      int rc = cuda_fail(e, "srk_graph_load: out-degrees");
-      srk_graph_free(g);
-      return rc;
-    }
+  if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
+    int rc = cuda_fail(e, "srk_graph_load");
+    srk_graph_free(g);
+    return rc;
   }
   *out = g;
   return SRK_OK;

@@ -31,10 +31,10 @@ struct srk_graph {
   // 2, only when forced by SRK_ADJ_CSR): no packed copy; nodes are their ids
   // and a step reads row_ptr and col.
   uint32_t *adj = nullptr;
-  int32_t *npos = nullptr;   // narrow layout: ranks, n (owned),
-  int32_t *order = nullptr;  //   and the nodes by rank, n (owned)
-  uint2 *hub = nullptr;      // narrow layout: hub records, n_hubs (owned)
-  uint32_t *ctab = nullptr;  // narrow layout: list starts by degree (owned)
+  int32_t *npos = nullptr;   // narrow layout (in adj's block): ranks, n,
+  int32_t *order = nullptr;  //   the nodes by rank, n,
+  uint2 *hub = nullptr;      //   hub records, n_hubs,
+  uint32_t *ctab = nullptr;  //   and list starts by degree
   int32_t n_hubs = 0;        // narrow layout: H
   int32_t pos_bits = 1;      // narrow layout: ranks < 2^pos_bits
   uint32_t deg_max = 1;      // narrow layout: largest degree code
@@ -43,7 +43,7 @@ struct srk_graph {
   // whose score can be nonzero.
   int32_t *act = nullptr;
   int32_t n_act = 0;
-  int32_t *out_deg = nullptr;  // out-degrees by id, n (owned)
+  int32_t *out_deg = nullptr;  // out-degrees by id, n (in act's block)
   // Launch shape of the batched target kernel chosen by the autotuner
   // (-1: not tuned yet).
   int batch_cfg = -1;
