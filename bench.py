@@ -238,7 +238,7 @@ def kernel_source_sha256():
     import hashlib
     import re
     h = hashlib.sha256()
-    for name in ("srk_query.cu", "srk_device.cuh", "srk_graph.cu"):
+    for name in ("srk_lockstep.cu", "srk_device.cuh", "srk_graph.cu"):
         with open(os.path.join(ROOT, "paper_2304_04015_gb300", "csrc", name)) as f:
             text = f.read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
@@ -251,7 +251,7 @@ def recorded_profile():
     """The committed ncu record of the target-walk kernel, if it was taken on
     the current kernel sources, else None."""
     try:
-        with open(os.path.join(ROOT, "profiles", "k_target_walks_rmat20_traffic.json")) as f:
+        with open(os.path.join(ROOT, "profiles", "k_lockstep_rmat20_traffic.json")) as f:
             rec = json.load(f)
         return rec if rec.get("kernel_sources_sha256") == kernel_source_sha256() else None
     except Exception:
@@ -393,7 +393,7 @@ def run_batch(args, rank, world):
     peak, peak_kind = load_peaks()
     achieved = st.target_steps * BYTES_PER_STEP / t_batch / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": None, "kernel": "kb_target_walks",
+                "frac": achieved / peak, "traffic": None, "kernel": "k_lockstep",
                 "peak_kind": peak_kind + " (HBM copy)", "bytes_per_unit": BYTES_PER_STEP,
                 "unit_name": "target-walk step",
                 "note": "whole batch time (the source phases are a few percent)"}
@@ -652,7 +652,7 @@ def run_serve(args, rank, world):
     peak, peak_kind = load_peaks()
     achieved = st.target_steps * BYTES_PER_STEP / st.wall_s / 1e9 if st.wall_s else 0.0
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": None, "kernel": "k_target_walks",
+                "frac": achieved / peak, "traffic": None, "kernel": "k_lockstep",
                 "peak_kind": peak_kind + " (HBM copy)", "bytes_per_unit": BYTES_PER_STEP,
                 "unit_name": "target-walk step",
                 "note": "over the serving run's wall time (includes idle gaps)"}
@@ -947,12 +947,13 @@ def main():
                                                             by_op)),
                   "kernel_steps_per_s": target_steps_per_s,
                   "frac_of_graph_sized_probe": target_steps_per_s / l2_rate,
-                  "note": "one scattered 4-byte adjacency read per target-walk step; "
+                  "note": "target-walk steps against scattered 4-byte reads; steps that "
+                          "an end filter rules out count but read nothing; "
                           "probe = srk_probe_gather, independent random loads at full "
                           "occupancy on an array the size of the adjacency"}
     fits_l2 = adj_b <= l2_b
     hbm_frac = hbm_achieved / peak_hbm
-    common = {"kernel": "k_target_walks", "traffic": traffic,
+    common = {"kernel": "k_lockstep", "traffic": traffic,
               "traffic_unit": "DRAM bytes per launch (ncu, recorded for these kernel sources)",
               "kernel_ms_per_launch": float(np.mean(k_ms)),
               "kernel_share_of_query": float(np.sum(k_ms) / np.sum(q_ms)),
@@ -962,21 +963,26 @@ def main():
                            "bytes_per_unit": BYTES_PER_STEP,
                            "unit_name": "target-walk step (row_ptr pair + one entry)"}}
     if l2_rate is not None:
+        # each probe load misses L1 and takes one L2 sector.  A step takes fewer:
+        # first steps read lists held in shared memory, and last steps that an end
+        # filter rules out read nothing (they count as steps), so the ratio is
+        # taken in sectors where a capture of these sources records them, and in
+        # steps (an upper bound of the reads) where none does.
+        sps = recorded_l2_sectors()
+        rate = target_steps_per_s * (1.0 if sps is None else sps)
         roofline = {"bound": "l2_gather" if fits_l2 else "hbm_gather",
-                    "achieved": target_steps_per_s / 1e9, "peak": l2_rate / 1e9,
-                    "unit": "Gloads/s", "frac": target_steps_per_s / l2_rate,
+                    "achieved": rate / 1e9, "peak": l2_rate / 1e9,
+                    "unit": "Gloads/s" if sps is None else "Gsectors/s",
+                    "frac": rate / l2_rate,
                     "peak_kind": "measured live: random 4-byte gather probe on an array the "
                                  "size of the adjacency (%d MB)" % (adj_b >> 20),
-                    "unit_name": "target-walk step (one dependent scattered adjacency load)",
+                    "unit_name": "target-walk step (at most one scattered adjacency load)"
+                                 if sps is None else "L2 sector requested by L1 (one per "
+                                 "scattered adjacency load)",
                     **common}
-        sps = recorded_l2_sectors()
         if sps is not None:
-            # each probe load misses L1 and takes one L2 sector; a step of the
-            # kernel takes fewer (some of its loads hit L1)
             roofline["l2_sectors"] = {
-                "per_step": sps, "achieved": target_steps_per_s * sps / 1e9,
-                "peak": l2_rate / 1e9, "unit": "Gsectors/s",
-                "frac": target_steps_per_s * sps / l2_rate,
+                "per_step": sps, "steps_per_s": target_steps_per_s,
                 "source": "L2 sectors requested by L1 per step from the recorded ncu "
                           "capture of these kernel sources"}
     else:
@@ -1024,7 +1030,9 @@ def main():
                                  "in-neighbours returns after the source phases"},
             "roofline": roofline, "gather_roofline": gather, "cpu_baseline": base,
             "e2e": e2e, "clocks": clk,
-            "gpu_launches": 9 * launches,
+            # k_source, k_edges, k_lockstep, k_finish; literal: k_source,
+            # k_hit_table, k_literal_walks
+            "gpu_launches": (3 if args.literal_shuffle else 4) * launches,
             "wall_s_timed_loop": t_wall, "graph_gen_s": t_gen}
     if rank == 0:
         print(json.dumps(line), flush=True)

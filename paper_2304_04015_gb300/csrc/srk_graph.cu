@@ -441,7 +441,7 @@ constexpr int kCodeBits = 11;
 // by id.  Expected visits (k_visit_*): 25 p_1 + 15 p_2 + 9 p_3, the landing
 // mass of the first three steps weighted by survival at c = 0.6 (the layout
 // does not depend on a query's c).  The layout is a function of the graph alone
-// and is made on the device: R-MAT 20 loads in 2.1 ms and R-MAT 22 in 5.1 ms,
+// and is made on the device: R-MAT 20 loads in 1.8 ms and R-MAT 22 in 5.0 ms,
 // where an order sorted on the host took 61 and 282 ms.
 static int build_narrow(srk_graph *g, int dev) {
   const int32_t n = g->n;

@@ -25,21 +25,23 @@
 //   draws u's step for those only.
 //
 // What bounds it (GB300): the misses of the scattered list reads, one 32-byte
-// sector each, 3.1e11 per second with the graph in L2; then issue slots.  At
-// R-MAT 20, eps = 0.02 (10,975 pairs, 546,406 targets): 0.93 sectors and 109
-// warp instructions per 32 pairs and targets, where a warp per target took
-// about 2.0 sectors and 189.  One query 31.5 ms instead of 42.3 ms; R-MAT 16
-// 2.11 ms instead of 2.58 ms; 100,003 nodes with uniform lists of 12, eps =
-// 0.03, 2.17 ms instead of 2.90 ms; R-MAT 22 at eps = 0.05, bound by DRAM (64
-// bytes fetched per missing sector), 51-55 ms instead of 60 ms.
+// sector each, of which a plain random gather gets 3.1e11 per second with the
+// graph in L2, then issue slots and the latency of a walk's chain of reads.  At
+// R-MAT 20, eps = 0.02 (10,941 pairs, 546,406 targets): 1.17 sectors a pair
+// and target and 104 warp instructions per pair and 32 targets (2.0 and 189
+// with a warp per target), 2.4e11 sectors per second, 54 % of the issue slots.
+// One query 29.2 ms instead of 42.3 ms; R-MAT 16 2.10 ms instead of 2.57 ms;
+// 100,003 nodes with uniform lists of 12, eps = 0.03, 1.97 ms instead of 2.92
+// ms; R-MAT 22 at eps = 0.05, bound by DRAM (64 bytes fetched per missing
+// sector), 49-55 ms instead of 55-62 ms.
 //
 // Launch shape: 2 blocks of 448 threads per SM, 3 targets a thread (72
 // registers).  Measured at R-MAT 20 in an earlier state of the kernel: 1 target
 // x 704 threads 44.7 ms, 2 x 512 39.9, 3 x 448 38.2, 4 x 384 38.2, 5 x 320 41:
 // several targets share a pair's uniform work, and their chains of dependent
-// loads overlap.  Shared memory is kept to about 76 KB a block, since the rest
-// of the SM's 256 KB holds the lines of reads in flight: 92 KB of it cost
-// nothing against 124 KB, 60 KB 10 %, 28 KB half the speed.
+// loads overlap.  Shared memory is kept to 64 KB a block, since the rest of the
+// SM's 256 KB holds the lines of reads in flight: 92 KB of it cost nothing
+// against 124 KB, 60 KB 10 %, 28 KB half the speed.
 #include <stdint.h>
 #include <string.h>
 
