@@ -11,8 +11,8 @@
 // launched as one.  The walk kernel's launch shape (targets per thread) is
 // chosen per graph by timing the candidates on the first units of the first
 // batch (autotuner).  (One persistent launch over all (source, target) items,
-// a warp each, took 86.2 ms for 24 sources of mixed eps on R-MAT 16, where this
-// takes 61.8 ms.)  With shared target walks (SRK_OPT_SHARED_WALKS) the batches hold
+// a warp each, took 68.4 ms for 24 sources of mixed eps on R-MAT 16, where this
+// takes 51.5 ms.)  With shared target walks (SRK_OPT_SHARED_WALKS) the batches hold
 // up to 64 sources and the target walks run once for all of them
 // (k_lock_shared, srk_lockstep.cu).
 #include <stdint.h>
