@@ -894,17 +894,21 @@ k_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ bounds
 // table's signature: 1024 bits, one L1 line that all the block's warps read,
 // so at most 6 % of the walks that meet nobody go to the table (with a 64-bit
 // signature in a register, the form before, half of them did).
-// A warp per target with lanes over pairs took 10.4 ms for 48 sources on R-MAT
-// 18, eps = 0.05; this takes 6.2 ms, with 54 % of the issue slots and 62 % of the
-// request cycles to the L2 in use; 2 targets a thread 6.6
-// ms, 1 8.6 ms.
-constexpr int kSharedTargets = 3;  // per thread
+// A warp per target with lanes over pairs took 10.3 ms for 48 sources on R-MAT
+// 18, eps = 0.05; this takes 6.3 ms, with 54 % of the issue slots and 62 % of the
+// request cycles to the L2 in use; 2 targets a thread 6.6 ms, 1 8.6 ms.  The
+// wide layout, whose lists take twice the room and whose targets come by id,
+// wants fewer lists in the L2 between two of their first steps: 48 sources on
+// R-MAT 21 and 24, 378 and 33.1 queries/s with 2 targets a thread, 372 and 32.3
+// with 3, 357 and 33.1 with 1.
+constexpr int kSharedTargets = 3;  // per thread, at most
+constexpr int shared_targets(int layout) { return layout == kWide ? 2 : kSharedTargets; }
 
 template <int kLayout, bool kCount>
 __global__ void __launch_bounds__(kLockThreads, kLockBlocks)
 k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ act, int32_t n_act,
               const __grid_constant__ SharedWalks Q) {
-  constexpr int kT = kSharedTargets;
+  constexpr int kT = shared_targets(kLayout);
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ LockShared S;
   __shared__ int64_t rowbase[SRK_MAX_LEN + 2];
@@ -1209,8 +1213,11 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   // length: the short ones all fit its shared memory, the heavy units come
   // first.  By id for a part of them.
   const int32_t *act = nr == g->n && g->layout == kNarrow ? g->order : g->act;
-  // shape 0: kLockTargets targets a thread; 1: one (too few to give it several)
-  const bool one = shape < 0 ? nr <= kLockThreads : shape == 1;
+  // shape 0: kLockTargets targets a thread; 1: one, where there are too few to
+  // give it several, and on the wide layout, where fewer of the targets' own
+  // lists then compete for the L2 (R-MAT 24, eps = 0.05: 4.59 queries/s against
+  // 4.25; R-MAT 21, 50.6 against 50.1)
+  const bool one = shape < 0 ? nr <= kLockThreads || g->layout == kWide : shape == 1;
   if (g->layout == kWide) {
     if (count) launch_lockstep<kWide, true>(V, act, bounds, Q, one, grid, st);
     else launch_lockstep<kWide, false>(V, act, bounds, Q, one, grid, st);

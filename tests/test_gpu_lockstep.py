@@ -90,3 +90,28 @@ def test_short_target_ranges_without_filters(srk, lo, hi):
     for a, b in zip(got[:4], (ref.scores, ref.count, ref.wsum, ref.steps)):
         assert np.array_equal(a[lo:hi].astype(b.dtype), b[lo:hi])
     assert got[4].target_steps == int(ref.steps[lo:hi].sum())
+
+
+@pytest.mark.parametrize("n", [447, 449, 895, 897, 1793])
+def test_target_blocks_wide(srk, n):
+    """8-byte entries: one target per thread for a query, two for shared walks."""
+    import torch
+    rp, col = ring_lists(n, 3, n)
+    dev = torch.device("cuda:0")
+    kw = dict(z_override=500.0, L_override=12)
+    sources, c = [0, n // 2, n - 1], 0.6
+    out = torch.empty((3, n), dtype=torch.float64, device=dev)
+    cnt = torch.empty((3, n), dtype=torch.int32, device=dev)
+    with srk.srk_graph_load(torch.from_numpy(rp).to(dev), torch.from_numpy(col).to(dev),
+                            layout="wide") as g:
+        for shared in (False, True):
+            if shared:
+                srk.srk_multi_source(g, sources, c, [0.5] * 3, 3, out, cnt, shared_walks=True, **kw)
+            else:
+                for i, s in enumerate(sources):
+                    srk.srk_single_source(g, s, c, 0.5, 3, out[i], cnt[i], **kw)
+            torch.cuda.synchronize()
+            for i, s in enumerate(sources):
+                ref = oracle_query(rp, col, s, 0.5, 3, shared_walks=shared, **kw)
+                assert np.array_equal(out[i].cpu().numpy(), ref.scores)
+                assert np.array_equal(cnt[i].cpu().numpy().view(np.uint32), ref.count)
