@@ -641,8 +641,9 @@ extern "C" int srk_graph_load(const int32_t *row_ptr, const int32_t *col,
     // Layout by size: 4-byte entries while n + m needs 28 bits at most (degree
     // codes of 9 bits at R-MAT 23), 8-byte entries beyond, which carry the full
     // degree.  Forced at R-MAT 24 and 25 (codes of 8 and 7 bits), 4-byte entries
-    // give 4.93 and 2.30 queries/s at eps = 0.05 against 4.25 and 2.12: half
-    // the bytes weigh more than the hubs' records.  The default stays where
+    // give 4.93 and 2.30 queries/s at eps = 0.05 against 4.59 and 2.12 (the
+    // latter with 3 targets a thread): half the bytes weigh more than the
+    // hubs' records.  The default stays where
     // callers find it documented.  The CSR layout is only taken when asked for.
     g->layout = (flags & SRK_ADJ_WIDE)     ? 1
                 : (flags & SRK_ADJ_CSR)    ? 2
