@@ -45,6 +45,8 @@ k_sort_scatter(const int32_t *__restrict__ keys, const int32_t *__restrict__ val
   __syncthreads();
   const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
   for (int r = 0; r < kSortItems; ++r) {
+    // the last tile's rounds past the end: most of them on a small graph
+    if (tile0 + (int64_t)r * kSortBlock >= m) break;
     const int64_t i = tile0 + (int64_t)r * kSortBlock + t;
     const bool valid = i < m;
     int32_t key = 0, val = 0, d = 256;  // 256: no key in this slot
