@@ -42,6 +42,10 @@
  *   (a cudaStream_t; NULL = the legacy default stream).
  * Determinism: identical graph, source, c, eps, seed and options give
  *   bit-identical counts, weight sums and scores, whatever the launch shape.
+ * Waits: the walk kernels fetch a query's end filters into shared memory ahead of
+ *   their use.  A wait for them gives up after 2^20 polls, or as many as the
+ *   environment variable SRK_WAIT_POLLS says (0 to 2^20; 0: at once); the
+ *   filters are then read from global memory, with the same results.
  * Threads: queries only read the graph, so concurrent queries on different
  *   streams are safe.  Each call allocates its scratch from a library-owned
  *   stream-ordered pool on the stream it runs on.

@@ -43,6 +43,7 @@
 // SM's 256 KB holds the lines of reads in flight: 92 KB of it cost nothing
 // against 124 KB, 60 KB 10 %, 28 KB half the speed.
 #include <stdint.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
@@ -68,6 +69,7 @@ struct LockQuery {
   int32_t s;
   int32_t min_cap;              // pairs below this cap are not walked here
   int32_t max_units;            // units beyond these are not walked
+  int32_t polls;                // of a wait for filters before it gives up
 };
 
 // -------------------------------------------------- asynchronous copies --
@@ -134,15 +136,17 @@ struct LockShared {
   uint32_t sums[4];
   uint32_t warp_sum[kLockWarps];
   int32_t unit;
-  int32_t broken;  // a wait gave up: filters are read from global memory from here on
+  int32_t broken;  // a wait gave up: filters are read from global memory
 };
 
-// Waits, a bounded time, for the phase of parity ph.
-__device__ __forceinline__ bool lock_wait(LockShared &S, uint64_t *bar, uint32_t ph) {
-  if (mbar_try(bar, ph)) return *(volatile int32_t *)&S.broken == 0;
-  for (int spin = 0; spin < (1 << 20); ++spin) {
+// Waits, `polls` polls at most, for the phase of parity ph; false when this or
+// another wait of the block gave up.
+constexpr int32_t kWaitPolls = 1 << 20;
+__device__ __forceinline__ bool lock_wait(LockShared &S, uint64_t *bar, uint32_t ph,
+                                          int32_t polls) {
+  for (int32_t i = 0; i < polls; ++i) {
+    if (mbar_try(bar, ph)) return *(volatile int32_t *)&S.broken == 0;
     if (*(volatile int32_t *)&S.broken) return false;
-    if (mbar_try(bar, ph)) return true;
   }
   *(volatile int32_t *)&S.broken = 1;
   return false;
@@ -450,17 +454,22 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
 
 // Pairs first, first + stride, ... (len of them) for the block's targets; seq
 // counts the groups of this block.  Warp 0 forms the groups: the next pairs
-// whose filters fit a stage.
+// whose filters fit a stage.  `staged`: the pairs have filters, and no wait of an
+// earlier unit gave up (the same in every thread).  When a wait gives up, the
+// block's warps read the filters from global memory instead, one warp after the
+// other as each comes to a wait; none frees a stage from then on, so warp 0 forms
+// no group into a stage in use, waits for those that it has formed before it
+// leaves, and no later unit forms any.
 template <int kT, bool kCount, class GA, class E>
 __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
                                                const LockQuery &Q, LockShared &S,
                                                uint32_t *ring, uint4 *queues, const E *lists,
                                                int32_t first, int32_t stride, int32_t len,
-                                               uint32_t &seq, LockTargets<kT> &X) {
+                                               bool staged, uint32_t &seq, LockTargets<kT> &X) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const bool filtered = Q.min_cap == 2;
   LockQueue B{smem_addr(queues + wid * kQueue), 0, lanes_below_mask()};
-  int32_t issued = 0;  // warp 0: pairs in the groups formed so far
+  int32_t issued = 0;     // warp 0: pairs in the groups formed so far,
+  uint32_t formed = seq;  //   and the number of the next group
   auto issue = [&](uint32_t n) {  // warp 0: form group n and fetch its filters
     if (issued >= len) return;
     const uint32_t sg = n % kStages;
@@ -486,23 +495,24 @@ __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
       bulk_load(ring + sg * kStageWords + incl - words, Q.bits + filter_place(f),
                 4u * (uint32_t)words, &S.full[sg]);
     issued += count;
+    formed = n + 1;
   };
   const uint32_t seq0 = seq;
-  if (filtered && wid == 0)
+  if (staged && wid == 0)
     for (uint32_t q = 0; q < kStages - 1; ++q) issue(seq0 + q);
   int4 nrec = Q.rec[first];
   int32_t nh = lane < nrec.y ? Q.H[nrec.z + lane] : 0;
   LockFilter F;
-  F.landed = filtered;
+  F.landed = staged;
   for (int32_t gk = 0; gk < len; ++seq) {
     const uint32_t sg = seq % kStages;
     int32_t ge = len;
     if (F.landed) {
       if (wid == 0 &&
           __all_sync(0xffffffffu, seq == seq0 || lock_wait(S, &S.empty[(seq - 1) % kStages],
-                                                           ((seq - 1) / kStages) & 1u)))
+                                                           ((seq - 1) / kStages) & 1u, Q.polls)))
         issue(seq + kStages - 1);
-      F.landed = lock_wait(S, &S.full[sg], (seq / kStages) & 1u);
+      F.landed = lock_wait(S, &S.full[sg], (seq / kStages) & 1u, Q.polls);
       F.landed = __all_sync(0xffffffffu, F.landed);
       if (F.landed) ge = gk + S.pairs[sg];
     }
@@ -534,6 +544,10 @@ __device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
     }
   }
   if (B.n > 0) lock_drain(G, T, Q, B, B.n, X.u);
+  if (staged && wid == 0 && !F.landed)  // copies in flight, which nobody waited for
+    for (uint32_t q = max(seq0, formed > kStages ? formed - kStages : 0u); q < formed; ++q)
+      for (int32_t i = 0; i < kWaitPolls && !mbar_try(&S.full[q % kStages], (q / kStages) & 1u); ++i) {
+      }
 }
 
 // ------------------------------------------------------- edges, and walks --
@@ -811,6 +825,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   uint32_t seq = 0;
   for (;;) {
     __syncthreads();
+    const bool staged = Q.min_cap == 2 && *(volatile int32_t *)&S.broken == 0;
     if (threadIdx.x == 0) S.unit = atomicAdd(bounds, 1);
     if (threadIdx.x < 4) S.sums[threadIdx.x] = 0;
     __syncthreads();
@@ -820,8 +835,8 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
     const int32_t first = (int32_t)(unit / n_tb), len = (n_pairs - first + n_chunks - 1) / n_chunks;
     LockTargets<kT> X;
     lock_targets(G, V.row_ptr, S, lists, act, act_lo + tb * T, act_hi, Q.s, len >= 32, X);
-    lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len, seq,
-                               X);
+    lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len,
+                               staged, seq, X);
 #pragma unroll
     for (int t = 0; t < kT; ++t) {
       if (kCount && X.st[t]) {
@@ -1170,6 +1185,14 @@ static void launch_lockstep(const GraphView &V, const int32_t *act, int32_t *bou
                                                                                      Q);
 }
 
+// Polls of a wait for filters: 2^20, or the environment variable SRK_WAIT_POLLS.
+static int32_t wait_polls() {
+  const char *env = getenv("SRK_WAIT_POLLS");
+  if (!env || !*env) return kWaitPolls;
+  const long v = strtol(env, nullptr, 10);
+  return v < 0 || v > kWaitPolls ? kWaitPolls : (int32_t)v;
+}
+
 double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t max_units) {
   const int32_t T = kLockThreads * (shape == 1 ? 1 : kLockTargets);
   const int32_t n_tb = (g->n_act + T - 1) / T;
@@ -1206,6 +1229,7 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   Q.s = t.s;
   Q.min_cap = F.slots ? 2 : 1;
   Q.max_units = max_units;
+  Q.polls = wait_polls();
   if (timing) cudaEventRecord(timing[0], st);
   const int grid = sm_count(dev) * kLockBlocks;
   // The targets: by rank where all of them are wanted (the narrow layout ranks

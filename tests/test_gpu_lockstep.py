@@ -115,3 +115,15 @@ def test_target_blocks_wide(srk, n):
                 ref = oracle_query(rp, col, s, 0.5, 3, shared_walks=shared, **kw)
                 assert np.array_equal(out[i].cpu().numpy(), ref.scores)
                 assert np.array_equal(cnt[i].cpu().numpy().view(np.uint32), ref.count)
+
+
+@pytest.mark.parametrize("polls", ["0", "1"])
+def test_waits_for_filters_that_give_up(srk, monkeypatch, polls):
+    """SRK_WAIT_POLLS = 0: every block's first wait gives up, so the filters are
+    read from global memory from then on; 1: some waits may.  Integers: equal."""
+    rp, col = ring_lists(5000, 12, 8)
+    kw = dict(z_override=4000.0, L_override=14)
+    ref = oracle_query(rp, col, 9, 0.5, 21, **kw)
+    monkeypatch.setenv("SRK_WAIT_POLLS", polls)
+    for _ in range(3):
+        assert_parity(gpu_query(srk, rp, col, 9, 0.5, 21, **kw), ref)
