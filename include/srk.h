@@ -119,8 +119,9 @@ typedef struct srk_stats {
     int32_t L;              /* truncation length */
     int32_t n_walks;        /* N_tot = sum_l N_l, walks per node and pairs per target */
     int32_t n_active_pairs; /* pairs whose both walks take >= 1 step */
-    int32_t batch_shape;    /* srk_multi_source: index of the persistent kernel's
-                               launch shape the autotuner chose; else -1 */
+    int32_t batch_shape;    /* srk_multi_source: index of the walk kernels' launch
+                               shape (0: several targets a thread, 1: one);
+                               else -1 */
     uint64_t source_steps;  /* steps taken by the source's walks */
     uint64_t target_steps;  /* target-walk steps taken over all targets (with
                                SRK_OPT_SHARED_WALKS in srk_multi_source: the
@@ -239,13 +240,11 @@ int srk_single_source(const srk_graph *g, int32_t s, double c, double eps,
  * key is derived from its source).  The sources run in batches sized by
  * a scratch budget (a quarter of free device memory, at most 8 GiB, or the
  * byte count in the environment variable SRK_BATCH_BYTES): one
- * launch per source-side phase for the whole batch, then one persistent
- * launch per source over its targets, captured in a CUDA graph unless
+ * launch for the source side of the whole batch, then persistent launches over
+ * the targets of groups of sources, captured in a CUDA graph unless
  * opt->flags has SRK_OPT_NO_GRAPH.  Sources none of whose walk pairs can meet
  * (e.g. no in-neighbours) and targets without in-neighbours produce no work;
- * their scores are written directly.  The persistent kernel's launch shape is
- * picked per graph by timing the candidate shapes on the first units of work
- * of the first call (kept in the handle).  The call
+ * their scores are written directly.  The call
  * synchronises the stream at the end of every batch.  With
  * SRK_OPT_SHARED_WALKS the batches hold up to 64 sources, grouped by walk
  * budget with the sources without in-neighbours last (the call first reads

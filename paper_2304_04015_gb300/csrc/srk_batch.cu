@@ -1,20 +1,16 @@
 // srk_multi_source: many single-source queries with uneven walk budgets.
 //
-// The sources are processed in batches sized by a memory budget.  Each batch
-// runs the source-side steps a2-a3 of all its sources with one launch per
-// phase (thread g of a phase finds its source by a binary search over the
-// prefix of the sources' walk counts); then every source's targets are walked
-// as srk_single_source walks them (enqueue_walks, srk_lockstep.cu), so the
-// results are identical.  Sources whose walks never leave the source (no pair
-// can meet) find no work there: their score rows are prefilled (1 at the
-// source, 0 elsewhere).  A batch's launches are captured in a CUDA graph and
-// launched as one.  The walk kernel's launch shape (targets per thread) is
-// chosen per graph by timing the candidates on the first units of the first
-// batch (autotuner).  (One persistent launch over all (source, target) items,
-// a warp each, took 68.4 ms for 24 sources of mixed eps on R-MAT 16, where this
-// takes 51.5 ms.)  With shared target walks (SRK_OPT_SHARED_WALKS) the batches hold
-// up to 64 sources and the target walks run once for all of them
-// (k_lock_shared, srk_lockstep.cu).
+// The sources are processed in batches sized by a memory budget.  One launch runs
+// the source side (steps a2-a3) of all a batch's sources, a cluster each
+// (srk_source.cu).  Their targets are then walked as srk_single_source walks them
+// (srk_lockstep.cu), so the results are identical, a group of sources at a time:
+// one launch each for the group's end nodes, edges, walks and scores, but that a
+// source whose walks fill the GPU by themselves has a walk launch of its own.
+// Sources whose walks never leave the source (no pair can meet) find no work
+// there: their score rows are prefilled (1 at the source, 0 elsewhere).  A batch's
+// launches are captured in a CUDA graph and launched as one.  With shared target
+// walks (SRK_OPT_SHARED_WALKS) the batches hold up to 64 sources and the target
+// walks run once for all of them (k_lock_shared, srk_lockstep.cu).
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
@@ -207,57 +203,6 @@ int source_in_degrees(const srk_graph *g, const int32_t *sources, int32_t k, cud
 
 }  // namespace srk
 
-namespace {
-
-// The launch shape (enqueue_walks) that walks the first units of a batch's
-// first source with pairs the fastest, per target and pair; stays -1 when no
-// source has any.  Leaves the source side to be run again.
-template <class SourceSide, class Walks>
-int tune_shape(const srk_graph *g, const std::vector<BatchSrc> &src, SourceSide &source_side,
-               Walks &walks, cudaStream_t st, int *shape) {
-  int rc = source_side(st);
-  if (rc) return rc;
-  int32_t pick = -1;
-  for (size_t b = 0; b < src.size() && pick < 0; ++b) {
-    int32_t pairs = 0;
-    cudaError_t e = cudaMemcpyAsync(&pairs, small_view(src[b].w.small).cnt + 1, sizeof pairs,
-                                    cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "batched query: reading the pair counts");
-    if (pairs > 0) pick = (int32_t)b;
-  }
-  if (pick < 0) return SRK_OK;
-  cudaEvent_t ev[2] = {nullptr, nullptr};
-  cudaError_t e = cudaEventCreate(&ev[0]);
-  if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
-  if (e != cudaSuccess) rc = cuda_fail(e, "batched query: creating the autotuner's events");
-  double best = 0.0;
-  for (int sh = 0; sh < kWalkShapes && rc == SRK_OK; ++sh) {
-    if (sh > 0) rc = source_side(st);
-    const int32_t units = sm_count(g->device) * 2;  // about one round of the grid
-    if (rc == SRK_OK) rc = walks(pick, st, ev, sh, units);
-    int32_t cnt[3] = {0, 0, 0};
-    float ms = 0.f;
-    if (rc == SRK_OK) {
-      e = cudaMemcpyAsync(cnt, small_view(src[(size_t)pick].w.small).cnt, sizeof cnt,
-                          cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-      if (e != cudaSuccess) rc = cuda_fail(e, "batched query: autotuner");
-    }
-    const double rate = walk_units_work(g, sh, cnt[2] > 0 ? cnt[2] : cnt[1], units) / std::max(1e-6f, ms);
-    if (rc == SRK_OK && rate > best) {
-      best = rate;
-      *shape = sh;
-    }
-  }
-  if (ev[0]) cudaEventDestroy(ev[0]);
-  if (ev[1]) cudaEventDestroy(ev[1]);
-  return rc;
-}
-
-}  // namespace
-
 extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
                                 int32_t k, double c, const double *eps,
                                 uint64_t seed, const srk_opts *opt,
@@ -344,7 +289,8 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     // sources [i0, i1) form this batch
     size_t need = 0;
     int32_t i1 = i0;
-    std::vector<size_t> ws_off;
+    std::vector<size_t> ws_off, ends;  // sources' places; bytes of their end filters,
+    size_t most = 0;                   //   and the most of them
     int64_t sh_L = 1, sh_N = 0;  // shared walks: the tables' extent so far
     std::vector<int32_t> pmin((size_t)SRK_MAX_LEN + 2, INT32_MAX);
     while (i1 < k && !(shared && i1 - i0 >= 64)) {
@@ -367,7 +313,10 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       const size_t b = align256(plan(t1, &w, nullptr)) +
                        (d_scores ? 0 : align256(8 * n)) + (d_counts ? 0 : align256(4 * n)) +
                        (shared ? align256(8 * (size_t)t1.N_tot) : 0);
-      if (i1 > i0 && need + b + sb > budget) break;
+      const size_t f = shared ? 0 : align256(filter_bytes(g, t1, g->n));
+      if (i1 > i0 && need + b + sb + std::max(most, f) > budget) break;
+      most = std::max(most, f);
+      ends.push_back(f);
       sh_L = L1;
       sh_N = N1;
       if (shared)
@@ -407,18 +356,33 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     const size_t head = align256(sizeof(BatchSrc) * kb) + align256(sizeof(QueryTab) * kb) +
                         align256(sizeof(int64_t) * (kb + 1)) + 256 + align256(m_bytes) +
                         align256(r_bytes) + align256(g_bytes) + align256(h_bytes) +
-                        align256(c_bytes) + align256(sizeof(SourceJob) * (size_t)kb);
-    // end filters: one region, which the sources use one after the other
-    size_t extra = 0;
-    for (int32_t b = i0; b < i1 && !shared; ++b)
-      extra = std::max(extra, filter_bytes(g, tabs[(size_t)b], g->n));
+                        align256(c_bytes) + align256(sizeof(SourceJob) * (size_t)kb) +
+                        align256(sizeof(WalkJob) * (size_t)kb) + align256(4 * (size_t)kb);
+    // End filters: one region, which groups of sources use one after the other,
+    // in what the scratch budget leaves.
+    size_t room = 0;
+    for (size_t f : ends) room += f;
+    room = std::min(room, budget > need ? (budget - need) & ~(size_t)255 : 0);
     char *base = nullptr;
-    cudaError_t e = cudaMallocFromPoolAsync((void **)&base, head + need + extra, mp, st);
-    if (e == cudaErrorMemoryAllocation && extra > 0) {  // the walks can do without
+    cudaError_t e = cudaMallocFromPoolAsync((void **)&base, head + need + room, mp, st);
+    if (e == cudaErrorMemoryAllocation && room > 0) {  // the walks can do without
       cudaGetLastError();
-      extra = 0;
+      room = 0;
       e = cudaMallocFromPoolAsync((void **)&base, head + need, mp, st);
     }
+    // groups: [groups[q], groups[q + 1]), as many sources as the region holds
+    std::vector<int32_t> groups(1, 0);
+    size_t held = 0;
+    for (int32_t b = 0; b < kb && !shared; ++b) {
+      if (b > groups.back() &&
+          (b - groups.back() >= kWalkGroup || held + ends[(size_t)b] > room)) {
+        groups.push_back(b);
+        held = 0;
+      }
+      held += ends[(size_t)b];
+    }
+    groups.push_back(kb);
+    const int32_t n_groups = (int32_t)groups.size() - 1;
     if (e != cudaSuccess) { rc = cuda_fail(e, "batch workspace allocation"); break; }
     BatchSrc *d_src = (BatchSrc *)base;
     QueryTab *d_tab = (QueryTab *)(base + align256(sizeof(BatchSrc) * kb));
@@ -431,6 +395,8 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     uint4 *d_T = (uint4 *)((char *)d_sig + align256(g_bytes));
     SharedSrc *d_ssrc = (SharedSrc *)((char *)d_T + align256(h_bytes));
     SourceJob *d_jobs = (SourceJob *)((char *)d_ssrc + align256(c_bytes));
+    WalkJob *d_walks = (WalkJob *)((char *)d_jobs + align256(sizeof(SourceJob) * (size_t)kb));
+    int32_t *d_units = (int32_t *)((char *)d_walks + align256(sizeof(WalkJob) * (size_t)kb));
     // shared walks: d_ctr[0] = target counter, d_ctr[1] = steps
     char *ws_base = base + head;
     std::vector<BatchSrc> hsrc((size_t)kb);
@@ -463,6 +429,19 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     std::vector<SourceJob> jobs;
     for (int32_t b = 0; b < kb; ++b)
       jobs.push_back(SourceJob{hsrc[(size_t)b].w, hsrc[(size_t)b].tab});
+    std::vector<WalkJob> walks;
+    for (int32_t q = 0; q < n_groups && !shared; ++q) {
+      size_t at = 0;
+      for (int32_t b = groups[(size_t)q]; b < groups[(size_t)q + 1]; ++b) {
+        const BatchSrc &S = hsrc[(size_t)b];
+        const QueryTab &t = tabs[(size_t)(i0 + b)];
+        Filters F;
+        const size_t f = std::min(ends[(size_t)b], room - at);
+        plan_filters(g, t, S.w, g->n, f, &F, ws_base + need + at);
+        at += f;
+        walks.push_back(walk_job(g, t, S.w, F, Outputs{S.scores, S.counts, nullptr, nullptr}));
+      }
+    }
     std::vector<SharedSrc> ssrc;
     for (int32_t b = 0; shared && b < kb; ++b) {
       const BatchSrc &S = hsrc[(size_t)b];
@@ -474,6 +453,8 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(SourceJob) * kb, cudaMemcpyHostToDevice,
                              st)) != cudaSuccess ||
+        (!shared && (e = cudaMemcpyAsync(d_walks, walks.data(), sizeof(WalkJob) * kb,
+                                         cudaMemcpyHostToDevice, st)) != cudaSuccess) ||
         (e = cudaMemcpyAsync(d_src, hsrc.data(), sizeof(BatchSrc) * kb,
                              cudaMemcpyHostToDevice, st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(d_off, hoff.data(), sizeof(int64_t) * (kb + 1),
@@ -505,7 +486,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     const int gw = (int)std::max<int64_t>(1, std::min<int64_t>((A.total_walks + 255) / 256,
                                                                 (int64_t)sms * 8));
     auto enqueue_source_side = [&](cudaStream_t s2) {
-      int r = enqueue_sources(g, d_jobs, kb, shared, s2);
+      int r = enqueue_sources(g, d_jobs, kb, Jmax, shared, s2);
       if (shared) {
         cudaMemsetAsync(d_ctr, 0, 256, s2);
         cudaMemsetAsync(d_M, 0, m_bytes, s2);
@@ -537,43 +518,23 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       SW.steps = count ? d_ctr + 1 : nullptr;
       SW.counter = reinterpret_cast<int32_t *>(d_ctr);
     }
-    auto enqueue_source = [&](int32_t b, cudaStream_t s2, const cudaEvent_t *timing, int shape,
-                              int32_t max_units) {
-      const BatchSrc &S = hsrc[(size_t)b];
-      const QueryTab &t = tabs[(size_t)(i0 + b)];
-      const Outputs o{S.scores, S.counts, nullptr, nullptr};
-      Filters F;
-      plan_filters(g, t, S.w, g->n, extra, &F, ws_base + need);
-      int r = enqueue_ends(g, S.w, F, s2);
-      if (r == SRK_OK)
-        r = enqueue_walks(g, t, S.w, F, o, count, s2, timing, 0, (int32_t)n, shape, max_units);
-      return r;
-    };
-    // autotune the walk kernel's launch shape on the first batch with pairs
-    int shape = g->batch_cfg;
-    if (!shared && shape < 0) {
-      rc = tune_shape(g, hsrc, enqueue_source_side, enqueue_source, st, &shape);
-      if (rc) {
-        cudaFreeAsync(base, st);
-        break;
-      }
-      if (shape >= 0) const_cast<srk_graph *>(g)->batch_cfg = shape;
-    }
     auto enqueue_all = [&](cudaStream_t s2) {
       int r = enqueue_source_side(s2);
       if (r) return r;
-      if (shared)
-        r = enqueue_shared_walks(g, SW, s2);
-      else
-        for (int32_t b = 0; b < kb && r == SRK_OK; ++b)
-          r = enqueue_source(b, s2, nullptr, shape, INT32_MAX);
+      if (shared) return enqueue_shared_walks(g, SW, s2);
+      cudaMemsetAsync(d_units, 0, 4 * (size_t)n_groups, s2);
+      for (int32_t q = 0; q < n_groups && r == SRK_OK; ++q) {
+        const int32_t b = groups[(size_t)q];
+        r = enqueue_walk_group(g, walks.data() + b, d_walks + b, groups[(size_t)q + 1] - b, Jmax,
+                               d_units + q, count, s2);
+      }
       return r;
     };
     if (use_graph) {
       // The batch is captured every time (its buffers move), but the graph's
       // executable is kept in the handle and only updated with the new
-      // parameters while the launch sequence keeps its shape (same kernels,
-      // same order); otherwise it is instantiated anew.
+      // parameters for a batch of as many sources while the launch sequence keeps
+      // its shape (same kernels, same order); otherwise it is instantiated anew.
       std::lock_guard<std::mutex> lk(capture_mutex(dev));
       srk_graph *gm = const_cast<srk_graph *>(g);
       cudaGraph_t graph = nullptr;
@@ -587,7 +548,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       }
       if (e == cudaSuccess && gm->batch_exec) {
         cudaGraphExecUpdateResultInfo info;
-        if (cudaGraphExecUpdate(gm->batch_exec, graph, &info) != cudaSuccess) {
+        if (gm->batch_k != kb || cudaGraphExecUpdate(gm->batch_exec, graph, &info) != cudaSuccess) {
           cudaGetLastError();  // a different shape: instantiate below
           cudaGraphExecDestroy(gm->batch_exec);
           gm->batch_exec = nullptr;
@@ -596,6 +557,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         }
       }
       if (e == cudaSuccess && !gm->batch_exec) e = cudaGraphInstantiate(&gm->batch_exec, graph, 0);
+      gm->batch_k = kb;
       if (e == cudaSuccess) e = cudaGraphLaunch(gm->batch_exec, cs);
       if (e == cudaSuccess) e = cudaEventRecord(ev_out, cs);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev_out, 0);
@@ -653,7 +615,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = cuda_fail(e, "srk_multi_source");
   }
-  total.batch_shape = g->batch_cfg;
+  total.batch_shape = shared ? -1 : walk_shape(g, g->n_act);
   if (rc == SRK_OK && opt && opt->stats) *opt->stats = total;
   return rc;
 }

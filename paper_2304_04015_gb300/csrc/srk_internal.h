@@ -44,12 +44,10 @@ struct srk_graph {
   int32_t *act = nullptr;
   int32_t n_act = 0;
   int32_t *out_deg = nullptr;  // out-degrees by id, n (in act's block)
-  // Launch shape of the batched target kernel chosen by the autotuner
-  // (-1: not tuned yet).
-  int batch_cfg = -1;
   // Executable of the last captured batch (srk_multi_source with a CUDA
-  // graph), updated in place for the next batch of the same shape.
+  // graph), of batch_k sources, updated in place for the next batch of as many.
   cudaGraphExec_t batch_exec = nullptr;
+  int32_t batch_k = 0;
   // Topology of the linearised form (edge owners, a transpose, list size
   // classes), built by the first srk_linear_fwd on the graph.
   struct srk_lin_topo *lin = nullptr;
@@ -206,16 +204,18 @@ size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, i
 // The source side of queries (srk_source.cu).  enqueue_source: one query, steps
 // a2-a3 to the pair records (the cap rows only with the literal shuffle) and
 // the end nodes of F.  enqueue_sources: of k queries, to the pair records or,
-// with `shared`, to sigma.  enqueue_ends: the end nodes of one of them.
+// with `shared`, to sigma.  enqueue_ends: the end nodes of k of them.  N: the most
+// walks that one of the k has.
 struct SourceJob {
   Workspace w;
   const QueryTab *tab;  // device
 };
 int enqueue_source(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
                    int32_t u_begin, int32_t u_end, cudaStream_t st);
-int enqueue_sources(const srk_graph *g, const SourceJob *jobs, int32_t k, bool shared,
+int enqueue_sources(const srk_graph *g, const SourceJob *jobs, int32_t k, int32_t N, bool shared,
                     cudaStream_t st);
-int enqueue_ends(const srk_graph *g, const Workspace &w, const Filters &F, cudaStream_t st);
+struct WalkJob;
+int enqueue_ends(const srk_graph *g, const WalkJob *jobs, int32_t k, int32_t N, cudaStream_t st);
 
 // Carves `base` (or only sizes the plan when base is null); returns the
 // number of bytes one query of table `t` needs.
@@ -233,17 +233,46 @@ int single_source(const srk_graph *g, int32_t s, double c, double eps, uint64_t 
 // Bytes of `extra` scratch a query of n_targets targets makes use of (it does
 // with less, or none: its end nodes then have fewer filters, or none).
 size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets);
+// What the target walks of a query need (srk_lockstep.cu).
+struct LockQuery {
+  const int4 *rec;              // per pair {j, cap, first node in H, filter}
+  const unsigned long long *w;  // per pair: its quantised weight
+  const int32_t *H;             // nodes of the pairs' source walks, steps 1..cap
+  const uint32_t *bits;         // the filters
+  const int32_t *cnt;           // cnt[i]: pairs with cap >= i (longest first)
+  unsigned long long *W;        // per target: weight sum
+  uint32_t *counts;             // per target: meetings, or null
+  uint32_t *steps;              // per target: steps, or null
+  unsigned long long *steps_total;
+  uint32_t key;                 // walk key of the target walks
+  uint32_t rk[10];              //   and its round keys
+  int32_t s;
+  int32_t min_cap;              // pairs below this cap are not walked here
+  int32_t polls;                // of a wait for filters before it gives up
+};
 // Steps a4-a5 after the source side (the pair records of w and the end nodes
 // of F are made, the outputs of the range cleared): srk_lockstep.cu.
 int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
                   const Outputs &o, bool count, cudaStream_t st,
-                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end, int shape = -1,
-                  int32_t max_units = INT32_MAX);
-// Launch shapes of the walks: 0 and up, -1 for the default of the target count.
-// max_units bounds the units of work walked (the autotuner's trials), and
-// walk_units_work is the targets x pairs of that many units over all targets.
-constexpr int kWalkShapes = 2;
-double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t max_units);
+                  const cudaEvent_t *timing, int32_t u_begin, int32_t u_end);
+// The same, and the end nodes before it, for a group of queries over all targets
+// (at most kWalkGroup, their pair records made and their rows prefilled): `jobs` on
+// the device, `host` their copy, N the most walks of one of them, `counter` a device
+// word that is zero.
+struct WalkJob {
+  Workspace w;
+  Filters F;
+  LockQuery Q;
+  double z;
+  int32_t alone;  // its targets are walked by a launch of their own
+};
+constexpr int32_t kWalkGroup = 256;
+WalkJob walk_job(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
+                 const Outputs &o);
+int enqueue_walk_group(const srk_graph *g, const WalkJob *host, const WalkJob *jobs, int32_t k,
+                       int32_t N, int32_t *counter, bool count, cudaStream_t st);
+// Launch shape of the walks of n_targets targets: 0, several a thread, or 1, one.
+int walk_shape(const srk_graph *g, int64_t n_targets);
 // Shared target walks of up to 64 sources (srk_batch.cu makes the tables).
 struct SharedSrc {
   const unsigned long long *wj;  // quantised Lemma 7 weight of pair j

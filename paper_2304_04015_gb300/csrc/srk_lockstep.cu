@@ -53,24 +53,14 @@
 
 namespace srk {
 
-// What the lockstep kernel needs of one query.
-struct LockQuery {
-  const int4 *rec;              // per pair {j, cap, first node in H, filter}
-  const unsigned long long *w;  // per pair: its quantised weight
-  const int32_t *H;             // nodes of the pairs' source walks, steps 1..cap
-  const uint32_t *bits;         // the filters
-  const int32_t *cnt;           // cnt[i]: pairs with cap >= i (longest first)
-  unsigned long long *W;        // per target: weight sum
-  uint32_t *counts;             // per target: meetings, or null
-  uint32_t *steps;              // per target: steps, or null
-  unsigned long long *steps_total;
-  uint32_t key;                 // walk key of the target walks
-  uint32_t rk[10];              //   and its round keys
-  int32_t s;
-  int32_t min_cap;              // pairs below this cap are not walked here
-  int32_t max_units;            // units beyond these are not walked
-  int32_t polls;                // of a wait for filters before it gives up
-};
+// A query of a group, which a block holds in shared memory: its round keys are
+// made as they are needed (kernel parameters have them as constant operands).
+struct GroupQuery : LockQuery {};
+__device__ __forceinline__ uint32_t round_key(const GroupQuery &Q, int r) {
+  return Q.key + (uint32_t)r * kPhiloxW0;
+}
+template <class QT>
+__device__ __forceinline__ uint32_t round_key(const QT &Q, int r) { return Q.rk[r]; }
 
 // -------------------------------------------------- asynchronous copies --
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
@@ -157,16 +147,17 @@ __device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &hi, u
       : "=r"(hi), "=r"(lo) : "r"(a), "r"(b));
 }
 
-// philox2 with the round keys given (kernel parameters: constant operands).
-__device__ __forceinline__ void philox2k(const uint32_t (&rk)[10], uint32_t c0, uint32_t c1,
-                                         uint32_t &x0, uint32_t &x1) {
+// philox2 with the round keys of a query.
+template <class QT>
+__device__ __forceinline__ void philox2k(const QT &Q, uint32_t c0, uint32_t c1, uint32_t &x0,
+                                         uint32_t &x1) {
   x0 = c0;
   x1 = c1;
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
     uint32_t hi, lo;
     mul_wide(kPhilox2M, x0, hi, lo);
-    x0 = hi ^ x1 ^ rk[r];
+    x0 = hi ^ x1 ^ round_key(Q, r);
     x1 = lo;
   }
 }
@@ -304,9 +295,9 @@ struct LockQueue {
   uint32_t below;  // the mask of the lower lanes
 };
 
-template <int kT, class GA>
-__device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, const LockQuery &Q, LockQueue &B, int take,
-                                           const int32_t (&u)[kT]) {
+template <int kT, class GA, class QT>
+__device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, const QT &Q,
+                                           LockQueue &B, int take, const int32_t (&u)[kT]) {
   __syncwarp();
   const int lane = threadIdx.x & 31;
   B.n -= take;
@@ -328,7 +319,7 @@ __device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, con
     const auto e = word_entry(G, it.x);
     b = lock_next(G, T, true, e, entry_pos(G, e), deg[0]);
   }
-  philox2k(Q.rk, walk_ctr0(i, j), (uint32_t)v, x0[0], x1[0]);
+  philox2k(Q, walk_ctr0(i, j), (uint32_t)v, x0[0], x1[0]);
   if (!(i & 1)) x0[0] = x1[0];
   lock_index(x0, deg, Q.key, i, j, vv, idx);
   if (deg[0]) {
@@ -343,9 +334,9 @@ __device__ __forceinline__ void lock_drain(const GA &G, const LockTables &T, con
 
 // One pair (index j, nodes h at steps 1..cap, step 1..32 in the lanes' h32)
 // for the thread's targets; kCap = cap, or 0 for any up to 32, or -1 for any.
-template <int kCap, int kT, bool kCount, class GA, class E>
-__device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, const LockQuery &Q, const LockFilter &F,
-                                          uint32_t lists, int32_t a, uint32_t j, int cap_,
+template <int kCap, int kT, bool kCount, class GA, class E, class QT>
+__device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, const QT &Q,
+                                          const LockFilter &F, uint32_t lists, int32_t a, uint32_t j, int cap_,
                                           int32_t h32, const int32_t *__restrict__ h,
                                           LockTargets<kT> &X, LockQueue &B) {
   const int cap = kCap > 0 ? kCap : cap_;
@@ -355,7 +346,7 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
   E e[kT];
 #pragma unroll
   for (int t = 0; t < kT; ++t) {
-    philox2k(Q.rk, j, (uint32_t)X.u[t], x0[t], x1[t]);
+    philox2k(Q, j, (uint32_t)X.u[t], x0[t], x1[t]);
     deg[t] = X.d[t];
   }
   lock_index(x0, deg, Q.key, 1, j, X.u, idx);
@@ -441,7 +432,7 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
     if (!(i & 1)) {
 #pragma unroll
       for (int t = 0; t < kT; ++t)
-        philox2k(Q.rk, walk_ctr0(i + 1, j), (uint32_t)X.u[t], x0[t], x1[t]);
+        philox2k(Q, walk_ctr0(i + 1, j), (uint32_t)X.u[t], x0[t], x1[t]);
       lock_index(x0, deg, Q.key, i + 1, j, X.u, idx);
     } else {
       lock_index(x1, deg, Q.key, i + 1, j, X.u, idx);
@@ -460,9 +451,9 @@ __device__ __forceinline__ void lock_pair(const GA &G, const LockTables &T, cons
 // other as each comes to a wait; none frees a stage from then on, so warp 0 forms
 // no group into a stage in use, waits for those that it has formed before it
 // leaves, and no later unit forms any.
-template <int kT, bool kCount, class GA, class E>
-__device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T,
-                                               const LockQuery &Q, LockShared &S,
+template <int kT, bool kCount, class GA, class E, class QT>
+__device__ __forceinline__ void lockstep_walks(const GA &G, const LockTables &T, const QT &Q,
+                                               LockShared &S,
                                                uint32_t *ring, uint4 *queues, const E *lists,
                                                int32_t first, int32_t stride, int32_t len,
                                                bool staged, uint32_t &seq, LockTargets<kT> &X) {
@@ -584,11 +575,13 @@ __device__ __forceinline__ void last_steps(const Filters &F, const int4 *__restr
   }
 }
 
-__global__ void __launch_bounds__(256)
-k_edges(Filters F, GraphView V, int64_t m, const int32_t *__restrict__ cnt,
-        const int4 *__restrict__ rec, const unsigned long long *__restrict__ pair_w, uint32_t key,
-        int32_t s, int32_t u_begin, int32_t u_end, unsigned long long *__restrict__ W,
-        uint32_t *__restrict__ counts) {
+__device__ __forceinline__ void walk_edges(const Filters &F, const GraphView &V, int64_t m,
+                                           const int32_t *__restrict__ cnt,
+                                           const int4 *__restrict__ rec,
+                                           const unsigned long long *__restrict__ pair_w,
+                                           uint32_t key, int32_t s, int32_t u_begin, int32_t u_end,
+                                           unsigned long long *__restrict__ W,
+                                           uint32_t *__restrict__ counts) {
   if (cnt[1] == 0) return;  // no pair can meet
   const int lane = threadIdx.x & 31;
   const int32_t *__restrict__ row_ptr = V.row_ptr;
@@ -684,6 +677,22 @@ k_edges(Filters F, GraphView V, int64_t m, const int32_t *__restrict__ cnt,
       }
     }
   }
+}
+
+__global__ void __launch_bounds__(256)
+k_edges(const __grid_constant__ Filters F, const __grid_constant__ GraphView V, int64_t m,
+        const int32_t *cnt, const int4 *rec, const unsigned long long *pair_w, uint32_t key,
+        int32_t s, int32_t u_begin, int32_t u_end, unsigned long long *W, uint32_t *counts) {
+  walk_edges(F, V, m, cnt, rec, pair_w, key, s, u_begin, u_end, W, counts);
+}
+
+// For a group of queries (blockIdx.y: the query).
+__global__ void __launch_bounds__(256)
+k_edges_group(const __grid_constant__ GraphView V, int64_t m, const WalkJob *__restrict__ jobs) {
+  const WalkJob &J = jobs[blockIdx.y];
+  const Filters F = J.F;
+  if (F.slots)
+    walk_edges(F, V, m, J.Q.cnt, J.Q.rec, J.Q.w, J.Q.key, J.Q.s, 0, V.n, J.Q.W, J.Q.counts);
 }
 
 // Into how many strided sets the pairs are cut, so that sets x target blocks
@@ -784,6 +793,48 @@ __device__ __forceinline__ void lock_targets(const GA &G, const int32_t *__restr
   }
 }
 
+// A block's dynamic shared memory, its tables filled and its barriers made (to be
+// followed by a __syncthreads); the lists of E begin at the returned ring's end.
+template <int kLayout>
+__device__ __forceinline__ uint32_t *lock_setup(const GraphView &V, unsigned char *dyn,
+                                                LockShared &S, LockTables &tabs, uint4 *&queues) {
+  uint32_t *ring = reinterpret_cast<uint32_t *>(dyn);
+  queues = reinterpret_cast<uint4 *>(ring + kStages * kStageWords + kListWords);
+  uint2 *hub = reinterpret_cast<uint2 *>(queues + kQueue * kLockWarps);
+  uint32_t *ctab = reinterpret_cast<uint32_t *>(hub + kHubCache);
+  tabs = LockTables{smem_addr(ctab), smem_addr(hub), 0u};
+  if (threadIdx.x < kStages) {
+    mbar_init(&S.full[threadIdx.x], 1);
+    mbar_init(&S.empty[threadIdx.x], kLockWarps);
+  }
+  if (threadIdx.x == 0) S.broken = 0;
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if constexpr (kLayout == kNarrow) {
+    tabs.n_hub = (uint32_t)min(V.n_hubs, kHubCache);
+    for (uint32_t i = threadIdx.x; i < tabs.n_hub; i += kLockThreads) hub[i] = V.hub[i];
+    for (uint32_t i = threadIdx.x; i <= V.deg_max; i += kLockThreads) ctab[i] = V.ctab[i];
+  }
+  return ring;
+}
+
+// The steps of a unit's targets, to their totals and the thread's.
+template <int kT>
+__device__ __forceinline__ void add_steps(const LockTargets<kT> &X, uint32_t *steps,
+                                          unsigned long long &total) {
+#pragma unroll
+  for (int t = 0; t < kT; ++t)
+    if (X.st[t]) {
+      if (steps) atomicAdd(&steps[X.u[t]], X.st[t]);
+      total += X.st[t];
+    }
+}
+// A thread's total of steps, summed over its warp, to *steps_total.
+__device__ __forceinline__ void add_total(unsigned long long total,
+                                          unsigned long long *steps_total) {
+  for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+  if ((threadIdx.x & 31) == 0 && total) atomicAdd(steps_total, total);
+}
+
 // The walks.  A unit of work is a block of targets and a strided set of
 // pairs; blocks take units from a counter.  A unit's targets keep their lists
 // in shared memory where they fit, for their first steps.  W[u] (in the scores
@@ -796,31 +847,17 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   __shared__ LockShared S;
   const auto G = adj_view<kLayout>(V);
   using E = decltype(adj_entry(G, 0, 0u));
-  uint32_t *ring = reinterpret_cast<uint32_t *>(dyn);
-  E *lists = reinterpret_cast<E *>(ring + kStages * kStageWords);
-  uint4 *queues = reinterpret_cast<uint4 *>(ring + kStages * kStageWords + kListWords);
-  uint2 *hub = reinterpret_cast<uint2 *>(queues + kQueue * kLockWarps);
-  uint32_t *ctab = reinterpret_cast<uint32_t *>(hub + kHubCache);
-  LockTables tabs{smem_addr(ctab), smem_addr(hub), 0u};
   const int32_t act_lo = bounds[2], act_hi = bounds[1];
   const int32_t n_pairs = Q.cnt[Q.min_cap], n_t = act_hi - act_lo;
   if (n_pairs == 0 || n_t <= 0) return;
   const int32_t T = kLockThreads * kT, n_tb = (n_t + T - 1) / T;
   const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
-  const int64_t units = min((int64_t)n_tb * n_chunks, (int64_t)Q.max_units);
+  const int64_t units = (int64_t)n_tb * n_chunks;
   if ((int64_t)blockIdx.x >= units) return;
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x < kStages) {
-    mbar_init(&S.full[threadIdx.x], 1);
-    mbar_init(&S.empty[threadIdx.x], kLockWarps);
-  }
-  if (threadIdx.x == 0) S.broken = 0;
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  if constexpr (kLayout == kNarrow) {
-    tabs.n_hub = (uint32_t)min(V.n_hubs, kHubCache);
-    for (uint32_t i = threadIdx.x; i < tabs.n_hub; i += kLockThreads) hub[i] = V.hub[i];
-    for (uint32_t i = threadIdx.x; i <= V.deg_max; i += kLockThreads) ctab[i] = V.ctab[i];
-  }
+  LockTables tabs;
+  uint4 *queues;
+  uint32_t *ring = lock_setup<kLayout>(V, dyn, S, tabs, queues);
+  E *lists = reinterpret_cast<E *>(ring + kStages * kStageWords);
   unsigned long long total = 0;
   uint32_t seq = 0;
   for (;;) {
@@ -837,17 +874,103 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
     lock_targets(G, V.row_ptr, S, lists, act, act_lo + tb * T, act_hi, Q.s, len >= 32, X);
     lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len,
                                staged, seq, X);
-#pragma unroll
-    for (int t = 0; t < kT; ++t) {
-      if (kCount && X.st[t]) {
-        if (Q.steps) atomicAdd(&Q.steps[X.u[t]], X.st[t]);
-        total += X.st[t];
-      }
+    if (kCount) add_steps(X, Q.steps, total);
+  }
+  if (kCount) add_total(total, Q.steps_total);
+}
+
+// The walks of a group of queries, all targets: the units of all of them that are
+// not `alone`, one query's after the other's, from one counter.  Queries that are
+// small by themselves fill the GPU together: a batch of 64 of eps = 0.05 on 2,000
+// nodes with 8 in-neighbours each took 3.54 ms with launches of their own and 1.34
+// ms with a warp per target and query, now 1.05 ms.  A query's unit is a block of
+// targets and so many pairs that the group has kGroupRounds units a block; less
+// work goes in one round of units of up to kGroupRound pairs.  (A batch of 8
+// queries on 900 nodes, eps = 0.1: 0.190 ms with units of 4 pairs and more, 0.219 of
+// 16; 8, 16 or 32 rounds differ by less than 2 %.)
+constexpr int kGroupRounds = 16, kGroupRound = 64, kGroupPairs = 4;
+template <int kLayout, bool kCount, int kT>
+__global__ void __launch_bounds__(kLockThreads, kLockBlocks)
+k_lockstep_group(const __grid_constant__ GraphView V, const int32_t *__restrict__ act, int32_t n_t,
+                 const WalkJob *__restrict__ jobs, int32_t k, int32_t *__restrict__ counter) {
+  extern __shared__ __align__(128) unsigned char dyn[];
+  __shared__ LockShared S;
+  __shared__ GroupQuery Q;
+  __shared__ int32_t chunks[kWalkGroup];    // strided sets of pairs by query,
+  __shared__ int32_t end[kWalkGroup];       //   and where its units end
+  __shared__ int32_t job;
+  __shared__ unsigned long long all_pairs;
+  static_assert(kWalkGroup <= kLockThreads && kWalkGroup % 32 == 0, "a thread per query");
+  const auto G = adj_view<kLayout>(V);
+  using E = decltype(adj_entry(G, 0, 0u));
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int32_t T = kLockThreads * kT, n_tb = (n_t + T - 1) / T;
+  int32_t pairs = 0;
+  if ((int32_t)threadIdx.x < k && !jobs[threadIdx.x].alone)
+    pairs = jobs[threadIdx.x].Q.cnt[jobs[threadIdx.x].Q.min_cap];
+  if (threadIdx.x == 0) all_pairs = 0;
+  __syncthreads();
+  if (pairs > 0) atomicAdd(&all_pairs, (unsigned long long)pairs);
+  __syncthreads();
+  if (all_pairs == 0 || n_t <= 0) return;
+  {
+    const unsigned long long per_block = all_pairs * (unsigned)n_tb / gridDim.x;
+    const unsigned long long want = max(per_block / kGroupRounds,
+                                        min(per_block, (unsigned long long)kGroupRound));
+    const int32_t unit = (int32_t)max(min(want, (unsigned long long)SRK_MAX_WALKS),
+                                      (unsigned long long)kGroupPairs);
+    const int32_t ch = (pairs + unit - 1) / unit;
+    int32_t incl = ch * n_tb;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) S.warp_sum[wid] = (uint32_t)incl;
+    __syncthreads();
+    for (int w = 0; w < wid; ++w) incl += (int32_t)S.warp_sum[w];
+    if (threadIdx.x < kWalkGroup) {
+      chunks[threadIdx.x] = ch;
+      end[threadIdx.x] = incl;
     }
   }
-  if (kCount) {
-    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    if (lane == 0 && total) atomicAdd(Q.steps_total, total);
+  LockTables tabs;
+  uint4 *queues;
+  uint32_t *ring = lock_setup<kLayout>(V, dyn, S, tabs, queues);
+  E *lists = reinterpret_cast<E *>(ring + kStages * kStageWords);
+  uint32_t seq = 0;
+  for (;;) {
+    __syncthreads();
+    const bool whole = *(volatile int32_t *)&S.broken == 0;
+    if (threadIdx.x == 0) {
+      const int32_t unit = atomicAdd(counter, 1);
+      int32_t lo = 0, hi = k;  // the first query whose units end past this one
+      while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (end[mid] <= unit) lo = mid + 1;
+        else hi = mid;
+      }
+      job = lo;
+      S.unit = unit - (lo < k ? end[lo] - chunks[lo] * n_tb : 0);
+    }
+    if (threadIdx.x < 4) S.sums[threadIdx.x] = 0;
+    __syncthreads();
+    if (job >= k) break;
+    for (int i = threadIdx.x; i < (int)(sizeof(LockQuery) / 8); i += kLockThreads)
+      reinterpret_cast<uint64_t *>(&Q)[i] = reinterpret_cast<const uint64_t *>(&jobs[job].Q)[i];
+    __syncthreads();
+    const int32_t n_chunks = chunks[job], tb = S.unit % n_tb, first = S.unit / n_tb;
+    const int32_t n_pairs = Q.cnt[Q.min_cap], len = (n_pairs - first + n_chunks - 1) / n_chunks;
+    const bool staged = whole && Q.min_cap == 2;
+    LockTargets<kT> X;
+    lock_targets(G, V.row_ptr, S, lists, act, tb * T, n_t, Q.s, len >= 32, X);
+    uint32_t none = 0;  // (groups are numbered by the units that form some)
+    lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len,
+                               staged, staged ? seq : none, X);
+    if (kCount) {
+      unsigned long long total = 0;
+      add_steps(X, nullptr, total);
+      add_total(total, Q.steps_total);
+    }
   }
 }
 
@@ -870,12 +993,15 @@ __device__ __forceinline__ void finish_tile(double *__restrict__ row, int64_t u0
   __syncthreads();
 }
 
-// Scores of a query, and the steps of the pairs that k_edges decided.
-__global__ void __launch_bounds__(256)
-k_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ bounds,
-         const int32_t *__restrict__ cnt, int32_t s, int32_t u_begin, int32_t u_end, double z,
-         int32_t skipped, double *__restrict__ scores, unsigned long long *__restrict__ wsums,
-         uint32_t *__restrict__ steps, unsigned long long *__restrict__ steps_total) {
+// Scores of a query, and the steps of the pairs that k_edges decided for the
+// n_t targets with in-neighbours of the range.
+__device__ __forceinline__ void finish_query(const int32_t *__restrict__ row_ptr, int32_t n_t,
+                                             const int32_t *__restrict__ cnt, int32_t s,
+                                             int32_t u_begin, int32_t u_end, double z,
+                                             bool skipped, double *__restrict__ scores,
+                                             unsigned long long *__restrict__ wsums,
+                                             uint32_t *__restrict__ steps,
+                                             unsigned long long *__restrict__ steps_total) {
   __shared__ uint16_t list[kFinishTile];
   __shared__ int32_t n_list;
   // pairs of cap 1 decided per edge: one step each of every target
@@ -894,10 +1020,26 @@ k_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ bounds
     if (threadIdx.x == 0 && s >= u0 && s < u1) scores[s] = 1.0;
   }
   if (one && blockIdx.x == 0 && threadIdx.x == 0) {
-    int64_t t = bounds[1] - bounds[2];
+    int64_t t = n_t;
     if (s >= u_begin && s < u_end && row_ptr[s + 1] > row_ptr[s]) --t;
     atomicAdd(steps_total, (unsigned long long)t * one);
   }
+}
+
+__global__ void __launch_bounds__(256)
+k_finish(const int32_t *row_ptr, const int32_t *bounds, const int32_t *cnt, int32_t s,
+         int32_t u_begin, int32_t u_end, double z, int32_t skipped, double *scores,
+         unsigned long long *wsums, uint32_t *steps, unsigned long long *steps_total) {
+  finish_query(row_ptr, bounds[1] - bounds[2], cnt, s, u_begin, u_end, z, skipped != 0, scores,
+               wsums, steps, steps_total);
+}
+
+// For a group of queries (blockIdx.y: the query).
+__global__ void __launch_bounds__(256)
+k_finish_group(const int32_t *row_ptr, int32_t n, int32_t n_t, const WalkJob *__restrict__ jobs) {
+  const WalkJob &J = jobs[blockIdx.y];
+  finish_query(row_ptr, n_t, J.Q.cnt, J.Q.s, 0, n, J.z, J.F.slots != nullptr,
+               reinterpret_cast<double *>(J.Q.W), nullptr, nullptr, J.Q.steps_total);
 }
 
 // ---------------------------------------------------- shared target walks --
@@ -990,7 +1132,7 @@ k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ a
       E e[kT];
 #pragma unroll
       for (int t = 0; t < kT; ++t) {
-        philox2k(Q.rk, (uint32_t)j, (uint32_t)X.u[t], x0[t], x1[t]);
+        philox2k(Q, (uint32_t)j, (uint32_t)X.u[t], x0[t], x1[t]);
         gone[t] = make_uint2(0u, 0u);
         deg[t] = X.d[t];
         if (any_own) {
@@ -1060,7 +1202,7 @@ k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ a
         if (!(i & 1)) {
 #pragma unroll
           for (int t = 0; t < kT; ++t)
-            philox2k(Q.rk, walk_ctr0(i + 1, (uint32_t)j), (uint32_t)X.u[t], x0[t], x1[t]);
+            philox2k(Q, walk_ctr0(i + 1, (uint32_t)j), (uint32_t)X.u[t], x0[t], x1[t]);
           lock_index(x0, deg, Q.key, i + 1, (uint32_t)j, X.u, idx);
         } else {
           lock_index(x1, deg, Q.key, i + 1, (uint32_t)j, X.u, idx);
@@ -1165,6 +1307,10 @@ static cudaError_t allow_lock_t() {
   set((const void *)k_lockstep<kLayout, true, 1>);
   set((const void *)k_lockstep<kLayout, false, kLockTargets>);
   set((const void *)k_lockstep<kLayout, true, kLockTargets>);
+  set((const void *)k_lockstep_group<kLayout, false, 1>);
+  set((const void *)k_lockstep_group<kLayout, true, 1>);
+  set((const void *)k_lockstep_group<kLayout, false, kLockTargets>);
+  set((const void *)k_lockstep_group<kLayout, true, kLockTargets>);
   set((const void *)k_lock_shared<kLayout, false>);
   set((const void *)k_lock_shared<kLayout, true>);
   return e;
@@ -1177,13 +1323,41 @@ cudaError_t allow_lockstep(int layout) {
 
 template <int kLayout, bool kCount>
 static void launch_lockstep(const GraphView &V, const int32_t *act, int32_t *bounds,
-                            const LockQuery &Q, bool one, int grid, cudaStream_t st) {
-  if (one)
+                            const LockQuery &Q, int shape, int grid, cudaStream_t st) {
+  if (shape == 1)
     k_lockstep<kLayout, kCount, 1><<<grid, kLockThreads, kLockSmem, st>>>(V, act, bounds, Q);
   else
     k_lockstep<kLayout, kCount, kLockTargets><<<grid, kLockThreads, kLockSmem, st>>>(V, act, bounds,
                                                                                      Q);
 }
+
+// For a group of queries.
+template <int kLayout, bool kCount>
+static void launch_group(const GraphView &V, const int32_t *act, int32_t n_act,
+                         const WalkJob *jobs, int32_t k, int32_t *counter, int shape, int grid,
+                         cudaStream_t st) {
+  if (shape == 1)
+    k_lockstep_group<kLayout, kCount, 1><<<grid, kLockThreads, kLockSmem, st>>>(V, act, n_act, jobs,
+                                                                                k, counter);
+  else
+    k_lockstep_group<kLayout, kCount, kLockTargets><<<grid, kLockThreads, kLockSmem, st>>>(
+        V, act, n_act, jobs, k, counter);
+}
+
+// Calls launch<layout, count>(...) for a graph.
+#define SRK_BY_LAYOUT(launch, ...)                                       \
+  do {                                                                   \
+    if (g->layout == kWide) {                                            \
+      if (count) launch<kWide, true>(__VA_ARGS__);                       \
+      else launch<kWide, false>(__VA_ARGS__);                            \
+    } else if (g->layout == kCsr) {                                      \
+      if (count) launch<kCsr, true>(__VA_ARGS__);                        \
+      else launch<kCsr, false>(__VA_ARGS__);                             \
+    } else {                                                             \
+      if (count) launch<kNarrow, true>(__VA_ARGS__);                     \
+      else launch<kNarrow, false>(__VA_ARGS__);                          \
+    }                                                                    \
+  } while (0)
 
 // Polls of a wait for filters: 2^20, or the environment variable SRK_WAIT_POLLS.
 static int32_t wait_polls() {
@@ -1193,34 +1367,17 @@ static int32_t wait_polls() {
   return v < 0 || v > kWaitPolls ? kWaitPolls : (int32_t)v;
 }
 
-double walk_units_work(const srk_graph *g, int shape, int32_t n_pairs, int32_t max_units) {
-  const int32_t T = kLockThreads * (shape == 1 ? 1 : kLockTargets);
-  const int32_t n_tb = (g->n_act + T - 1) / T;
-  if (n_tb == 0 || n_pairs == 0) return 0.0;
-  const int32_t chunks = lock_chunks(n_pairs, n_tb, sm_count(g->device) * kLockBlocks);
-  const double units = (double)n_tb * chunks;
-  return (double)g->n_act * n_pairs * std::min(1.0, (double)max_units / units);
-}
-
-int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
-                  const Outputs &o, bool count, cudaStream_t st, const cudaEvent_t *timing,
-                  int32_t u_begin, int32_t u_end, int shape, int32_t max_units) {
-  const int dev = g->device;
-  const int64_t nr = (int64_t)u_end - u_begin;
-  const GraphView V = view_of(g);
+static LockQuery lock_query(const QueryTab &t, const Workspace &w, const Filters &F,
+                            const Outputs &o) {
   const Small sm = small_view(w.small);
-  int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
-  unsigned long long *W = reinterpret_cast<unsigned long long *>(o.scores);
-  if (F.slots)
-    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, sm.cnt, w.rec(), w.pair_w, t.tkey,
-                                                      t.s, u_begin, u_end, W, o.counts);
   LockQuery Q;
+  memset(&Q, 0, sizeof Q);
   Q.rec = w.rec();
   Q.w = w.pair_w;
   Q.H = w.Hc;
   Q.bits = F.bits;
   Q.cnt = sm.cnt;
-  Q.W = W;
+  Q.W = reinterpret_cast<unsigned long long *>(o.scores);
   Q.counts = o.counts;
   Q.steps = o.steps;
   Q.steps_total = sm.ctr;
@@ -1228,8 +1385,30 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   for (int r = 0; r < 10; ++r) Q.rk[r] = t.tkey + (uint32_t)r * kPhiloxW0;
   Q.s = t.s;
   Q.min_cap = F.slots ? 2 : 1;
-  Q.max_units = max_units;
   Q.polls = wait_polls();
+  return Q;
+}
+
+// kLockTargets targets a thread (shape 0), or one (1) where there are too few to
+// give it several, and on the wide layout, where fewer of the targets' own
+// lists then compete for the L2 (R-MAT 24, eps = 0.05: 4.59 queries/s against
+// 4.25; R-MAT 21, 50.6 against 50.1).
+int walk_shape(const srk_graph *g, int64_t n_targets) {
+  return n_targets <= kLockThreads || g->layout == kWide ? 1 : 0;
+}
+
+int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
+                  const Outputs &o, bool count, cudaStream_t st, const cudaEvent_t *timing,
+                  int32_t u_begin, int32_t u_end) {
+  const int dev = g->device;
+  const int64_t nr = (int64_t)u_end - u_begin;
+  const GraphView V = view_of(g);
+  const Small sm = small_view(w.small);
+  int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
+  const LockQuery Q = lock_query(t, w, F, o);
+  if (F.slots)
+    k_edges<<<grid_for(g->m, 256, dev), 256, 0, st>>>(F, V, g->m, sm.cnt, w.rec(), w.pair_w, t.tkey,
+                                                      t.s, u_begin, u_end, Q.W, o.counts);
   if (timing) cudaEventRecord(timing[0], st);
   const int grid = sm_count(dev) * kLockBlocks;
   // The targets: by rank where all of them are wanted (the narrow layout ranks
@@ -1237,21 +1416,7 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   // length: the short ones all fit its shared memory, the heavy units come
   // first.  By id for a part of them.
   const int32_t *act = nr == g->n && g->layout == kNarrow ? g->order : g->act;
-  // shape 0: kLockTargets targets a thread; 1: one, where there are too few to
-  // give it several, and on the wide layout, where fewer of the targets' own
-  // lists then compete for the L2 (R-MAT 24, eps = 0.05: 4.59 queries/s against
-  // 4.25; R-MAT 21, 50.6 against 50.1)
-  const bool one = shape < 0 ? nr <= kLockThreads || g->layout == kWide : shape == 1;
-  if (g->layout == kWide) {
-    if (count) launch_lockstep<kWide, true>(V, act, bounds, Q, one, grid, st);
-    else launch_lockstep<kWide, false>(V, act, bounds, Q, one, grid, st);
-  } else if (g->layout == kCsr) {
-    if (count) launch_lockstep<kCsr, true>(V, act, bounds, Q, one, grid, st);
-    else launch_lockstep<kCsr, false>(V, act, bounds, Q, one, grid, st);
-  } else {
-    if (count) launch_lockstep<kNarrow, true>(V, act, bounds, Q, one, grid, st);
-    else launch_lockstep<kNarrow, false>(V, act, bounds, Q, one, grid, st);
-  }
+  SRK_BY_LAYOUT(launch_lockstep, V, act, bounds, Q, walk_shape(g, nr), grid, st);
   if (timing) cudaEventRecord(timing[1], st);
   if (nr > 0)
     k_finish<<<grid_for(nr, kFinishTile, dev), 256, 0, st>>>(g->row_ptr, bounds, sm.cnt, t.s,
@@ -1260,6 +1425,58 @@ int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, con
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
   return SRK_OK;
+}
+
+// Queries of more pairs x targets than this fill the GPU by themselves and are walked
+// by k_lockstep, whose query is a kernel parameter.  R-MAT 16, 16 queries: of 7e7
+// 6.05 ms with launches of their own, 5.39 ms as a group; of 4e8 29.9 and 29.9; with
+// those of 2e9 in a batch 70.0 and 73.2.
+constexpr double kAlonePairs = 5e8;
+
+WalkJob walk_job(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
+                 const Outputs &o) {
+  WalkJob J;
+  memset(&J, 0, sizeof J);
+  J.w = w;
+  J.F = F;
+  J.Q = lock_query(t, w, F, o);
+  J.z = t.z;
+  const int64_t pairs = t.L >= J.Q.min_cap ? t.N_tot - t.P[J.Q.min_cap] : 0;  // at most
+  J.alone = (double)pairs * g->n_act > kAlonePairs ? 1 : 0;
+  return J;
+}
+
+int enqueue_walk_group(const srk_graph *g, const WalkJob *host, const WalkJob *jobs, int32_t k,
+                       int32_t N, int32_t *counter, bool count, cudaStream_t st) {
+  const int dev = g->device, sms = sm_count(dev), grid = sms * kLockBlocks;
+  const GraphView V = view_of(g);
+  bool ends = false, together = false;
+  for (int32_t b = 0; b < k; ++b) {
+    ends |= host[b].F.slots != nullptr;
+    together |= host[b].alone == 0;
+  }
+  if (ends) {
+    const int rc = enqueue_ends(g, jobs, k, N, st);
+    if (rc) return rc;
+    // (a group's queries share the SMs: longer runs of edges a warp)
+    const dim3 by((unsigned)std::min(grid_for(g->m, 256, dev), std::max(8, sms * 16 / k)),
+                  (unsigned)k);
+    k_edges_group<<<by, 256, 0, st>>>(V, g->m, jobs);
+  }
+  const int32_t *act = g->layout == kNarrow ? g->order : g->act;  // (see enqueue_walks)
+  const int shape = walk_shape(g, g->n_act);
+  if (together)
+    SRK_BY_LAYOUT(launch_group, V, act, g->n_act, jobs, k, counter, shape, grid, st);
+  for (int32_t b = 0; b < k; ++b)
+    if (host[b].alone) {
+      int32_t *bounds = reinterpret_cast<int32_t *>(small_view(host[b].w.small).ctr + 2);
+      SRK_BY_LAYOUT(launch_lockstep, V, act, bounds, host[b].Q, shape, grid, st);
+    }
+  const dim3 by((unsigned)std::min(grid_for(g->n, kFinishTile, dev), std::max(4, sms * 8 / k)),
+                (unsigned)k);
+  k_finish_group<<<by, 256, 0, st>>>(g->row_ptr, g->n, g->n_act, jobs);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? SRK_OK : cuda_fail(e, "kernel launch");
 }
 
 int enqueue_shared_walks(const srk_graph *g, const SharedWalks &Q, cudaStream_t st) {

@@ -14,7 +14,7 @@
 // step of t's list.
 //
 // One cluster of 8 blocks of 1024 threads runs a query's phases with a cluster
-// barrier between them, one cluster per query of a batch.  Each phase is a few
+// barrier between them, one cluster (of 1 to 8 blocks) per query of a batch.  Each phase is a few
 // dependent reads of a few thousand threads, so it is the number of phases and
 // the price of each step from one to the next that count: as 12 kernels the
 // source side took 72 us at 2,018 walks and 139 us at 18,234, now 39 and 102 (of
@@ -41,16 +41,16 @@ struct SourceShared {
   int32_t R[SRK_MAX_LEN + 2];      // nodes of the longer pairs
 };
 
-// Phases of one query by cluster `c`, to sigma (kRows false) or to the cap rows
+// Phases of one query by cluster `c` of `blocks`, to sigma (kRows false) or to the cap rows
 // and, but for the literal shuffle, the pair records.
 template <bool kRows>
-__device__ __forceinline__ void source_phases(cg::cluster_group &c, SourceShared &S,
+__device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, SourceShared &S,
                                               const GraphView &V, const QueryTab &t,
                                               const Workspace &w, const int32_t *act,
                                               int32_t n_act, int32_t u_begin, int32_t u_end) {
   const int32_t N = t.N_tot, L = t.L;
   const int32_t tid = (int32_t)c.block_rank() * kSourceThreads + (int32_t)threadIdx.x;
-  constexpr int32_t nth = kSourceBlocks * kSourceThreads;
+  const int32_t nth = blocks * kSourceThreads;
   const Small sm = small_view(w.small);
   int32_t *head = w.grp_cnt, *next = w.rank;  // the lists of steps by k
   for (int i = threadIdx.x; i <= L + 1; i += kSourceThreads) {
@@ -200,10 +200,10 @@ __device__ __forceinline__ void source_phases(cg::cluster_group &c, SourceShared
 
 // The end nodes of a query's pairs into the table and the bitmap (cleared
 // before), room for every node's list and filter, and the pairs' places there.
-__device__ __forceinline__ void end_phases(cg::cluster_group &c, const Workspace &w,
+__device__ __forceinline__ void end_phases(cg::cluster_group &c, int blocks, const Workspace &w,
                                            const Filters &F) {
   const int32_t tid = (int32_t)c.block_rank() * kSourceThreads + (int32_t)threadIdx.x;
-  constexpr int32_t nth = kSourceBlocks * kSourceThreads;
+  const int32_t nth = blocks * kSourceThreads;
   const Small sm = small_view(w.small);
   const int32_t n1 = sm.cnt[1], n2 = sm.cnt[2];  // pairs, and those of cap 2 and more
   int4 *rec = w.rec();
@@ -257,11 +257,11 @@ __device__ __forceinline__ void end_phases(cg::cluster_group &c, const Workspace
 }
 
 // Zeros F's slots, bitmap and counters (16-byte words).
-__device__ __forceinline__ void clear_ends(cg::cluster_group &c, const Filters &F) {
+__device__ __forceinline__ void clear_ends(cg::cluster_group &c, int blocks, const Filters &F) {
   const int32_t tid = (int32_t)c.block_rank() * kSourceThreads + (int32_t)threadIdx.x;
   uint4 *p = reinterpret_cast<uint4 *>(F.slots);
   const int64_t n = ((char *)F.ctl + 256 - (char *)F.slots) / 16;
-  for (int64_t i = tid; i < n; i += kSourceBlocks * kSourceThreads) p[i] = make_uint4(0, 0, 0, 0);
+  for (int64_t i = tid; i < n; i += blocks * kSourceThreads) p[i] = make_uint4(0, 0, 0, 0);
 }
 
 __global__ void __cluster_dims__(kSourceBlocks, 1, 1) __launch_bounds__(kSourceThreads)
@@ -270,30 +270,36 @@ k_source(const __grid_constant__ GraphView V, const __grid_constant__ QueryTab t
          const int32_t *act, int32_t n_act, int32_t u_begin, int32_t u_end) {
   __shared__ SourceShared S;
   cg::cluster_group c = cg::this_cluster();
-  if (F.slots) clear_ends(c, F);
-  source_phases<true>(c, S, V, t, w, act, n_act, u_begin, u_end);
+  if (F.slots) clear_ends(c, kSourceBlocks, F);
+  source_phases<true>(c, kSourceBlocks, S, V, t, w, act, n_act, u_begin, u_end);
   if (F.slots) {
     c.sync();
-    end_phases(c, w, F);
+    end_phases(c, kSourceBlocks, w, F);
   }
 }
 
+// The queries of a batch, a cluster each.
 template <bool kRows>
-__global__ void __cluster_dims__(kSourceBlocks, 1, 1) __launch_bounds__(kSourceThreads)
+__global__ void __launch_bounds__(kSourceThreads)
 k_sources(const __grid_constant__ GraphView V, const SourceJob *__restrict__ jobs,
           const int32_t *act, int32_t n_act) {
   __shared__ SourceShared S;
   cg::cluster_group c = cg::this_cluster();
-  const SourceJob &job = jobs[blockIdx.x / kSourceBlocks];
-  source_phases<kRows>(c, S, V, *job.tab, job.w, act, n_act, 0, V.n);
+  const int blocks = (int)c.num_blocks();
+  const SourceJob &job = jobs[blockIdx.x / blocks];
+  source_phases<kRows>(c, blocks, S, V, *job.tab, job.w, act, n_act, 0, V.n);
 }
 
-__global__ void __cluster_dims__(kSourceBlocks, 1, 1) __launch_bounds__(kSourceThreads)
-k_ends(const __grid_constant__ Workspace w, const __grid_constant__ Filters F) {
+// The end nodes of a group of queries, a cluster each.
+__global__ void __launch_bounds__(kSourceThreads) k_ends(const WalkJob *__restrict__ jobs) {
   cg::cluster_group c = cg::this_cluster();
-  clear_ends(c, F);
+  const int blocks = (int)c.num_blocks();
+  const Workspace w = jobs[blockIdx.x / blocks].w;
+  const Filters F = jobs[blockIdx.x / blocks].F;
+  if (!F.slots) return;  // the whole cluster
+  clear_ends(c, blocks, F);
   c.sync();
-  end_phases(c, w, F);
+  end_phases(c, blocks, w, F);
 }
 
 // ------------------------------------------------------------ host side --
@@ -310,20 +316,47 @@ int enqueue_source(const srk_graph *g, const QueryTab &t, const Workspace &w, co
   return launched("source walks: launch");
 }
 
-int enqueue_sources(const srk_graph *g, const SourceJob *jobs, int32_t k, bool shared,
-                    cudaStream_t st) {
-  const int grid = kSourceBlocks * k;
-  if (shared)
-    k_sources<false><<<grid, kSourceThreads, 0, st>>>(view_of(g), jobs, g->act, g->n_act);
-  else
-    k_sources<true><<<grid, kSourceThreads, 0, st>>>(view_of(g), jobs, g->act, g->n_act);
-  return launched("source walks: launch");
+// Launches `kernel` with a cluster for each of k queries.  The cluster's size: the
+// queries run in rounds over the SMs (a block each), and a round takes about two
+// units of time and one for each walk of a thread.  64 queries of 435 walks take 107
+// us with clusters of 8 blocks and 30 us with clusters of 2.
+template <class... Par, class... Arg>
+static cudaError_t launch_clusters(void (*kernel)(Par...), const srk_graph *g, int32_t k, int32_t N,
+                                   cudaStream_t st, Arg... arg) {
+  const int64_t sms = sm_count(g->device);
+  int blocks = 1;
+  int64_t least = INT64_MAX;
+  for (int b = 1; b <= kSourceBlocks; b *= 2) {
+    const int64_t rounds = ((int64_t)k * b + sms - 1) / sms,
+                  time = rounds * (2 + (N + b * kSourceThreads - 1) / (b * kSourceThreads));
+    if (time <= least) {
+      least = time;
+      blocks = b;
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(blocks * k));
+  cfg.blockDim = dim3(kSourceThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)blocks;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Par(arg)...);
 }
 
-int enqueue_ends(const srk_graph *, const Workspace &w, const Filters &F, cudaStream_t st) {
-  if (!F.slots) return SRK_OK;
-  k_ends<<<kSourceBlocks, kSourceThreads, 0, st>>>(w, F);
-  return launched("end nodes: launch");
+int enqueue_sources(const srk_graph *g, const SourceJob *jobs, int32_t k, int32_t N, bool shared,
+                    cudaStream_t st) {
+  const cudaError_t e = launch_clusters(shared ? k_sources<false> : k_sources<true>, g, k, N, st,
+                                        view_of(g), jobs, (const int32_t *)g->act, g->n_act);
+  return e == cudaSuccess ? SRK_OK : cuda_fail(e, "source walks: launch");
+}
+
+int enqueue_ends(const srk_graph *g, const WalkJob *jobs, int32_t k, int32_t N, cudaStream_t st) {
+  const cudaError_t e = launch_clusters(k_ends, g, k, N, st, jobs);
+  return e == cudaSuccess ? SRK_OK : cuda_fail(e, "end nodes: launch");
 }
 
 }  // namespace srk

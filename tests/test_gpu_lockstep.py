@@ -127,3 +127,104 @@ def test_waits_for_filters_that_give_up(srk, monkeypatch, polls):
     monkeypatch.setenv("SRK_WAIT_POLLS", polls)
     for _ in range(3):
         assert_parity(gpu_query(srk, rp, col, 9, 0.5, 21, **kw), ref)
+
+
+def batch_and_singles(srk, g, n, sources, eps, seed, **kw):
+    """Dense batch outputs and the same queries one by one, as (scores, counts)."""
+    import torch
+    dev = torch.device("cuda:0")
+    k = len(sources)
+    out = [(torch.full((k, n), -3.0, dtype=torch.float64, device=dev),
+            torch.full((k, n), 7, dtype=torch.int32, device=dev)) for _ in range(2)]
+    st = srk.SrkStats()
+    srk.srk_multi_source(g, sources, 0.6, eps, seed, *out[0], stats=st, **kw)
+    steps = 0
+    for i, s in enumerate(sources):
+        one = srk.SrkStats()
+        srk.srk_single_source(g, s, 0.6, eps[i], seed, out[1][0][i], out[1][1][i], stats=one)
+        steps += one.target_steps
+    torch.cuda.synchronize()
+    return out, st.target_steps, steps
+
+
+# 256 sources to a group, one cluster of 1 to 8 blocks a source; sources of 5e8 pairs
+# x targets are walked by launches of their own beside the others of their group
+@pytest.mark.parametrize("n,k,eps", [(2, 3, [0.9]), (447, 1, [0.2]), (449, 33, [0.3, 0.1]),
+                                     (1345, 255, [0.4]), (1000, 256, [0.3]), (1000, 257, [0.3, 0.5]),
+                                     (20000, 5, [0.008, 0.3, 0.1])])
+def test_groups_of_sources(srk, n, k, eps):
+    import torch
+    rp, col = ring_lists(n, 5 if n > 5 else 1, n)
+    if n >= 1000:  # every third node loses its list: no targets, and sources that meet nobody
+        keep = np.repeat(np.arange(n) % 3 != 2, 5)
+        col = col[keep]
+        rp = np.concatenate([[0], np.cumsum(5 * (np.arange(n) % 3 != 2))]).astype(np.int32)
+    eps = [eps[i % len(eps)] for i in range(k)]
+    if n == 2:
+        eps = [0.9] * k
+    sources = [(i * 7) % n for i in range(k)]
+    kw = dict(z_override=20.0) if n == 2 else {}
+    dev = torch.device("cuda:0")
+    with srk.srk_graph_load(torch.from_numpy(rp).to(dev), torch.from_numpy(col).to(dev)) as g:
+        if n == 2:
+            out = torch.empty((k, n), dtype=torch.float64, device=dev)
+            srk.srk_multi_source(g, sources, 0.6, eps, 5, out, **kw)
+            torch.cuda.synchronize()
+            for i, s in enumerate(sources):
+                assert np.array_equal(out[i].cpu().numpy(),
+                                      oracle_query(rp, col, s, 0.9, 5, **kw).scores)
+            return
+        for kw in ({}, dict(no_graph=True)):
+            (a, b), steps, want = batch_and_singles(srk, g, n, sources, eps, 5, **kw)
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and steps == want
+        ref = oracle_query(rp, col, sources[-1], eps[-1], 5)
+        assert np.array_equal(a[0][k - 1].cpu().numpy(), ref.scores)
+
+
+@pytest.mark.parametrize("layout", ["narrow", "wide", "csr"])
+@pytest.mark.parametrize("budget", [None, 1 << 20, 3 << 20, 6 << 20])
+def test_groups_within_a_scratch_budget(srk, monkeypatch, layout, budget):
+    """Budgets that leave room for no filters, for some, and for some groups."""
+    import torch
+    from srk_inputs import rmat_in_csr
+    rp, col = rmat_in_csr(13, seed=4)
+    n = rp.size - 1
+    sources = [int(s) for s in np.argsort(-np.diff(rp), kind="stable")[:24]]
+    eps = [0.1, 0.07, 0.2] * 8
+    dev = torch.device("cuda:0")
+    if budget:
+        monkeypatch.setenv("SRK_BATCH_BYTES", str(budget))
+    with srk.srk_graph_load(torch.from_numpy(rp).to(dev), torch.from_numpy(col).to(dev),
+                            layout=layout) as g:
+        (a, b), steps, want = batch_and_singles(srk, g, n, sources, eps, 8)
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and steps == want
+
+
+def test_small_sources_of_a_batch_run_together(srk):
+    """64 queries that are small by themselves, as one batch: well below the time
+    of as many calls (0.57 to 0.63 of it when the batch ran them one by one)."""
+    import time
+
+    import torch
+    from srk_inputs import er_in_csr
+    rp, col = er_in_csr(2000, 8.0, seed=2)
+    n = rp.size - 1
+    dev = torch.device("cuda:0")
+    sources = [int(s) for s in np.flatnonzero(np.diff(rp) > 0)[:64]]
+    out = torch.empty((64, n), dtype=torch.float64, device=dev)
+
+    def best_of(f):
+        times = []
+        for _ in range(8):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            f()
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t0)
+        return min(times)
+
+    with srk.srk_graph_load(torch.from_numpy(rp).to(dev), torch.from_numpy(col).to(dev)) as g:
+        batch = best_of(lambda: srk.srk_multi_source(g, sources, 0.6, [0.1] * 64, 7, out))
+        loop = best_of(lambda: [srk.srk_single_source(g, s, 0.6, 0.1, 7, out[i])
+                                for i, s in enumerate(sources)])
+    assert batch < 0.4 * loop
