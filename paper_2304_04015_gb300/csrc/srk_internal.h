@@ -68,13 +68,24 @@ struct GraphView {
   int32_t pos_bits;
   uint32_t deg_max;
   int32_t n, n_hubs, layout;
+  int32_t far;  // the adjacency does not fit the L2
 };
 
 namespace srk {
 
+// Bytes of the adjacency that the walks read.
+inline int64_t adj_bytes(const srk_graph *g) {
+  return g->layout == 1 ? 8 * ((int64_t)g->n + g->m) : 4 * ((int64_t)(g->layout == 2 ? g->n : 0) + g->m);
+}
+// Adjacencies of more than this do not fit the L2 (129 MB in all, of which the
+// walks' other data has a part; between 72 and 143 MB nothing was measured).
+constexpr int64_t kNearBytes = 96ll << 20;
+
 inline GraphView view_of(const srk_graph *g) {
-  return GraphView{g->row_ptr, g->col,      g->adj,     g->npos, g->order,  g->hub,
-                   g->ctab,    g->pos_bits, g->deg_max, g->n,    g->n_hubs, g->layout};
+  return GraphView{g->row_ptr, g->col,    g->adj,      g->npos,
+                   g->order,   g->hub,    g->ctab,     g->pos_bits,
+                   g->deg_max, g->n,      g->n_hubs,   g->layout,
+                   adj_bytes(g) > kNearBytes ? 1 : 0};
 }
 
 // The output function of SplitMix64 (Steele, Lea, Flood, OOPSLA 2014) and

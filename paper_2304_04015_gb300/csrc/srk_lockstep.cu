@@ -696,16 +696,17 @@ k_edges_group(const __grid_constant__ GraphView V, int64_t m, const WalkJob *__r
 }
 
 // Into how many strided sets the pairs are cut, so that sets x target blocks
-// are units of equal work: up to 16 a block, of at least 128 pairs where there
-// are as many, and as near below a whole number of rounds over the grid as a
+// are units of equal work: up to `rounds_most` a block, of at least 128 pairs where
+// there are as many, and as near below a whole number of rounds over the grid as a
 // count within a quarter of the largest gets.
-__host__ __device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb,
-                                                       int32_t grid) {
+__device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb, int32_t grid,
+                                               int32_t rounds_most) {
   const int64_t per_block = (int64_t)n_pairs * n_tb / grid;
-  const int32_t rounds = per_block < 256 ? 1 : per_block < 2048 ? (int32_t)(per_block / 128) : 16;
+  const int32_t rounds = per_block < 256 ? 1 : (int32_t)min(per_block / 128, (int64_t)rounds_most);
   int32_t most = rounds * grid / n_tb;
   if (most > n_pairs) most = n_pairs;
   if (most < 1) most = 1;
+  if (rounds > 16) return most;  // the last round weighs little
   int32_t best = most;
   float fill = 0.0f;
   for (int32_t c = most, k = 0; c > 0 && c >= most - most / 4 && k < 16; --c, ++k) {
@@ -717,6 +718,23 @@ __host__ __device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t
     }
   }
   return best;
+}
+
+// Block of targets and strided set of pairs of a unit.  On a graph beyond the L2
+// units that follow one another have the same targets, and there are many sets of
+// pairs, so that the blocks at work hold few targets between them and those
+// targets' lists stay in the L2, where most first steps read them.  On the others the
+// targets run first: the narrow layout has them by rank, so the heavy units come
+// first.  With the targets first everywhere: R-MAT 22, eps = 0.05, 52.1 ms instead of
+// 46.3; wide layout, ER lists of 16, 3 queries, 2^20 nodes (143 MB) 54.6 instead of 44.2
+// (a warp per target: 44.5), 2^21 165 instead of 129 (157); 48 queries with shared
+// walks, R-MAT 24, 1535 instead of 1407 (1520).
+constexpr int kRounds = 16, kFarRounds = 256;
+__device__ __forceinline__ void split_unit(bool far, int32_t unit, int32_t n_tb, int32_t n_chunks,
+                                           int32_t &tb, int32_t &first) {
+  const int32_t by = far ? n_chunks : n_tb, q = unit / by, r = unit - q * by;
+  tb = far ? q : r;
+  first = far ? r : q;
 }
 
 // The targets act[from .. to) of a block (all but `skip`), at most kT a thread;
@@ -851,7 +869,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   const int32_t n_pairs = Q.cnt[Q.min_cap], n_t = act_hi - act_lo;
   if (n_pairs == 0 || n_t <= 0) return;
   const int32_t T = kLockThreads * kT, n_tb = (n_t + T - 1) / T;
-  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
+  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x, V.far ? kFarRounds : kRounds);
   const int64_t units = (int64_t)n_tb * n_chunks;
   if ((int64_t)blockIdx.x >= units) return;
   LockTables tabs;
@@ -866,10 +884,10 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
     if (threadIdx.x == 0) S.unit = atomicAdd(bounds, 1);
     if (threadIdx.x < 4) S.sums[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t unit = S.unit;
-    if (unit >= units) break;
-    const int32_t tb = (int32_t)(unit % n_tb);
-    const int32_t first = (int32_t)(unit / n_tb), len = (n_pairs - first + n_chunks - 1) / n_chunks;
+    if (S.unit >= units) break;
+    int32_t tb, first;
+    split_unit(V.far, S.unit, n_tb, n_chunks, tb, first);
+    const int32_t len = (n_pairs - first + n_chunks - 1) / n_chunks;
     LockTargets<kT> X;
     lock_targets(G, V.row_ptr, S, lists, act, act_lo + tb * T, act_hi, Q.s, len >= 32, X);
     lockstep_walks<kT, kCount>(G, tabs, Q, S, ring, queues, (const E *)lists, first, n_chunks, len,
@@ -888,7 +906,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
 // work goes in one round of units of up to kGroupRound pairs.  (A batch of 8
 // queries on 900 nodes, eps = 0.1: 0.190 ms with units of 4 pairs and more, 0.219 of
 // 16; 8, 16 or 32 rounds differ by less than 2 %.)
-constexpr int kGroupRounds = 16, kGroupRound = 64, kGroupPairs = 4;
+constexpr int kGroupRounds = 16, kGroupRound = 64, kFarGroupRound = 128, kGroupPairs = 4;
 template <int kLayout, bool kCount, int kT>
 __global__ void __launch_bounds__(kLockThreads, kLockBlocks)
 k_lockstep_group(const __grid_constant__ GraphView V, const int32_t *__restrict__ act, int32_t n_t,
@@ -915,8 +933,9 @@ k_lockstep_group(const __grid_constant__ GraphView V, const int32_t *__restrict_
   if (all_pairs == 0 || n_t <= 0) return;
   {
     const unsigned long long per_block = all_pairs * (unsigned)n_tb / gridDim.x;
-    const unsigned long long want = max(per_block / kGroupRounds,
-                                        min(per_block, (unsigned long long)kGroupRound));
+    const unsigned rounds = V.far ? kFarRounds : kGroupRounds;
+    const unsigned long long round = V.far ? kFarGroupRound : kGroupRound;
+    const unsigned long long want = max(per_block / rounds, min(per_block, round));
     const int32_t unit = (int32_t)max(min(want, (unsigned long long)SRK_MAX_WALKS),
                                       (unsigned long long)kGroupPairs);
     const int32_t ch = (pairs + unit - 1) / unit;
@@ -958,7 +977,9 @@ k_lockstep_group(const __grid_constant__ GraphView V, const int32_t *__restrict_
     for (int i = threadIdx.x; i < (int)(sizeof(LockQuery) / 8); i += kLockThreads)
       reinterpret_cast<uint64_t *>(&Q)[i] = reinterpret_cast<const uint64_t *>(&jobs[job].Q)[i];
     __syncthreads();
-    const int32_t n_chunks = chunks[job], tb = S.unit % n_tb, first = S.unit / n_tb;
+    const int32_t n_chunks = chunks[job];
+    int32_t tb, first;
+    split_unit(V.far, S.unit, n_tb, n_chunks, tb, first);
     const int32_t n_pairs = Q.cnt[Q.min_cap], len = (n_pairs - first + n_chunks - 1) / n_chunks;
     const bool staged = whole && Q.min_cap == 2;
     LockTargets<kT> X;
@@ -1081,7 +1102,7 @@ k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ a
   const int32_t n_pairs = Q.J - Q.j0;
   if (n_pairs <= 0 || n_act <= 0) return;
   const int32_t T = kLockThreads * kT, n_tb = (n_act + T - 1) / T;
-  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x);
+  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x, V.far ? kFarRounds : kRounds);
   const int64_t units = (int64_t)n_tb * n_chunks;
   if ((int64_t)blockIdx.x >= units) return;
   const int lane = threadIdx.x & 31;
@@ -1103,9 +1124,9 @@ k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ a
     }
     if (threadIdx.x < 4) S.sums[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t unit = S.unit;
-    if (unit >= units) break;
-    const int32_t tb = (int32_t)(unit % n_tb), first = (int32_t)(unit / n_tb);
+    if (S.unit >= units) break;
+    int32_t tb, first;
+    split_unit(V.far, S.unit, n_tb, n_chunks, tb, first);
     LockTargets<kT> X;
     lock_targets(G, V.row_ptr, S, lists, act, tb * T, n_act, -1, (n_pairs - first) / n_chunks >= 32,
                  X);
@@ -1390,11 +1411,13 @@ static LockQuery lock_query(const QueryTab &t, const Workspace &w, const Filters
 }
 
 // kLockTargets targets a thread (shape 0), or one (1) where there are too few to
-// give it several, and on the wide layout, where fewer of the targets' own
-// lists then compete for the L2 (R-MAT 24, eps = 0.05: 4.59 queries/s against
-// 4.25; R-MAT 21, 50.6 against 50.1).
+// give it several, and on the wide layout far beyond the L2, where fewer of the
+// targets' own lists then compete for it.  Wide layout, ms for 3 queries, 3 targets
+// a thread and one: 2^20 nodes with lists of 16 (143 MB) 25.1 and 32.7 (R-MAT), 44.2 and
+// 53.4 (ER); 2^21 (285 MB) 77.2 and 80.8, 138 and 133; 2^23 153 and 145, 319 and 289.
 int walk_shape(const srk_graph *g, int64_t n_targets) {
-  return n_targets <= kLockThreads || g->layout == kWide ? 1 : 0;
+  const bool far = g->layout == kWide && 8 * ((int64_t)g->n + g->m) > (256ll << 20);
+  return n_targets <= kLockThreads || far ? 1 : 0;
 }
 
 int enqueue_walks(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,

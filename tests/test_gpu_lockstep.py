@@ -228,3 +228,48 @@ def test_small_sources_of_a_batch_run_together(srk):
         loop = best_of(lambda: [srk.srk_single_source(g, s, 0.6, 0.1, 7, out[i])
                                 for i, s in enumerate(sources)])
     assert batch < 0.4 * loop
+
+
+@pytest.fixture(scope="module")
+def far_graph(srk):
+    """Lists of 13 on 2^20 nodes, with the wide layout (117 MB: beyond the L2, units of
+    one target block in a row) and the narrow one (54 MB: within it)."""
+    import torch
+    n, d = 1 << 20, 13
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(6)
+    col = torch.randint(0, n, (n * d,), generator=gen, device="cuda").to(torch.int32)
+    rp = torch.arange(0, n * d + 1, d, dtype=torch.int32, device="cuda")
+    with srk.srk_graph_load(rp, col, layout="wide") as far, \
+            srk.srk_graph_load(rp, col, layout="narrow") as near:
+        yield n, rp, col, far, near
+
+
+@pytest.mark.parametrize("lo,hi", [(0, 1 << 20), (0, (1 << 20) - 1), (5, 453), (1000, 90001)])
+def test_far_and_near_adjacency_agree(srk, far_graph, lo, hi):
+    import torch
+    n, rp, col, far, near = far_graph
+    out = []
+    for g in (far, near):
+        sc = torch.zeros(n, dtype=torch.float64, device="cuda")
+        ct, st = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(2))
+        ws = torch.zeros(n, dtype=torch.int64, device="cuda")
+        srk.srk_single_source(g, 77, 0.6, 0.12, 3, sc, ct, ws, step_counts=st, target_range=(lo, hi))
+        out.append((sc, ct, ws, st))
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(*out))
+    some = np.unique(np.linspace(lo, hi - 1, 300).astype(np.int32))
+    ref = oracle_query(rp.cpu().numpy(), col.cpu().numpy(), 77, 0.12, 3, targets=some)
+    assert np.array_equal(out[0][0].cpu().numpy()[some], ref.scores)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+def test_far_and_near_batches_agree(srk, far_graph, shared):
+    import torch
+    n, rp, col, far, near = far_graph
+    sources, eps = [1, 77, 500000], [0.2, 0.12, 0.3]
+    out = [torch.empty((3, n), dtype=torch.float64, device="cuda") for _ in range(2)]
+    for g, o in zip((far, near), out):
+        srk.srk_multi_source(g, sources, 0.6, eps, 9, o, shared_walks=shared)
+    torch.cuda.synchronize()
+    assert torch.equal(*out)
