@@ -1274,10 +1274,14 @@ size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, i
   F->rank1 = w.succ;
   // They cost a pass over the edges and save about a last step in every pair
   // and target, some hundred times less each: not for fewer than 8 pairs x
-  // targets an edge (a short target range, a tiny z).  Beyond 2^20 walks the
-  // table of end nodes would outgrow the caches.
+  // targets an edge (a short target range, a tiny z).  More than 2^20 end nodes
+  // would take a table of more than 32 MB.  (So many walks do not: 1.2e6 on R-MAT 16
+  // take 110 ms with filters, 178 without and 168 with a warp per target; 5e6 on 1,000
+  // nodes 28.3, 31.7 and 134 ms.  On fewer targets k_edges, which then has long lists of
+  // pairs for a few edges, was not measured with as many.)
   const int64_t pairs = t.L >= 1 ? t.N_tot - t.P[1] : 0;
-  if (t.literal || pairs == 0 || g->m == 0 || t.N_tot > (1 << 20) ||
+  if (t.literal || pairs == 0 || g->m == 0 || std::min<int64_t>(pairs, g->n) > (1 << 20) ||
+      (t.N_tot > (1 << 20) && n_targets < 1000) ||
       (double)pairs * (double)n_targets < 8.0 * (double)g->m)
     return 0;
   int sb = 5;
