@@ -313,7 +313,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       const size_t b = align256(plan(t1, &w, nullptr)) +
                        (d_scores ? 0 : align256(8 * n)) + (d_counts ? 0 : align256(4 * n)) +
                        (shared ? align256(8 * (size_t)t1.N_tot) : 0);
-      const size_t f = shared ? 0 : align256(filter_bytes(g, t1, g->n));
+      const size_t f = shared ? 0 : align256(filter_bytes(g, t1, walk_way(g, t1, n, true)));
       if (i1 > i0 && need + b + sb + std::max(most, f) > budget) break;
       most = std::max(most, f);
       ends.push_back(f);
@@ -437,7 +437,7 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
         const QueryTab &t = tabs[(size_t)(i0 + b)];
         Filters F;
         const size_t f = std::min(ends[(size_t)b], room - at);
-        plan_filters(g, t, S.w, g->n, f, &F, ws_base + need + at);
+        plan_filters(g, t, S.w, walk_way(g, t, n, true), f, &F, ws_base + need + at);
         at += f;
         walks.push_back(walk_job(g, t, S.w, F, Outputs{S.scores, S.counts, nullptr, nullptr}));
       }

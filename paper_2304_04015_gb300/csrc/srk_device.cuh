@@ -447,7 +447,74 @@ __device__ __forceinline__ int32_t feistel_pi(const FeistelShape &f, const Feist
 
 // All pairs of target u (list base b_u, degree deg_u > 0) walked by one warp
 // with lane refill; per-lane totals of meetings c, weight W and steps st are
-// added to the arguments (not reduced across the warp).  Pair a (index j,
+// added to the arguments (not reduced across the warp).  Pair a (index j) walks target
+// walk j, for the pairs' cap at most (a >= cnt[i + 1]: step i was its last).
+template <class GA>
+__device__ __forceinline__ void walk_target(const GA &G, const PairSet &S, uint32_t u,
+                                            int32_t b_u, uint32_t deg_u, uint32_t &c,
+                                            unsigned long long &W, uint32_t &st) {
+  int32_t next = 0;  // first unassigned pair (warp-uniform)
+  bool live = false;
+  int32_t a = 0, i = 1, b = 0;
+  uint32_t deg = 0, j = 0;
+  for (;;) {
+    const uint32_t idle = __ballot_sync(0xffffffffu, !live);
+    if (idle) {
+      if (!live) {
+        a = next + __popc(idle & lanes_below_mask());
+        if (a < S.n_pairs) {
+          live = true;
+          j = (uint32_t)S.pair_j[a];
+          i = 1;
+          b = b_u;
+          deg = deg_u;
+        }
+      }
+      next += __popc(idle);
+    }
+    if (!__any_sync(0xffffffffu, live)) break;
+    if (live) {
+      uint32_t x0, x1;
+      philox2(S.key, walk_ctr0(i, j), u, x0, x1);
+      // odd step i
+      auto e = step_entry(G, b, x0, deg, S.key, i, j, u);
+      int32_t x = entry_pos(G, e);
+      ++st;
+      const int2 r1 = S.rc[i];
+      if (x == S.Hc[r1.x + a]) {
+        ++c;
+        W += S.pair_w[a];
+        live = false;
+      } else if (a >= r1.y) {
+        live = false;  // cap reached
+      } else {
+        b = entry_next(G, e, x, deg);
+        if (deg == 0) {
+          live = false;  // no in-neighbours: the walk ends
+        } else {
+          // even step i + 1
+          e = step_entry(G, b, x1, deg, S.key, i + 1, j, u);
+          x = entry_pos(G, e);
+          ++st;
+          const int2 r2 = S.rc[i + 1];
+          if (x == S.Hc[r2.x + a]) {
+            ++c;
+            W += S.pair_w[a];
+            live = false;
+          } else if (a >= r2.y) {
+            live = false;
+          } else {
+            b = entry_next(G, e, x, deg);
+            if (deg == 0) live = false;
+            i += 2;
+          }
+        }
+      }
+    }
+  }
+}
+
+// walk_target with the literal shuffle.  Pair a (index j,
 // source length l1 stored in pair_w[a]) walks target walk t = pi_u(j) of length l2 = stratum(t),
 // walk replica t; it ends after min(l2, source cap) steps; a meeting adds
 // round(a(l1) a(l2) 2^32).  P (stratum prefix, shared memory) and a (Lemma 7

@@ -207,14 +207,19 @@ struct Filters {
   int slot_bits, bloom_bits;
   int32_t max_units;
 };
+// How the targets of a query are walked: in lockstep with end filters or without
+// (srk_lockstep.cu), or by a warp each (k_target_walks, srk_query.cu).  `batch`: a
+// source of a batch, over all targets (never by warps).
+enum class WalkWay { kFilters, kPlain, kWarps };
+WalkWay walk_way(const srk_graph *g, const QueryTab &t, int64_t n_targets, bool batch);
 // The query's end nodes and filters in `avail` bytes at `extra` (0 bytes or a
-// null pointer: none); returns the bytes taken.
-size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, int64_t n_targets,
+// null pointer: none), where its way is kFilters; returns the bytes taken.
+size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, WalkWay way,
                     size_t avail, Filters *F, char *extra);
 
 // The source side of queries (srk_source.cu).  enqueue_source: one query, steps
-// a2-a3 to the pair records (the cap rows only with the literal shuffle) and
-// the end nodes of F.  enqueue_sources: of k queries, to the pair records or,
+// a2-a3 to the pair records (with `rows` to the cap rows only) and the end nodes of
+// F.  enqueue_sources: of k queries, to the pair records or,
 // with `shared`, to sigma.  enqueue_ends: the end nodes of k of them.  N: the most
 // walks that one of the k has.
 struct SourceJob {
@@ -222,7 +227,7 @@ struct SourceJob {
   const QueryTab *tab;  // device
 };
 int enqueue_source(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
-                   int32_t u_begin, int32_t u_end, cudaStream_t st);
+                   bool rows, int32_t u_begin, int32_t u_end, cudaStream_t st);
 int enqueue_sources(const srk_graph *g, const SourceJob *jobs, int32_t k, int32_t N, bool shared,
                     cudaStream_t st);
 struct WalkJob;
@@ -241,9 +246,9 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
 int single_source(const srk_graph *g, int32_t s, double c, double eps, uint64_t seed,
                   const srk_opts *opt, double *scores, uint32_t *meet_counts,
                   uint64_t *weight_sums, void *cuda_stream, size_t extra_limit);
-// Bytes of `extra` scratch a query of n_targets targets makes use of (it does
+// Bytes of `extra` scratch a query makes use of (it does
 // with less, or none: its end nodes then have fewer filters, or none).
-size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets);
+size_t filter_bytes(const srk_graph *g, const QueryTab &t, WalkWay way);
 // What the target walks of a query need (srk_lockstep.cu).
 struct LockQuery {
   const int4 *rec;              // per pair {j, cap, first node in H, filter}

@@ -1265,25 +1265,63 @@ k_finish_rows(const SharedSrc *__restrict__ src, int32_t n) {
 // Returns the bytes taken.
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, int64_t n_targets,
+WalkWay walk_way(const srk_graph *g, const QueryTab &t, int64_t n_targets, bool batch) {
+  const int64_t pairs = t.L >= 1 ? t.N_tot - t.P[1] : 0;
+  if (t.literal || pairs == 0 || g->m == 0) return WalkWay::kPlain;
+  // Filters cost a pass over the edges and save about a last step in every pair and
+  // target.  Where they don't pay, and on some adjacencies that the caches hold less
+  // of, a warp per target is the fastest: it reads the target's list from L1 for all
+  // its first steps.  The lines, in pairs x targets with in-neighbours an edge, ms
+  // with filters, without and with warps (lists of 16, part of the targets):
+  //   R-MAT 18 narrow (16 MB)   4.9: 0.26 0.25 0.26;  13: 0.36 0.40 0.40
+  //   R-MAT 18 csr (17 MB)      1.1: 0.20 0.15 0.20;  4.9: 0.30 0.30 0.29;  13: 0.44 0.51 0.48
+  //   R-MAT 20 narrow (64 MB)   1.2: 0.45 0.27 0.29;  4.9: 0.72 0.68 0.64;  13: 1.15 1.32 1.18
+  //   ER 2^20 narrow            2.2: 0.41 0.42 0.41;  7: 0.78 1.06 0.90;  24: 2.09 3.02 2.35
+  //   R-MAT 22 narrow (268 MB)  4.5: 3.30 3.89 2.91;  12: 6.39 8.00 6.05;  36: 18.7 25.9 20.3
+  //   R-MAT 20 wide (143 MB)    13: 1.59 2.17 1.38;  39: 4.35 6.70 4.17;  78: 8.49 13.8 8.66
+  //   ER 2^20 wide              24: 3.20 5.30 2.90;  72: 8.30 14.7 7.89;  143: 15.3 28.9 15.3
+  //   R-MAT 23 wide (1.1 GB)    3: 8.59 12.6 7.67;  9: 24.8 41.7 26.0
+  //   R-MAT 20 csr (72 MB)      13: 1.56 1.91 1.40;  39: 4.23 5.78 4.17;  78: 8.37 12.3 8.59
+  //   R-MAT 22 csr (285 MB)     3: 3.68 4.41 2.50;  9: 8.83 11.3 8.05;  18: 17.5 24.1 17.0
+  const int64_t bytes = adj_bytes(g);
+  const bool small = bytes <= (48ll << 20), far = bytes > kNearBytes;
+  const double targets = (double)n_targets * (double)g->n_act / (double)g->n,
+               rate = (double)pairs * targets / (double)g->m;
+  // (a small adjacency's line was measured in targets of any kind: 1,000 nodes with
+  // lists of 16, L = 2, 126 pairs 53 us without filters, 66 with)
+  double least = 6.0;
+  if (small) least = 8.0 * (double)g->n_act / (double)g->n;
+  else if (batch) least = g->layout == kNarrow && !far ? 6.0 : 1.5;
+  else if (g->layout == kNarrow) least = far ? 16.0 : 6.0;
+  else if (g->layout == kCsr) least = far ? 1e30 : 40.0;
+  else least = bytes <= (256ll << 20) ? 75.0 : 6.0;
+  // with L = 1 the pass over the edges is all there is (R-MAT 20, 4.3: 0.11 ms, 1.15
+  // without)
+  if (t.L == 1 && !small) least = 0.5;
+  // More than 2^20 end nodes would take a table of more than 32 MB.  (So many walks do
+  // not: 1.2e6 on R-MAT 16 take 110 ms with filters, 178 without and 168 with a warp per
+  // target; 5e6 on 1,000 nodes 28.3, 31.7 and 134 ms.  On fewer targets k_edges, which
+  // then has long lists of pairs for a few edges, was not measured with as many.)
+  const bool fit = std::min<int64_t>(pairs, g->n) <= (1 << 20) &&
+                   (t.N_tot <= (1 << 20) || n_targets >= 1000);
+  if (fit && rate >= least) return WalkWay::kFilters;
+  // Fewer than 128 pairs are too few rounds for a warp's lanes, and on adjacencies that
+  // the caches do hold lockstep without filters is the faster down to few targets.
+  if (batch || pairs < 128) return WalkWay::kPlain;
+  const double few = g->layout == kNarrow ? (small ? 1e30 : far ? 0.0 : 2.0)
+                     : bytes <= (12ll << 20) ? 1e30 : small ? 3.0 : 0.0;
+  return rate < few ? WalkWay::kPlain : WalkWay::kWarps;
+}
+
+size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, WalkWay way,
                     size_t avail, Filters *F, char *base) {
   memset(F, 0, sizeof *F);
   // (arrays of the shuffle, free by then)
   F->list1 = w.items;
   F->slot_of = w.first;
   F->rank1 = w.succ;
-  // They cost a pass over the edges and save about a last step in every pair
-  // and target, some hundred times less each: not for fewer than 8 pairs x
-  // targets an edge (a short target range, a tiny z).  More than 2^20 end nodes
-  // would take a table of more than 32 MB.  (So many walks do not: 1.2e6 on R-MAT 16
-  // take 110 ms with filters, 178 without and 168 with a warp per target; 5e6 on 1,000
-  // nodes 28.3, 31.7 and 134 ms.  On fewer targets k_edges, which then has long lists of
-  // pairs for a few edges, was not measured with as many.)
-  const int64_t pairs = t.L >= 1 ? t.N_tot - t.P[1] : 0;
-  if (t.literal || pairs == 0 || g->m == 0 || std::min<int64_t>(pairs, g->n) > (1 << 20) ||
-      (t.N_tot > (1 << 20) && n_targets < 1000) ||
-      (double)pairs * (double)n_targets < 8.0 * (double)g->m)
-    return 0;
+  if (way != WalkWay::kFilters) return 0;
+  const int64_t pairs = t.N_tot - t.P[1];
   int sb = 5;
   while (((int64_t)1 << sb) < 2 * std::min<int64_t>(pairs, g->n)) ++sb;
   F->slot_bits = sb;
@@ -1304,11 +1342,11 @@ size_t plan_filters(const srk_graph *g, const QueryTab &t, const Workspace &w, i
   return fixed + unit * (size_t)F->max_units;
 }
 
-size_t filter_bytes(const srk_graph *g, const QueryTab &t, int64_t n_targets) {
+size_t filter_bytes(const srk_graph *g, const QueryTab &t, WalkWay way) {
   Filters F;
   Workspace w;
   memset(&w, 0, sizeof w);
-  return plan_filters(g, t, w, n_targets, SIZE_MAX, &F, nullptr);
+  return plan_filters(g, t, w, way, SIZE_MAX, &F, nullptr);
 }
 
 

@@ -4,7 +4,8 @@
 //   a2-a3 enqueue_source (srk_source.cu) the source's walks, their shuffle and
 //                        the walk pairs, sorted by step cap (descending)
 //   a4-a5 enqueue_walks  (srk_lockstep.cu) the targets' walks
-//       k_literal_walks  the same with the literal target shuffle, on a
+//       k_target_walks   the same by a warp per target, with the literal target
+//                        shuffle and where that is faster (walk_way), on a
 //                        step-major hit table (k_hit_table): row i holds, for
 //                        every pair that can still meet at step i, the source
 //                        walk's node at step i
@@ -52,12 +53,13 @@ k_hit_table(const __grid_constant__ QueryTab tab, GraphView V, const int32_t *__
   }
 }
 
-// ---------------------------------- steps a4-a5 with the literal shuffle --
+// -------------------------------------- steps a4-a5 by a warp per target --
 // Each warp takes targets u from a global counter.  Its 32 lanes walk the
 // target's pairs a = 0, 1, ... of the cap-sorted list; a lane whose walk ends
 // takes the next unassigned pair at once (lane refill), so walks that end
-// early (cap, meeting, no in-neighbours) do not idle the warp.  (Pairs differ
-// from target to target here, so the lockstep form has nothing to share.)
+// early (cap, meeting, no in-neighbours) do not idle the warp.  (With the literal
+// shuffle pairs differ from target to target, so the lockstep form has nothing to
+// share.)
 // Walks run on the packed adjacency.  Pair a (original index
 // j) walks from u: one Philox2x32-10 block, counter (((i-1)>>1) << 24 | j, u)
 // under the target walks' key, serves the odd step i (word 0) and the even
@@ -97,17 +99,17 @@ struct LiteralArgs {
 // 8 blocks of 256 threads per SM (32 registers): the kernel is bound by the
 // rate of scattered L1 misses, and full occupancy keeps the most misses in
 // flight.
-template <int kLayout>
+template <int kLayout, bool kLiteral>
 __global__ void __launch_bounds__(256, 8)
-k_literal_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ LiteralArgs X) {
+k_target_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ LiteralArgs X) {
   __shared__ int2 rc[SRK_MAX_LEN + 3];  // {R[i], cnt[i+1]}, one load per step
-  __shared__ int32_t Psh[SRK_MAX_LEN + 2];
+  __shared__ int32_t Psh[kLiteral ? SRK_MAX_LEN + 2 : 1];
   {
     const Small sm = small_view(const_cast<int32_t *>(A.small_base));
     for (int i = threadIdx.x; i <= A.L + 2; i += blockDim.x) {
       rc[i] = make_int2((i <= A.L + 1) ? sm.R[i] : 0,
                         (i + 1 <= A.L + 1) ? sm.cnt[i + 1] : 0);  // cnt[L+1] = cnt[L+2] = 0
-      if (i <= A.L + 1) Psh[i] = X.P[i];
+      if (kLiteral && i <= A.L + 1) Psh[i] = X.P[i];
     }
   }
   __syncthreads();
@@ -121,11 +123,12 @@ k_literal_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ Li
   S.Hc = A.Hc;
   S.n_pairs = rc[0].y;  // cnt[1]
   S.key = A.walk_key;
-  const FeistelShape fs =
-      feistel_shape(A.N_tot, ((uint64_t)A.key1 << 32) | A.key0, (uint32_t)A.s);
+  FeistelShape fs;
+  if constexpr (kLiteral)
+    fs = feistel_shape(A.N_tot, ((uint64_t)A.key1 << 32) | A.key0, (uint32_t)A.s);
   unsigned long long warp_steps = 0;
-  // the active targets act[counter .. act_hi) (k_rows set the counter to the
-  // range's first index and act_hi beside it); the outputs of the others
+  // the active targets act[counter .. act_hi) (the source side set the counter to
+  // the range's first index and act_hi beside it); the outputs of the others
   // were cleared before the launch, and s's score is 1
   if (blockIdx.x == 0 && threadIdx.x == 0 && A.s >= A.u_begin && A.s < A.u_end)
     A.scores[A.s] = 1.0;
@@ -142,9 +145,13 @@ k_literal_walks(const __grid_constant__ TargetArgs A, const __grid_constant__ Li
     unsigned long long W = 0;
     uint32_t deg_u = 0;
     const int32_t b_u = node_start(G, A.view.row_ptr, u, deg_u);
-    if (u != A.s && deg_u > 0)
-      walk_target_literal(G, S, fs, Psh, A.L, X.a, (uint32_t)u, b_u, deg_u, lanes_below, c, W,
-                          st);
+    if (u != A.s && deg_u > 0) {
+      if constexpr (kLiteral)
+        walk_target_literal(G, S, fs, Psh, A.L, X.a, (uint32_t)u, b_u, deg_u, lanes_below, c, W,
+                            st);
+      else
+        walk_target(G, S, (uint32_t)u, b_u, deg_u, c, W, st);
+    }
     for (int off = 16; off > 0; off >>= 1) {
       c += __shfl_xor_sync(0xffffffffu, c, off);
       st += __shfl_xor_sync(0xffffffffu, st, off);
@@ -205,7 +212,7 @@ static int target_grid(int device) {
   static int blocks_per_sm[64] = {};
   int b = (device >= 0 && device < 64) ? blocks_per_sm[device] : 0;
   if (!b) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_literal_walks<kNarrow>, 256, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_target_walks<kNarrow, false>, 256, 0) !=
             cudaSuccess || b < 1)
       b = 1;
     if (device >= 0 && device < 64) blocks_per_sm[device] = b;
@@ -221,8 +228,10 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
   const int dev = g->device;
   cudaError_t e = cudaSuccess;
   Filters F;
-  plan_filters(g, t, w, (int64_t)u_end - u_begin, extra ? extra_bytes : 0, &F, extra);
-  const int rc = enqueue_source(g, t, w, F, u_begin, u_end, st);
+  const WalkWay way = walk_way(g, t, (int64_t)u_end - u_begin, false);
+  const bool warps = t.literal || way == WalkWay::kWarps;
+  plan_filters(g, t, w, way, extra ? extra_bytes : 0, &F, extra);
+  const int rc = enqueue_source(g, t, w, F, warps, u_begin, u_end, st);
   if (rc) return rc;
   // targets without in-neighbours have zero outputs (and s, if it is one of
   // them, the score 1): clear the range, then walk only the active targets
@@ -231,13 +240,13 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
     e = cudaMemsetAsync(o.scores + u_begin, 0, sizeof(double) * nr, st);
     if (e == cudaSuccess && o.counts)
       e = cudaMemsetAsync(o.counts + u_begin, 0, sizeof(uint32_t) * nr, st);
-    if (e == cudaSuccess && o.wsums && t.literal)
+    if (e == cudaSuccess && o.wsums && warps)
       e = cudaMemsetAsync(o.wsums + u_begin, 0, sizeof(unsigned long long) * nr, st);
     if (e == cudaSuccess && o.steps)
       e = cudaMemsetAsync(o.steps + u_begin, 0, sizeof(uint32_t) * nr, st);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the outputs of the target range");
   }
-  if (t.literal) {
+  if (warps) {
     const GraphView V = view_of(g);
     k_hit_table<<<grid_for(t.N_tot, 256, dev), 256, 0, st>>>(t, V, w.sigma, w.seff, w.spos, w.small, w.pair_j, w.pair_w,
                                     w.Hc);
@@ -269,9 +278,16 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
     memcpy(X.a, t.a, sizeof X.a);
     if (timing) cudaEventRecord(timing[0], st);
     const int tg = target_grid(dev);
-    if (g->layout == kWide) k_literal_walks<kWide><<<tg, 256, 0, st>>>(A, X);
-    else if (g->layout == kCsr) k_literal_walks<kCsr><<<tg, 256, 0, st>>>(A, X);
-    else k_literal_walks<kNarrow><<<tg, 256, 0, st>>>(A, X);
+    if (g->layout == kWide) {
+      if (t.literal) k_target_walks<kWide, true><<<tg, 256, 0, st>>>(A, X);
+      else k_target_walks<kWide, false><<<tg, 256, 0, st>>>(A, X);
+    } else if (g->layout == kCsr) {
+      if (t.literal) k_target_walks<kCsr, true><<<tg, 256, 0, st>>>(A, X);
+      else k_target_walks<kCsr, false><<<tg, 256, 0, st>>>(A, X);
+    } else {
+      if (t.literal) k_target_walks<kNarrow, true><<<tg, 256, 0, st>>>(A, X);
+      else k_target_walks<kNarrow, false><<<tg, 256, 0, st>>>(A, X);
+    }
     if (timing) cudaEventRecord(timing[1], st);
     e = cudaGetLastError();
     return e == cudaSuccess ? SRK_OK : cuda_fail(e, "kernel launch");
@@ -367,7 +383,8 @@ int srk::single_source(const srk_graph *g, int32_t s, double c, double eps, uint
   cudaMemPool_t mp = pool(g->device);
   if (!mp) return fail(SRK_ECUDA, "cannot create the device memory pool");
   const size_t o_extra = ws;
-  size_t extra = std::min(extra_limit, filter_bytes(g, t, (int64_t)(u_end - u_begin)));
+  size_t extra =
+      std::min(extra_limit, filter_bytes(g, t, walk_way(g, t, (int64_t)u_end - u_begin, false)));
   char *base = nullptr;
   cudaError_t e = cudaMallocFromPoolAsync((void **)&base, ws + extra, mp, st);
   if (e == cudaErrorMemoryAllocation && extra > 0) {  // the query can do without filters

@@ -296,7 +296,7 @@ extern "C" int srk_server_submit(srk_server *srv, int32_t graph, int32_t s, doub
   r.tag = tag;
   r.host_scores = host_scores;
   r.bytes = bytes;
-  r.extra = filter_bytes(g, t, g->n);
+  r.extra = filter_bytes(g, t, walk_way(g, t, g->n, false));
   r.pairs = pairs;
   r.t_submit = Clock::now();
   std::lock_guard<std::mutex> lk(srv->mu);

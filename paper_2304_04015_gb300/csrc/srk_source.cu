@@ -42,10 +42,10 @@ struct SourceShared {
 };
 
 // Phases of one query by cluster `c` of `blocks`, to sigma (kRows false) or to the cap rows
-// and, but for the literal shuffle, the pair records.
+// and, unless only the `rows` are wanted, the pair records.
 template <bool kRows>
-__device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, SourceShared &S,
-                                              const GraphView &V, const QueryTab &t,
+__device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, bool rows,
+                                              SourceShared &S, const GraphView &V, const QueryTab &t,
                                               const Workspace &w, const int32_t *act,
                                               int32_t n_act, int32_t u_begin, int32_t u_end) {
   const int32_t N = t.N_tot, L = t.L;
@@ -123,7 +123,7 @@ __device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, 
   c.sync();
 
   // cnt[i]: pairs with cap >= i (longest first); R[i]: where the nodes of the
-  // pairs of cap i begin or, for the literal shuffle, row i of the hit table
+  // pairs of cap i begin or, where only the rows are wanted, row i of the hit table
   for (int i = threadIdx.x; i <= L + 1; i += kSourceThreads)
     S.cnt[i] = i >= 1 && i <= L ? sm.cap_hist[i] : 0;
   __syncthreads();
@@ -140,7 +140,7 @@ __device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, 
     S.cnt[L + 1] = 0;
     S.R[0] = 0;
     S.R[L + 1] = r;
-    if (t.literal) {
+    if (rows) {
       r = 0;
       for (int i = 1; i <= L + 1; ++i) {
         S.R[i] = r;
@@ -169,13 +169,13 @@ __device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, 
       int32_t *bounds = reinterpret_cast<int32_t *>(sm.ctr + 2);
       if (threadIdx.x == 0) {
         bounds[2] = lo;
-        bounds[0] = t.literal ? lo : 0;  // the walk kernel's counter: targets, or units
+        bounds[0] = rows ? lo : 0;  // the walk kernel's counter: targets, or units
       } else {
         bounds[1] = lo;
       }
     }
   }
-  if (t.literal) return;
+  if (rows) return;
 
   // the pair records
   int4 *rec = w.rec();
@@ -266,12 +266,12 @@ __device__ __forceinline__ void clear_ends(cg::cluster_group &c, int blocks, con
 
 __global__ void __cluster_dims__(kSourceBlocks, 1, 1) __launch_bounds__(kSourceThreads)
 k_source(const __grid_constant__ GraphView V, const __grid_constant__ QueryTab t,
-         const __grid_constant__ Workspace w, const __grid_constant__ Filters F,
+         const __grid_constant__ Workspace w, const __grid_constant__ Filters F, bool rows,
          const int32_t *act, int32_t n_act, int32_t u_begin, int32_t u_end) {
   __shared__ SourceShared S;
   cg::cluster_group c = cg::this_cluster();
   if (F.slots) clear_ends(c, kSourceBlocks, F);
-  source_phases<true>(c, kSourceBlocks, S, V, t, w, act, n_act, u_begin, u_end);
+  source_phases<true>(c, kSourceBlocks, rows, S, V, t, w, act, n_act, u_begin, u_end);
   if (F.slots) {
     c.sync();
     end_phases(c, kSourceBlocks, w, F);
@@ -287,7 +287,7 @@ k_sources(const __grid_constant__ GraphView V, const SourceJob *__restrict__ job
   cg::cluster_group c = cg::this_cluster();
   const int blocks = (int)c.num_blocks();
   const SourceJob &job = jobs[blockIdx.x / blocks];
-  source_phases<kRows>(c, blocks, S, V, *job.tab, job.w, act, n_act, 0, V.n);
+  source_phases<kRows>(c, blocks, false, S, V, *job.tab, job.w, act, n_act, 0, V.n);
 }
 
 // The end nodes of a group of queries, a cluster each.
@@ -310,9 +310,9 @@ static int launched(const char *what) {
 }
 
 int enqueue_source(const srk_graph *g, const QueryTab &t, const Workspace &w, const Filters &F,
-                   int32_t u_begin, int32_t u_end, cudaStream_t st) {
-  k_source<<<kSourceBlocks, kSourceThreads, 0, st>>>(view_of(g), t, w, F, g->act, g->n_act, u_begin,
-                                                     u_end);
+                   bool rows, int32_t u_begin, int32_t u_end, cudaStream_t st) {
+  k_source<<<kSourceBlocks, kSourceThreads, 0, st>>>(view_of(g), t, w, F, rows, g->act, g->n_act,
+                                                     u_begin, u_end);
   return launched("source walks: launch");
 }
 

@@ -273,3 +273,33 @@ def test_far_and_near_batches_agree(srk, far_graph, shared):
         srk.srk_multi_source(g, sources, 0.6, eps, 9, o, shared_walks=shared)
     torch.cuda.synchronize()
     assert torch.equal(*out)
+
+
+@pytest.mark.parametrize("z,part", [(1137.0, 1), (1137.0, 2), (1137.0, 20), (1137.0, 60), (100.0, 1),
+                                    (100.0, 7)])
+def test_ways_to_walk_agree(srk, far_graph, z, part):
+    """Lists of 13 on 2^20 nodes: as the targets get fewer the layouts go over from end
+    filters to a warp per target and to lockstep without filters, at lines of their
+    own (117, 54 and 58 MB; 68, 34, 3.4, 1.1, 6 and 0.9 pairs x targets an edge)."""
+    import torch
+    n, rp, col, far, near = far_graph
+    lo, hi = n // 9, n // 9 + (n - n // 9) // part
+    if part == 1:
+        lo, hi = 0, n
+    some = np.unique(np.linspace(lo, hi - 1, 100).astype(np.int32))
+    ref = oracle_query(rp.cpu().numpy(), col.cpu().numpy(), 77, 0.12, 3, targets=some, z_override=z)
+    with srk.srk_graph_load(rp, col, layout="csr") as csr:
+        for g in (far, near, csr):
+            sc = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+            ct, st = (torch.full((n,), 9, dtype=torch.int32, device="cuda") for _ in range(2))
+            ws = torch.full((n,), 9, dtype=torch.int64, device="cuda")
+            stats = srk.SrkStats()
+            srk.srk_single_source(g, 77, 0.6, 0.12, 3, sc, ct, ws, step_counts=st, stats=stats,
+                                  z_override=z, target_range=(lo, hi))
+            assert np.array_equal(sc.cpu().numpy()[some], ref.scores)
+            assert np.array_equal(ct.cpu().numpy()[some].view(np.uint32), ref.count)
+            assert np.array_equal(ws.cpu().numpy()[some].view(np.uint64), ref.wsum)
+            assert np.array_equal(st.cpu().numpy()[some].astype(np.uint64), ref.steps)
+            assert stats.target_steps == int(st[lo:hi].sum())
+            assert bool((sc[:lo] == -1.0).all()) and bool((sc[hi:] == -1.0).all())
+            assert bool((ct[:lo] == 9).all()) and bool((ws[hi:] == 9).all())
