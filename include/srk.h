@@ -433,7 +433,8 @@ typedef struct srk_server srk_server;
 typedef struct srk_server_report {
     uint64_t submitted, admitted, shed, completed, failed;
     uint64_t target_steps;   /* walk steps of completed requests */
-    uint64_t reserved_peak;  /* most device memory held by admitted requests */
+    uint64_t reserved_peak;  /* most device memory held by admitted requests, or, if
+                                more, by running ones with their end filters */
     double p50_ms, p99_ms, mean_ms, max_ms;
     double wall_s;           /* first submission to last completion */
     double queries_per_s;    /* completed / wall_s */

@@ -114,6 +114,7 @@ static void worker_main(srk_server *srv, int device) {
       srv->running_bytes += r.bytes;
       if (srv->reserved + srv->extra_bytes + r.extra <= srv->budget) srv->extra_bytes += r.extra;
       else r.extra = 0;
+      srv->reserved_peak = std::max(srv->reserved_peak, srv->running_bytes + srv->extra_bytes);
     }
     const srk_graph *g = srv->graphs[(size_t)r.graph];
     double *d_scores = nullptr;

@@ -90,3 +90,15 @@ def test_latency_target_admission(srk, graphs):
     assert all(adm_zero)
     assert sum(adm_busy) < len(busy)
     assert st.completed == st.admitted == sum(adm_busy) + len(zero)
+
+
+def test_reserved_peak_covers_the_filters(srk, graphs):
+    """One request at a time: the peak covers what the pool handed out for it (two
+    blocks, which the pool rounds up to 512 bytes each)."""
+    g, n = graphs[1]
+    with srk.srk_server_create([g], mem_budget=1 << 30, n_workers=1) as srv:
+        _, used, _ = srk.srk_pool_stats(0, reset_high=True)
+        assert srk.srk_server_submit(srv, 0, 3, 0.6, 0.05, 1)
+        srk.srk_server_drain(srv)
+        _, _, high = srk.srk_pool_stats(0)
+        assert 0 < high - used <= srk.srk_server_stats(srv).reserved_peak + 1024
