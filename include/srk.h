@@ -271,8 +271,8 @@ int srk_multi_source(const srk_graph *g, const int32_t *sources, int32_t k,
  *   top_count  : NULL or k int32 (device): entries filled, min(top, nnz);
  *   nnz        : NULL or k int64 (device): targets with a nonzero score.
  * The scores are exactly those of srk_multi_source (same options, including
- * SRK_OPT_SHARED_WALKS).  Sources run in chunks whose dense rows fit a
- * scratch budget (an eighth of free device memory, at most 16 GiB, or the
+ * SRK_OPT_SHARED_WALKS).  Sources run in chunks whose dense rows, with 8 KB
+ * each of selection histograms, fit a scratch budget (an eighth of free device memory, at most 16 GiB, or the
  * byte count in SRK_TOPK_ROWS_BYTES; a multiple of 64 rows when 64 or more
  * fit); with SRK_OPT_SHARED_WALKS the chunks take the sources with
  * in-neighbours by eps, descending, and the others last (sources outside

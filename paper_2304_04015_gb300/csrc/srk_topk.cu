@@ -293,7 +293,7 @@ extern "C" int srk_multi_source_topk(const srk_graph *g, const int32_t *sources,
       (top_count && !is_device_ptr(top_count)) || (nnz && !is_device_ptr(nnz)))
     return fail(SRK_EINVAL, "srk_multi_source_topk takes device output pointers");
   const int64_t n = g->n;
-  // chunk of sources whose dense rows fit the scratch budget
+  // chunk of sources whose dense rows, with their histograms, fit the scratch budget
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
   size_t budget = std::max<size_t>((size_t)64 << 20, std::min<size_t>((size_t)16 << 30, free_b / 8));
@@ -301,7 +301,7 @@ extern "C" int srk_multi_source_topk(const srk_graph *g, const int32_t *sources,
     const unsigned long long v = strtoull(env, nullptr, 10);
     if (v > 0) budget = (size_t)v;
   }
-  int32_t R = (int32_t)std::max<int64_t>(1, std::min<int64_t>(k, (int64_t)(budget / (8 * (size_t)n))));
+  int32_t R = (int32_t)std::max<int64_t>(1, std::min<int64_t>(k, (int64_t)(budget / (8 * (size_t)n + 4 * kBins))));
   if (R >= 64 && R < k) R -= R % 64;  // whole batches of shared target walks
   const int32_t n_chunks = (int32_t)((n + kChunk - 1) / kChunk);
   int P = 1;

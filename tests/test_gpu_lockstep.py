@@ -303,3 +303,38 @@ def test_ways_to_walk_agree(srk, far_graph, z, part):
             assert stats.target_steps == int(st[lo:hi].sum())
             assert bool((sc[:lo] == -1.0).all()) and bool((sc[hi:] == -1.0).all())
             assert bool((ct[:lo] == 9).all()) and bool((ws[hi:] == 9).all())
+
+
+def pool_peak(srk, f):
+    """Bytes that the library's pool handed out at most while f ran."""
+    import torch
+    torch.cuda.synchronize()
+    _, used, _ = srk.srk_pool_stats(0, reset_high=True)
+    f()
+    torch.cuda.synchronize()
+    return srk.srk_pool_stats(0)[2] - used
+
+
+def test_scratch_budgets_hold(srk, monkeypatch):
+    """SRK_BATCH_BYTES bounds the batch's scratch with its filters (the descriptors of 64
+    sources, 4 KB each, come on top), SRK_TOPK_ROWS_BYTES the top-k rows with their
+    histograms (per row some 200 bytes, and a batch of one small source, on top)."""
+    import torch
+    from srk_inputs import rmat_in_csr
+    rp, col = rmat_in_csr(13, seed=4)
+    n = rp.size - 1
+    dev = torch.device("cuda:0")
+    sources = [int(s) for s in np.argsort(-np.diff(rp), kind="stable")[:64]]
+    out = torch.empty((64, n), dtype=torch.float64, device=dev)
+    with srk.srk_graph_load(torch.from_numpy(rp).to(dev), torch.from_numpy(col).to(dev)) as g:
+        for mb in (2, 4, 16):
+            monkeypatch.setenv("SRK_BATCH_BYTES", str(mb << 20))
+            peak = pool_peak(srk, lambda: srk.srk_multi_source(g, sources, 0.6, [0.1] * 64, 7, out))
+            assert 0 < peak <= (mb << 20) + 64 * 4096 + 65536
+        monkeypatch.setenv("SRK_BATCH_BYTES", "1")
+        budget = 64 * 8 * n
+        monkeypatch.setenv("SRK_TOPK_ROWS_BYTES", str(budget))
+        o = [torch.empty((64, 10), dtype=t, device=dev) for t in (torch.int32, torch.float64)]
+        peak = pool_peak(srk, lambda: srk.srk_multi_source_topk(
+            g, sources, 0.6, [0.5] * 64, 7, 10, *o, z_override=60.0))
+        assert 0 < peak <= budget + 64 * 256 + (200 << 10)
