@@ -230,15 +230,25 @@ def variant_suffix(args):
     return ("_literal" if args.literal_shuffle else "") + ("_warmup" if args.warmup_rule else "")
 
 
+# The code that decides what the target-walk kernel reads: the kernel itself, the
+# pairs and filters it gets, and the layout of the adjacency.
+KERNEL_SOURCES = ("srk_lockstep.cu", "srk_device.cuh", "srk_internal.h", "srk_source.cu",
+                  "srk_graph.cu")
+PROFILE = os.path.join(ROOT, "profiles", "k_lockstep_rmat20_traffic.json")
+
+
+def kernel_name(args):
+    """The kernel that walks the targets of this run's queries."""
+    return "k_target_walks" if args.literal_shuffle else "k_lockstep"
+
+
 def kernel_source_sha256():
-    """sha256 over the code the target-walk kernel is compiled from and the
-    code that lays out the adjacency it reads (the kernel file, the device
-    header, the graph loader), with comments and whitespace removed, so that
+    """sha256 over KERNEL_SOURCES with comments and whitespace removed, so that
     an edit of the prose alone keeps a traffic record valid."""
     import hashlib
     import re
     h = hashlib.sha256()
-    for name in ("srk_lockstep.cu", "srk_device.cuh", "srk_graph.cu"):
+    for name in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2304_04015_gb300", "csrc", name)) as f:
             text = f.read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
@@ -247,29 +257,32 @@ def kernel_source_sha256():
     return h.hexdigest()
 
 
-def recorded_profile():
+def recorded_profile(args, layout):
     """The committed ncu record of the target-walk kernel, if it was taken on
-    the current kernel sources, else None."""
+    the current kernel sources and is of this run's kernel, adjacency layout and
+    sample rule (4-byte entries, no option), else None."""
+    if variant_suffix(args) or layout != "narrow":
+        return None
     try:
-        with open(os.path.join(ROOT, "profiles", "k_lockstep_rmat20_traffic.json")) as f:
+        with open(PROFILE) as f:
             rec = json.load(f)
         return rec if rec.get("kernel_sources_sha256") == kernel_source_sha256() else None
     except Exception:
         return None
 
 
-def recorded_traffic():
+def recorded_traffic(args, layout):
     """DRAM bytes per target-walk step of the target-walk kernel, from the
-    committed ncu summary, if it was taken on the current kernel sources."""
-    rec = recorded_profile()
+    committed ncu summary, if it applies to this run."""
+    rec = recorded_profile(args, layout)
     if rec is None:
         return None
     return float(rec["dram_bytes_per_launch"]) / float(rec["target_steps_of_launch"])
 
 
-def recorded_l2_sectors():
-    """L2 sectors requested by L1 per target-walk step (ncu, current sources)."""
-    rec = recorded_profile()
+def recorded_l2_sectors(args, layout):
+    """L2 sectors requested by L1 per target-walk step, likewise."""
+    rec = recorded_profile(args, layout)
     if rec is None or "l2_sectors_from_l1_of_launch" not in rec:
         return None
     return float(rec["l2_sectors_from_l1_of_launch"]) / float(rec["target_steps_of_launch"])
@@ -331,8 +344,8 @@ def cpu_baseline_mix(graphs_np, queries, budget_s):
 
 
 def run_batch(args, rank, world):
-    """Batched multi-source (srk_multi_source, one persistent launch per
-    batch) against the plain path (one srk_single_source per source) on the
+    """Batched multi-source (srk_multi_source, persistent launches per
+    group of sources) against the plain path (one srk_single_source per source) on the
     same sources and eps: R-MAT scale --batch-scale, 4096 sources of which a
     third have top in-degree, a third median in-degree and a third none,
     eps per source from {0.05, 0.02, 0.01}; the first --batch-sources of the
@@ -393,7 +406,8 @@ def run_batch(args, rank, world):
     peak, peak_kind = load_peaks()
     achieved = st.target_steps * BYTES_PER_STEP / t_batch / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": None, "kernel": "k_lockstep",
+                "frac": achieved / peak, "traffic": None,
+                "kernel": "k_lock_shared" if sw else "k_lockstep, k_lockstep_group",
                 "peak_kind": peak_kind + " (HBM copy)", "bytes_per_unit": BYTES_PER_STEP,
                 "unit_name": "target-walk step",
                 "note": "whole batch time (the source phases are a few percent)"}
@@ -439,7 +453,7 @@ def run_batch_topk(args, srk, torch, dev, g, rp, n, m, sources, eps, pick, t_gen
     nz = torch.empty(k, dtype=torch.int64, device=dev)
     sw = args.shared_walks
     srk.srk_multi_source_topk(g, sources[:3], C, eps[:3], QUERY_SEED, top, tn[:3], ts[:3],
-                              shared_walks=sw)   # warm-up (autotuner)
+                              shared_walks=sw)   # warm-up
     torch.cuda.synchronize()
     st = srk.SrkStats()
     ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
@@ -927,7 +941,7 @@ def main():
     kern_s = float(np.sum(k_ms)) / 1e3
     target_steps_per_s = tgt_steps / kern_s
     hbm_achieved = tgt_steps * BYTES_PER_STEP / kern_s / 1e9
-    per_step = recorded_traffic()
+    per_step = recorded_traffic(args, layout)
     launches = args.steps * n_src
     traffic = per_step * tgt_steps / launches if per_step is not None else None
     adj_b = adjacency_bytes(layout, n, m)
@@ -953,7 +967,7 @@ def main():
                           "occupancy on an array the size of the adjacency"}
     fits_l2 = adj_b <= l2_b
     hbm_frac = hbm_achieved / peak_hbm
-    common = {"kernel": "k_lockstep", "traffic": traffic,
+    common = {"kernel": kernel_name(args), "traffic": traffic,
               "traffic_unit": "DRAM bytes per launch (ncu, recorded for these kernel sources)",
               "kernel_ms_per_launch": float(np.mean(k_ms)),
               "kernel_share_of_query": float(np.sum(k_ms) / np.sum(q_ms)),
@@ -968,7 +982,7 @@ def main():
         # filter rules out read nothing (they count as steps), so the ratio is
         # taken in sectors where a capture of these sources records them, and in
         # steps (an upper bound of the reads) where none does.
-        sps = recorded_l2_sectors()
+        sps = recorded_l2_sectors(args, layout)
         rate = target_steps_per_s * (1.0 if sps is None else sps)
         roofline = {"bound": "l2_gather" if fits_l2 else "hbm_gather",
                     "achieved": rate / 1e9, "peak": l2_rate / 1e9,
@@ -1031,7 +1045,7 @@ def main():
             "roofline": roofline, "gather_roofline": gather, "cpu_baseline": base,
             "e2e": e2e, "clocks": clk,
             # k_source, k_edges, k_lockstep, k_finish; literal: k_source,
-            # k_hit_table, k_literal_walks
+            # k_hit_table, k_target_walks
             "gpu_launches": (3 if args.literal_shuffle else 4) * launches,
             "wall_s_timed_loop": t_wall, "graph_gen_s": t_gen}
     if rank == 0:
