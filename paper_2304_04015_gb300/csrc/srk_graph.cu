@@ -258,8 +258,15 @@ __global__ void k_visit_acc(const unsigned long long *__restrict__ p, int32_t n,
     acc[v] += (unsigned long long)w * p[v];
 }
 
-// Sort key of node v in the narrow layout: its degree code, descending, then
-// its visits, descending, by their leading ten bits (exponent and mantissa).
+// Sort key of a node in the narrow layout: its degree code, descending, then
+// its visits w, descending, by their leading ten bits (exponent and mantissa).
+__device__ __forceinline__ uint32_t rank_key(uint32_t code, uint32_t dmax, unsigned long long w) {
+  const int e = w ? 64 - __clzll((long long)w) : 0;  // 0..64
+  const uint32_t heat = (uint32_t)e << 9 | (e > 10 ? (uint32_t)(w >> (e - 10)) & 511u
+                                                   : (uint32_t)(w << (10 - e)) & 511u);
+  return (dmax - code) << 16 | (0xFFFFu - heat);
+}
+
 __global__ void k_rank_keys(const int32_t *__restrict__ row_ptr, int32_t n, uint32_t dmax,
                             const unsigned long long *__restrict__ vis,
                             int32_t *__restrict__ key, int32_t *__restrict__ id,
@@ -270,17 +277,91 @@ __global__ void k_rank_keys(const int32_t *__restrict__ row_ptr, int32_t n, uint
   __syncthreads();
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
     const uint32_t d = (uint32_t)(row_ptr[v + 1] - row_ptr[v]), code = d < dmax ? d : dmax;
-    const unsigned long long w = vis[v];
-    const int e = w ? 64 - __clzll((long long)w) : 0;  // 0..64
-    const uint32_t heat = (uint32_t)e << 9 | (e > 10 ? (uint32_t)(w >> (e - 10)) & 511u
-                                                     : (uint32_t)(w << (10 - e)) & 511u);
-    key[v] = (int32_t)((dmax - code) << 16 | (0xFFFFu - heat));
+    key[v] = (int32_t)rank_key(code, dmax, vis[v]);
     id[v] = (int32_t)v;
     atomicAdd(&hist[code], 1);
   }
   __syncthreads();
   for (uint32_t c = threadIdx.x; c <= dmax; c += blockDim.x)
     if (hist[c]) atomicAdd(&count[c], hist[c]);
+}
+
+// The visits, keys and order of a small graph (at most kRankNodes nodes, one block):
+// what the kernels above and the radix sort do for a large one in 27 launches, which
+// on 1,000 nodes made up a third of the load.  p, q: scratch of n words each.
+constexpr int32_t kRankNodes = 4096, kRankEdges = 65536;
+__global__ void __launch_bounds__(1024)
+k_rank_small(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int32_t n,
+             int32_t m, int32_t n_act, uint32_t dmax, const int32_t *__restrict__ owner,
+             unsigned long long *p, unsigned long long *q, int32_t *__restrict__ order,
+             int32_t *__restrict__ count) {
+  constexpr int kPer = kRankNodes / 1024;
+  __shared__ unsigned long long s[kRankNodes];  // key << 32 | id
+  const int t = threadIdx.x;
+  unsigned long long acc[kPer];
+  uint32_t deg[kPer];
+  const unsigned long long unit = (1ull << 40) / (unsigned long long)(n_act > 0 ? n_act : 1);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int32_t v = t + 1024 * k;
+    acc[k] = 0;
+    deg[k] = v < n ? (uint32_t)(row_ptr[v + 1] - row_ptr[v]) : 0u;
+    if (v < n) p[v] = deg[k] ? unit : 0ull;
+  }
+  for (uint32_t c = t; c <= dmax; c += 1024) count[c] = 0;
+#pragma unroll 1
+  for (int step = 0; step < 3; ++step) {
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int32_t v = t + 1024 * k;
+      if (v < n) {
+        if (deg[k] > 1) p[v] /= (unsigned long long)deg[k];
+        q[v] = 0ull;
+      }
+    }
+    __syncthreads();
+    for (int32_t e = t; e < m; e += 1024) {
+      const unsigned long long share = p[owner[e]];
+      if (share) atomicAdd(&q[col[e]], share);
+    }
+    __syncthreads();
+    const unsigned long long w = step == 0 ? 25ull : step == 1 ? 15ull : 9ull;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int32_t v = t + 1024 * k;
+      if (v < n) acc[k] += w * q[v];
+    }
+    unsigned long long *const x = p;
+    p = q;
+    q = x;
+  }
+  int32_t size = 2;  // of the sort
+  while (size < n) size <<= 1;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int32_t v = t + 1024 * k;
+    if (v < n) {
+      const uint32_t code = deg[k] < dmax ? deg[k] : dmax;
+      s[v] = (unsigned long long)rank_key(code, dmax, acc[k]) << 32 | (uint32_t)v;
+      atomicAdd(&count[code], 1);
+    } else if (v < size) {
+      s[v] = ~0ull;
+    }
+  }
+  for (int32_t run = 2; run <= size; run <<= 1)
+    for (int32_t d = run >> 1; d > 0; d >>= 1) {
+      __syncthreads();
+      for (int32_t i = t; i < size / 2; i += 1024) {
+        const int32_t a = 2 * i - (i & (d - 1)), b = a + d;  // bit d of a is clear
+        const unsigned long long x = s[a], y = s[b];
+        if ((x > y) == ((a & run) == 0)) {
+          s[a] = y;
+          s[b] = x;
+        }
+      }
+    }
+  __syncthreads();
+  for (int32_t i = t; i < n; i += 1024) order[i] = (int32_t)(uint32_t)s[i];
 }
 
 // npos of the ranked nodes; the hubs' degrees by rank.
@@ -468,24 +549,27 @@ static int build_narrow(srk_graph *g, int dev) {
   int32_t *owner = (int32_t *)at, *sort_tmp = (int32_t *)(at + mb),
           *count = (int32_t *)(at + mb + sort_b);
   const int bn = sm_count(dev) * 4, bm = sm_count(dev) * 8;
-  cudaMemsetAsync(acc, 0, 8 * (size_t)n, 0);
-  cudaMemsetAsync(count, 0, sizeof(int32_t) * ((size_t)dmax + 1), 0);
   if (m > 0) k_owners<<<bm, 256>>>(g->row_ptr, n, owner);
-  k_visit_init<<<bn, 256>>>(g->row_ptr, n, g->n_act, p);
-  const unsigned int w[3] = {25u, 15u, 9u};
-  for (int k = 0; k < 3; ++k) {
-    cudaMemsetAsync(q, 0, 8 * (size_t)n, 0);
-    k_visit_share<<<bn, 256>>>(g->row_ptr, n, p);
-    if (m > 0) k_visit_step<<<bm, 256>>>(owner, g->col, m, p, q);
-    k_visit_acc<<<bn, 256>>>(q, n, w[k], acc);
-    std::swap(p, q);
+  const int32_t *order = vA;
+  if (n <= kRankNodes && m <= kRankEdges) {
+    k_rank_small<<<1, 1024>>>(g->row_ptr, g->col, n, (int32_t)m, g->n_act, dmax, owner, p, q, vA,
+                              count);
+  } else {
+    cudaMemsetAsync(acc, 0, 8 * (size_t)n, 0);
+    cudaMemsetAsync(count, 0, sizeof(int32_t) * ((size_t)dmax + 1), 0);
+    k_visit_init<<<bn, 256>>>(g->row_ptr, n, g->n_act, p);
+    const unsigned int w[3] = {25u, 15u, 9u};
+    for (int k = 0; k < 3; ++k) {
+      cudaMemsetAsync(q, 0, 8 * (size_t)n, 0);
+      k_visit_share<<<bn, 256>>>(g->row_ptr, n, p);
+      if (m > 0) k_visit_step<<<bm, 256>>>(owner, g->col, m, p, q);
+      k_visit_acc<<<bn, 256>>>(q, n, w[k], acc);
+      std::swap(p, q);
+    }
+    k_rank_keys<<<bn, 256, sizeof(int32_t) * ((size_t)dmax + 1)>>>(g->row_ptr, n, dmax, acc, kA,
+                                                                   vA, count);
+    if (radix_sort(kA, vA, kB, vB, n, 16 + std::min(32 - pb, kCodeBits), sort_tmp, 0)) order = vB;
   }
-  k_rank_keys<<<bn, 256, sizeof(int32_t) * ((size_t)dmax + 1)>>>(g->row_ptr, n, dmax, acc, kA, vA,
-                                                                 count);
-  const int32_t *order = radix_sort(kA, vA, kB, vB, n, 16 + std::min(32 - pb, kCodeBits), sort_tmp,
-                                    0)
-                             ? vB
-                             : vA;
   // list starts by degree, from the number of nodes of each code
   std::vector<int32_t> cnt((size_t)dmax + 1);
   e = cudaMemcpy(cnt.data(), count, sizeof(int32_t) * cnt.size(), cudaMemcpyDeviceToHost);

@@ -338,3 +338,18 @@ def test_scratch_budgets_hold(srk, monkeypatch):
         peak = pool_peak(srk, lambda: srk.srk_multi_source_topk(
             g, sources, 0.6, [0.5] * 64, 7, 10, *o, z_override=60.0))
         assert 0 < peak <= budget + 64 * 256 + (200 << 10)
+
+
+@pytest.mark.parametrize("n,d", [(1, 1), (3, 2), (1024, 5), (1025, 40), (4095, 16), (4096, 16),
+                                 (4096, 17), (4097, 3)])
+def test_graphs_ranked_by_one_block(srk, n, d):
+    """At most 4,096 nodes and 65,536 edges; lists of 0, d or 2 d entries."""
+    rng = np.random.default_rng(n + d)
+    deg = np.array([0, d, 2 * d])[rng.integers(0, 3, size=n)] if n > 3 else np.full(n, d)
+    if (n, d) in ((4096, 16), (4096, 17)):
+        deg = np.full(n, d)
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
+    col = rng.integers(0, n, size=int(rp[-1])).astype(np.int32)
+    s = int(np.flatnonzero(deg)[0])
+    kw = dict(z_override=300.0, L_override=10)
+    assert_parity(gpu_query(srk, rp, col, s, 0.5, 3, **kw), oracle_query(rp, col, s, 0.5, 3, **kw))
