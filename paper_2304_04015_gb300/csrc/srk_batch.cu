@@ -41,8 +41,6 @@ struct BatchArgs {
   int32_t k;
   int64_t total_walks;
   GraphView view;
-  uint32_t key0, key1;
-  uint32_t shared_key;  // walk key of the shared target walks
   uint2 *M;       // shared walks: M[j (Lmax + 1) + i - 1] bit b = pair j of batch source b
                   // may still meet at step i (cap_b(j) >= i)
   uint32_t *sig;  // shared walks: 32 words per meeting table, bit sig_bit(node) set for
@@ -55,7 +53,6 @@ struct BatchArgs {
                   // linear probing from slot_of(node)
   const int64_t *rowbase;  // shared walks: rowbase[i] = tables before step i - Pmin_i
   int32_t tbits;  // shared walks: log2 of the slots per table (>= 2 k)
-  int32_t Jmax;   // shared walks: the largest N_tot of the batch
   int32_t Lmax;   // shared walks: the largest L of the batch
 };
 
@@ -414,18 +411,18 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       BatchSrc &S = hsrc[(size_t)b];
       char *wb = ws_base + ws_off[(size_t)b];
       const size_t core = align256(plan(t, &S.w, wb));
-      char *extra = wb + core;
+      char *outs = wb + core;
       S.tab = d_tab + b;
       const size_t row = (size_t)row_of[(size_t)(i0 + b)];
-      S.scores = d_scores ? scores + row * n : (double *)extra;
-      if (!d_scores) extra += align256(8 * n);
+      S.scores = d_scores ? scores + row * n : (double *)outs;
+      if (!d_scores) outs += align256(8 * n);
       S.counts = !meet_counts ? nullptr
-                 : (d_counts ? meet_counts + row * n : (uint32_t *)extra);
-      if (meet_counts && !d_counts) extra += align256(4 * n);
+                 : (d_counts ? meet_counts + row * n : (uint32_t *)outs);
+      if (meet_counts && !d_counts) outs += align256(4 * n);
       S.wj = nullptr;
       if (shared) {
-        S.wj = (unsigned long long *)extra;
-        extra += align256(8 * (size_t)t.N_tot);
+        S.wj = (unsigned long long *)outs;
+        outs += align256(8 * (size_t)t.N_tot);
       }
       S.s = t.s;
       S.L = t.L;
@@ -481,16 +478,12 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
     A.k = kb;
     A.total_walks = hoff[(size_t)kb];
     A.view = view_of(g);
-    A.key0 = (uint32_t)seed;
-    A.key1 = (uint32_t)(seed >> 32);
-    A.shared_key = walk_key(seed, kSharedWalkKey);
     A.M = d_M;
     A.sig = d_sig;
     A.T = d_T;
     A.rowbase = d_rowbase;
     A.tbits = tbits;
     A.Lmax = Lmax;
-    A.Jmax = Jmax;
     const int gw = (int)std::max<int64_t>(1, std::min<int64_t>((A.total_walks + 255) / 256,
                                                                 (int64_t)sms * 8));
     auto enqueue_source_side = [&](cudaStream_t s2) {
@@ -521,8 +514,8 @@ extern "C" int srk_multi_source(const srk_graph *g, const int32_t *sources,
       SW.j0 = j0;
       SW.J = Jmax;
       SW.Lmax = Lmax;
-      SW.key = A.shared_key;
-      for (int r = 0; r < 10; ++r) SW.rk[r] = A.shared_key + (uint32_t)r * kPhiloxW0;
+      SW.key = walk_key(seed, kSharedWalkKey);
+      for (int r = 0; r < 10; ++r) SW.rk[r] = SW.key + (uint32_t)r * kPhiloxW0;
       SW.steps = count ? d_ctr + 1 : nullptr;
       SW.counter = reinterpret_cast<int32_t *>(d_ctr);
     }

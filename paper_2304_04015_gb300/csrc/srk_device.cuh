@@ -133,10 +133,10 @@ __device__ __forceinline__ int stratum_of(const int32_t *P, int L, int32_t r) {
 namespace srk {
 
 // Control block of one query (int32 words): cap histogram, row sizes cnt[i]
-// (pairs with cap >= i), hit-table row offsets R[i], per-cap cursors, then
-// four uint64 slots: [0] target steps, [1] source steps, [2] the target
-// kernel's work counter (low word; the batched path's item counter uses the
-// whole slot) and the end of its active-target range (high word), [3] spare.
+// (pairs with cap >= i), row offsets R[i] (source_phases), per-cap cursors, then
+// four uint64 slots: [0] target steps, [1] source steps, [2] the walk kernel's
+// work counter (low word) and the end of its active-target range (high word), [3]
+// the beginning of that range (low word).
 constexpr int kRowWords = SRK_MAX_LEN + 2;
 constexpr int kSmallWords = 4 * kRowWords;
 constexpr int kSmallBytes = 4 * kSmallWords + 32;

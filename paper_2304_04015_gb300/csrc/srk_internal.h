@@ -167,12 +167,12 @@ int sm_count(int device);
 
 // Scratch of one query, carved from one device block (srk_query.cu).
 struct Workspace {
-  int32_t *spos, *seff, *kdraw, *grp_cnt, *rank, *grp_off, *items, *first,
-      *succ, *sigma, *pair_j, *Hc, *small;
+  // the shuffle's draws, and its lists of steps by draw, are in the room of the pair
+  // records, which are made after it
+  int32_t *spos, *seff, *kdraw, *head, *next, *items, *first, *succ, *sigma, *pair_j, *Hc, *small;
   unsigned long long *pair_w;
   size_t bytes;
-  // the pair records {j, cap, first node in Hc, filter}, longest pairs first:
-  // 16 bytes a pair in kdraw to grp_off, which the shuffle no longer needs then
+  // the pair records {j, cap, first node in Hc, filter}, longest pairs first
   __host__ __device__ int4 *rec() const { return reinterpret_cast<int4 *>(kdraw); }
 };
 

@@ -30,10 +30,10 @@
 // R-MAT 20, eps = 0.02 (10,941 pairs, 546,406 targets): 1.17 sectors a pair
 // and target and 104 warp instructions per pair and 32 targets (2.0 and 189
 // with a warp per target), 2.4e11 sectors per second, 54 % of the issue slots.
-// One query 29.2 ms instead of 42.3 ms; R-MAT 16 2.10 ms instead of 2.57 ms;
-// 100,003 nodes with uniform lists of 12, eps = 0.03, 1.97 ms instead of 2.92
+// One query 29.0 ms instead of 42.4 ms; R-MAT 16 1.99 ms instead of 2.56 ms;
+// 100,003 nodes with uniform lists of 12, eps = 0.03, 1.98 ms instead of 2.95
 // ms; R-MAT 22 at eps = 0.05, bound by DRAM (64 bytes fetched per missing
-// sector), 49-55 ms instead of 55-62 ms.
+// sector), 46-48 ms instead of 61-62 ms.
 //
 // Launch shape: 2 blocks of 448 threads per SM, 3 targets a thread (72
 // registers).  Measured at R-MAT 20 in an earlier state of the kernel: 1 target
@@ -650,6 +650,8 @@ __device__ __forceinline__ void walk_edges(const Filters &F, const GraphView &V,
       }
       const bool todo = S.cnt1 > 0 && u >= u_begin && u < u_end && u != s;
       // a few pairs: each lane decides its edge's; many: the warp's lanes share them
+      // (3 queries with L = 1, ER lists of 16 on 100,003 nodes: 0.167 ms when more than
+      // one pair is shared, 0.162 from 9 on, 0.229 from 65 on)
       uint32_t c = 0;
       unsigned long long ws = 0;
       if (todo && S.cnt1 <= 8)
@@ -1078,7 +1080,8 @@ k_finish_group(const int32_t *row_ptr, int32_t n, int32_t n_t, const WalkJob *__
 // wide layout, whose lists take twice the room and whose targets come by id,
 // wants fewer lists in the L2 between two of their first steps: 48 sources on
 // R-MAT 21 and 24, 378 and 33.1 queries/s with 2 targets a thread, 372 and 32.3
-// with 3, 357 and 33.1 with 1.
+// with 3, 357 and 33.1 with 1 (with the targets first; in split_unit's order for
+// graphs beyond the L2 2 targets a thread give 437 and 34.1).
 constexpr int kSharedTargets = 3;  // per thread, at most
 constexpr int shared_targets(int layout) { return layout == kWide ? 2 : kSharedTargets; }
 

@@ -71,7 +71,7 @@ k_hit_table(const __grid_constant__ QueryTab tab, GraphView V, const int32_t *__
 // (s~(s,s) = 1).
 struct TargetArgs {
   GraphView view;
-  int32_t n, s, L;
+  int32_t s, L;
   uint32_t walk_key;       // walk key of the target walks (the source's or the shared one)
   uint32_t key0, key1;
   double z;
@@ -186,10 +186,9 @@ size_t plan(const QueryTab &t, Workspace *w, char *base) {
   };
   w->spos = (int32_t *)take(4 * N * Ls);
   w->seff = (int32_t *)take(4 * N);
-  w->kdraw = (int32_t *)take(4 * N);
-  w->grp_cnt = (int32_t *)take(4 * N);
-  w->rank = (int32_t *)take(4 * N);
-  w->grp_off = (int32_t *)take(4 * (N + 1));
+  w->kdraw = (int32_t *)take(sizeof(int4) * N);  // the pair records
+  w->head = w->kdraw + N;
+  w->next = w->kdraw + 2 * N;
   w->items = (int32_t *)take(4 * N);
   w->first = (int32_t *)take(4 * N);
   w->succ = (int32_t *)take(4 * N);
@@ -252,7 +251,6 @@ int enqueue_query(const srk_graph *g, const QueryTab &t, const Workspace &w,
                                     w.Hc);
     TargetArgs A;
     A.view = V;
-    A.n = g->n;
     A.s = t.s;
     A.walk_key = t.tkey;
     A.L = t.L;

@@ -52,7 +52,7 @@ __device__ __forceinline__ void source_phases(cg::cluster_group &c, int blocks, 
   const int32_t tid = (int32_t)c.block_rank() * kSourceThreads + (int32_t)threadIdx.x;
   const int32_t nth = blocks * kSourceThreads;
   const Small sm = small_view(w.small);
-  int32_t *head = w.grp_cnt, *next = w.rank;  // the lists of steps by k
+  int32_t *const head = w.head, *const next = w.next;  // the lists of steps by k
   for (int i = threadIdx.x; i <= L + 1; i += kSourceThreads) {
     S.P[i] = t.P[i];
     S.hist[i] = 0;
