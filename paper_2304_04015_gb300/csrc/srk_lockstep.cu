@@ -688,8 +688,9 @@ k_edges(const __grid_constant__ Filters F, const __grid_constant__ GraphView V, 
   walk_edges(F, V, m, cnt, rec, pair_w, key, s, u_begin, u_end, W, counts);
 }
 
-// For a group of queries (blockIdx.y: the query).
-__global__ void __launch_bounds__(256)
+// For a group of queries (blockIdx.y: the query).  (5 blocks an SM, 48 registers: 62 as
+// the compiler takes them leave 3 to 4, and cost 2 to 4 % of a batch on 2,000 nodes.)
+__global__ void __launch_bounds__(256, 5)
 k_edges_group(const __grid_constant__ GraphView V, int64_t m, const WalkJob *__restrict__ jobs) {
   const WalkJob &J = jobs[blockIdx.y];
   const Filters F = J.F;
@@ -698,17 +699,22 @@ k_edges_group(const __grid_constant__ GraphView V, int64_t m, const WalkJob *__r
 }
 
 // Into how many strided sets the pairs are cut, so that sets x target blocks
-// are units of equal work: up to `rounds_most` a block, of at least 128 pairs where
-// there are as many, and as near below a whole number of rounds over the grid as a
-// count within a quarter of the largest gets.
+// are units of equal work: up to 16 a block, of at least 128 pairs where there are as
+// many, and as near below a whole number of rounds over the grid as a count within
+// a quarter of the largest gets; on a graph beyond the L2 up to 1,024 a block, of at
+// least 32 pairs (see split_unit).
+constexpr int kRounds = 16, kUnitPairs = 128, kFarRounds = 1024, kFarUnitPairs = 32;
 __device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb, int32_t grid,
-                                               int32_t rounds_most) {
+                                               bool far) {
   const int64_t per_block = (int64_t)n_pairs * n_tb / grid;
-  const int32_t rounds = per_block < 256 ? 1 : (int32_t)min(per_block / 128, (int64_t)rounds_most);
+  const int32_t least = far ? kFarUnitPairs : kUnitPairs;
+  const int32_t rounds = per_block < 2 * least
+                             ? 1
+                             : (int32_t)min(per_block / least, (int64_t)(far ? kFarRounds : kRounds));
   int32_t most = rounds * grid / n_tb;
   if (most > n_pairs) most = n_pairs;
   if (most < 1) most = 1;
-  if (rounds > 16) return most;  // the last round weighs little
+  if (rounds > kRounds) return most;  // the last round weighs little
   int32_t best = most;
   float fill = 0.0f;
   for (int32_t c = most, k = 0; c > 0 && c >= most - most / 4 && k < 16; --c, ++k) {
@@ -727,11 +733,11 @@ __device__ __forceinline__ int32_t lock_chunks(int32_t n_pairs, int32_t n_tb, in
 // pairs, so that the blocks at work hold few targets between them and those
 // targets' lists stay in the L2, where most first steps read them.  On the others the
 // targets run first: the narrow layout has them by rank, so the heavy units come
-// first.  With the targets first everywhere: R-MAT 22, eps = 0.05, 52.1 ms instead of
-// 46.3; wide layout, ER lists of 16, 3 queries, 2^20 nodes (143 MB) 54.6 instead of 44.2
-// (a warp per target: 44.5), 2^21 165 instead of 129 (157); 48 queries with shared
-// walks, R-MAT 24, 1535 instead of 1407 (1520).
-constexpr int kRounds = 16, kFarRounds = 256;
+// first.  With the targets first everywhere: wide layout, ER lists of 16, 3 queries,
+// 2^20 nodes (143 MB) 54.6 ms, 2^21 165; 48 queries with shared walks, R-MAT 24, 1535.  So,
+// with sets of 128 pairs, 44.2 (a warp per target: 44.5), 129 (157) and 1407 (1520).
+// Sets of 128, 64 and 32 pairs, one query: R-MAT 22, eps = 0.05, 35.4, 33.9 and 32.8 ms
+// (43.8); ER 2^22, eps = 0.1, 29.3, 27.5 and 26.1 (31.3), on the CSR 40.7, 38.9 and 37.8 (39.6).
 __device__ __forceinline__ void split_unit(bool far, int32_t unit, int32_t n_tb, int32_t n_chunks,
                                            int32_t &tb, int32_t &first) {
   const int32_t by = far ? n_chunks : n_tb, q = unit / by, r = unit - q * by;
@@ -871,7 +877,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
   const int32_t n_pairs = Q.cnt[Q.min_cap], n_t = act_hi - act_lo;
   if (n_pairs == 0 || n_t <= 0) return;
   const int32_t T = kLockThreads * kT, n_tb = (n_t + T - 1) / T;
-  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x, V.far ? kFarRounds : kRounds);
+  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x, V.far != 0);
   const int64_t units = (int64_t)n_tb * n_chunks;
   if ((int64_t)blockIdx.x >= units) return;
   LockTables tabs;
@@ -908,7 +914,7 @@ k_lockstep(const __grid_constant__ GraphView V, const int32_t *__restrict__ act,
 // work goes in one round of units of up to kGroupRound pairs.  (A batch of 8
 // queries on 900 nodes, eps = 0.1: 0.190 ms with units of 4 pairs and more, 0.219 of
 // 16; 8, 16 or 32 rounds differ by less than 2 %.)
-constexpr int kGroupRounds = 16, kGroupRound = 64, kFarGroupRound = 128, kGroupPairs = 4;
+constexpr int kGroupRounds = 16, kGroupRound = 64, kGroupPairs = 4;
 template <int kLayout, bool kCount, int kT>
 __global__ void __launch_bounds__(kLockThreads, kLockBlocks)
 k_lockstep_group(const __grid_constant__ GraphView V, const int32_t *__restrict__ act, int32_t n_t,
@@ -936,7 +942,7 @@ k_lockstep_group(const __grid_constant__ GraphView V, const int32_t *__restrict_
   {
     const unsigned long long per_block = all_pairs * (unsigned)n_tb / gridDim.x;
     const unsigned rounds = V.far ? kFarRounds : kGroupRounds;
-    const unsigned long long round = V.far ? kFarGroupRound : kGroupRound;
+    const unsigned long long round = V.far ? kFarUnitPairs : kGroupRound;
     const unsigned long long want = max(per_block / rounds, min(per_block, round));
     const int32_t unit = (int32_t)max(min(want, (unsigned long long)SRK_MAX_WALKS),
                                       (unsigned long long)kGroupPairs);
@@ -1105,7 +1111,7 @@ k_lock_shared(const __grid_constant__ GraphView V, const int32_t *__restrict__ a
   const int32_t n_pairs = Q.J - Q.j0;
   if (n_pairs <= 0 || n_act <= 0) return;
   const int32_t T = kLockThreads * kT, n_tb = (n_act + T - 1) / T;
-  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x, V.far ? kFarRounds : kRounds);
+  const int32_t n_chunks = lock_chunks(n_pairs, n_tb, gridDim.x, V.far != 0);
   const int64_t units = (int64_t)n_tb * n_chunks;
   if ((int64_t)blockIdx.x >= units) return;
   const int lane = threadIdx.x & 31;
@@ -1280,12 +1286,16 @@ WalkWay walk_way(const srk_graph *g, const QueryTab &t, int64_t n_targets, bool 
   //   R-MAT 18 csr (17 MB)      1.1: 0.20 0.15 0.20;  4.9: 0.30 0.30 0.29;  13: 0.44 0.51 0.48
   //   R-MAT 20 narrow (64 MB)   1.2: 0.45 0.27 0.29;  4.9: 0.72 0.68 0.64;  13: 1.15 1.32 1.18
   //   ER 2^20 narrow            2.2: 0.41 0.42 0.41;  7: 0.78 1.06 0.90;  24: 2.09 3.02 2.35
-  //   R-MAT 22 narrow (268 MB)  4.5: 3.30 3.89 2.91;  12: 6.39 8.00 6.05;  36: 18.7 25.9 20.3
-  //   R-MAT 20 wide (143 MB)    13: 1.59 2.17 1.38;  39: 4.35 6.70 4.17;  78: 8.49 13.8 8.66
-  //   ER 2^20 wide              24: 3.20 5.30 2.90;  72: 8.30 14.7 7.89;  143: 15.3 28.9 15.3
-  //   R-MAT 23 wide (1.1 GB)    3: 8.59 12.6 7.67;  9: 24.8 41.7 26.0
+  //   R-MAT 22 narrow (268 MB)  1.1: 1.39 1.11 0.94;  3: 3.08 - 2.32;  12: 5.28 8.00 6.08
+  //   ER 2^22 narrow            0.6: - 1.01 0.71;  6.8: 4.95 8.40 5.39;  20: 13.6 23.9 15.8
+  //   R-MAT 20 wide (143 MB)    13: 1.58 2.17 1.38;  39: 3.88 6.70 4.19;  78: 7.79 13.8 8.70
+  //   ER 2^20 wide              2.2: 0.52 0.66 0.48;  24: 2.61 5.30 2.86;  72: 7.06 14.7 7.79
+  //   R-MAT 23 wide (1.1 GB)    3: 7.94 12.6 7.66;  9: 24.2 41.7 26.0
+  //   ER 2^23 wide              7: 15.0 30.0 18.4
   //   R-MAT 20 csr (72 MB)      13: 1.56 1.91 1.40;  39: 4.23 5.78 4.17;  78: 8.37 12.3 8.59
-  //   R-MAT 22 csr (285 MB)     3: 3.68 4.41 2.50;  9: 8.83 11.3 8.05;  18: 17.5 24.1 17.0
+  //   R-MAT on 1.7e6 csr (102 MB)  71: 16.8 - 15.7;  ER on 1.5e6 csr (97 MB)  143: 27.8 - 29.0
+  //   R-MAT 22 csr (285 MB)     3: 3.71 4.41 2.55;  9: 8.09 11.3 8.16;  18: 16.5 24.1 17.2
+  //   ER 2^22 csr               6.8: 6.84 10.8 6.86;  20: 19.2 31.7 20.0
   const int64_t bytes = adj_bytes(g);
   const bool small = bytes <= (48ll << 20), far = bytes > kNearBytes;
   const double targets = (double)n_targets * (double)g->n_act / (double)g->n,
@@ -1295,9 +1305,9 @@ WalkWay walk_way(const srk_graph *g, const QueryTab &t, int64_t n_targets, bool 
   double least = 6.0;
   if (small) least = 8.0 * (double)g->n_act / (double)g->n;
   else if (batch) least = g->layout == kNarrow && !far ? 6.0 : 1.5;
-  else if (g->layout == kNarrow) least = far ? 16.0 : 6.0;
-  else if (g->layout == kCsr) least = far ? 1e30 : 40.0;
-  else least = bytes <= (256ll << 20) ? 75.0 : 6.0;
+  else if (g->layout == kNarrow) least = 6.0;
+  else if (g->layout == kCsr) least = !far ? 40.0 : bytes <= (200ll << 20) ? 80.0 : 9.0;
+  else least = bytes <= (256ll << 20) ? 20.0 : 6.0;
   // with L = 1 the pass over the edges is all there is (R-MAT 20, 4.3: 0.11 ms, 1.15
   // without)
   if (t.L == 1 && !small) least = 0.5;

@@ -280,7 +280,7 @@ def test_far_and_near_batches_agree(srk, far_graph, shared):
 def test_ways_to_walk_agree(srk, far_graph, z, part):
     """Lists of 13 on 2^20 nodes: as the targets get fewer the layouts go over from end
     filters to a warp per target and to lockstep without filters, at lines of their
-    own (117, 54 and 58 MB; 68, 34, 3.4, 1.1, 6 and 0.9 pairs x targets an edge)."""
+    own (117, 54 and 58 MB; 68, 30, 3, 1, 6 and 0.8 pairs x targets an edge)."""
     import torch
     n, rp, col, far, near = far_graph
     lo, hi = n // 9, n // 9 + (n - n // 9) // part
