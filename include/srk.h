@@ -84,7 +84,7 @@ extern "C" {
                                   pseudo-random, so the independence of the
                                   pairings across targets that Section 5.2
                                   has is approximated, not reproduced.  About
-                                  3.6x slower than the default pairing */
+                                  5x slower than the default pairing */
 
 #define SRK_OPT_SHARED_WALKS 8  /* target walks keyed by (node, replica) alone:
                                   walk r of target u draws its steps under the

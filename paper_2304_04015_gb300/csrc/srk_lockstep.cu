@@ -33,7 +33,7 @@
 // One query 29.0 ms instead of 42.4 ms; R-MAT 16 1.99 ms instead of 2.56 ms;
 // 100,003 nodes with uniform lists of 12, eps = 0.03, 1.98 ms instead of 2.95
 // ms; R-MAT 22 at eps = 0.05, bound by DRAM (64 bytes fetched per missing
-// sector), 46-48 ms instead of 61-62 ms.
+// sector), 41-44 ms instead of 57-62 ms.
 //
 // Launch shape: 2 blocks of 448 threads per SM, 3 targets a thread (72
 // registers).  Measured at R-MAT 20 in an earlier state of the kernel: 1 target
@@ -1087,7 +1087,7 @@ k_finish_group(const int32_t *row_ptr, int32_t n, int32_t n_t, const WalkJob *__
 // wants fewer lists in the L2 between two of their first steps: 48 sources on
 // R-MAT 21 and 24, 378 and 33.1 queries/s with 2 targets a thread, 372 and 32.3
 // with 3, 357 and 33.1 with 1 (with the targets first; in split_unit's order for
-// graphs beyond the L2 2 targets a thread give 437 and 34.1).
+// graphs beyond the L2 2 targets a thread give 435 and 34.2).
 constexpr int kSharedTargets = 3;  // per thread, at most
 constexpr int shared_targets(int layout) { return layout == kWide ? 2 : kSharedTargets; }
 
